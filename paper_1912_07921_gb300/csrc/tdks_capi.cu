@@ -215,44 +215,39 @@ void sweep_common(const tdks_system *s, SweepParams &p, const double A[3], int s
   p.do_obs = 0;
 }
 
-// Tensor map over a packed array for the TMA sweep of `mode` (box depth = planes per copy).
-bool encode_map(const tdks_system *s, const void *ptr, int mode, CUtensorMap *out, bool lockstep, int tx, int ty) {
+// Tiled map of `rank` dimensions over 8-byte elements.  The x axis and a point's contiguous values
+// (64 bytes of a packed array, 16 of a point record) form one innermost dimension, so that a tile
+// row is one run of bytes for the copy engine instead of one 64-byte (or 16-byte) run per point.
+// Coordinates along it are x * 8 (packed) or x * 2 (records), always a multiple of 16 bytes.
+static bool encode_tiled(const void *ptr, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
+                         const cuuint32_t *box, CUtensorMap *out) {
   EncodeTiledFn fn = encode_fn();
   if (!fn || (reinterpret_cast<uintptr_t>(ptr) & 15) != 0) return false;
-  const cuuint64_t dims[5] = {16, (cuuint64_t)s->nx, (cuuint64_t)s->ny, (cuuint64_t)s->nz, (cuuint64_t)s->n_kb};
-  const cuuint64_t strides[4] = {64, 64ull * s->nx, 64ull * s->nx * s->ny, 64ull * (cuuint64_t)s->N};
-  const cuuint32_t box[5] = {16, (cuuint32_t)(tx + 2 * s->M), (cuuint32_t)(ty + 2 * s->M),
-                             (cuuint32_t)tma_planes(s->prec, mode, lockstep), 1};
   const cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<void *>(ptr), dims, strides, box, es,
+  return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, rank, const_cast<void *>(ptr), dims, strides, box, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Map over a packed array with a box of bx x by points and z depth `depth`.
+bool encode_op_map(const tdks_system *s, const void *ptr, CUtensorMap *out, int bx, int by, int depth) {
+  const cuuint64_t dims[4] = {8ull * s->nx, (cuuint64_t)s->ny, (cuuint64_t)s->nz, (cuuint64_t)s->n_kb};
+  const cuuint64_t strides[3] = {64ull * s->nx, 64ull * s->nx * s->ny, 64ull * (cuuint64_t)s->N};
+  const cuuint32_t box[4] = {8u * bx, (cuuint32_t)by, (cuuint32_t)depth, 1};
+  return encode_tiled(ptr, 4, dims, strides, box, out);
+}
+
+// Map over a packed array for the halo planes of the TMA sweep of `mode` (box depth = planes per copy).
+bool encode_map(const tdks_system *s, const void *ptr, int mode, CUtensorMap *out, bool lockstep, int tx, int ty) {
+  return encode_op_map(s, ptr, out, tx + 2 * s->M, ty + 2 * s->M, tma_planes(s->prec, mode, lockstep));
 }
 
 // Map over the per-point records, tile box of the mode's depth.
 bool encode_aux_map(const tdks_system *s, int mode, CUtensorMap *out, bool lockstep, int tx, int ty) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn || (reinterpret_cast<uintptr_t>(s->aux) & 15) != 0) return false;
-  const cuuint64_t dims[4] = {4, (cuuint64_t)s->nx, (cuuint64_t)s->ny, (cuuint64_t)s->nz};
-  const cuuint64_t strides[3] = {16, 16ull * s->nx, 16ull * s->nx * s->ny};
-  const cuuint32_t box[4] = {4, (cuuint32_t)tx, (cuuint32_t)ty, (cuuint32_t)tma_planes(s->prec, mode, lockstep)};
-  const cuuint32_t es[4] = {1, 1, 1, 1};
-  return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, s->aux, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Map over a packed array with the tile box (no halo) of z depth `depth`.
-bool encode_op_map(const tdks_system *s, const void *ptr, CUtensorMap *out, int tx, int ty, int depth) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn || (reinterpret_cast<uintptr_t>(ptr) & 15) != 0) return false;
-  const cuuint64_t dims[5] = {16, (cuuint64_t)s->nx, (cuuint64_t)s->ny, (cuuint64_t)s->nz, (cuuint64_t)s->n_kb};
-  const cuuint64_t strides[4] = {64, 64ull * s->nx, 64ull * s->nx * s->ny, 64ull * (cuuint64_t)s->N};
-  const cuuint32_t box[5] = {16, (cuuint32_t)tx, (cuuint32_t)ty, (cuuint32_t)depth, 1};
-  const cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<void *>(ptr), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint64_t dims[3] = {2ull * s->nx, (cuuint64_t)s->ny, (cuuint64_t)s->nz};
+  const cuuint64_t strides[2] = {16ull * s->nx, 16ull * s->nx * s->ny};
+  const cuuint32_t box[3] = {2u * tx, (cuuint32_t)ty, (cuuint32_t)tma_planes(s->prec, mode, lockstep)};
+  return encode_tiled(s->aux, 3, dims, strides, box, out);
 }
 
 bool encode_sweep_maps(const tdks_system *s, const void *in, int mode, SweepMaps *out, bool lockstep, int sweep) {

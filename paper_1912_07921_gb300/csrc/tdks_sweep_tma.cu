@@ -35,7 +35,7 @@ __device__ __forceinline__ void tma_sweep_body(const Src &src) {
   constexpr int QN = 2 * M + U;   // z-queue entries
   constexpr int LP = 2 * M / U;   // priming centre loads per item
   extern __shared__ unsigned char smem_raw[];
-  unsigned char *cbase = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
+  unsigned char *cbase = smem_raw + ((0u - smem_u32(smem_raw)) & 127u);
   unsigned char *hbase = cbase + (size_t)SC * G::CSLOT_BYTES;
   unsigned char *obase = hbase + (size_t)SH * G::HSLOT_BYTES;
   __shared__ __align__(8) uint64_t cfull[SC];

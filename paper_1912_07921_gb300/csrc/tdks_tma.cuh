@@ -83,21 +83,21 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t *bar, uint32_t parit
   }
   return true;
 }
-__device__ __forceinline__ void tma_load_5d(void *dst, const CUtensorMap *tmap, uint64_t *bar, int c0, int c1,
-                                            int c2, int c3, int c4) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(bar))
-      : "memory");
-}
-
 __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *tmap, uint64_t *bar, int c0, int c1,
                                             int c2, int c3) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
       "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar))
+      : "memory");
+}
+
+__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *tmap, uint64_t *bar, int c0, int c1,
+                                            int c2) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -295,8 +295,7 @@ struct Loader {
       mbar_expect_tx(&cfull[slot], G::CSLOT_BYTES);
       int zc = c.z0 - M + U * c.l;
       if (c.wrap) zc -= floordiv_i(zc, c.nz) * c.nz;  // (U = 1 for periodic cells)
-      tma_load_5d(cbase + (size_t)slot * G::CSLOT_BYTES, &mp->ctr, &cfull[slot], 0, c.tx * TX, c.ty * TY, zc,
-                  c.kb);
+      tma_load_4d(cbase + (size_t)slot * G::CSLOT_BYTES, &mp->ctr, &cfull[slot], 8 * c.tx * TX, c.ty * TY, zc, c.kb);
     } else if (kind == 1) {
       const int slot = (int)(c.issued % SH);
       unsigned char *dst = hbase + (size_t)slot * G::HSLOT_BYTES;
@@ -308,21 +307,21 @@ struct Loader {
       const uint32_t bytes = G::IN_BYTES + G::AUX_BYTES + (uint32_t)(sl + sr) * G::STRIPX_BYTES +
                              (uint32_t)(st + sb) * G::STRIPY_BYTES;
       mbar_expect_tx(&hfull[slot], bytes);
-      tma_load_5d(dst, &mp->in, &hfull[slot], 0, x0 - M, y0 - M, zp, c.kb);
-      tma_load_4d(dst + G::IN_BYTES, &mp->aux, &hfull[slot], 0, x0, y0, zp);
+      tma_load_4d(dst, &mp->in, &hfull[slot], 8 * (x0 - M), y0 - M, zp, c.kb);
+      tma_load_3d(dst + G::IN_BYTES, &mp->aux, &hfull[slot], 2 * x0, y0, zp);
       if constexpr (G::STRIP_BYTES > 0) {
         unsigned char *sd = dst + G::IN_BYTES + G::AUX_BYTES;
-        if (sl) tma_load_5d(sd, &mp->sx, &hfull[slot], 0, c.nx - M, y0 - M, zp, c.kb);
-        if (sr) tma_load_5d(sd + G::STRIPX_BYTES, &mp->sx, &hfull[slot], 0, 0, y0 - M, zp, c.kb);
-        if (st) tma_load_5d(sd + 2 * G::STRIPX_BYTES, &mp->sy, &hfull[slot], 0, x0, c.ny - M, zp, c.kb);
-        if (sb) tma_load_5d(sd + 2 * G::STRIPX_BYTES + G::STRIPY_BYTES, &mp->sy, &hfull[slot], 0, x0, 0, zp, c.kb);
+        if (sl) tma_load_4d(sd, &mp->sx, &hfull[slot], 8 * (c.nx - M), y0 - M, zp, c.kb);
+        if (sr) tma_load_4d(sd + G::STRIPX_BYTES, &mp->sx, &hfull[slot], 0, y0 - M, zp, c.kb);
+        if (st) tma_load_4d(sd + 2 * G::STRIPX_BYTES, &mp->sy, &hfull[slot], 8 * x0, c.ny - M, zp, c.kb);
+        if (sb) tma_load_4d(sd + 2 * G::STRIPX_BYTES + G::STRIPY_BYTES, &mp->sy, &hfull[slot], 8 * x0, 0, zp, c.kb);
       }
     } else {
       const int slot = (int)(c.issued % SO);
       unsigned char *dst = obase + (size_t)slot * G::OP_BYTES;
       mbar_expect_tx(&ofull[slot], G::OP_BYTES);
       for (int j = 0; j < 4; j++)
-        tma_load_5d(dst + j * G::OPT_BYTES, &mp->op[j], &ofull[slot], 0, c.tx * TX, c.ty * TY, c.z0 + c.l, c.kb);
+        tma_load_4d(dst + j * G::OPT_BYTES, &mp->op[j], &ofull[slot], 8 * c.tx * TX, c.ty * TY, c.z0 + c.l, c.kb);
     }
     c.issued++;
     c.l++;
@@ -497,7 +496,7 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
   constexpr int LP = 2 * M / U;   // priming centre loads per item
   constexpr int IR = 16;          // claimed-item ring (the producer runs at most a few items ahead)
   extern __shared__ unsigned char smem_raw[];
-  unsigned char *cbase = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
+  unsigned char *cbase = smem_raw + ((0u - smem_u32(smem_raw)) & 127u);
   unsigned char *hbase = cbase + (size_t)SC * G::CSLOT_BYTES;
   unsigned char *obase = hbase + (size_t)SH * G::HSLOT_BYTES;
   __shared__ __align__(8) uint64_t cfull[SC], cempty[SC];
