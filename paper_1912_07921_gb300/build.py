@@ -12,7 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libtdks.so")
 SOURCES = ["tdks_sweep.cu", "tdks_sweep_tma.cu", "tdks_sweep_ws1.cu", "tdks_sweep_ws2.cu", "tdks_sweep_ws3.cu",
-           "tdks_sweep_ws4.cu", "tdks_sweep_ws5.cu",
+           "tdks_sweep_ws4.cu", "tdks_sweep_ws5.cu", "tdks_sweep_ws6.cu", "tdks_sweep_ws7.cu", "tdks_sweep_ws8.cu",
            "tdks_aux.cu", "tdks_capi.cu", "tdks_batch.cu", "tdks_noalloc.cu",
            "tdks_checkpoint.cu", "tdks_probe.cu",
            "tdks_tsurff.cu", "tdks_hartree.cu", "tdks_heat.cu"]

@@ -87,7 +87,7 @@ int enqueue_substep(tdks_batch *b) {
     BatchSweepArgs a{b->d_sweep[k], b->d_maps, k, b->d_item_begin[k],
                       n, b->total_items[k], b->d_work, b->d_item_sys[k]};
     const int mode = k == 0 ? MODE_FIRST : (k == 3 ? MODE_LAST : MODE_MID);
-    e = launch_sweep_tma_batch(b->M, b->prec, mode, a, b->work, b->shape[k]);
+    e = launch_sweep_tma_batch(b->M, b->prec, mode, a, b->work, kernel_shape(b->sys[0], b->shape[k], k));
     if (e != cudaSuccess) return fail(TDKS_EDEVICE, std::string("batched sweep: ") + cudaGetErrorString(e));
     if (k == 0) {
       e = launch_batch_tail(b->d_aux, b->d_clock, n, 0, b->work);
@@ -129,7 +129,7 @@ int build_sweep_tables(tdks_batch *b, bool tune) {
     bool ok = true;
     for (int k = 0; k < 4 && ok; k++) {
       int tx = 16, ty = 8;
-      ws_shape_info(b->shape[k], &tx, &ty, nullptr, nullptr);
+      ws_shape_info(kernel_shape(s, b->shape[k], k), &tx, &ty, nullptr, nullptr);
       s->tx = tx; s->ty = ty; s->zc = s->nz;
       ok = encode_sweep_maps(s, ins[k], modes[k], &maps[4 * i + k], false);
       SweepParams p{};
@@ -154,7 +154,7 @@ int build_sweep_tables(tdks_batch *b, bool tune) {
     if (!ok) return fail(TDKS_EDEVICE, "tensor map encoding failed");
     // the warp-specialised sweep writes one partial record per consumer warp and item
     int warps = 8;
-    ws_shape_info(b->shape[0], nullptr, nullptr, nullptr, &warps);
+    ws_shape_info(kernel_shape(s, b->shape[0], 0), nullptr, nullptr, nullptr, &warps);
     b->aux_h[i].n_items = sp[0].back().n_items * warps;
   }
   for (int k = 0; k < 4; k++) {
@@ -404,10 +404,10 @@ int tdks_batch_autotune(tdks_batch_t b, int reps, double *ms) {
     for (int k = 0; k < 4 && !rc; k++) {
       BatchSweepArgs a{b->d_sweep[k], b->d_maps, k, b->d_item_begin[k],
                       n, b->total_items[k], b->d_work, b->d_item_sys[k]};
-      cudaError_t e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, sh);  // warm-up
+      cudaError_t e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, kernel_shape(b->sys[0], sh, k));  // warm-up
       cudaEventRecord(e0, b->work);
       for (int r = 0; r < reps && e == cudaSuccess; r++)
-        e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, sh);
+        e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, kernel_shape(b->sys[0], sh, k));
       cudaEventRecord(e1, b->work);
       if (e != cudaSuccess) { rc = fail(TDKS_EDEVICE, std::string("batched sweep: ") + cudaGetErrorString(e)); break; }
       if (cudaEventSynchronize(e1) != cudaSuccess) { rc = fail(TDKS_EDEVICE, "batch autotune timing"); break; }

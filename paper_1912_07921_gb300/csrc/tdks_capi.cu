@@ -132,11 +132,15 @@ static bool tma_path(const tdks_system *s) {
   return ws_path(s) || (s->path == 2 && s->bc == TDKS_BC_ZERO && tma_supported(s->M, s->tx, s->ty));
 }
 
+int kernel_shape(const tdks_system *s, int shape, int sweep) {
+  return ws_kernel_shape(shape, s->M, s->prec, s->bc == TDKS_BC_BLOCH, s->nx, s->ny, sweep == 3);
+}
+
 // Tile of a sweep: the warp-specialised TMA sweep's shape, else the system's tile.
 static void sweep_tile(const tdks_system *s, int sweep, int &tx, int &ty) {
   tx = s->tx;
   ty = s->ty;
-  if (sweep >= 0 && ws_path(s)) ws_shape_info(s->wshape[sweep], &tx, &ty, nullptr, nullptr);
+  if (sweep >= 0 && ws_path(s)) ws_shape_info(kernel_shape(s, s->wshape[sweep], sweep), &tx, &ty, nullptr, nullptr);
 }
 
 void sweep_geometry(const tdks_system *s, SweepParams &p, int sweep) {
@@ -293,7 +297,7 @@ int run_sweep(tdks_system *s, int mode, SweepParams &p, const SweepMaps *tm, int
   cudaError_t e;
   const bool tma = tm && tma_path(s);
   const bool ws = tma && s->path == 0;
-  const int shape = (ws && sweep >= 0) ? s->wshape[sweep] : 0;
+  const int shape = (ws && sweep >= 0) ? kernel_shape(s, s->wshape[sweep], sweep) : 0;
   if (tma)
     e = launch_sweep_tma(s->M, s->prec, mode, s->tx, s->ty, *tm, p, 0, s->stream, !ws, shape);
   else
@@ -984,7 +988,7 @@ static int tune_launch(tdks_system *s, int sweep) {
   if (!encode_sweep_maps(s, p.in, mode, &tm, false, sweep)) return fail(TDKS_EDEVICE, "tensor map encoding failed");
   if (mode == MODE_LAST) {
     int tx = 16, ty = 8;
-    ws_shape_info(s->wshape[sweep], &tx, &ty, nullptr, nullptr);
+    ws_shape_info(kernel_shape(s, s->wshape[sweep], sweep), &tx, &ty, nullptr, nullptr);
     const void *ops[4] = {s->term[0], s->term[1], s->term[0], s->term[1]};
     for (int j = 0; j < 4; j++)
       if (!encode_op_map(s, ops[j], &tm.op[j], tx, ty)) return fail(TDKS_EDEVICE, "tensor map encoding failed");

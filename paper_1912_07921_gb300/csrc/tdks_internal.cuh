@@ -291,8 +291,12 @@ cudaError_t launch_sweep_tma(int M, int prec, int mode, int tx, int ty, const Sw
 // block with `warps` consumer warps, each thread computing `rows` y-adjacent points.
 // Shape 0 (16 x 8, two points per thread, eight consumer warps) is the default and the one
 // the batched sweep uses.  Null outputs are skipped; false for a shape out of range.
-constexpr int WS_SHAPES = 6;
+constexpr int WS_SHAPES = 9;
 bool ws_shape_info(int shape, int *tx, int *ty, int *rows, int *warps);
+// The shape whose kernel a sweep of `shape` runs: shapes 5 to 8 exist for some systems only, the others
+// run one that does.  Tiles, tensor maps and record counts follow the result.
+// last: the sweep of the last Taylor term.
+int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last);
 bool tma_supported(int M, int tx, int ty);
 int tma_planes(int prec, int mode, bool lockstep = false);
 int lda_blocks(long N);

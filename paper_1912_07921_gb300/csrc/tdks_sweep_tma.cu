@@ -65,7 +65,7 @@ __device__ __forceinline__ void tma_sweep_body(const Src &src) {
   }
   __syncthreads();
 
-  const Loader<M, TX, TY, U, G, SC, SH, SO, Src> ld{src, n_my, cbase, hbase, obase, cfull, hfull, ofull};
+  const Loader<M, TX, TY, U, U, G, SC, SH, SO, Src> ld{src, n_my, cbase, hbase, obase, cfull, hfull, ofull};
   // the cursors live in shared memory: only thread 0 uses them, and registers are scarce
   __shared__ LoadCursor cur[3];
   LoadCursor &cc = cur[0], &hc = cur[1], &oc = cur[2];
@@ -257,6 +257,9 @@ extern template cudaError_t launch_ws_batch_shape<2>(int, int, int, const BatchS
 extern template cudaError_t launch_ws_batch_shape<3>(int, int, int, const BatchSweepArgs &, cudaStream_t);
 extern template cudaError_t launch_ws_batch_shape<4>(int, int, int, const BatchSweepArgs &, cudaStream_t);
 extern template cudaError_t launch_ws_batch_shape<5>(int, int, int, const BatchSweepArgs &, cudaStream_t);
+extern template cudaError_t launch_ws_batch_shape<6>(int, int, int, const BatchSweepArgs &, cudaStream_t);
+extern template cudaError_t launch_ws_batch_shape<7>(int, int, int, const BatchSweepArgs &, cudaStream_t);
+extern template cudaError_t launch_ws_batch_shape<8>(int, int, int, const BatchSweepArgs &, cudaStream_t);
 template cudaError_t launch_ws_batch_shape<0>(int, int, int, const BatchSweepArgs &, cudaStream_t);
 
 cudaError_t launch_sweep_tma_batch(int M, int prec, int mode, const BatchSweepArgs &a, cudaStream_t s, int shape) {
@@ -268,6 +271,9 @@ cudaError_t launch_sweep_tma_batch(int M, int prec, int mode, const BatchSweepAr
     case 3: return launch_ws_batch_shape<3>(M, prec, mode, a, s);
     case 4: return launch_ws_batch_shape<4>(M, prec, mode, a, s);
     case 5: return launch_ws_batch_shape<5>(M, prec, mode, a, s);
+    case 6: return launch_ws_batch_shape<6>(M, prec, mode, a, s);
+    case 7: return launch_ws_batch_shape<7>(M, prec, mode, a, s);
+    case 8: return launch_ws_batch_shape<8>(M, prec, mode, a, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -293,15 +299,23 @@ extern template cudaError_t launch_ws_shape<4>(int, int, int, int, const SweepMa
                                                  cudaStream_t);
 extern template cudaError_t launch_ws_shape<5>(int, int, int, int, const SweepMaps &, const SweepParams &, int,
                                                  cudaStream_t);
+extern template cudaError_t launch_ws_shape<6>(int, int, int, int, const SweepMaps &, const SweepParams &, int,
+                                                 cudaStream_t);
+extern template cudaError_t launch_ws_shape<8>(int, int, int, int, const SweepMaps &, const SweepParams &, int,
+                                                 cudaStream_t);
+extern template cudaError_t launch_ws_shape<7>(int, int, int, int, const SweepMaps &, const SweepParams &, int,
+                                                 cudaStream_t);
 template cudaError_t launch_ws_shape<0>(int, int, int, int, const SweepMaps &, const SweepParams &, int, cudaStream_t);
 
+// (rows: 16-byte vectors' worth of points per thread)
 template <int SHAPE>
 static void shape_of(int *tx, int *ty, int *rows, int *warps) {
   typedef WsShape<SHAPE> S;
+  constexpr bool small = C64Shape<SHAPE>::ONLY && C64Shape<SHAPE>::P == P_C64S;
   if (tx) *tx = S::TX;
   if (ty) *ty = S::TY;
-  if (rows) *rows = S::R;
-  if (warps) *warps = WsWarps<S::TX, S::TY, S::R>::CW;
+  if (rows) *rows = S::R * S::RX / (S::RX == 2 && small ? 2 : 1);
+  if (warps) *warps = WsWarps<S::TX, S::TY, S::R, small ? 8 : 4, S::RX>::CW;
 }
 
 bool ws_shape_info(int shape, int *tx, int *ty, int *rows, int *warps) {
@@ -311,17 +325,22 @@ bool ws_shape_info(int shape, int *tx, int *ty, int *rows, int *warps) {
     case 2: shape_of<2>(tx, ty, rows, warps); return true;
     case 3: shape_of<3>(tx, ty, rows, warps); return true;
     case 4: shape_of<4>(tx, ty, rows, warps); return true;
-    case 5: {
-      // complex64 systems: 8 one-complex vectors per point (complex128 runs shape 2, also 12 warps)
-      typedef WsShape<5> S;
-      if (tx) *tx = S::TX;
-      if (ty) *ty = S::TY;
-      if (rows) *rows = S::R;
-      if (warps) *warps = WsWarps<S::TX, S::TY, S::R, 8>::CW;
-      return true;
-    }
+    case 5: shape_of<5>(tx, ty, rows, warps); return true;
+    case 6: shape_of<6>(tx, ty, rows, warps); return true;
+    case 7: shape_of<7>(tx, ty, rows, warps); return true;
+    case 8: shape_of<8>(tx, ty, rows, warps); return true;
   }
   return false;
+}
+
+int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last) {
+  if (shape < 5) return shape;
+  if (prec != P_C64) return 2;                                       // the FP64 pipe bounds every shape alike
+  if (shape == 5) return bloch ? 2 : 5;
+  if (bloch && (M != 2 || nx % 2 != 0 || ny % 2 != 0)) return 2;     // blocks must not straddle a face
+  if (last) return 2;                                                // their operands would not fit
+  if (shape == 7 && M != 2) return 6;                                // its z queues would not fit
+  return shape;
 }
 
 cudaError_t launch_sweep_tma(int M, int prec, int mode, int tx, int ty, const SweepMaps &maps, const SweepParams &p,
@@ -342,6 +361,9 @@ cudaError_t launch_sweep_tma(int M, int prec, int mode, int tx, int ty, const Sw
     case 3: return launch_ws_shape<3>(M, prec, mode, b, maps, p, grid, s);
     case 4: return launch_ws_shape<4>(M, prec, mode, b, maps, p, grid, s);
     case 5: return launch_ws_shape<5>(M, prec, mode, b, maps, p, grid, s);
+    case 6: return launch_ws_shape<6>(M, prec, mode, b, maps, p, grid, s);
+    case 7: return launch_ws_shape<7>(M, prec, mode, b, maps, p, grid, s);
+    case 8: return launch_ws_shape<8>(M, prec, mode, b, maps, p, grid, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -145,6 +145,8 @@ double envelope_of(const tdks_system *s, double t, double *denv);
 // warp-specialised TMA sweep takes that sweep's tile shape; -1: the system's tile (16x8 on
 // the TMA path)
 bool ws_path(const tdks_system *s);
+// the kernel shape behind tile shape `shape` in Taylor-term sweep `sweep` of this system
+int kernel_shape(const tdks_system *s, int shape, int sweep);
 void sweep_geometry(const tdks_system *s, tdks::SweepParams &p, int sweep = -1);
 void sweep_common(const tdks_system *s, tdks::SweepParams &p, const double A[3], int sweep = -1);
 long n_items_of(const tdks_system *s);

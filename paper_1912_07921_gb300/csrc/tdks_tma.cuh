@@ -150,23 +150,23 @@ struct TmaGeom {
   static constexpr uint32_t AUX_BYTES = (uint32_t)TX * TY * 16 * U;
   static constexpr uint32_t STRIPX_BYTES = (uint32_t)M * SY * OVC * 16;   // beyond x = 0 or x = nx - 1
   static constexpr uint32_t STRIPY_BYTES = (uint32_t)TX * M * OVC * 16;   // beyond y = 0 or y = ny - 1
-  static constexpr uint32_t STRIP_BYTES = BL ? 2 * (STRIPX_BYTES + STRIPY_BYTES) : 0;
+  static constexpr uint32_t STRIP1_BYTES = BL ? 2 * (STRIPX_BYTES + STRIPY_BYTES) : 0;  // of one plane
+  static constexpr uint32_t STRIP_BYTES = STRIP1_BYTES * U;
   static constexpr uint32_t OPT_BYTES = (uint32_t)CPLANE * 16;       // one operand tile
   static constexpr uint32_t OP_BYTES = 4 * OPT_BYTES;
   static constexpr int SO = OPS ? 2 : 0;
   // (the last term's 4 operand tiles leave taller tiles room for few centre slots)
-  static constexpr int SC = U == 1 ? (OPS ? (TX * TY > 128 ? 2 : 4) : 6) : 4;
+  static constexpr int SC = U == 1 ? (OPS ? (TX * TY > 128 ? 2 : 4) : (TX * TY > 256 ? 3 : 6)) : (OVC * TX * TY > 512 ? 3 : 4);
   static constexpr size_t BUDGET = 227 * 1024 - 2048;                // dynamic smem available
   static constexpr size_t HALO_ROOM = BUDGET - 128 - (size_t)SO * OP_BYTES - (size_t)SC * CSLOT_BYTES;
   // periodic cells, first Taylor term (NLG): the non-local rows of the plane's sphere points,
   // gathered into the slot by the patcher warp, where two slots still fit (else the consumers
   // load them).  (The larger slot leaves fewer halo slots: the faster middle and last sweeps
   // measured slower with it, the first sweep, with its current gradients, faster.)
-  static constexpr uint32_t NL_STAGE = (uint32_t)TX * TY * OVC * 16;
+  static constexpr uint32_t NL_STAGE = (uint32_t)TX * TY * OVC * 16 * U;
   static constexpr bool NLS = BL && NLG && HALO_ROOM / (IN_BYTES + AUX_BYTES + STRIP_BYTES + NL_STAGE) >= 2;
   static constexpr uint32_t NL_BYTES = NLS ? NL_STAGE : 0;
   static constexpr uint32_t HSLOT_BYTES = IN_BYTES + AUX_BYTES + STRIP_BYTES + NL_BYTES;
-  static_assert(!BL || U == 1, "periodic cells take one plane per iteration");
   static constexpr int SH_FIT = (int)(HALO_ROOM / HSLOT_BYTES);
   static constexpr int SH = SH_FIT < 8 ? SH_FIT : 8;
   static constexpr size_t SMEM = (size_t)SC * CSLOT_BYTES + (size_t)SH * HSLOT_BYTES + (size_t)SO * OP_BYTES + 128;
@@ -249,8 +249,8 @@ __device__ __forceinline__ int loads_of(int kind, int z0, int z1) {
   return z1 - z0;
 }
 
-// The producer side of the rings (thread 0 only).
-template <int M, int TX, int TY, int U, class G, int SC, int SH, int SO, class Src>
+// The producer side of the rings (one thread).  D: planes per copy (the z depth of the maps' boxes).
+template <int M, int TX, int TY, int U, int D, class G, int SC, int SH, int SO, class Src>
 struct Loader {
   Src src;
   long n_my;
@@ -289,41 +289,50 @@ struct Loader {
 
   // issue the load the cursor is positioned on
   __device__ __forceinline__ void emit(LoadCursor &c, int kind) const {
+    emit_at(c, kind, (int)(c.issued % (kind == 0 ? SC : (kind == 1 ? SH : SO))));
+    c.issued++;
+  }
+
+  // the same into ring slot `slot`
+  __device__ __forceinline__ void emit_at(LoadCursor &c, int kind, int slot) const {
     const SweepMaps *mp = src.maps_of(c.sys);
     if (kind == 0) {
-      const int slot = (int)(c.issued % SC);
       mbar_expect_tx(&cfull[slot], G::CSLOT_BYTES);
-      int zc = c.z0 - M + U * c.l;
-      if (c.wrap) zc -= floordiv_i(zc, c.nz) * c.nz;  // (U = 1 for periodic cells)
-      tma_load_4d(cbase + (size_t)slot * G::CSLOT_BYTES, &mp->ctr, &cfull[slot], 8 * c.tx * TX, c.ty * TY, zc, c.kb);
+#pragma unroll
+      for (int u = 0; u < U; u += D) {
+        int zc = c.z0 - M + U * c.l + u;
+        if (c.wrap) zc -= floordiv_i(zc, c.nz) * c.nz;  // (D = 1 for periodic cells)
+        tma_load_4d(cbase + (size_t)slot * G::CSLOT_BYTES + (size_t)u * G::CPLANE * 16, &mp->ctr, &cfull[slot],
+                    8 * c.tx * TX, c.ty * TY, zc, c.kb);
+      }
     } else if (kind == 1) {
-      const int slot = (int)(c.issued % SH);
       unsigned char *dst = hbase + (size_t)slot * G::HSLOT_BYTES;
-      const int zp = c.z0 + U * c.l;
       const int x0 = c.tx * TX, y0 = c.ty * TY;
       // periodic cell: the strips this tile's halo crosses (the slot holds zeros there)
       const bool sl = G::STRIP_BYTES && c.wrap && x0 - M < 0, sr = G::STRIP_BYTES && c.wrap && x0 + TX + M > c.nx;
       const bool st = G::STRIP_BYTES && c.wrap && y0 - M < 0, sb = G::STRIP_BYTES && c.wrap && y0 + TY + M > c.ny;
-      const uint32_t bytes = G::IN_BYTES + G::AUX_BYTES + (uint32_t)(sl + sr) * G::STRIPX_BYTES +
-                             (uint32_t)(st + sb) * G::STRIPY_BYTES;
+      const uint32_t bytes = G::IN_BYTES + G::AUX_BYTES + (uint32_t)U * ((uint32_t)(sl + sr) * G::STRIPX_BYTES +
+                                                                         (uint32_t)(st + sb) * G::STRIPY_BYTES);
       mbar_expect_tx(&hfull[slot], bytes);
-      tma_load_4d(dst, &mp->in, &hfull[slot], 8 * (x0 - M), y0 - M, zp, c.kb);
-      tma_load_3d(dst + G::IN_BYTES, &mp->aux, &hfull[slot], 2 * x0, y0, zp);
-      if constexpr (G::STRIP_BYTES > 0) {
-        unsigned char *sd = dst + G::IN_BYTES + G::AUX_BYTES;
-        if (sl) tma_load_4d(sd, &mp->sx, &hfull[slot], 8 * (c.nx - M), y0 - M, zp, c.kb);
-        if (sr) tma_load_4d(sd + G::STRIPX_BYTES, &mp->sx, &hfull[slot], 0, y0 - M, zp, c.kb);
-        if (st) tma_load_4d(sd + 2 * G::STRIPX_BYTES, &mp->sy, &hfull[slot], 8 * x0, c.ny - M, zp, c.kb);
-        if (sb) tma_load_4d(sd + 2 * G::STRIPX_BYTES + G::STRIPY_BYTES, &mp->sy, &hfull[slot], 8 * x0, 0, zp, c.kb);
+#pragma unroll
+      for (int u = 0; u < U; u += D) {
+        const int zp = c.z0 + U * c.l + u;
+        tma_load_4d(dst + (size_t)u * G::PLANE * 16, &mp->in, &hfull[slot], 8 * (x0 - M), y0 - M, zp, c.kb);
+        tma_load_3d(dst + G::IN_BYTES + (size_t)u * TX * TY * 16, &mp->aux, &hfull[slot], 2 * x0, y0, zp);
+        if constexpr (G::STRIP_BYTES > 0) {
+          unsigned char *sd = dst + G::IN_BYTES + G::AUX_BYTES + (size_t)u * G::STRIP1_BYTES;
+          if (sl) tma_load_4d(sd, &mp->sx, &hfull[slot], 8 * (c.nx - M), y0 - M, zp, c.kb);
+          if (sr) tma_load_4d(sd + G::STRIPX_BYTES, &mp->sx, &hfull[slot], 0, y0 - M, zp, c.kb);
+          if (st) tma_load_4d(sd + 2 * G::STRIPX_BYTES, &mp->sy, &hfull[slot], 8 * x0, c.ny - M, zp, c.kb);
+          if (sb) tma_load_4d(sd + 2 * G::STRIPX_BYTES + G::STRIPY_BYTES, &mp->sy, &hfull[slot], 8 * x0, 0, zp, c.kb);
+        }
       }
     } else {
-      const int slot = (int)(c.issued % SO);
       unsigned char *dst = obase + (size_t)slot * G::OP_BYTES;
       mbar_expect_tx(&ofull[slot], G::OP_BYTES);
       for (int j = 0; j < 4; j++)
         tma_load_4d(dst + j * G::OPT_BYTES, &mp->op[j], &ofull[slot], 8 * c.tx * TX, c.ty * TY, c.z0 + c.l, c.kb);
     }
-    c.issued++;
     c.l++;
   }
 };
@@ -352,19 +361,39 @@ struct Loader {
 // 2M x-arm loads, 2M/4 y-arm loads and one queue load of 8 bytes, against 2M, (2M+2)/2 and
 // one of 16 bytes for two values in the two-complex shapes: about a third fewer shared-memory
 // bytes per value.  Complex128 systems and periodic cells run shape 5 as shape 2.
+//
+// Shapes 6 and 7 give a thread a block of 2 x 2 points (RX = 2 x-adjacent, R = 2 y-adjacent): the
+// block shares its x-arm loads too, 2M per row and 2M per column for four points, so a value costs
+// 2M + 1 shared loads where two y-adjacent points cost 3M + 2 and one point 4M + 1.  The block's
+// inner neighbours come from the z queues.  To keep the loads free of bank conflicts (a point is 64
+// bytes, half of the banks) the odd blocks of a row are mirrored: their first point is the right
+// one and their x offsets count downwards, so that two blocks side by side always read different
+// halves of the banks.  The x arm is symmetric, so mirrored values are the same bit for bit.
 template <int SHAPE> struct WsShape;
-template <> struct WsShape<0> { static constexpr int TX = 16, TY = 8, R = 2; };   //  8 consumer warps
-template <> struct WsShape<1> { static constexpr int TX = 16, TY = 12, R = 4; };  //  6
-template <> struct WsShape<2> { static constexpr int TX = 16, TY = 12, R = 2; };  // 12
-template <> struct WsShape<3> { static constexpr int TX = 16, TY = 8, R = 1; };   // 16
-template <> struct WsShape<4> { static constexpr int TX = 14, TY = 8, R = 2; };   //  7
-template <> struct WsShape<5> { static constexpr int TX = 16, TY = 12, R = 4; };  // 12 (complex64, 8-byte vectors)
-template <int TX, int TY, int R, int OV = OVC> struct WsWarps {
-  static constexpr int CW = OV * TX * TY / (32 * R);       // consumer warps
-  static constexpr int THREADS = 32 * CW + 32;             // + the producer warp
-  // consumer thread t owns vector t % OV of point (t / OV) % TX of row group t / (OV TX), whose
-  // R rows are y-adjacent: the row groups must fill the tile and the warps exactly
-  static_assert(TY % R == 0 && CW * 32 == OV * TX * (TY / R), "row groups must fill the tile and the warps");
+template <> struct WsShape<0> { static constexpr int U = 1, TX = 16, TY = 8, R = 2, RX = 1; };   //  8 consumer warps
+template <> struct WsShape<1> { static constexpr int U = 1, TX = 16, TY = 12, R = 4, RX = 1; };  //  6
+template <> struct WsShape<2> { static constexpr int U = 1, TX = 16, TY = 12, R = 2, RX = 1; };  // 12
+template <> struct WsShape<3> { static constexpr int U = 1, TX = 16, TY = 8, R = 1, RX = 1; };   // 16
+template <> struct WsShape<4> { static constexpr int U = 1, TX = 14, TY = 8, R = 2, RX = 1; };   //  7
+template <> struct WsShape<5> { static constexpr int U = 1, TX = 16, TY = 12, R = 4, RX = 1; };  // 12 (complex64, 8-byte vectors)
+template <> struct WsShape<6> { static constexpr int U = 2, TX = 16, TY = 12, R = 2, RX = 1; };  // 12 (complex64, terms 1-3)
+template <> struct WsShape<7> { static constexpr int U = 1, TX = 16, TY = 24, R = 2, RX = 2; };  // 12 (complex64, order 4, terms 1-3)
+template <> struct WsShape<8> { static constexpr int U = 2, TX = 16, TY = 12, R = 2, RX = 2; };  // 12 (complex64, 8-byte vectors, terms 1-3)
+template <int TX, int TY, int R, int OV = OVC, int RX = 1, bool SPL = false> struct WsWarps {
+  static constexpr int CW = OV * TX * TY / (32 * R * RX);  // consumer warps
+  // Blocks of 2 x 2 points want more registers than 65536 / threads: their twelve consumer warps and the
+  // four service warps start with 128 per thread each, all there are, and the service warpgroup
+  // gives most of its share to the consumers, whose z queues would spill at 128 (M = 4: 72 of them):
+  // 384 * 152 + 128 * 56 = 512 * 128.
+  static constexpr bool SPLIT = RX == 2 || SPL;
+  static_assert(!SPLIT || CW == 12, "the register split is for twelve consumer warps");
+  static constexpr int CONSUMER_REGS = 152, PRODUCER_REGS = 56;
+  static constexpr int THREADS = 32 * CW + 128;            // + three producer warps and the patcher
+  // consumer thread t owns vector t % OV of block (t / OV) % (TX / RX) of row group t / (OV TX / RX),
+  // whose R rows are y-adjacent: the row groups must fill the tile and the warps exactly
+  static_assert(TY % R == 0 && TX % RX == 0 && CW * 32 == OV * (TX / RX) * (TY / R),
+                "row groups must fill the tile and the warps");
+  static_assert(RX == 1 || (RX == 2 && R == 2), "blocks are columns of R points or 2 x 2 points");
 };
 
 // H at R y-adjacent points (rows 0 .. R-1) of one plane, from their z queues Q[r] and
@@ -397,7 +426,7 @@ __device__ __forceinline__ void stencil_rows(const typename VT<P>::S *W, typenam
 // Bloch phase of one wrap, e^{i ang} = c + i s, in the compute precision.
 template <int P>
 __device__ __forceinline__ void bloch_phase(double ang, typename VT<P>::S &c, typename VT<P>::S &s) {
-  if constexpr (P == P_C64) {
+  if constexpr (P != P_C128) {
     float sn, cs;
     sincosf((float)ang, &sn, &cs);
     c = pk2(cs, cs);
@@ -415,7 +444,7 @@ __device__ __forceinline__ typename VT<P>::V apply_phase(typename VT<P>::S c, ty
                                                          typename VT<P>::V a) {
   typedef VT<P> T;
   if (w < 0) {
-    if constexpr (P == P_C64) s ^= SIGN2; else s = -s;
+    if constexpr (P != P_C128) s ^= SIGN2; else s = -s;
   }
   for (int i = w < 0 ? -w : w; i > 0; i--) a = T::cmul(c, s, a);
   return a;
@@ -477,7 +506,88 @@ __device__ __forceinline__ void stencil_rows_bloch(const SweepParams &p, const t
   }
 }
 
-template <int M, int P, int MODE, int TX, int TY, int R, int U, bool BATCH, int BLOCH, class Src>
+// H at a 2 x 2 block of points (point q = 2 r + c: row r, column c) from their z queues Q[q] and
+// the halo plane, S0 = the block's first point's vector.  sx = +-OV: the vector stride from column 0 to
+// column 1 (mirrored blocks count x downwards).  Same terms and summation order as stencil_point.
+// Inner neighbours come from the queues: in a finite box points of the block beyond the grid are zero
+// there as in the halo plane; a periodic cell takes this shape only where nx and ny are even, so that a
+// block lies inside the cell or outside it as a whole.
+template <int M, int P, int BLOCH, int QB, int QN>
+__device__ __forceinline__ void stencil_block(const SweepParams &p, const typename VT<P>::S *W,
+                                              typename W0T<P>::type w0, const typename VT<P>::V (*Q)[QN],
+                                              const typename VT<P>::V *S0, int SXO, int sx,
+                                              const typename VT<P>::R *ve, typename VT<P>::V *acc,
+                                              typename VT<P>::V (*gax)[3], bool need_grad, bool grads) {
+  typedef VT<P> T;
+  typedef typename T::V V;
+  typename T::S A3[3] = {};
+  if (BLOCH && need_grad) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) A3[a] = T::bc(a == 0 && sx < 0 ? -p.A[a] : p.A[a]);
+  }
+  V gsum[4];
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    acc[q] = T::mul(T::diag(ve[q], w0), Q[q][(QB + M) % QN]);
+    if (BLOCH) {
+      gsum[q] = T::zero();
+      gax[q][0] = gax[q][1] = gax[q][2] = T::zero();
+    }
+  }
+  // outer neighbours of the last distance: x- of row r, x+ of row r; y- of column c, y+ of column c
+  V xl[2], xh[2], yl[2], yh[2];
+#pragma unroll
+  for (int i = 0; i < 2; i++) {
+    xl[i] = Q[2 * i][(QB + M) % QN];
+    xh[i] = Q[2 * i + 1][(QB + M) % QN];
+    yl[i] = Q[i][(QB + M) % QN];
+    yh[i] = Q[2 + i][(QB + M) % QN];
+  }
+#pragma unroll
+  for (int m = 1; m <= M; m++) {
+    V xln[2], xhn[2], yln[2], yhn[2];
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+      xln[i] = (S0 - m * sx)[i * SXO];
+      xhn[i] = (S0 + (m + 1) * sx)[i * SXO];
+      yln[i] = (S0 + i * sx)[-m * SXO];
+      yhn[i] = (S0 + i * sx)[(m + 1) * SXO];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const int r = q >> 1, c = q & 1;
+      const V xm = c == 0 ? xln[r] : xl[r], xp = c == 0 ? xh[r] : xhn[r];
+      const V ym = r == 0 ? yln[c] : yl[c], yp = r == 0 ? yh[c] : yhn[c];
+      const V zm = Q[q][(QB + M - m) % QN], zp = Q[q][(QB + M + m) % QN];
+      const V s6 = T::add(T::add(T::add(zm, zp), T::add(xm, xp)), T::add(ym, yp));
+      acc[q] = T::fma(W[m], s6, acc[q]);
+      if (BLOCH && need_grad) {
+        const V dx = T::sub(xp, xm), dy = T::sub(yp, ym), dz = T::sub(zp, zm);
+        const typename T::S gm = T::bc(p.gw[m]);
+        const V dA = T::fma(A3[0], dx, T::fma(A3[1], dy, T::mul(A3[2], dz)));
+        gsum[q] = T::fma(gm, dA, gsum[q]);
+        if (grads) {
+          gax[q][0] = T::fma(sx < 0 ? T::bc(-p.gw[m]) : gm, dx, gax[q][0]);
+          gax[q][1] = T::fma(gm, dy, gax[q][1]);
+          gax[q][2] = T::fma(gm, dz, gax[q][2]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+      xl[i] = xln[i];
+      xh[i] = xhn[i];
+      yl[i] = yln[i];
+      yh[i] = yhn[i];
+    }
+  }
+  if (BLOCH && need_grad) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) acc[q] = T::add(acc[q], T::negi(gsum[q]));
+  }
+}
+
+template <int M, int P, int MODE, int TX, int TY, int R, int RX, int U, bool BATCH, int BLOCH, class Src>
 __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work) {
   typedef VT<P> T;
   typedef typename T::V V;
@@ -489,7 +599,8 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
   static_assert(!OPS || U == 1, "the last Taylor term takes one plane per iteration");
   constexpr int OV = T::OV;       // thread vectors per (point, batch)
   constexpr int CPL = TX * TY * OV;  // thread vectors per centre plane or operand tile
-  constexpr int CW = WsWarps<TX, TY, R, OV>::CW;
+  constexpr int CW = WsWarps<TX, TY, R, OV, RX>::CW;
+  constexpr int NP = R * RX;      // points per consumer thread
   constexpr int SC = G::SC, SH = G::SH;
   constexpr int SO = G::SO > 0 ? G::SO : 1;
   constexpr int QN = 2 * M + U;   // z-queue entries
@@ -524,102 +635,87 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
   }
   __syncthreads();  // the only CTA-wide barrier: from here on the warps run decoupled
 
-  if (warp == CW) {
-    // ---- producer: claim items, and issue every ring's loads as soon as a slot is free ----
-    // (failure injection: a withholding producer does nothing, so the other warps' waits
-    // run out; no copy is in flight and nothing needs draining)
+  typedef WsWarps<TX, TY, R, OV, RX, U == 2> WW;
+  if (warp >= CW) {
+  if constexpr (WW::SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(WW::PRODUCER_REGS));
+  // ---- producers: one warp per ring (warp CW the centre planes, CW + 1 the halo planes, CW + 2 the
+  // last term's operands), each refilling its ring's slots in order as they are released.  One warp
+  // for all three rings polled them in turn and set the pace of the CTA: ~1450 cycles per plane with
+  // the consumers' stencil taken out, whatever the tile.  The centre producer, which runs ahead of
+  // the others, claims the items.
+  // (failure injection: withholding producers do nothing, so the other warps' waits run out; no copy
+  // is in flight and nothing needs draining)
+  auto serve = [&](auto kind_c) {
+    constexpr int KIND = decltype(kind_c)::value;
+    constexpr int S = KIND == 0 ? SC : (KIND == 1 ? SH : SO);
+    uint64_t *full = KIND == 0 ? cfull : (KIND == 1 ? hfull : ofull);
+    uint64_t *empty = KIND == 0 ? cempty : (KIND == 1 ? hempty : oempty);
+    const Loader<M, TX, TY, U, 1, G, SC, SH, SO, Src> ld{src, 0, cbase, hbase, obase, cfull, hfull, ofull};
+    RingPos rp;
+    unsigned issued = 0;
+    bool gave_up = false;
+    for (unsigned seq = 0; !gave_up; seq++) {
+      if constexpr (KIND == 0) {
+        const unsigned int t = atomicAdd(work, 1u);
+        // every CTA ends with one claim past the last item: the launch's last claim returns the
+        // counter to zero for the next launch
+        if ((long)t == n_items_all + (long)gridDim.x - 1) atomicExch(work, 0u);
+        s_item[seq % IR] = (long)t < n_items_all ? (long)t : -1;
+        mbar_arrive(&ibar[seq % IR]);
+      } else if (!mbar_wait_or_abort(&ibar[seq % IR], (seq / IR) & 1u, abort_flag)) {
+        gave_up = true;
+        break;
+      }
+      const long it = s_item[seq % IR];
+      if (it < 0) break;
+      const SweepParams *qp = nullptr;
+      const SweepMaps *mq = nullptr;
+      long local = 0;
+      src.item(it, qp, mq, local);
+      LoadCursor cu{};
+      int z1 = 0;
+      item_geom(*qp, local, cu.tx, cu.ty, cu.kb, cu.z0, z1);
+      cu.sys = src.sys_of(it);
+      cu.nx = qp->nx;
+      cu.ny = qp->ny;
+      cu.nz = qp->nz;
+      cu.wrap = qp->bloch;
+      const int n = loads_of<M, U>(KIND, cu.z0, z1);
+      for (cu.l = 0; cu.l < n;) {
+        // the slot is free once the consumers have released its previous use (at once the first time)
+        if (!mbar_wait_or_abort(&empty[rp.slot], rp.phase ^ 1u, abort_flag)) {
+          gave_up = true;
+          break;
+        }
+        // (the patcher warp writes halo slots: its writes come before the copy that follows them)
+        if (BLOCH && KIND == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        ld.emit_at(cu, KIND, rp.slot);
+        rp.next<S>();
+        issued++;
+      }
+    }
+    if (gave_up) *abort_flag = 1;
+    // copies still in flight must land before the CTA's shared memory goes away
+    for (unsigned j = issued > S ? issued - S : 0; j < issued; j++)
+      mbar_wait_bounded(&full[j % S], (j / S) & 1u, DRAIN_LIMIT_CYCLES);
+  };
+  if (warp >= CW && warp < CW + 3) {
     if (lane == 0 && !src.withhold()) {
-      const Loader<M, TX, TY, U, G, SC, SH, SO, Src> ld{src, 0, cbase, hbase, obase, cfull, hfull, ofull};
-      LoadCursor c[3];
-      bool done[3] = {false, false, !OPS};
-      for (int k = 0; k < 3; k++) c[k] = LoadCursor{-1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-      long claimed = 0;  // claims made (their items are in s_item)
-      // position cursor k on its next load; false if it has none yet (or none at all)
-      auto position = [&](int k) -> bool {
-        LoadCursor &cu = c[k];
-        while (!done[k] && cu.l >= cu.n) {
-          const long ns = cu.ii + 1;
-          if (ns >= claimed) {
-            if (k != 0) return false;  // the centre cursor, always ahead, makes the claims
-            const unsigned int t = atomicAdd(work, 1u);
-            // every CTA ends with one claim past the last item: the launch's last claim
-            // returns the counter to zero for the next launch
-            if ((long)t == n_items_all + (long)gridDim.x - 1) atomicExch(work, 0u);
-            s_item[claimed % IR] = (long)t < n_items_all ? (long)t : -1;
-            mbar_arrive(&ibar[claimed % IR]);
-            claimed++;
-          }
-          const long it = s_item[ns % IR];
-          if (it < 0) {
-            done[k] = true;
-            break;
-          }
-          const SweepParams *qp = nullptr;
-          const SweepMaps *mq = nullptr;
-          long local = 0;
-          src.item(it, qp, mq, local);
-          int z1 = 0;
-          item_geom(*qp, local, cu.tx, cu.ty, cu.kb, cu.z0, z1);
-          cu.sys = src.sys_of(it);
-          cu.ii = ns;
-          cu.l = 0;
-          cu.n = loads_of<M, U>(k, cu.z0, z1);
-          cu.nx = qp->nx;
-          cu.ny = qp->ny;
-          cu.nz = qp->nz;
-          cu.wrap = qp->bloch;
-        }
-        return !done[k];
-      };
-      long long idle_since = clock64();
-      for (;;) {
-        bool left = false, progressed = false;
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-          if (done[k]) continue;
-          left = true;
-          if (!position(k)) continue;
-          const int S = k == 0 ? SC : (k == 1 ? SH : SO);
-          uint64_t *empty = k == 0 ? cempty : (k == 1 ? hempty : oempty);
-          const long n = c[k].issued;
-          // slot n % S is free once the consumers have released its previous use
-          if (n >= S && !mbar_test(&empty[n % S], (uint32_t)(((n / S) - 1) & 1))) continue;
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          ld.emit(c[k], k);
-          progressed = true;
-        }
-        if (!left) break;
-        if (progressed) {
-          idle_since = clock64();
-        } else {
-          if (*abort_flag || clock64() - idle_since > WAIT_LIMIT_CYCLES) {
-            *abort_flag = 1;
-            break;
-          }
-          __nanosleep(32);
-        }
-      }
-      // copies still in flight must land before the CTA's shared memory goes away
-      for (int k = 0; k < 3; k++) {
-        if (k == 2 && !OPS) continue;
-        const int S = k == 0 ? SC : (k == 1 ? SH : SO);
-        uint64_t *full = k == 0 ? cfull : (k == 1 ? hfull : ofull);
-        const long n = c[k].issued;
-        for (long j = n > S ? n - S : 0; j < n; j++)
-          mbar_wait_bounded(&full[j % S], (uint32_t)((j / S) & 1), DRAIN_LIMIT_CYCLES);
-      }
+      if (warp == CW) serve(std::integral_constant<int, 0>{});
+      if (warp == CW + 1) serve(std::integral_constant<int, 1>{});
+      if (OPS && warp == CW + 2) serve(std::integral_constant<int, 2>{});
     }
     return;
   }
 
-  if (BLOCH && warp == CW + 1) {
+  if (BLOCH && warp == CW + 3) {
     // ---- patcher (periodic cells): for each output plane of each item, once the halo slot
     // has landed, write the Bloch-phased periodic images of the strips beyond the cell's
     // x and y faces into the halo box (where the TMA box holds zeros), then release the
     // slot to the consumers -----------------------------------------------------------------
     RingPos rp;
-    for (long seq = 0;; seq++) {
-      if (!mbar_wait_or_abort(&ibar[seq % IR], (uint32_t)((seq / IR) & 1), abort_flag)) {
+    for (unsigned seq = 0;; seq++) {
+      if (!mbar_wait_or_abort(&ibar[seq % IR], (seq / IR) & 1u, abort_flag)) {
         *abort_flag = 1;
         break;
       }
@@ -639,55 +735,60 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
       bloch_phase<P>(p.kvec[3 * kidx] * p.L[0], cx, sx);
       bloch_phase<P>(p.kvec[3 * kidx + 1] * p.L[1], cy, sy);
       constexpr int VB = (int)sizeof(V);  // bytes per thread vector
-      constexpr int SLB = (int)((G::IN_BYTES + G::AUX_BYTES) / VB);
-      constexpr int SRB = SLB + (int)(G::STRIPX_BYTES / VB);
+      constexpr int SRB = (int)(G::STRIPX_BYTES / VB);
       constexpr int STB = SRB + (int)(G::STRIPX_BYTES / VB);
       constexpr int SBB = STB + (int)(G::STRIPY_BYTES / VB);
       bool gave_up = false;
-      for (int z = z0; z < z1; z++) {
+      for (int z = z0; z < z1; z += U) {
         const int hs = rp.slot;
         if (!mbar_wait_or_abort(&hfull[hs], rp.phase, abort_flag)) {
           gave_up = true;
           break;
         }
-        V *box = reinterpret_cast<V *>(hbase + (size_t)hs * G::HSLOT_BYTES);
-        if (sl || sr) {
-          // box columns c with grid x = x0 - M + c beyond x = 0 (c < M) or beyond x = nx - 1
-          const int cr0 = nx - x0 + M;  // first box column past the last grid column
-          for (int i = lane; i < 2 * G::SY * M * OV; i += 32) {
-            const int v = i % OV, j = (i / OV) % M, row = (i / (OV * M)) % G::SY, side = i / (OV * M * G::SY);
-            if (side == 0 ? !sl : !sr) continue;
-            const int c = side == 0 ? j : cr0 + j;
-            if (c >= G::SX) continue;
-            const V a = box[(side == 0 ? SLB : SRB) + (row * M + j) * OV + v];
-            box[(row * G::SX + c) * OV + v] = apply_phase<P>(cx, sx, side == 0 ? -1 : 1, a);
+#pragma unroll 1
+        for (int u = 0; u < U; u++) {
+          unsigned char *slot = hbase + (size_t)hs * G::HSLOT_BYTES;
+          V *box = reinterpret_cast<V *>(slot + (size_t)u * G::PLANE * 16);
+          const V *strips = reinterpret_cast<const V *>(slot + G::IN_BYTES + G::AUX_BYTES + (size_t)u * G::STRIP1_BYTES);
+          if (sl || sr) {
+            // box columns c with grid x = x0 - M + c beyond x = 0 (c < M) or beyond x = nx - 1
+            const int cr0 = nx - x0 + M;  // first box column past the last grid column
+            for (int i = lane; i < 2 * G::SY * M * OV; i += 32) {
+              const int v = i % OV, j = (i / OV) % M, row = (i / (OV * M)) % G::SY, side = i / (OV * M * G::SY);
+              if (side == 0 ? !sl : !sr) continue;
+              const int c = side == 0 ? j : cr0 + j;
+              if (c >= G::SX) continue;
+              const V a = strips[(side == 0 ? 0 : SRB) + (row * M + j) * OV + v];
+              box[(row * G::SX + c) * OV + v] = apply_phase<P>(cx, sx, side == 0 ? -1 : 1, a);
+            }
+          }
+          if (st || sb) {
+            // box rows rr with grid y = y0 - M + rr beyond y = 0 (rr < M) or beyond y = ny - 1,
+            // over the tile's columns (the star stencil never reads the corners)
+            const int rb0 = ny - y0 + M;
+            for (int i = lane; i < 2 * M * TX * OV; i += 32) {
+              const int v = i % OV, c = (i / OV) % TX, j = (i / (OV * TX)) % M, side = i / (OV * TX * M);
+              if (side == 0 ? !st : !sb) continue;
+              const int rr = side == 0 ? j : rb0 + j;
+              if (rr >= G::SY) continue;
+              const V a = strips[(side == 0 ? STB : SBB) + (j * TX + c) * OV + v];
+              box[(rr * G::SX + c + M) * OV + v] = apply_phase<P>(cy, sy, side == 0 ? -1 : 1, a);
+            }
+          }
+          if (G::NLS && p.has_proj) {
+            // the plane's non-local rows: row r0 of each sphere point (points outside every
+            // sphere are never read from here), in 16-byte units whatever the size of a vector
+            const PointAux *ax = reinterpret_cast<const PointAux *>(slot + G::IN_BYTES) + u * TX * TY;
+            ulonglong2 *nla = reinterpret_cast<ulonglong2 *>(slot + G::IN_BYTES + G::AUX_BYTES + G::STRIP_BYTES) +
+                              u * TX * TY * OVC;
+            const ulonglong2 *nlk = reinterpret_cast<const ulonglong2 *>(p.nl) + (long)kb * (p.n_ent + 1) * OVC;
+            for (int i = lane; i < TX * TY * OVC; i += 32) {
+              const PointAux a = ax[i / OVC];
+              if (a.r1 > a.r0) cp_async_16(nla + i, nlk + (long)a.r0 * OVC + i % OVC);
+            }
           }
         }
-        if (st || sb) {
-          // box rows rr with grid y = y0 - M + rr beyond y = 0 (rr < M) or beyond y = ny - 1,
-          // over the tile's columns (the star stencil never reads the corners)
-          const int rb0 = ny - y0 + M;
-          for (int i = lane; i < 2 * M * TX * OV; i += 32) {
-            const int v = i % OV, c = (i / OV) % TX, j = (i / (OV * TX)) % M, side = i / (OV * TX * M);
-            if (side == 0 ? !st : !sb) continue;
-            const int rr = side == 0 ? j : rb0 + j;
-            if (rr >= G::SY) continue;
-            const V a = box[(side == 0 ? STB : SBB) + (j * TX + c) * OV + v];
-            box[(rr * G::SX + c + M) * OV + v] = apply_phase<P>(cy, sy, side == 0 ? -1 : 1, a);
-          }
-        }
-        if (G::NLS && p.has_proj) {
-          // the plane's non-local rows: row r0 of each sphere point (points outside every
-          // sphere are never read from here)
-          const PointAux *ax = reinterpret_cast<const PointAux *>(hbase + (size_t)hs * G::HSLOT_BYTES + G::IN_BYTES);
-          V *nla = box + (G::IN_BYTES + G::AUX_BYTES + G::STRIP_BYTES) / VB;
-          const V *nlk = reinterpret_cast<const V *>(p.nl) + (long)kb * (p.n_ent + 1) * OV;
-          for (int i = lane; i < TX * TY * OV; i += 32) {
-            const PointAux a = ax[i / OV];
-            if (a.r1 > a.r0) cp_async_16(nla + i, nlk + (long)a.r0 * OV + i % OV);
-          }
-          cp_async_arrive(&hready[hs]);
-        }
+        if (G::NLS && p.has_proj) cp_async_arrive(&hready[hs]);
         __syncwarp();
         if (lane == 0) mbar_arrive(&hready[hs]);
         rp.next<SH>();
@@ -700,22 +801,29 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
     cp_async_wait_all();  // no copy may land after the CTA's shared memory is gone
     return;
   }
+  return;
+  }
+  if constexpr (WW::SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(WW::CONSUMER_REGS));
 
   // ---- consumers: no barrier between warps; a warp that gives up stops, and the others
   // give up at their next wait ----------------------------------------------------------------
+  // (point q = RX r + c of the thread's block: row r, column c; odd blocks of a row are mirrored)
   const int v = tid % OV;
-  const int lx = (tid / OV) % TX;
-  const int ly0 = R * (tid / (OV * TX));
-  const int hs0 = ((ly0 + M) * G::SX + (lx + M)) * OV + v;   // row 0's vector in a halo plane
-  const int tsl0 = ly0 * TX + lx;                             // row 0's point in a tile
-  const int csl0 = tsl0 * OV + v;                             // row 0's vector in a centre plane
+  const int lb = (tid / OV) % (TX / RX);                      // block of the row
+  const int sx = RX == 2 && (lb & 1) ? -OV : OV;              // vector stride from column 0 to column 1
+  const int lx = RX * lb + (sx < 0 ? 1 : 0);                  // column 0's x
+  const int ly0 = R * (tid / (OV * (TX / RX)));
+  const int hs0 = ((ly0 + M) * G::SX + (lx + M)) * OV + v;   // point 0's vector in a halo plane
+  const int tsl0 = ly0 * TX + lx;                             // point 0 in a tile
+  const int csl0 = tsl0 * OV + v;                             // point 0's vector in a centre plane
+  const int dx1 = sx < 0 ? -1 : 1;                            // points from column 0 to column 1
   constexpr int SXO = G::SX * OV;
 
   RingPos rc, rh, ro;  // ring positions of the next centre / halo / operand load
   bool aborted = false;
   int *errp = src.err0();  // then the current item's system's
-  for (long seq = 0;; seq++) {
-    if (!mbar_wait_or_abort(&ibar[seq % IR], (uint32_t)((seq / IR) & 1), abort_flag)) {
+  for (unsigned seq = 0;; seq++) {
+    if (!mbar_wait_or_abort(&ibar[seq % IR], (seq / IR) & 1u, abort_flag)) {
       aborted = true;
       break;
     }
@@ -749,18 +857,18 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
     if constexpr (BLOCH) bloch_phase<P>(p.kvec[3 * kidx + 2] * p.L[2], cz, sz);
     const bool need_grad = BLOCH && p.grad_mask != 0;
     const bool grads = BLOCH && MODE == MODE_FIRST && (p.grad_mask & 8);
-    bool own[R];
+    bool own[NP];
 #pragma unroll
-    for (int r = 0; r < R; r++) own[r] = gx < nx && gy0 + r < ny;
+    for (int q = 0; q < NP; q++) own[q] = gx + (q % RX) * dx1 < nx && gy0 + q / RX < ny;
     const int nl = loads_of<M, U>(0, z0, z1);
-    // vector index of row 0's point in the first output plane (advances one plane per output)
+    // vector index of point 0 in the first output plane (advances one plane per output)
     long idx = ((long)kb * N + ((long)z0 * ny + gy0) * nx + gx) * OV + v;
     const long row = (long)nx * OV;
-    V Q[R][QN];
+    V Q[NP][QN];
 #pragma unroll
-    for (int r = 0; r < R; r++)
+    for (int q = 0; q < NP; q++)
 #pragma unroll
-      for (int j = 0; j < QN; j++) Q[r][j] = T::zero();
+      for (int j = 0; j < QN; j++) Q[q][j] = T::zero();
     ObsAcc<P> oa;
 
     int l = 0;
@@ -777,14 +885,15 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
 #pragma unroll
       for (int u = 0; u < U; u++) {
 #pragma unroll
-        for (int r = 0; r < R; r++) Q[r][(RQ + u) % QN] = cslot[u * CPL + csl0 + r * TX * OV];
+        for (int q = 0; q < NP; q++)
+          Q[q][(RQ + u) % QN] = (cslot + (q % RX) * sx)[u * CPL + csl0 + (q / RX) * TX * OV];
         if constexpr (BLOCH) {
           // a plane beyond a z face was loaded from its periodic image: apply the Bloch phase
           const int zq = z0 - M + U * l + u;
           if ((unsigned)zq >= (unsigned)p.nz) {
             const int wz = floordiv_i(zq, p.nz);
 #pragma unroll
-            for (int r = 0; r < R; r++) Q[r][(RQ + u) % QN] = apply_phase<P>(cz, sz, wz, Q[r][(RQ + u) % QN]);
+            for (int q = 0; q < NP; q++) Q[q][(RQ + u) % QN] = apply_phase<P>(cz, sz, wz, Q[q][(RQ + u) % QN]);
           }
         }
       }
@@ -830,42 +939,46 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
         static_for<0, U>([&](auto uc) {
           constexpr int u = decltype(uc)::value;
           constexpr int QB = (RQ + U + u) % QN;  // queue position of plane (zf + u) - M
-          Rv ve[R];
-          V nlv[R], acc[R];
+          Rv ve[NP];
+          V nlv[NP], acc[NP];
 #pragma unroll
-          for (int r = 0; r < R; r++) {
-            const PointAux a = ax[u * TX * TY + tsl0 + r * TX];
-            ve[r] = *reinterpret_cast<const Rv *>(&a.veff);
+          for (int q = 0; q < NP; q++) {
+            const PointAux a = (ax + (q % RX) * dx1)[u * TX * TY + tsl0 + (q / RX) * TX];
+            ve[q] = *reinterpret_cast<const Rv *>(&a.veff);
             if constexpr (G::NLS) {
               // (gathered into the slot by the patcher warp)
               const V *nla = reinterpret_cast<const V *>(hslot + G::IN_BYTES + G::AUX_BYTES + G::STRIP_BYTES);
-              nlv[r] = has_proj && a.r1 > a.r0 ? nla[(tsl0 + r * TX) * OV + v] : T::zero();
+              nlv[q] = has_proj && a.r1 > a.r0 ? (nla + (q % RX) * sx)[(u * TX * TY + tsl0 + (q / RX) * TX) * OV + v] : T::zero();
             } else {
-              nlv[r] = has_proj ? nl_term<P>(nlk, n_ent, a.r0, a.r1) : T::zero();
+              nlv[q] = has_proj ? nl_term<P>(nlk, n_ent, a.r0, a.r1) : T::zero();
             }
           }
-          V gax[BLOCH ? R : 1][3];
-          if constexpr (BLOCH) {
-            stencil_rows_bloch<M, P, QB, QN, R>(p, W, w0, Q, xs, hs0, SXO, ve, acc, gax, need_grad, grads);
+          [[maybe_unused]] V gax[BLOCH ? NP : 1][3];
+          if constexpr (RX == 2) {
+            stencil_block<M, P, BLOCH, QB, QN>(p, W, w0, Q, xs + u * G::SX * G::SY * OV + hs0, SXO, sx, ve, acc, gax,
+                                               need_grad, grads);
+          } else if constexpr (BLOCH) {
+            stencil_rows_bloch<M, P, QB, QN, R>(p, W, w0, Q, xs + u * G::SX * G::SY * OV, hs0, SXO, ve, acc, gax, need_grad, grads);
           } else {
             stencil_rows<M, P, QB, QN, R>(W, w0, Q, xs + u * G::SX * G::SY * OV, hs0, SXO, ve, acc);
           }
           const long iu = idx + (long)u * plane_pts * OV;
 #pragma unroll
-          for (int r = 0; r < R; r++) {
-            const bool live = own[r] && (zf + u < z1);
-            if (has_proj) acc[r] = T::add(acc[r], nlv[r]);
-            const V c0 = Q[r][(QB + M) % QN];
+          for (int q = 0; q < NP; q++) {
+            const bool live = own[q] && (zf + u < z1);
+            if (has_proj) acc[q] = T::add(acc[q], nlv[q]);
+            const V c0 = Q[q][(QB + M) % QN];
             if (MODE == MODE_FIRST && do_obs && live) {
-              oa.add_e(c0, acc[r]);
+              oa.add_e(c0, acc[q]);
               if constexpr (BLOCH) {
                 if (grads) {
 #pragma unroll
-                  for (int a = 0; a < 3; a++) oa.add_j(a, c0, gax[r][a]);
+                  for (int a = 0; a < 3; a++) oa.add_j(a, c0, gax[q][a]);
                 }
               }
             }
-            finish_point<P, MODE>(epi, CR, CI, live, iu + r * row, v, c0, acc[r], operands(csl0 + r * TX * OV));
+            finish_point<P, MODE>(epi, CR, CI, live, iu + (q / RX) * row + (q % RX) * sx, v, c0, acc[q],
+                                  operands(csl0 + (q / RX) * TX * OV + (q % RX) * sx));
           }
         });
         __syncwarp();
@@ -904,27 +1017,28 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
   }
 }
 
-template <int M, int P, int MODE, int TX, int TY, int R, int U, int BLOCH>
-__global__ void __launch_bounds__(WsWarps<TX, TY, R, VT<P>::OV>::THREADS + 32 * BLOCH, 1)
+template <int M, int P, int MODE, int TX, int TY, int R, int RX, int U, int BLOCH>
+__global__ void __launch_bounds__(WsWarps<TX, TY, R, VT<P>::OV, RX>::THREADS, 1)
 ws_sweep_kernel(const __grid_constant__ SweepMaps maps, const __grid_constant__ SweepParams p) {
   const SingleSrc src{&p, &maps};
-  ws_sweep_body<M, P, MODE, TX, TY, R, U, false, BLOCH>(src, p.work);
+  ws_sweep_body<M, P, MODE, TX, TY, R, RX, U, false, BLOCH>(src, p.work);
 }
 
-template <int M, int P, int MODE, int TX, int TY, int R, int U>
-__global__ void __launch_bounds__(WsWarps<TX, TY, R, VT<P>::OV>::THREADS, 1)
+template <int M, int P, int MODE, int TX, int TY, int R, int RX, int U>
+__global__ void __launch_bounds__(WsWarps<TX, TY, R, VT<P>::OV, RX>::THREADS, 1)
 ws_sweep_batch_kernel(const __grid_constant__ BatchSweepArgs a) {
   const BatchSrc src{&a};
-  ws_sweep_body<M, P, MODE, TX, TY, R, U, true, 0>(src, a.work);
+  ws_sweep_body<M, P, MODE, TX, TY, R, RX, U, true, 0>(src, a.work);
 }
 
 // Launch of the warp-specialised sweep of shape SHAPE for one system (one plane per
 // iteration; grid <= 0: one CTA per SM, at most one per work item).
 template <int SHAPE, int M, int P, int MODE, int BLOCH>
 static cudaError_t launch_ws_t(const SweepMaps &maps, const SweepParams &p, int grid, cudaStream_t s) {
-  constexpr int TX = WsShape<SHAPE>::TX, TY = WsShape<SHAPE>::TY, R = WsShape<SHAPE>::R;
-  typedef TmaGeom<M, TX, TY, 1, MODE == MODE_LAST, BLOCH != 0, MODE == MODE_FIRST> G;
-  auto k = ws_sweep_kernel<M, P, MODE, TX, TY, R, 1, BLOCH>;
+  constexpr int TX = WsShape<SHAPE>::TX, TY = WsShape<SHAPE>::TY, R = WsShape<SHAPE>::R, RX = WsShape<SHAPE>::RX;
+  constexpr int U = WsShape<SHAPE>::U;
+  typedef TmaGeom<M, TX, TY, U, MODE == MODE_LAST, BLOCH != 0, MODE == MODE_FIRST> G;
+  auto k = ws_sweep_kernel<M, P, MODE, TX, TY, R, RX, U, BLOCH>;
   static std::atomic<unsigned> attr_done{0};
   if (cudaError_t e = ensure_smem_attr(k, G::SMEM, attr_done)) return e;
   if (grid <= 0) {
@@ -933,7 +1047,7 @@ static cudaError_t launch_ws_t(const SweepMaps &maps, const SweepParams &p, int 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     grid = (int)(p.n_items < sms ? p.n_items : sms);
   }
-  k<<<grid, WsWarps<TX, TY, R, VT<P>::OV>::THREADS + 32 * BLOCH, G::SMEM, s>>>(maps, p);  // (+ the patcher warp)
+  k<<<grid, WsWarps<TX, TY, R, VT<P>::OV, RX>::THREADS, G::SMEM, s>>>(maps, p);
   return cudaGetLastError();
 }
 
@@ -941,9 +1055,10 @@ static cudaError_t launch_ws_t(const SweepMaps &maps, const SweepParams &p, int 
 // SM, at most one per work item) walk the items of every system of the batch.
 template <int SHAPE, int M, int P, int MODE>
 static cudaError_t launch_ws_batch_t(const BatchSweepArgs &a, cudaStream_t s) {
-  constexpr int TX = WsShape<SHAPE>::TX, TY = WsShape<SHAPE>::TY, R = WsShape<SHAPE>::R;
-  typedef TmaGeom<M, TX, TY, 1, MODE == MODE_LAST> G;
-  auto k = ws_sweep_batch_kernel<M, P, MODE, TX, TY, R, 1>;
+  constexpr int TX = WsShape<SHAPE>::TX, TY = WsShape<SHAPE>::TY, R = WsShape<SHAPE>::R, RX = WsShape<SHAPE>::RX;
+  constexpr int U = WsShape<SHAPE>::U;
+  typedef TmaGeom<M, TX, TY, U, MODE == MODE_LAST, false, MODE == MODE_FIRST> G;
+  auto k = ws_sweep_batch_kernel<M, P, MODE, TX, TY, R, RX, U>;
   static std::atomic<unsigned> attr_done{0};
   if (cudaError_t e = ensure_smem_attr(k, G::SMEM, attr_done)) return e;
   int dev = 0, sms = 0;
@@ -951,9 +1066,20 @@ static cudaError_t launch_ws_batch_t(const BatchSweepArgs &a, cudaStream_t s) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = (int)(a.total_items < sms ? a.total_items : sms);
   if (grid <= 0) return cudaSuccess;
-  k<<<grid, WsWarps<TX, TY, R, VT<P>::OV>::THREADS, G::SMEM, s>>>(a);
+  k<<<grid, WsWarps<TX, TY, R, VT<P>::OV, RX>::THREADS, G::SMEM, s>>>(a);
   return cudaGetLastError();
 }
+
+// Shapes 5 to 7 are complex64 kernels; what runs where is decided by ws_kernel_shape, which the
+// launchers below rely on: shape 5 finite boxes, 6 (order 4 or 8) and 7 (order 4) also periodic
+// cells of order 4.  Shapes 5 and 6 compute one complex value per thread vector, shape 7 two.
+template <int SHAPE> struct C64Shape {
+  static constexpr bool ONLY = SHAPE >= 5;
+  static constexpr int P = SHAPE == 7 || SHAPE == 6 ? P_C64 : P_C64S;
+  static constexpr bool M4 = SHAPE != 7;       // has order-8 kernels
+  static constexpr bool CELL = SHAPE >= 6;     // has periodic-cell kernels (order 4)
+  static constexpr bool LAST = SHAPE == 5;     // has last-term kernels
+};
 
 template <int SHAPE>
 cudaError_t launch_ws_batch_shape(int M, int prec, int mode, const BatchSweepArgs &a, cudaStream_t s) {
@@ -964,11 +1090,20 @@ cudaError_t launch_ws_batch_shape(int M, int prec, int mode, const BatchSweepArg
     case MODE_LAST: return launch_ws_batch_t<SHAPE, MM, PP, MODE_LAST>(a, s);     \
   }                                                                               \
   return cudaErrorInvalidValue;
-  if constexpr (SHAPE == 5) {
-    // complex64: one complex value per thread vector; complex128 runs shape 2
-    if (prec != P_C64) return launch_ws_batch_shape<2>(M, prec, mode, a, s);
-    if (M == 2) { TDKS_WSB_MODES(2, P_C64S) }
-    if (M == 4) { TDKS_WSB_MODES(4, P_C64S) }
+  if constexpr (C64Shape<SHAPE>::ONLY) {
+    if (prec != P_C64) return cudaErrorInvalidValue;
+    constexpr int P = C64Shape<SHAPE>::P;
+    if constexpr (C64Shape<SHAPE>::LAST) {
+      if (M == 2 && mode == MODE_LAST) return launch_ws_batch_t<SHAPE, 2, P, MODE_LAST>(a, s);
+      if constexpr (C64Shape<SHAPE>::M4)
+        if (M == 4 && mode == MODE_LAST) return launch_ws_batch_t<SHAPE, 4, P, MODE_LAST>(a, s);
+    }
+    if (M == 2 && mode == MODE_FIRST) return launch_ws_batch_t<SHAPE, 2, P, MODE_FIRST>(a, s);
+    if (M == 2 && mode == MODE_MID) return launch_ws_batch_t<SHAPE, 2, P, MODE_MID>(a, s);
+    if constexpr (C64Shape<SHAPE>::M4) {
+      if (M == 4 && mode == MODE_FIRST) return launch_ws_batch_t<SHAPE, 4, P, MODE_FIRST>(a, s);
+      if (M == 4 && mode == MODE_MID) return launch_ws_batch_t<SHAPE, 4, P, MODE_MID>(a, s);
+    }
   } else {
     if (M == 2) {
       if (prec == P_C64) { TDKS_WSB_MODES(2, P_C64) } else { TDKS_WSB_MODES(2, P_C128) }
@@ -1007,18 +1142,25 @@ static cudaError_t launch_ws_bc(int M, int prec, int mode, const SweepMaps &maps
 template <int SHAPE>
 cudaError_t launch_ws_shape(int M, int prec, int mode, int bloch, const SweepMaps &maps, const SweepParams &p,
                             int grid, cudaStream_t s) {
-  if constexpr (SHAPE == 5) {
-    // complex64 finite boxes: one complex value per thread vector; the rest run shape 2
-    if (bloch || prec != P_C64) return launch_ws_shape<2>(M, prec, mode, bloch, maps, p, grid, s);
-#define TDKS_WS5_MODES(MM)                                                                       \
+  if constexpr (C64Shape<SHAPE>::ONLY) {
+    constexpr int P = C64Shape<SHAPE>::P;
+    if (prec != P_C64) return cudaErrorInvalidValue;
+#define TDKS_WS5_MODES(MM, BL)                                                                   \
   switch (mode) {                                                                                \
-    case MODE_FIRST: return launch_ws_t<5, MM, P_C64S, MODE_FIRST, 0>(maps, p, grid, s);         \
-    case MODE_MID: return launch_ws_t<5, MM, P_C64S, MODE_MID, 0>(maps, p, grid, s);             \
-    case MODE_LAST: return launch_ws_t<5, MM, P_C64S, MODE_LAST, 0>(maps, p, grid, s);           \
+    case MODE_FIRST: return launch_ws_t<SHAPE, MM, P, MODE_FIRST, BL>(maps, p, grid, s);         \
+    case MODE_MID: return launch_ws_t<SHAPE, MM, P, MODE_MID, BL>(maps, p, grid, s);             \
+    case MODE_LAST:                                                                              \
+      if constexpr (C64Shape<SHAPE>::LAST) return launch_ws_t<SHAPE, MM, P, MODE_LAST, BL>(maps, p, grid, s); \
   }                                                                                              \
   return cudaErrorInvalidValue;
-    if (M == 2) { TDKS_WS5_MODES(2) }
-    if (M == 4) { TDKS_WS5_MODES(4) }
+    if constexpr (C64Shape<SHAPE>::CELL) {
+      if (bloch && M == 2) { TDKS_WS5_MODES(2, 1) }
+    }
+    if (bloch) return cudaErrorInvalidValue;
+    if (M == 2) { TDKS_WS5_MODES(2, 0) }
+    if constexpr (C64Shape<SHAPE>::M4) {
+      if (M == 4) { TDKS_WS5_MODES(4, 0) }
+    }
 #undef TDKS_WS5_MODES
     return cudaErrorInvalidValue;
   } else {
