@@ -115,9 +115,11 @@ struct tdks_system {
   double ts_vol[7] = {0, 0, 0, 0, 0, 0, 0};
   double ts_trel = 0.0, ts_t0 = 0.0;
   bool ts_started = false;
-  // Hartree term (xc = TDKS_XC_LDA_X_HARTREE): padded transform buffer and transformed kernel
-  // (hp[] points per axis), the potential v_H (N doubles); the density goes through n_total
-  double2 *d_hbuf = nullptr, *d_hkern = nullptr;
+  // Hartree term (xc = TDKS_XC_LDA_X_HARTREE), transforms of hp[] points per axis: the half spectrum of
+  // the density, the twiddle tables, the kernel's transform on the half spectrum and the potential
+  // v_H (N doubles); the density goes through n_total
+  double2 *d_hbuf = nullptr, *d_htw = nullptr;
+  double *d_hkern = nullptr;
   double *d_vh = nullptr;
   int hp[3] = {0, 0, 0};
   // clock used by batched propagation: state time, step length, sub-steps per step
