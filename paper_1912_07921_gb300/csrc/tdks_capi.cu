@@ -154,15 +154,26 @@ void sweep_geometry(const tdks_system *s, SweepParams &p, int sweep) {
   int zc = s->zc;
   const bool dynamic = ws_path(s);
   if (zc <= 0 && dynamic) {
-    // warp-specialised TMA sweep: CTAs claim items from a counter, so the cost is the total
-    // work spread over the SMs (the 2M priming planes of an item only load a centre tile,
-    // about a quarter of an output plane each) plus half an item of tail; the items of
-    // one column's z chunks are claimed one after another and share their halo planes in L2.
+    // warp-specialised TMA sweep: CTAs claim items from a counter, one CTA per SM.  The time lies
+    // between that of whole rounds of equal items and that of the work spread evenly plus half an
+    // item of tail.  complex128 (bound by the FP64 pipe, items all alike): the rounds decide; of the
+    // medium molecule's middle term 8 planes measured 1.547 ms, 24 1.585 ms (5% of its last round
+    // empty).  complex64 (edge tiles are shorter): both count; periodic cell 16 of 64 planes 203 us,
+    // 32 204, 64 220; shapes that take two planes at a time want an even number.  An item's priming
+    // planes and set-up cost it ~2 output planes of a complex64 sweep of order 8; next to the FP64
+    // arithmetic of a complex128 plane they are small.
     const long per_plane = (long)p.n_tx * p.n_ty * p.n_kb;
+    const bool c64 = s->prec == TDKS_C64;
+    const int step = sweep >= 0 ? ws_shape_planes(kernel_shape(s, s->wshape[sweep], sweep)) : 1;
+    const double extra = c64 ? 0.5 * s->M : 0.3, spread = c64 ? 1.0 : 0.1;
     double best = -1.0;
-    for (int c = 1; c <= s->nz; c++) {
+    for (int n = 1; n <= s->nz; n++) {
+      int c = (s->nz + n - 1) / n;
+      c = (c + step - 1) / step * step;
       const long items = per_plane * ((s->nz + c - 1) / c);
-      const double cost = (double)items * (c + 0.25 * 2 * s->M) / 152.0 + 0.5 * c;
+      const double even = (double)items * (c + extra) / 152.0 + 0.5 * c;
+      const double rounds = (double)((items + 151) / 152) * (c + extra);
+      const double cost = rounds + spread * even;
       if (best < 0.0 || cost < best) { best = cost; zc = c; }
     }
   } else if (zc <= 0) {

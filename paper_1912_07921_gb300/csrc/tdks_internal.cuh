@@ -81,9 +81,10 @@ struct SweepParams {
   // stencil: H = w0 c + sum_m w[m] (sum of the 6 neighbours at distance m) + ...
   double w[MAXM + 1];         // w[0] = -3 c_0 / (2 h^2), w[m] = -c_m / (2 h^2)
   double gw[MAXM + 1];        // gradient weights d_m / h
-  double cr, ci;              // out = (cr + i ci) * (H in)
+  double coef;                // out = coef H in, or i coef H in (coef_im)
+  int coef_im;
   float wf[MAXM + 1];         // w rounded to FP32 (complex64 sweeps)
-  float crf, cif;             // cr, ci rounded to FP32
+  float coeff;                // coef rounded to FP32
   const void *in;             // stencil input (psi storage in MODE_FIRST, term storage else)
   void *out;                  // term output (MODE_FIRST / MODE_MID)
   void *psi;                  // MODE_LAST: state (complex128, or the hi part of a complex64
@@ -115,12 +116,12 @@ struct SweepParams {
                               // between launches: the launch's last claim resets it)
 };
 
-// Sets the Taylor coefficient (cr + i ci) with its FP32 copies.
+// Sets the coefficient cr + i ci, one of which is zero (H itself, or -i tau/k of a Taylor term), with
+// its FP32 copy.
 inline void set_coef(SweepParams &p, double cr, double ci) {
-  p.cr = cr;
-  p.ci = ci;
-  p.crf = (float)cr;
-  p.cif = (float)ci;
+  p.coef_im = cr == 0.0;
+  p.coef = p.coef_im ? ci : cr;
+  p.coeff = (float)p.coef;
 }
 
 struct GatherParams {
@@ -297,6 +298,8 @@ bool ws_shape_info(int shape, int *tx, int *ty, int *rows, int *warps);
 // run one that does.  Tiles, tensor maps and record counts follow the result.
 // last: the sweep of the last Taylor term.
 int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last);
+// planes a shape's kernel takes per iteration
+int ws_shape_planes(int shape);
 bool tma_supported(int M, int tx, int ty);
 int tma_planes(int prec, int mode, bool lockstep = false);
 int lda_blocks(long N);

@@ -62,7 +62,8 @@ sweep_kernel(const SweepParams p) {
 #pragma unroll
   for (int m = 0; m <= M; m++) W[m] = T::coef(p.w[m], p.wf[m]);
   const typename W0T<P>::type w0 = P == P_C64 ? (typename W0T<P>::type)p.wf[0] : (typename W0T<P>::type)p.w[0];
-  const S CR = T::coef(p.cr, p.crf), CI = T::coef(p.ci, p.cif);
+  const bool kim = p.coef_im != 0;
+  const typename T::K KC = T::kcoef(p.coef, p.coeff, kim);
   const bool need_grad = BLOCH && (p.grad_mask != 0);
   const bool grads = BLOCH && MODE == MODE_FIRST && (p.grad_mask & 8);
 
@@ -176,7 +177,7 @@ sweep_kernel(const SweepParams p) {
           for (int a = 0; a < 3; a++) oa.add_j(a, Q[M], gax[a]);
         }
       }
-      finish_point<P, MODE>(p, CR, CI, own, idx, v, kidx, Q[M], acc, lop);
+      finish_point<P, MODE>(p, KC, kim, own, idx, v, kidx, Q[M], acc, lop);
       // plane z+1 into the other buffer
       V *Sn = sm + (buf ^ 1) * PLANE;
       Sn[csl] = Q[M + 1];

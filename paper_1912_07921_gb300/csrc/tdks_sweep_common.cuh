@@ -96,10 +96,11 @@ stencil_point(const SweepParams &p, const typename VT<P>::S *W, typename W0T<P>:
 
 // Non-local (Kleinman-Bylander) term of a point, precomputed per sphere point by the
 // projector step: nlk = the item's (kb, v) column of nl; row r0 for points with entries,
-// the zero row n_ent for the others (a branch-free load that can be issued early).
+// zero for the others (a predicated load: it can be issued early, and a warp none of whose points
+// is in a sphere, most warps of a molecule, does not wait for it).
 template <int P>
-__device__ __forceinline__ typename VT<P>::V nl_term(const typename VT<P>::V *nlk, int n_ent, int r0, int r1) {
-  return VT<P>::ld(nlk + (long)(r1 > r0 ? r0 : n_ent) * VT<P>::OV);
+__device__ __forceinline__ typename VT<P>::V nl_term(const typename VT<P>::V *nlk, int r0, int r1) {
+  return VT<P>::ld_if(r1 > r0, nlk + (long)r0 * VT<P>::OV);
 }
 template <int P>
 __device__ __forceinline__ const typename VT<P>::V *nl_column(const SweepParams &p, int kb, int v) {
@@ -131,15 +132,15 @@ __device__ __forceinline__ Epi make_epi(const SweepParams &p, int kidx) {
   return Epi{p.out, p.psi, p.psi_lo, p.dens_part, p.wocc[kidx]};
 }
 
-// Epilogue of one output vector.  idx = vector index ((kb*N + pt)*OVC + v); (CR, CI) = the
-// Taylor coefficient, converted to the compute precision once per work item.
+// Epilogue of one output vector.  idx = vector index ((kb*N + pt)*OVC + v); KC, im = the
+// Taylor coefficient (real or imaginary), converted to the compute precision once per work item.
 template <int P, int MODE>
-__device__ __forceinline__ void finish_point(const Epi &ep, typename VT<P>::S CR, typename VT<P>::S CI, bool own,
+__device__ __forceinline__ void finish_point(const Epi &ep, typename VT<P>::K KC, bool im, bool own,
                                              long idx, int v, typename VT<P>::V c0, typename VT<P>::V acc,
                                              const LastOperands<P> &lo_ops) {
   typedef VT<P> T;
   typedef typename T::V V;
-  const V outv = T::cmul(CR, CI, acc);
+  const V outv = T::kmul(KC, im, acc);
   if (MODE != MODE_LAST) {
     if (own) reinterpret_cast<V *>(ep.out)[idx] = outv;
   } else {
@@ -156,10 +157,10 @@ __device__ __forceinline__ void finish_point(const Epi &ep, typename VT<P>::S CR
 }
 
 template <int P, int MODE>
-__device__ __forceinline__ void finish_point(const SweepParams &p, typename VT<P>::S CR, typename VT<P>::S CI,
+__device__ __forceinline__ void finish_point(const SweepParams &p, typename VT<P>::K KC, bool im,
                                              bool own, long idx, int v, int kidx, typename VT<P>::V c0,
                                              typename VT<P>::V acc, const LastOperands<P> &lo_ops) {
-  finish_point<P, MODE>(make_epi(p, kidx), CR, CI, own, idx, v, c0, acc, lo_ops);
+  finish_point<P, MODE>(make_epi(p, kidx), KC, im, own, idx, v, c0, acc, lo_ops);
 }
 
 // Block reduction of the observable partials of one work item into obs_part[item].

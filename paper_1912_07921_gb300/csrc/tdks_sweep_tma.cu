@@ -99,14 +99,14 @@ __device__ __forceinline__ void tma_sweep_body(const Src &src) {
 #pragma unroll
     for (int m = 0; m <= M; m++) W[m] = T::coef(p.w[m], p.wf[m]);
     const typename W0T<P>::type w0 = P == P_C64 ? (typename W0T<P>::type)p.wf[0] : (typename W0T<P>::type)p.w[0];
-    const S_ CR = T::coef(p.cr, p.crf), CI = T::coef(p.ci, p.cif);
+    const bool kim = p.coef_im != 0;
+    const typename T::K KC = T::kcoef(p.coef, p.coeff, kim);
     int tx, ty, kb, z0, z1;
     item_geom(p, local, tx, ty, kb, z0, z1);
     const int kidx = kb / p.n_batches;
     const Epi epi = make_epi(p, kidx);
     const bool has_proj = p.has_proj != 0, do_obs = p.do_obs != 0;
     const V *nlk = nl_column<P>(p, kb, v);
-    const int n_ent = p.n_ent;
     const int gx = tx * TX + lx, gy = ty * TY + ly;
     const bool own = gx < nx && gy < ny;
     const int nl = loads_of<M, U>(0, z0, z1);
@@ -152,7 +152,7 @@ __device__ __forceinline__ void tma_sweep_body(const Src &src) {
           constexpr int QB = (RQ + U + u) % QN;  // queue position of plane (zf + u) - M
           const PointAux a = ax[u * TX * TY + tsl];
           const R ve = *reinterpret_cast<const R *>(&a.veff);
-          const V nlv = has_proj ? nl_term<P>(nlk, n_ent, a.r0, a.r1) : T::zero();
+          const V nlv = has_proj ? nl_term<P>(nlk, a.r0, a.r1) : T::zero();
           V gax[3];
           V acc = stencil_point<M, P, 0, QB, QN>(p, W, w0, Q, xs + u * G::PLANE, hsl, G::SX * OVC, ve, false,
                                                  false, gax);
@@ -160,7 +160,7 @@ __device__ __forceinline__ void tma_sweep_body(const Src &src) {
           if (has_proj) acc = T::add(acc, nlv);
           const V c0 = Q[(QB + M) % QN];
           if (MODE == MODE_FIRST && do_obs && live) oa.add_e(c0, acc);
-          finish_point<P, MODE>(epi, CR, CI, live, idx + (long)u * plane_pts * OVC, v, c0, acc, lop);
+          finish_point<P, MODE>(epi, KC, kim, live, idx + (long)u * plane_pts * OVC, v, c0, acc, lop);
         });
         idx += U * plane_pts * OVC;
       }
@@ -332,6 +332,8 @@ bool ws_shape_info(int shape, int *tx, int *ty, int *rows, int *warps) {
   }
   return false;
 }
+
+int ws_shape_planes(int shape) { return shape == 6 || shape == 8 ? 2 : 1; }
 
 int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last) {
   if (shape < 5) return shape;

@@ -842,19 +842,21 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
 #pragma unroll
     for (int m = 0; m <= M; m++) W[m] = T::coef(p.w[m], p.wf[m]);
     const typename W0T<P>::type w0 = P != P_C128 ? (typename W0T<P>::type)p.wf[0] : (typename W0T<P>::type)p.w[0];
-    const S_ CR = T::coef(p.cr, p.crf), CI = T::coef(p.ci, p.cif);
+    const bool kim = p.coef_im != 0;
+    const typename T::K KC = T::kcoef(p.coef, p.coeff, kim);
     int tx, ty, kb, z0, z1;
     item_geom(p, local, tx, ty, kb, z0, z1);
     const int kidx = kb / p.n_batches;
     const Epi epi = make_epi(p, kidx);
     const bool has_proj = p.has_proj != 0, do_obs = p.do_obs != 0;
     const V *nlk = nl_column<P>(p, kb, v);
-    const int n_ent = p.n_ent;
     const int gx = tx * TX + lx, gy0 = ty * TY + ly0;
     // periodic cell: the Bloch phase of one wrap along z, e^{i k_z L_z} = cz + i sz, applied to
     // the queue planes loaded from beyond a z face (the patcher warp handles x and y)
     S_ cz{}, sz{};
     if constexpr (BLOCH) bloch_phase<P>(p.kvec[3 * kidx + 2] * p.L[2], cz, sz);
+    S_ szm = sz;  // -sz: one wrap the other way
+    if constexpr (P != P_C128) szm ^= SIGN2; else szm = -szm;
     const bool need_grad = BLOCH && p.grad_mask != 0;
     const bool grads = BLOCH && MODE == MODE_FIRST && (p.grad_mask & 8);
     bool own[NP];
@@ -891,9 +893,10 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
           // a plane beyond a z face was loaded from its periodic image: apply the Bloch phase
           const int zq = z0 - M + U * l + u;
           if ((unsigned)zq >= (unsigned)p.nz) {
-            const int wz = floordiv_i(zq, p.nz);
+            // (nz >= M: the planes a live output reads are one wrap away)
+            const S_ s1 = zq < 0 ? szm : sz;
 #pragma unroll
-            for (int q = 0; q < NP; q++) Q[q][(RQ + u) % QN] = apply_phase<P>(cz, sz, wz, Q[q][(RQ + u) % QN]);
+            for (int q = 0; q < NP; q++) Q[q][(RQ + u) % QN] = T::cmul(cz, s1, Q[q][(RQ + u) % QN]);
           }
         }
       }
@@ -950,7 +953,7 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
               const V *nla = reinterpret_cast<const V *>(hslot + G::IN_BYTES + G::AUX_BYTES + G::STRIP_BYTES);
               nlv[q] = has_proj && a.r1 > a.r0 ? (nla + (q % RX) * sx)[(u * TX * TY + tsl0 + (q / RX) * TX) * OV + v] : T::zero();
             } else {
-              nlv[q] = has_proj ? nl_term<P>(nlk, n_ent, a.r0, a.r1) : T::zero();
+              nlv[q] = has_proj ? nl_term<P>(nlk, a.r0, a.r1) : T::zero();
             }
           }
           [[maybe_unused]] V gax[BLOCH ? NP : 1][3];
@@ -977,7 +980,7 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
                 }
               }
             }
-            finish_point<P, MODE>(epi, CR, CI, live, iu + (q / RX) * row + (q % RX) * sx, v, c0, acc[q],
+            finish_point<P, MODE>(epi, KC, kim, live, iu + (q / RX) * row + (q % RX) * sx, v, c0, acc[q],
                                   operands(csl0 + (q / RX) * TX * OV + (q % RX) * sx));
           }
         });

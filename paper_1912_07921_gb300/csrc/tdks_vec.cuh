@@ -108,9 +108,22 @@ template <> struct VT<P_C128> {
   static __device__ __forceinline__ V cmul(S cr, S ci, V a) {
     return make_double2(cr * a.x - ci * a.y, cr * a.y + ci * a.x);
   }
+  // k a or i k a (k real): K = (k, k) or (-k, k), im = the second
+  typedef double2 K;
+  static __device__ __forceinline__ K kcoef(double d, float, bool im) { return make_double2(im ? -d : d, d); }
+  static __device__ __forceinline__ V kmul(K k, bool im, V a) {
+    return make_double2(k.x * (im ? a.y : a.x), k.y * (im ? a.x : a.y));
+  }
   // -i a
   static __device__ __forceinline__ V negi(V a) { return make_double2(a.y, -a.x); }
   static __device__ __forceinline__ V ld(const V *p) { return __ldg(p); }
+  // *p where on, else zero; no branch, and no wait where no lane of the warp loads
+  static __device__ __forceinline__ V ld_if(bool on, const V *p) {
+    V a = zero();
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %3, 0;\n\t@q ld.global.nc.v2.f64 {%0, %1}, [%2];\n\t}"
+        : "+d"(a.x), "+d"(a.y) : "l"(p), "r"((int)on));
+    return a;
+  }
   static __device__ __forceinline__ void to_d(V a, double2 *o) { o[0] = a; }
   static constexpr int CPV = 1;  // complex values per vector
   static constexpr int OV = 4;   // vectors per (point, batch): 64 bytes
@@ -132,11 +145,26 @@ template <> struct VT<P_C64> {
   static __device__ __forceinline__ V cmul(S cr, S ci, V a) {
     return make_ulonglong2(fma2(ci, ipos2(a.x), mul2(cr, a.x)), fma2(ci, ipos2(a.y), mul2(cr, a.y)));
   }
+  typedef u64 K;
+  static __device__ __forceinline__ K kcoef(double, float f, bool im) { return pk2(im ? -f : f, f); }
+  static __device__ __forceinline__ u64 kmul1(K k, bool im, u64 a) {
+    const float2 f = up2(a);
+    return mul2(k, im ? pk2(f.y, f.x) : a);
+  }
+  static __device__ __forceinline__ V kmul(K k, bool im, V a) {
+    return make_ulonglong2(kmul1(k, im, a.x), kmul1(k, im, a.y));
+  }
   static __device__ __forceinline__ V negi(V a) {
     float2 p = up2(a.x), q = up2(a.y);
     return make_ulonglong2(pk2(p.y, -p.x), pk2(q.y, -q.x));
   }
   static __device__ __forceinline__ V ld(const V *p) { return __ldg(p); }
+  static __device__ __forceinline__ V ld_if(bool on, const V *p) {
+    V a = zero();
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %3, 0;\n\t@q ld.global.nc.v2.u64 {%0, %1}, [%2];\n\t}"
+        : "+l"(a.x), "+l"(a.y) : "l"(p), "r"((int)on));
+    return a;
+  }
   static __device__ __forceinline__ void to_d(V a, double2 *o) {
     float2 p = up2(a.x), q = up2(a.y);
     o[0] = make_double2(p.x, p.y);
@@ -161,11 +189,23 @@ template <> struct VT<P_C64S> {
   static __device__ __forceinline__ V mul(S s, V a) { return mul2(s, a); }
   static __device__ __forceinline__ V fma(S s, V a, V c) { return fma2(s, a, c); }
   static __device__ __forceinline__ V cmul(S cr, S ci, V a) { return fma2(ci, ipos2(a), mul2(cr, a)); }
+  typedef u64 K;
+  static __device__ __forceinline__ K kcoef(double, float f, bool im) { return pk2(im ? -f : f, f); }
+  static __device__ __forceinline__ V kmul(K k, bool im, V a) {
+    const float2 f = up2(a);
+    return mul2(k, im ? pk2(f.y, f.x) : a);
+  }
   static __device__ __forceinline__ V negi(V a) {
     const float2 p = up2(a);
     return pk2(p.y, -p.x);
   }
   static __device__ __forceinline__ V ld(const V *p) { return __ldg(reinterpret_cast<const unsigned long long *>(p)); }
+  static __device__ __forceinline__ V ld_if(bool on, const V *p) {
+    V a = 0ull;
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q ld.global.nc.u64 %0, [%1];\n\t}"
+        : "+l"(a) : "l"(p), "r"((int)on));
+    return a;
+  }
   static __device__ __forceinline__ void to_d(V a, double2 *o) {
     const float2 p = up2(a);
     o[0] = make_double2(p.x, p.y);
