@@ -57,12 +57,12 @@ struct ProjEntry {
 };
 
 // One point of one face of the t-SURFF surface: its flat grid index, the face's normal
-// axis, the trapezoid weight times the sign of the outward normal, and its position.
+// axis, its grid indices, and the trapezoid weight times the sign of the outward normal.
 struct TsEntry {
   long cell;
   int ax;
+  int i[3];
   double ws;
-  double r[3];
 };
 
 // Per-point record read by the sweeps (16 bytes): the diagonal potential V_eff (double

@@ -111,6 +111,7 @@ struct tdks_system {
   tdks::TsEntry *d_ts_ent = nullptr;
   double *d_ts_p = nullptr;
   double2 *d_ts_G = nullptr, *d_ts_b = nullptr;
+  double2 *d_ts_E = nullptr, *d_ts_part = nullptr;  // Volkov factors per axis; the flux splits' sums
   int ts_np = 0, ts_ne = 0;
   double ts_vol[7] = {0, 0, 0, 0, 0, 0, 0};
   double ts_trel = 0.0, ts_t0 = 0.0;

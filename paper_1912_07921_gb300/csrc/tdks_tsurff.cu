@@ -10,9 +10,11 @@
 // the trapezoid rule over the configured steps.  The section notes that the method only
 // needs the gradient on the surface points: per step a gather kernel forms, at every surface
 // entry and orbital, w n.(phi, -i grad_h phi), and a flux kernel contracts them with the
-// Volkov factors of every momentum.
+// Volkov factors of every momentum (products of one factor per axis), the entries split over CTAs
+// whose sums are added in order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -61,61 +63,109 @@ __global__ void tsurff_gather_kernel(const TsGather g) {
   g.G1[t] = make_double2(en.ws * gy, -en.ws * gx);
 }
 
+// Volkov factors along each axis: E[p][i] = exp(-i k_p,a x_i) for the nx + ny + nz coordinates of a
+// momentum's three axes, so that a surface point's factor is a product of three (a sine and cosine
+// per momentum and point cost more than the contraction of a few orbitals).
+__global__ void tsurff_factor_kernel(const double *p, double ax, double ay, double az, int n_p, int nx, int ny,
+                                     int nz, double h, double2 *E) {
+  const int nt = nx + ny + nz;
+  const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (t >= (long)n_p * nt) return;
+  const int i = (int)(t % nt), pi = (int)(t / nt);
+  const int a = i < nx ? 0 : (i < nx + ny ? 1 : 2);
+  const int j = a == 0 ? i : (a == 1 ? i - nx : i - nx - ny), n = a == 0 ? nx : (a == 1 ? ny : nz);
+  const double k = p[3 * pi + a] + (a == 0 ? ax : (a == 1 ? ay : az));
+  double sn, cs;
+  sincos(k * ((j - 0.5 * (n - 1)) * h), &sn, &cs);
+  E[t] = make_double2(cs, -sn);
+}
+
 struct TsFlux {
-  int n_e, n_orb, n_p;
+  int n_e, n_orb, n_p, nt, off1, off2;  // nt = nx + ny + nz, off1 = nx, off2 = nx + ny
+  int splits, tile;        // CTAs along the entries; entries per shared-memory tile
   const TsEntry *ent;
-  const double2 *G0, *G1;
+  const double2 *G0, *G1, *E;
   const double *p;         // [n_p][3]
   double a[3], alpha[3], beta, t_rel, weight;
+  double2 *part;           // [splits][n_p][n_orb]
   double2 *b;              // [n_orb][n_p]
 };
 
-constexpr int TS_THREADS = 128;
+constexpr int TS_THREADS = 256;
+constexpr int TS_WMAX = 1024;  // Volkov factors of one shared-memory tile (momenta of the CTA x entries)
 
-// One momentum per CTA; threads over orbitals.  The Volkov factor exp(-i k_p.r_e) of a tile
-// of entries is formed once per CTA in shared memory.
+// Contraction sum_e W_pe (k_p,ax G0_eo + G1_eo) of one split of the entries, one (momentum, orbital)
+// pair per thread: 6 FP64 multiply-adds per entry and pair on GB300's 2-per-clock FP64 pipe, which
+// bounds it, so every lane holds a pair (pairs are numbered through, orbital fastest) and the entries
+// are split over enough CTAs to fill the GPU.  The tile's factors are formed once per CTA; G is read
+// through L1 in runs of orbitals.  One CTA per momentum with a thread per orbital, as before, left
+// 112 of 128 threads idle with 16 orbitals: 48^3 box, 400 momenta, 6.3 ms per flux.
 __global__ void __launch_bounds__(TS_THREADS) tsurff_flux_kernel(const TsFlux f) {
-  __shared__ double2 sW[TS_THREADS];
-  __shared__ double sK[TS_THREADS];
-  const int pi = blockIdx.x, tid = threadIdx.x;
-  const double px = f.p[3 * pi], py = f.p[3 * pi + 1], pz = f.p[3 * pi + 2];
-  const double k[3] = {px + f.a[0], py + f.a[1], pz + f.a[2]};
-  const double phase = 0.5 * ((px * px + py * py + pz * pz) * f.t_rel +
-                              2.0 * (px * f.alpha[0] + py * f.alpha[1] + pz * f.alpha[2]) + f.beta);
-  for (int o0 = 0; o0 < f.n_orb; o0 += TS_THREADS) {
-    const int o = o0 + tid;
-    double ar = 0.0, ai = 0.0;
-    for (int e0 = 0; e0 < f.n_e; e0 += TS_THREADS) {
-      const int e = e0 + tid;
-      if (e < f.n_e) {
-        const TsEntry en = f.ent[e];
-        double sn, cs;
-        sincos(k[0] * en.r[0] + k[1] * en.r[1] + k[2] * en.r[2], &sn, &cs);
-        sW[tid] = make_double2(cs, -sn);
-        sK[tid] = k[en.ax];
-      }
-      __syncthreads();
-      if (o < f.n_orb) {
-        const int ne = min(TS_THREADS, f.n_e - e0);
-        for (int j = 0; j < ne; j++) {
-          const long gi = (long)(e0 + j) * f.n_orb + o;
-          const double2 g0 = f.G0[gi], g1 = f.G1[gi], w = sW[j];
-          const double tr = sK[j] * g0.x + g1.x, ti = sK[j] * g0.y + g1.y;
-          ar += w.x * tr - w.y * ti;
-          ai += w.x * ti + w.y * tr;
-        }
-      }
-      __syncthreads();
+  __shared__ double2 sW[TS_WMAX];
+  __shared__ int sAx[TS_WMAX];
+  const long pairs = (long)f.n_p * f.n_orb, q0 = (long)blockIdx.x * TS_THREADS, q = q0 + threadIdx.x;
+  const bool live = q < pairs;
+  const int p0 = (int)(q0 / f.n_orb);
+  const int np = (int)(min(pairs - 1, q0 + TS_THREADS - 1) / f.n_orb) - p0 + 1;  // momenta of this CTA
+  const int pi = live ? (int)(q / f.n_orb) : p0, o = live ? (int)(q % f.n_orb) : 0, pl = pi - p0;
+  const double k0 = f.p[3 * pi] + f.a[0], k1 = f.p[3 * pi + 1] + f.a[1], k2 = f.p[3 * pi + 2] + f.a[2];
+  const int e_lo = (int)((long)f.n_e * blockIdx.y / f.splits), e_hi = (int)((long)f.n_e * (blockIdx.y + 1) / f.splits);
+  double ar = 0.0, ai = 0.0;
+  for (int e0 = e_lo; e0 < e_hi; e0 += f.tile) {
+    const int ne = min(f.tile, e_hi - e0);
+    __syncthreads();
+    for (int t = threadIdx.x; t < ne * np; t += TS_THREADS) {
+      const int j = t / np, m = t - j * np;
+      const TsEntry &en = f.ent[e0 + j];
+      const double2 *E = f.E + (long)(p0 + m) * f.nt;
+      const double2 x = E[en.i[0]], y = E[f.off1 + en.i[1]], z = E[f.off2 + en.i[2]];
+      const double2 xy = make_double2(x.x * y.x - x.y * y.y, x.x * y.y + x.y * y.x);
+      sW[t] = make_double2(xy.x * z.x - xy.y * z.y, xy.x * z.y + xy.y * z.x);
+      if (m == 0) sAx[j] = en.ax;
     }
-    if (o < f.n_orb) {
-      double sn, cs;
-      sincos(phase, &sn, &cs);
-      const double pref = 0.5 * f.weight * 0.063493635934240969;  // (2 pi)^(-3/2)
-      double2 &bo = f.b[(long)o * f.n_p + pi];
-      bo.x += pref * (cs * ar - sn * ai);
-      bo.y += pref * (cs * ai + sn * ar);
+    __syncthreads();
+    if (live) {
+      const double2 *g0 = f.G0 + (long)e0 * f.n_orb + o, *g1 = f.G1 + (long)e0 * f.n_orb + o;
+#pragma unroll 4
+      for (int j = 0; j < ne; j++) {
+        const double2 x = g0[(long)j * f.n_orb], y = g1[(long)j * f.n_orb], w = sW[j * np + pl];
+        const int ax = sAx[j];
+        const double k = ax == 0 ? k0 : (ax == 1 ? k1 : k2);
+        const double tr = k * x.x + y.x, ti = k * x.y + y.y;
+        ar += w.x * tr - w.y * ti;
+        ai += w.x * ti + w.y * tr;
+      }
     }
   }
+  if (live) f.part[(long)blockIdx.y * pairs + q] = make_double2(ar, ai);
+}
+
+// b += the splits' sums in order, times the time weight and the Volkov phase.
+__global__ void __launch_bounds__(TS_THREADS) tsurff_add_kernel(const TsFlux f) {
+  const long pairs = (long)f.n_p * f.n_orb, q = blockIdx.x * (long)TS_THREADS + threadIdx.x;
+  if (q >= pairs) return;
+  const int pi = (int)(q / f.n_orb), o = (int)(q % f.n_orb);
+  double ar = 0.0, ai = 0.0;
+  for (int s = 0; s < f.splits; s++) {
+    const double2 v = f.part[(long)s * pairs + q];
+    ar += v.x;
+    ai += v.y;
+  }
+  const double px = f.p[3 * pi], py = f.p[3 * pi + 1], pz = f.p[3 * pi + 2];
+  const double phase = 0.5 * ((px * px + py * py + pz * pz) * f.t_rel +
+                              2.0 * (px * f.alpha[0] + py * f.alpha[1] + pz * f.alpha[2]) + f.beta);
+  double sn, cs;
+  sincos(phase, &sn, &cs);
+  const double pref = 0.5 * f.weight * 0.063493635934240969;  // (2 pi)^(-3/2)
+  double2 &bo = f.b[(long)o * f.n_p + pi];
+  bo.x += pref * (cs * ar - sn * ai);
+  bo.y += pref * (cs * ai + sn * ar);
+}
+
+// CTAs along the entries: with the pair tiles, four to an SM, in whole rounds.
+int flux_splits(long pairs, int n_e) {
+  const long tiles = (pairs + TS_THREADS - 1) / TS_THREADS;
+  return (int)std::max(1L, std::min(std::min(64L, (long)n_e), 152L * 4 / tiles));
 }
 
 }  // namespace
@@ -124,6 +174,8 @@ namespace tdks_host {
 
 void tsurff_free(tdks_system *s) {
   cudaFree(s->d_ts_p); cudaFree(s->d_ts_ent); cudaFree(s->d_ts_G); cudaFree(s->d_ts_b);
+  cudaFree(s->d_ts_E); cudaFree(s->d_ts_part);
+  s->d_ts_E = s->d_ts_part = nullptr;
   s->d_ts_p = nullptr; s->d_ts_ent = nullptr; s->d_ts_G = nullptr; s->d_ts_b = nullptr;
   s->ts_np = 0;
   s->ts_ne = 0;
@@ -150,8 +202,19 @@ int tsurff_accumulate(tdks_system *s, double weight) {
   f.t_rel = s->ts_trel;
   f.weight = weight;
   f.b = s->d_ts_b;
-  tsurff_flux_kernel<<<s->ts_np, TS_THREADS, 0, s->stream>>>(f);
-  s->launches += 2;
+  f.E = s->d_ts_E; f.part = s->d_ts_part;
+  f.nt = s->nx + s->ny + s->nz; f.off1 = s->nx; f.off2 = s->nx + s->ny;
+  const long pairs = (long)s->ts_np * s->n_orb;
+  f.splits = flux_splits(pairs, s->ts_ne);
+  // (a CTA's 256 pairs belong to at most 255 / n_orb + 2 momenta, and to no more than there are)
+  f.tile = TS_WMAX / std::min(s->ts_np, (TS_THREADS - 1) / s->n_orb + 2);
+  const long nf = (long)s->ts_np * f.nt;
+  const unsigned tiles = (unsigned)((pairs + TS_THREADS - 1) / TS_THREADS);
+  tsurff_factor_kernel<<<(unsigned)((nf + 127) / 128), 128, 0, s->stream>>>(s->d_ts_p, f.a[0], f.a[1], f.a[2], s->ts_np,
+                                                                           s->nx, s->ny, s->nz, s->h, s->d_ts_E);
+  tsurff_flux_kernel<<<dim3(tiles, f.splits), TS_THREADS, 0, s->stream>>>(f);
+  tsurff_add_kernel<<<tiles, TS_THREADS, 0, s->stream>>>(f);
+  s->launches += 4;
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(TDKS_EDEVICE, std::string("t-SURFF flux: ") + cudaGetErrorString(e));
   return TDKS_OK;
@@ -216,7 +279,7 @@ extern "C" int tdks_set_tsurff(tdks_sys s, const int *box, int n_p, const double
         e.cell = ((long)ii[2] * s->ny + ii[1]) * s->nx + ii[0];
         e.ax = ax;
         e.ws = sgn * w;
-        for (int q = 0; q < 3; q++) e.r[q] = (ii[q] - 0.5 * (n[q] - 1)) * s->h;
+        for (int q = 0; q < 3; q++) e.i[q] = ii[q];
         ent.push_back(e);
       }
   }
@@ -228,6 +291,9 @@ extern "C" int tdks_set_tsurff(tdks_sys s, const int *box, int n_p, const double
   CU(cudaMalloc((void **)&s->d_ts_G, 2 * ent.size() * (size_t)s->n_orb * sizeof(double2)));
   CU(cudaMalloc((void **)&s->d_ts_b, (size_t)s->n_orb * n_p * sizeof(double2)));
   CU(cudaMemset(s->d_ts_b, 0, (size_t)s->n_orb * n_p * sizeof(double2)));
+  const long pairs = (long)s->n_orb * n_p;
+  CU(cudaMalloc((void **)&s->d_ts_E, (size_t)n_p * (s->nx + s->ny + s->nz) * sizeof(double2)));
+  CU(cudaMalloc((void **)&s->d_ts_part, (size_t)flux_splits(pairs, s->ts_ne) * pairs * sizeof(double2)));
   s->ts_np = n_p;
   for (int i = 0; i < 7; i++) s->ts_vol[i] = 0.0;
   s->ts_trel = 0.0;
