@@ -1,7 +1,11 @@
 // Auxiliary kernels of the TDKS library: Kleinman-Bylander gather-dot, density, LDA
 // exchange + effective potential, observable finalisation, layout packing.
+#include <cooperative_groups.h>
+
 #include "tdks_internal.cuh"
 #include "tdks_vec.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace tdks {
 
@@ -10,20 +14,24 @@ namespace tdks {
 //                                         exp(+i (k.T_u + A.d_u)) in(cell(u))[v]
 // (the <beta_aj|psi> of V_NL = sum |beta> D <beta|; the paper's norm-conserving
 // pseudopotentials, Sec. "Magneto-optics" and Sec. "Periodic systems", with synthetic
-// Gaussian-times-polynomial projectors).  Stage 1: n_chunks CTAs per (atom, kb), each
-// summing a contiguous share of the sphere with 64 point lanes x OVC vectors (warp
-// shuffles, then warps through shared memory in a fixed order); stage 2 adds the chunks in
-// order and applies D_aj h^3.  No atomics: the result does not depend on timing.
+// Gaussian-times-polynomial projectors).  n_chunks CTAs per (atom, kb), each summing a contiguous
+// share of the sphere with 64 point lanes x OVC vectors (warp shuffles, then warps through shared
+// memory in a fixed order); their sums are added in chunk order and take D_aj h^3.  For one system
+// the chunks of a unit are a thread-block cluster whose first CTA reads the others' sums from their
+// shared memory; a second launch for that sum, a chain of 16 dependent loads, took longer than the
+// gather itself (64^3, 4 atoms, 2 k-batches: 8.2 + 10 us against 9.5).  Batches keep two launches (their
+// units differ in size).  No atomics: the result does not depend on timing.
 // ---------------------------------------------------------------------------------
 constexpr int GATHER_THREADS = 256;
 
 int gather_chunks(long units) {
   const long want = (152L * 4 + units - 1) / units;
-  return (int)(want < 1 ? 1 : (want > 16 ? 16 : want));
+  return (int)(want < 1 ? 1 : (want > 8 ? 8 : want));  // (8 CTAs: the portable cluster size)
 }
 
+// (out: this CTA's 4 x OVC x 2 sums, index (j OVC + v) 2 + c)
 template <int P, int BLOCH>
-__device__ __forceinline__ void gather_body(const GatherParams &p, int a, int kb, int chunk) {
+__device__ __forceinline__ void gather_body(const GatherParams &p, int a, int kb, int chunk, double2 *out) {
   typedef VT<P> T;
   typedef typename T::V V;
   const int kidx = kb / p.n_batches;
@@ -45,16 +53,9 @@ __device__ __forceinline__ void gather_body(const GatherParams &p, int a, int kb
       const V x = T::ld(reinterpret_cast<const V *>(p.in) + ((long)kb * p.N + ca.x) * OVC + v);
       float c = 1.f, s = 0.f;
       if (phase) {
-        if (p.phase) {
-          const float2 ph = p.phase[(long)kidx * p.n_ent + e];
-          c = ph.x;
-          s = ph.y;
-        } else {
-          const ProjEntry &E = p.ent[e];
-          double ang = p.A[0] * E.d[0] + p.A[1] * E.d[1] + p.A[2] * E.d[2];
-          if (BLOCH) ang += p.kvec[3 * kidx] * E.T[0] + p.kvec[3 * kidx + 1] * E.T[1] + p.kvec[3 * kidx + 2] * E.T[2];
-          sincosf((float)ang, &s, &c);
-        }
+        const float2 ph = reinterpret_cast<const float2 *>(p.phase)[(long)kidx * p.n_ent + e];
+        c = ph.x;
+        s = ph.y;
       }
       const float2 x0 = up2(x.x), x1 = up2(x.y);
       const float2 y0 = make_float2(c * x0.x - s * x0.y, c * x0.y + s * x0.x);
@@ -71,9 +72,9 @@ __device__ __forceinline__ void gather_body(const GatherParams &p, int a, int kb
       const V x = T::ld(reinterpret_cast<const V *>(p.in) + pt * OVC + v);
       double c = 1.0, s = 0.0;
       if (phase) {
-        double ang = p.A[0] * E.d[0] + p.A[1] * E.d[1] + p.A[2] * E.d[2];
-        if (BLOCH) ang += p.kvec[3 * kidx] * E.T[0] + p.kvec[3 * kidx + 1] * E.T[1] + p.kvec[3 * kidx + 2] * E.T[2];
-        sincos(ang, &s, &c);
+        const double2 ph = reinterpret_cast<const double2 *>(p.phase)[(long)kidx * p.n_ent + e];
+        c = ph.x;
+        s = ph.y;
       }
       const double2 xd = *reinterpret_cast<const double2 *>(&x);
       const double xr = c * xd.x - s * xd.y, xi = c * xd.y + s * xd.x;
@@ -119,23 +120,16 @@ __device__ __forceinline__ void gather_body(const GatherParams &p, int a, int kb
       s0.x += red[w][j][vv][0].x; s0.y += red[w][j][vv][0].y;
       s1.x += red[w][j][vv][1].x; s1.y += red[w][j][vv][1].y;
     }
-    double2 *qp = p.qpart + ((((long)(kb * p.n_atoms + a) * p.n_chunks + chunk) * 4 + j) * OVC + vv) * 2;
-    qp[0] = s0;
-    qp[1] = s1;
+    out[2 * tid] = s0;
+    out[2 * tid + 1] = s1;
   }
 }
 
-// Stage 2 for one (atom, kb): thread (j, v) adds the chunk partials in order, times D h^3.
+// q of one (atom, kb, j, v) from its sums, times D h^3.
 template <int P>
-__device__ __forceinline__ void gather_finish(const GatherParams &p, int a, int kb, int t) {
+__device__ __forceinline__ void store_q(const GatherParams &p, int a, int kb, int t, double2 s0, double2 s1) {
   typedef typename VT<P>::V V;
   const int j = t / OVC, vv = t % OVC;
-  double2 s0 = make_double2(0.0, 0.0), s1 = make_double2(0.0, 0.0);
-  for (int c = 0; c < p.n_chunks; c++) {
-    const double2 *qp = p.qpart + ((((long)(kb * p.n_atoms + a) * p.n_chunks + c) * 4 + j) * OVC + vv) * 2;
-    s0.x += qp[0].x; s0.y += qp[0].y;
-    s1.x += qp[1].x; s1.y += qp[1].y;
-  }
   const double f = p.D[4 * a + j] * p.h3;
   V *q = reinterpret_cast<V *>(p.q) + ((long)(kb * p.n_atoms + a) * 4 + j) * OVC + vv;
   if constexpr (P == P_C64) {
@@ -145,17 +139,38 @@ __device__ __forceinline__ void gather_finish(const GatherParams &p, int a, int 
   }
 }
 
+// One system: a cluster of n_chunks CTAs per (atom, kb).
 template <int P, int BLOCH>
 __global__ void __launch_bounds__(GATHER_THREADS) gather_kernel(const GatherParams p) {
-  gather_body<P, BLOCH>(p, blockIdx.x / p.n_chunks, blockIdx.y, blockIdx.x % p.n_chunks);
+  __shared__ double2 part[4 * OVC * 2];
+  const int a = blockIdx.x / p.n_chunks, kb = blockIdx.y, chunk = blockIdx.x % p.n_chunks, t = threadIdx.x;
+  gather_body<P, BLOCH>(p, a, kb, chunk, part);
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  if (chunk == 0 && t < 4 * OVC) {
+    double2 s0 = part[2 * t], s1 = part[2 * t + 1];
+    for (int c = 1; c < p.n_chunks; c++) {
+      const double2 *r = cl.map_shared_rank(part, c);
+      const double2 x = r[2 * t], y = r[2 * t + 1];
+      s0.x += x.x; s0.y += x.y;
+      s1.x += y.x; s1.y += y.y;
+    }
+    store_q<P>(p, a, kb, t, s0, s1);
+  }
+  cl.sync();  // the others' shared memory stays until it has been read
 }
 
-// 16 threads per (atom, kb) unit, 8 units per CTA
+// Batches, stage 2 for one (atom, kb): thread (j, v) adds the chunk partials in order.
 template <int P>
-__global__ void __launch_bounds__(128) gather_finish_kernel(const GatherParams p) {
-  const long u = blockIdx.x * 8L + threadIdx.x / 16;
-  if (u >= (long)p.n_atoms * p.n_kb) return;
-  gather_finish<P>(p, (int)(u % p.n_atoms), (int)(u / p.n_atoms), threadIdx.x % 16);
+__device__ __forceinline__ void gather_finish(const GatherParams &p, int a, int kb, int t) {
+  const int j = t / OVC, vv = t % OVC;
+  double2 s0 = make_double2(0.0, 0.0), s1 = make_double2(0.0, 0.0);
+  for (int c = 0; c < p.n_chunks; c++) {
+    const double2 *qp = p.qpart + ((((long)(kb * p.n_atoms + a) * p.n_chunks + c) * 4 + j) * OVC + vv) * 2;
+    s0.x += qp[0].x; s0.y += qp[0].y;
+    s1.x += qp[1].x; s1.y += qp[1].y;
+  }
+  store_q<P>(p, a, kb, t, s0, s1);
 }
 
 // Non-local term at every point inside a sphere (the scatter half of V_nl):
@@ -186,18 +201,8 @@ __device__ __forceinline__ void nl_body(const GatherParams &p, long t, int kb) {
       x = T::fma(T::coef(0.0, b4.z), T::ld(qa + 2 * OVC), x);
       x = T::fma(T::coef(0.0, b4.w), T::ld(qa + 3 * OVC), x);
       if (phase) {
-        float sn, cs;
-        if (p.phase) {
-          const float2 ph = p.phase[(long)kidx * p.n_ent + ei];
-          cs = ph.x;
-          sn = ph.y;
-        } else {
-          const ProjEntry &E = p.ent[ei];
-          double ang = p.A[0] * E.d[0] + p.A[1] * E.d[1] + p.A[2] * E.d[2];
-          if (BLOCH) ang += p.kvec[3 * kidx] * E.T[0] + p.kvec[3 * kidx + 1] * E.T[1] + p.kvec[3 * kidx + 2] * E.T[2];
-          sincosf((float)ang, &sn, &cs);
-        }
-        x = T::cmul(pk2(cs, cs), pk2(-sn, -sn), x);
+        const float2 ph = reinterpret_cast<const float2 *>(p.phase)[(long)kidx * p.n_ent + ei];
+        x = T::cmul(pk2(ph.x, ph.x), pk2(-ph.y, -ph.y), x);
       }
     } else {
       const ProjEntry &E = p.ent[ei];
@@ -206,11 +211,8 @@ __device__ __forceinline__ void nl_body(const GatherParams &p, long t, int kb) {
 #pragma unroll
       for (int j = 1; j < 4; j++) x = T::fma(E.betad[j], T::ld(qa + j * OVC), x);
       if (phase) {
-        double ang = p.A[0] * E.d[0] + p.A[1] * E.d[1] + p.A[2] * E.d[2];
-        if (BLOCH) ang += p.kvec[3 * kidx] * E.T[0] + p.kvec[3 * kidx + 1] * E.T[1] + p.kvec[3 * kidx + 2] * E.T[2];
-        double sn, cs;
-        sincos(ang, &sn, &cs);
-        x = T::cmul(cs, -sn, x);
+        const double2 ph = reinterpret_cast<const double2 *>(p.phase)[(long)kidx * p.n_ent + ei];
+        x = T::cmul(ph.x, -ph.y, x);
       }
     }
     acc = T::add(acc, x);
@@ -244,7 +246,9 @@ gather_batch_kernel(const GatherParams *gp, const long *begin, const int *sys_of
   const GatherParams &p = gp[s];
   const long u = blockIdx.x - begin[s];
   const long unit = u / p.n_chunks;
-  gather_body<P, 0>(p, (int)(unit % p.n_atoms), (int)(unit / p.n_atoms), (int)(u % p.n_chunks));
+  const int chunk = (int)(u % p.n_chunks);
+  gather_body<P, 0>(p, (int)(unit % p.n_atoms), (int)(unit / p.n_atoms), chunk,
+                    p.qpart + ((long)(unit / p.n_atoms * p.n_atoms + unit % p.n_atoms) * p.n_chunks + chunk) * 8 * OVC);
 }
 
 template <int P>
@@ -308,12 +312,11 @@ constexpr int NLC_THREADS = 128;
 // systems; FP32 products and sums for complex64 systems (the FP64 pipe of GB300 is a small
 // fraction of its FP32 one; the lane sums meet in FP64)
 template <typename F>
-__device__ __forceinline__ void nl_current_lane(const NlCurrentParams &p, int a, int kb, int o, int lane, int lanes,
-                                                double *r) {
+__device__ __forceinline__ void nl_current_lane(const NlCurrentParams &p, int kb, int o, int e0, int e1, int lane,
+                                                int lanes, double *r) {
   const int kidx = kb / p.n_batches;
-  const double kx = p.kvec[3 * kidx], ky = p.kvec[3 * kidx + 1], kz = p.kvec[3 * kidx + 2];
   F pr[4] = {}, pi[4] = {}, qr[4][3] = {}, qi[4][3] = {};
-  for (int e = p.atom_begin[a] + lane; e < p.atom_begin[a + 1]; e += lanes) {
+  for (int e = e0 + lane; e < e1; e += lanes) {
     const ProjEntry &E = p.ent[e];
     const long i = ((long)kb * p.N + E.cell) * p.BS + o;
     F xr, xi;
@@ -326,9 +329,16 @@ __device__ __forceinline__ void nl_current_lane(const NlCurrentParams &p, int a,
       xr = hi.x + lo.x;
       xi = hi.y + lo.y;
     }
-    const double ang = kx * E.T[0] + ky * E.T[1] + kz * E.T[2] + p.A[0] * E.d[0] + p.A[1] * E.d[1] + p.A[2] * E.d[2];
     F sn, cs;
-    if constexpr (sizeof(F) == 8) sincos(ang, &sn, &cs); else sincosf((float)ang, &sn, &cs);
+    if constexpr (sizeof(F) == 8) {
+      const double2 ph = reinterpret_cast<const double2 *>(p.phase)[(long)kidx * p.n_ent + e];
+      cs = ph.x;
+      sn = ph.y;
+    } else {
+      const float2 ph = reinterpret_cast<const float2 *>(p.phase)[(long)kidx * p.n_ent + e];
+      cs = ph.x;
+      sn = ph.y;
+    }
     const F vr = cs * xr - sn * xi, vi = cs * xi + sn * xr;
     F b[4], d[3];
 #pragma unroll
@@ -358,22 +368,43 @@ __device__ __forceinline__ void nl_current_lane(const NlCurrentParams &p, int a,
   }
 }
 
+// A cluster of CTAs per (atom, k-batch), each summing a contiguous share of the atom's entries: with
+// one CTA a small cell's 72 units left half of the SMs idle.  The entries' phases come from the
+// projectors' table.  (8 atoms, 9 k-batches of complex128, with a sine and cosine per entry and lane:
+// 253 us per record.)
 __global__ void __launch_bounds__(NLC_THREADS) nl_current_kernel(const NlCurrentParams p) {
-  const int a = blockIdx.x, kb = blockIdx.y, t = threadIdx.x;
-  const int o = t % p.BS, lane = t / p.BS, lanes = NLC_THREADS / p.BS;
+  const int n_chunks = p.n_chunks, a = blockIdx.x / n_chunks, chunk = blockIdx.x % n_chunks, kb = blockIdx.y;
+  const int t = threadIdx.x, o = t % p.BS, lane = t / p.BS, lanes = NLC_THREADS / p.BS;
   const int kidx = kb / p.n_batches;
-  // sum over the lanes of each orbital in a fixed order
-  __shared__ double red[NLC_THREADS][32];
-  if (p.prec == P_C128) nl_current_lane<double>(p, a, kb, o, lane, lanes, red[t]);
-  else nl_current_lane<float>(p, a, kb, o, lane, lanes, red[t]);
+  // sum over the lanes of each orbital in a fixed order, then over the chunks
+  __shared__ double red[NLC_THREADS][33];
+  __shared__ double part[8][32];  // [orbital][component]
+  const int a0 = p.atom_begin[a], a1 = p.atom_begin[a + 1], len = (a1 - a0 + n_chunks - 1) / n_chunks;
+  const int e0 = a0 + chunk * len, e1 = min(a1, e0 + len);
+  if (p.prec == P_C128) nl_current_lane<double>(p, kb, o, e0, e1, lane, lanes, red[t]);
+  else nl_current_lane<float>(p, kb, o, e0, e1, lane, lanes, red[t]);
   __syncthreads();
-  if (t < p.BS) {
+  for (int i = t; i < 32 * p.BS; i += NLC_THREADS) {
+    const int oo = i % p.BS, c = i / p.BS;
+    double x = 0.0;
+    for (int l = 0; l < lanes; l++) x += red[l * p.BS + oo][c];
+    part[oo][c] = x;
+  }
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  if (chunk == 0 && t < p.BS) {
     double sum[32];
-    for (int c = 0; c < 32; c++) sum[c] = 0.0;
-    for (int l = 0; l < lanes; l++)
-      for (int c = 0; c < 32; c++) sum[c] += red[l * p.BS + t][c];
+#pragma unroll
+    for (int c = 0; c < 32; c++) sum[c] = part[t][c];
+    for (int q = 1; q < n_chunks; q++) {
+      const double *r = cl.map_shared_rank(&part[0][0], q) + 32 * t;
+#pragma unroll
+      for (int c = 0; c < 32; c++) sum[c] += r[c];
+    }
     double vel[3] = {0.0, 0.0, 0.0};
+#pragma unroll
     for (int j = 0; j < 4; j++)
+#pragma unroll
       for (int x = 0; x < 3; x++) {
         // Im(p^* q) = p_r q_i - p_i q_r
         const double im = sum[8 * j] * sum[8 * j + 3 + 2 * x] - sum[8 * j + 1] * sum[8 * j + 2 + 2 * x];
@@ -386,54 +417,85 @@ __global__ void __launch_bounds__(NLC_THREADS) nl_current_kernel(const NlCurrent
     out[2] = f * vel[1];
     out[3] = f * vel[2];
   }
+  cl.sync();  // the others' shared memory stays until it has been read
 }
 
-cudaError_t launch_nl_current(const NlCurrentParams &p, cudaStream_t s) {
-  nl_current_kernel<<<dim3(p.n_atoms, p.n_kb), NLC_THREADS, 0, s>>>(p);
-  return cudaGetLastError();
+cudaError_t launch_nl_current(const NlCurrentParams &q, cudaStream_t s) {
+  NlCurrentParams p = q;
+  p.n_chunks = gather_chunks((long)p.n_atoms * p.n_kb);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(p.n_atoms * p.n_chunks, p.n_kb);
+  cfg.blockDim = dim3(NLC_THREADS);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = p.n_chunks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, nl_current_kernel, p);
 }
 
+// Entry phases (cos, sin) of k.T + A.d, as the projector kernels read them: for complex64 systems the
+// FP32 sine and cosine of the FP64 angle, for complex128 FP64 ones.  (In FP64 a sine and cosine cost
+// more than an entry's products; formed in the kernels they were evaluated for every k-batch, vector
+// and Taylor term, and bounded them.)
+template <int P>
 __global__ void phase_table_kernel(const ProjEntry *ent, int n_ent, int n_k, const double *kvec, double Ax,
-                                   double Ay, double Az, int bloch, float2 *out) {
+                                   double Ay, double Az, int bloch, void *out) {
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= (long)n_ent * n_k) return;
   const int e = (int)(i % n_ent), k = (int)(i / n_ent);
   const ProjEntry &E = ent[e];
   double ang = Ax * E.d[0] + Ay * E.d[1] + Az * E.d[2];
   if (bloch) ang += kvec[3 * k] * E.T[0] + kvec[3 * k + 1] * E.T[1] + kvec[3 * k + 2] * E.T[2];
-  float sn, cs;
-  sincosf((float)ang, &sn, &cs);
-  out[i] = make_float2(cs, sn);
+  if constexpr (P == P_C64) {
+    float sn, cs;
+    sincosf((float)ang, &sn, &cs);
+    reinterpret_cast<float2 *>(out)[i] = make_float2(cs, sn);
+  } else {
+    double sn, cs;
+    sincos(ang, &sn, &cs);
+    reinterpret_cast<double2 *>(out)[i] = make_double2(cs, sn);
+  }
 }
 
-cudaError_t launch_phase_table(const ProjEntry *ent, int n_ent, int n_k, const double *kvec, const double A[3],
-                               int bloch, float2 *out, cudaStream_t s) {
+cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_k, const double *kvec,
+                               const double A[3], int bloch, void *out, cudaStream_t s) {
   const long n = (long)n_ent * n_k;
   if (n <= 0) return cudaSuccess;
-  phase_table_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ent, n_ent, n_k, kvec, A[0], A[1], A[2], bloch,
-                                                                 out);
+  const unsigned grid = (unsigned)((n + 127) / 128);
+  if (prec == P_C64)
+    phase_table_kernel<P_C64><<<grid, 128, 0, s>>>(ent, n_ent, n_k, kvec, A[0], A[1], A[2], bloch, out);
+  else
+    phase_table_kernel<P_C128><<<grid, 128, 0, s>>>(ent, n_ent, n_k, kvec, A[0], A[1], A[2], bloch, out);
+  return cudaGetLastError();
+}
+
+template <int P, int BLOCH>
+static cudaError_t launch_gather_t(const GatherParams &p, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(p.n_atoms * p.n_chunks, p.n_kb);
+  cfg.blockDim = dim3(GATHER_THREADS);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = p.n_chunks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaError_t e = cudaLaunchKernelEx(&cfg, gather_kernel<P, BLOCH>, p)) return e;
+  if (p.n_sp > 0) {
+    const dim3 grid((unsigned)(((long)p.n_sp * OVC + NL_THREADS - 1) / NL_THREADS), nl_kb_rows(p.n_kb));
+    nl_kernel<P, BLOCH><<<grid, NL_THREADS, 0, s>>>(p);
+  }
   return cudaGetLastError();
 }
 
 cudaError_t launch_gather(int prec, int bloch, const GatherParams &p, cudaStream_t s) {
   if (p.n_atoms <= 0) return cudaSuccess;
-  dim3 grid(p.n_atoms * p.n_chunks, p.n_kb);
-  const unsigned fgrid = (unsigned)(((long)p.n_atoms * p.n_kb + 7) / 8);
-  const dim3 ngrid((unsigned)(((long)p.n_sp * OVC + NL_THREADS - 1) / NL_THREADS), nl_kb_rows(p.n_kb));
-  if (prec == P_C64) {
-    if (bloch) gather_kernel<P_C64, 1><<<grid, GATHER_THREADS, 0, s>>>(p);
-    else gather_kernel<P_C64, 0><<<grid, GATHER_THREADS, 0, s>>>(p);
-    gather_finish_kernel<P_C64><<<fgrid, 128, 0, s>>>(p);
-    if (p.n_sp > 0 && bloch) nl_kernel<P_C64, 1><<<ngrid, NL_THREADS, 0, s>>>(p);
-    else if (p.n_sp > 0) nl_kernel<P_C64, 0><<<ngrid, NL_THREADS, 0, s>>>(p);
-  } else {
-    if (bloch) gather_kernel<P_C128, 1><<<grid, GATHER_THREADS, 0, s>>>(p);
-    else gather_kernel<P_C128, 0><<<grid, GATHER_THREADS, 0, s>>>(p);
-    gather_finish_kernel<P_C128><<<fgrid, 128, 0, s>>>(p);
-    if (p.n_sp > 0 && bloch) nl_kernel<P_C128, 1><<<ngrid, NL_THREADS, 0, s>>>(p);
-    else if (p.n_sp > 0) nl_kernel<P_C128, 0><<<ngrid, NL_THREADS, 0, s>>>(p);
-  }
-  return cudaGetLastError();
+  if (prec == P_C64) return bloch ? launch_gather_t<P_C64, 1>(p, s) : launch_gather_t<P_C64, 0>(p, s);
+  return bloch ? launch_gather_t<P_C128, 1>(p, s) : launch_gather_t<P_C128, 0>(p, s);
 }
 
 // ---------------------------------------------------------------------------------
@@ -513,10 +575,15 @@ cudaError_t launch_density(int prec, long N, int n_kb, int n_batches, const void
 // gauge, finite box) + |A|^2/2 (velocity gauge).  Per-block partial sums for the
 // observables: [int n, int n e_x, int n v_x, int x n, int y n, int z n] (before h^3).
 // ---------------------------------------------------------------------------------
-constexpr int LDA_THREADS = 256;
+constexpr int LDA_THREADS = 256;  // most threads of a CTA (and those of a batch's CTAs)
 
+// Threads per CTA of one system's launch: a small grid's points are spread over all SMs (a complex128
+// point's cube root is ~150 FP64 instructions at 2 per clock and SM: 24^3 points in 54 CTAs of 256
+// threads took 10.4 us, in 432 of 32 4.3 us).
+static int lda_threads(long N) { return N <= 608 * 32 ? 32 : (N <= 608 * 64 ? 64 : (N <= 608 * 256 ? 128 : LDA_THREADS)); }
 int lda_blocks(long N) {
-  long g = (N + LDA_THREADS - 1) / LDA_THREADS;
+  const int t = lda_threads(N);
+  const long g = (N + t - 1) / t;
   return (int)(g < 152 * 4 ? g : 152 * 4);
 }
 
@@ -621,20 +688,28 @@ __device__ __forceinline__ void lda_body(long N, int nx, int ny, int nz, double 
     }
   }
   if (!sums) return;  // (uniform over the grid: V_eff only, no record follows)
-  if constexpr (F32) {
-#pragma unroll
-    for (int c = 0; c < 6; c++) acc[c] = (double)fh[c] + (double)fl[c];
-  }
   __shared__ double red[LDA_THREADS / 32][6];
+#pragma unroll
   for (int i = 0; i < 6; i++) {
-    double x = acc[i];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    double x;
+    if constexpr (F32) {
+      // (lanes meet as double-float: five FP64 sums per value and warp cost more than the points)
+      float h = fh[i], l = fl[i];
+      for (int o = 16; o > 0; o >>= 1) {
+        const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
+        df_add_df(h, l, oh, ol);
+      }
+      x = (double)h + (double)l;
+    } else {
+      x = acc[i];
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    }
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][i] = x;
   }
   __syncthreads();
   if (threadIdx.x < 6) {
     double x = 0.0;
-    for (int w = 0; w < LDA_THREADS / 32; w++) x += red[w][threadIdx.x];
+    for (int w = 0; w < (int)blockDim.x / 32; w++) x += red[w][threadIdx.x];
     lda_part[blk * 6 + threadIdx.x] = x;
   }
 }
@@ -720,9 +795,9 @@ cudaError_t launch_rk4_finish(long n, void *psi, const void *acc, const void *k,
 cudaError_t launch_density_sum(int prec, long N, int n_kb, int n_batches, const double *wocc,
                                const double *dens_part, double *n_out, cudaStream_t s) {
   if (prec == P_C64)
-    density_sum_kernel<float><<<lda_blocks(N), LDA_THREADS, 0, s>>>(N, n_kb, n_batches, wocc, dens_part, n_out);
+    density_sum_kernel<float><<<lda_blocks(N), lda_threads(N), 0, s>>>(N, n_kb, n_batches, wocc, dens_part, n_out);
   else
-    density_sum_kernel<double><<<lda_blocks(N), LDA_THREADS, 0, s>>>(N, n_kb, n_batches, wocc, dens_part, n_out);
+    density_sum_kernel<double><<<lda_blocks(N), lda_threads(N), 0, s>>>(N, n_kb, n_batches, wocc, dens_part, n_out);
   return cudaGetLastError();
 }
 
@@ -807,10 +882,10 @@ cudaError_t launch_cfm_veff(int prec, int bloch, long N, int nx, int ny, int nz,
                             const double *vh, const double *n_in) {
   const int blocks = lda_blocks(N);
   if (prec == P_C64)
-    cfm_veff_kernel<float><<<blocks, LDA_THREADS, 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
+    cfm_veff_kernel<float><<<blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
                                                           vloc, xc, push, hist, E[0], E[1], E[2], aux, vh, n_in);
   else
-    cfm_veff_kernel<double><<<blocks, LDA_THREADS, 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
+    cfm_veff_kernel<double><<<blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
                                                            vloc, xc, push, hist, E[0], E[1], E[2], aux, vh, n_in);
   return cudaGetLastError();
 }
@@ -865,11 +940,11 @@ cudaError_t launch_lda(int prec, int bloch, long N, int nx, int ny, int nz, doub
                        double half_A2, PointAux *aux, double *lda_part, int n_blocks, cudaStream_t s,
                        const double *n_in, const double *vh, int sums) {
   if (prec == P_C64)
-    lda_kernel<float><<<n_blocks, LDA_THREADS, 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
+    lda_kernel<float><<<n_blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
                                                        vloc, xc, E[0], E[1], E[2], half_A2, aux, lda_part, n_in, vh,
                                                        sums);
   else
-    lda_kernel<double><<<n_blocks, LDA_THREADS, 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
+    lda_kernel<double><<<n_blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
                                                         vloc, xc, E[0], E[1], E[2], half_A2, aux, lda_part, n_in, vh,
                                                         sums);
   return cudaGetLastError();
@@ -903,11 +978,12 @@ __device__ __forceinline__ void write_record(const double O[4], const double Lq[
   rec[7] = field_val;
 }
 
-// Sum of the 10 per-thread values v over the CTA (FIN_THREADS threads): a fixed xor tree
+// Sum of the 10 per-thread values v over the CTA: a fixed xor tree
 // within each warp, then the warps in order; thread c < 10 returns component c.
-constexpr int FIN_THREADS = 128;
+constexpr int FIN_THREADS = 128;       // batches: one CTA per system
+constexpr int FIN_MAX_THREADS = 256;   // one system: a cluster of CTAs
 __device__ __forceinline__ double block_sum10(double v[10], int t) {
-  __shared__ double red[FIN_THREADS / 32][10];
+  __shared__ double red[FIN_MAX_THREADS / 32][10];
 #pragma unroll
   for (int c = 0; c < 10; c++) {
     double x = v[c];
@@ -917,7 +993,7 @@ __device__ __forceinline__ double block_sum10(double v[10], int t) {
   __syncthreads();
   double x = 0.0;
   if (t < 10)
-    for (int w = 0; w < FIN_THREADS / 32; w++) x += red[w][t];
+    for (int w = 0; w < (int)blockDim.x / 32; w++) x += red[w][t];
   return x;
 }
 
@@ -925,9 +1001,9 @@ __device__ __forceinline__ double block_sum10(double v[10], int t) {
 __device__ __forceinline__ double partial_sums(const double *obs_part, long i0, long i1, const double *lda_part,
                                                long l0, long l1, int t) {
   double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-  for (long i = i0 + t; i < i1; i += FIN_THREADS)
+  for (long i = i0 + t; i < i1; i += blockDim.x)
     for (int c = 0; c < 4; c++) v[c] += obs_part[i * 4 + c];
-  for (long i = l0 + t; i < l1; i += FIN_THREADS)
+  for (long i = l0 + t; i < l1; i += blockDim.x)
     for (int c = 0; c < 6; c++) v[4 + c] += lda_part[i * 6 + c];
   return block_sum10(v, t);
 }
@@ -945,29 +1021,33 @@ __device__ __forceinline__ void finalize_body(const double *obs_part, long n_ite
   if (t == 0) write_record(tot, tot + 4, rec, t_state, h3, occ, bloch, omega_cell, Ax, Ay, Az, field_val);
 }
 
-// Two stages for one system: CTA b of stage 1 sums the b-th contiguous share of the
-// partials; stage 2 adds the CTAs' sums in order.  The shares depend only on the counts,
-// so the record is the same on every run.
-__global__ void __launch_bounds__(FIN_THREADS)
-finalize_stage1_kernel(const double *obs_part, long n_items, const double *lda_part, int n_lda, double *fin_part) {
+// One system: a cluster of CTAs, CTA b of which sums the b-th contiguous share of the partials; the
+// first adds the CTAs' sums in order and writes the record (rec), or the 10 sums (sums).  The shares
+// depend only on the counts, so the record is the same on every run.  (Two launches with the sums
+// in between, 64 CTAs and one, took 7.4 + 4.0 us on the tiny molecule.)
+__global__ void __launch_bounds__(FIN_MAX_THREADS)
+finalize_kernel(const double *obs_part, long n_items, const double *lda_part, int n_lda, double *sums, double *rec,
+                double t_state, double h3, double occ, int bloch, double omega_cell, double Ax, double Ay, double Az,
+                double field_val) {
+  __shared__ double part[10], tot[10];
   const long b = blockIdx.x, nb = gridDim.x;
-  const double x = partial_sums(obs_part, n_items * b / nb, n_items * (b + 1) / nb, lda_part, n_lda * b / nb,
-                                n_lda * (b + 1) / nb, threadIdx.x);
-  if (threadIdx.x < 10) fin_part[b * 10 + threadIdx.x] = x;
-}
-
-__global__ void __launch_bounds__(32)
-finalize_stage2_kernel(const double *fin_part, int nb, double *rec, double t_state, double h3, double occ,
-                       int bloch, double omega_cell, double Ax, double Ay, double Az, double field_val) {
-  __shared__ double tot[10];
   const int t = threadIdx.x;
-  if (t < 10) {
-    double x = 0.0;
-    for (int b = 0; b < nb; b++) x += fin_part[b * 10 + t];
-    tot[t] = x;
+  const double x = partial_sums(obs_part, n_items * b / nb, n_items * (b + 1) / nb, lda_part, n_lda * b / nb,
+                                n_lda * (b + 1) / nb, t);
+  if (t < 10) part[t] = x;
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  if (b == 0) {
+    if (t < 10) {
+      double y = 0.0;
+      for (int c = 0; c < nb; c++) y += cl.map_shared_rank(part, c)[t];
+      if (sums) sums[t] = y;
+      else tot[t] = y;
+    }
+    __syncwarp();
+    if (!sums && t == 0) write_record(tot, tot + 4, rec, t_state, h3, occ, bloch, omega_cell, Ax, Ay, Az, field_val);
   }
-  __syncwarp();
-  if (t == 0) write_record(tot, tot + 4, rec, t_state, h3, occ, bloch, omega_cell, Ax, Ay, Az, field_val);
+  cl.sync();  // the CTAs' sums stay until they have been read
 }
 
 // Batched observable records: one CTA per system, at the first sub-step of each step.
@@ -1002,32 +1082,37 @@ cudaError_t launch_batch_tail(const BatchAux *aux, BatchClock *clk, int n_sys, i
   return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(32) finalize_sums_kernel(const double *fin_part, int nb, double *sums) {
-  const int t = threadIdx.x;
-  if (t < 10) {
-    double x = 0.0;
-    for (int b = 0; b < nb; b++) x += fin_part[b * 10 + t];
-    sums[t] = x;
-  }
-}
-
 __global__ void __launch_bounds__(32)
 record_from_sums_kernel(const double *sums, double *rec, double t_state, double h3, double occ, int bloch,
                         double omega_cell, double Ax, double Ay, double Az, double field_val) {
   if (threadIdx.x == 0) write_record(sums, sums + 4, rec, t_state, h3, occ, bloch, omega_cell, Ax, Ay, Az, field_val);
 }
 
-static int finalize_blocks(long n_items, int n_lda) {
-  const long want = (n_items + n_lda + 4L * FIN_THREADS - 1) / (4L * FIN_THREADS);
-  return (int)(want < 1 ? 1 : (want > FIN_BLOCKS ? FIN_BLOCKS : want));
+// CTAs of a record: one per 4 records a thread, at most a portable cluster's eight.
+static cudaError_t launch_finalize_cluster(const double *obs_part, long n_items, const double *lda_part, int n_lda,
+                                           double *sums, double *rec, double t_state, double h3, double occ,
+                                           int bloch, double omega_cell, double Ax, double Ay, double Az,
+                                           double field_val, cudaStream_t s) {
+  const long want = (n_items + n_lda + 4L * FIN_MAX_THREADS - 1) / (4L * FIN_MAX_THREADS);
+  const unsigned nb = (unsigned)(want < 1 ? 1 : (want > 8 ? 8 : want));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(nb);
+  cfg.blockDim = dim3(FIN_MAX_THREADS);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = nb;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, finalize_kernel, obs_part, n_items, lda_part, n_lda, sums, rec, t_state, h3, occ,
+                            bloch, omega_cell, Ax, Ay, Az, field_val);
 }
 
 cudaError_t launch_finalize_sums(const double *obs_part, long n_items, const double *lda_part, int n_lda,
-                                 double *fin_part, double *sums, cudaStream_t s) {
-  const int nb = finalize_blocks(n_items, n_lda);
-  finalize_stage1_kernel<<<nb, FIN_THREADS, 0, s>>>(obs_part, n_items, lda_part, n_lda, fin_part);
-  finalize_sums_kernel<<<1, 32, 0, s>>>(fin_part, nb, sums);
-  return cudaGetLastError();
+                                 double *sums, cudaStream_t s) {
+  return launch_finalize_cluster(obs_part, n_items, lda_part, n_lda, sums, nullptr, 0.0, 0.0, 1.0, 0, 1.0, 0.0, 0.0,
+                                 0.0, 0.0, s);
 }
 
 cudaError_t launch_record_from_sums(const double *sums, double *record, double t_state, double h3, double occ,
@@ -1040,13 +1125,9 @@ cudaError_t launch_record_from_sums(const double *sums, double *record, double t
 
 cudaError_t launch_finalize(const double *obs_part, long n_items, const double *lda_part, int n_lda,
                             double *record, double t_state, double h3, double occ, int bloch,
-                            double omega_cell, const double A[3], double field_val, double *fin_part,
-                            cudaStream_t s) {
-  const int nb = finalize_blocks(n_items, n_lda);
-  finalize_stage1_kernel<<<nb, FIN_THREADS, 0, s>>>(obs_part, n_items, lda_part, n_lda, fin_part);
-  finalize_stage2_kernel<<<1, 32, 0, s>>>(fin_part, nb, record, t_state, h3, occ, bloch, omega_cell, A[0], A[1],
-                                          A[2], field_val);
-  return cudaGetLastError();
+                            double omega_cell, const double A[3], double field_val, cudaStream_t s) {
+  return launch_finalize_cluster(obs_part, n_items, lda_part, n_lda, nullptr, record, t_state, h3, occ, bloch,
+                                 omega_cell, A[0], A[1], A[2], field_val, s);
 }
 
 // ---------------------------------------------------------------------------------

@@ -64,7 +64,7 @@ void batch_free(tdks_batch *b) {
 // partial buffer it fills), i.e. ~16 points per thread, so that the launch over all systems pays
 // each CTA's setup (system lookup, field, weight staging) a few times per SM rather than once per
 // CTA-sized run of points.
-static int lda_batch_blocks(long N) { return std::max(1, (lda_blocks(N) + 15) / 16); }
+static int lda_batch_blocks(long N) { return (int)std::max(1L, (std::min((N + 255) / 256, 608L) + 15) / 16); }
 
 // Kernels one sub-step launches: the LDA/V_eff kernel, per Taylor term the projector step
 // (gather stages 1 and 2 and the non-local term, where any system has atoms) and the sweep,

@@ -323,6 +323,21 @@ int run_sweep(tdks_system *s, int mode, SweepParams &p, const SweepMaps *tm, int
   return TDKS_OK;
 }
 
+// The entries' phases for vector potential A, built where they are not the ones at hand.
+int entry_phases(tdks_system *s, const double A[3], const void **out) {
+  const size_t bytes = (size_t)s->n_ent * s->n_k * (s->prec == TDKS_C64 ? sizeof(float2) : sizeof(double2));
+  if (!s->d_phase) CU(cudaMalloc(&s->d_phase, bytes));
+  if (!s->phase_ok || A[0] != s->phase_A[0] || A[1] != s->phase_A[1] || A[2] != s->phase_A[2]) {
+    CU(launch_phase_table(s->prec, s->d_ent, s->n_ent, s->n_k, s->d_kvec, A, s->bc == TDKS_BC_BLOCH, s->d_phase,
+                          s->stream));
+    s->launches++;
+    for (int a = 0; a < 3; a++) s->phase_A[a] = A[a];
+    s->phase_ok = true;
+  }
+  *out = s->d_phase;
+  return TDKS_OK;
+}
+
 int run_gather(tdks_system *s, const void *in, const double A[3]) {
   if (s->n_atoms <= 0) return TDKS_OK;
   GatherParams g{};
@@ -341,20 +356,11 @@ int run_gather(tdks_system *s, const void *in, const double A[3]) {
   g.nl = s->d_nl;
   g.phase = nullptr;
   const bool bloch = s->bc == TDKS_BC_BLOCH;
-  if (s->prec == TDKS_C64 && (bloch || g.A[0] != 0.0 || g.A[1] != 0.0 || g.A[2] != 0.0)) {
-    // the entries' phases for this vector potential, once for the Taylor terms that share it
-    if (!s->d_phase) CU(cudaMalloc((void **)&s->d_phase, (size_t)s->n_ent * s->n_k * sizeof(float2)));
-    if (!s->phase_ok || g.A[0] != s->phase_A[0] || g.A[1] != s->phase_A[1] || g.A[2] != s->phase_A[2]) {
-      CU(launch_phase_table(s->d_ent, s->n_ent, s->n_k, s->d_kvec, g.A, bloch, s->d_phase, s->stream));
-      s->launches++;
-      for (int a = 0; a < 3; a++) s->phase_A[a] = g.A[a];
-      s->phase_ok = true;
-    }
-    g.phase = s->d_phase;
-  }
+  if (bloch || g.A[0] != 0.0 || g.A[1] != 0.0 || g.A[2] != 0.0)
+    if (int rc = entry_phases(s, g.A, &g.phase)) return rc;
   Timed tm(s, 1);
   cudaError_t e = launch_gather(s->prec, bloch, g, s->stream);
-  s->launches += s->n_sp > 0 ? 3 : 2;  // gather stages 1 and 2, the non-local term
+  s->launches += s->n_sp > 0 ? 2 : 1;  // the gather, the non-local term
   if (e != cudaSuccess) return fail(TDKS_EDEVICE, std::string("projector gather: ") + cudaGetErrorString(e));
   return TDKS_OK;
 }
@@ -408,8 +414,10 @@ int run_finalize(tdks_system *s, double *rec, double t_state, const double E[3],
     NlCurrentParams q{};
     q.prec = s->prec; q.BS = s->BS; q.n_batches = s->n_batches; q.n_kb = s->n_kb; q.n_atoms = s->n_atoms;
     q.N = s->N; q.psi = s->psi; q.psi_lo = s->psi_lo; q.atom_begin = s->d_atom_begin; q.ent = s->d_ent;
-    q.D = s->d_D; q.kvec = s->d_kvec; q.wocc = s->d_wocc; q.h3 = h3;
-    for (int a = 0; a < 3; a++) q.A[a] = s->gauge == TDKS_GAUGE_VELOCITY ? A[a] : 0.0;
+    q.D = s->d_D; q.n_ent = s->n_ent; q.wocc = s->d_wocc; q.h3 = h3;
+    const double Av[3] = {s->gauge == TDKS_GAUGE_VELOCITY ? A[0] : 0.0, s->gauge == TDKS_GAUGE_VELOCITY ? A[1] : 0.0,
+                          s->gauge == TDKS_GAUGE_VELOCITY ? A[2] : 0.0};
+    if (int rc = entry_phases(s, Av, &q.phase)) return rc;
     q.out = s->obs_part + n_part * 4;
     cudaError_t e = launch_nl_current(q, s->stream);
     s->launches++;
@@ -420,9 +428,8 @@ int run_finalize(tdks_system *s, double *rec, double t_state, const double E[3],
   for (int a = 0; a < 3; a++) fv += (s->gauge == TDKS_GAUGE_VELOCITY ? A[a] : E[a]) * s->pol[a];
   const double Az[3] = {0, 0, 0};
   if (s->xfn) {  // state-parallel: band energy and currents summed over the ranks
-    cudaError_t e = launch_finalize_sums(s->obs_part, n_part, s->lda_part, lda_blocks(s->N), s->fin_part,
-                                         s->fin_sum, s->stream);
-    s->launches += 2;
+    cudaError_t e = launch_finalize_sums(s->obs_part, n_part, s->lda_part, lda_blocks(s->N), s->fin_sum, s->stream);
+    s->launches++;
     if (e != cudaSuccess) return fail(TDKS_EDEVICE, std::string("finalize: ") + cudaGetErrorString(e));
     if (int r = s->xfn(s->fin_sum, 4, (void *)s->stream, s->xctx))
       return fail(TDKS_EDEVICE, "exchange hook failed on the record sums (" + std::to_string(r) + ")");
@@ -435,8 +442,8 @@ int run_finalize(tdks_system *s, double *rec, double t_state, const double E[3],
   Timed tm(s, 2);
   cudaError_t e = launch_finalize(s->obs_part, n_part, s->lda_part, lda_blocks(s->N), rec, t_state, h3,
                                   s->occ, s->bc == TDKS_BC_BLOCH, omega_cell,
-                                  s->gauge == TDKS_GAUGE_VELOCITY ? A : Az, fv, s->fin_part, s->stream);
-  s->launches += 2;
+                                  s->gauge == TDKS_GAUGE_VELOCITY ? A : Az, fv, s->stream);
+  s->launches++;
   if (e != cudaSuccess) return fail(TDKS_EDEVICE, std::string("finalize: ") + cudaGetErrorString(e));
   return TDKS_OK;
 }
@@ -585,12 +592,17 @@ int tdks_create_grid(int nx, int ny, int nz, double h, int fd_order, int bc, int
     ALLOC(s->obs_part, (size_t)s->obs_cap * 4 * sizeof(double));
   }
   ALLOC(s->ring, (size_t)tdks_system::RING * TDKS_RECORD * sizeof(double));
-  ALLOC(s->fin_part, (size_t)FIN_BLOCKS * 10 * sizeof(double));
   ALLOC(s->obs_rec, TDKS_RECORD * sizeof(double));
   ALLOC(s->d_kvec, 3 * n_k * sizeof(double));
+  ALLOC(s->d_kphase, 3 * n_k * sizeof(double2));
   ALLOC(s->d_wocc, n_k * sizeof(double));
 #undef ALLOC
+  std::vector<double2> kphase(3 * n_k);
+  const double L[3] = {nx * h, ny * h, nz * h};
+  for (int i = 0; i < 3 * n_k; i++)
+    kphase[i] = make_double2(std::cos(s->kpts[i] * L[i % 3]), std::sin(s->kpts[i] * L[i % 3]));
   if (cudaMemcpy(s->d_kvec, s->kpts.data(), 3 * n_k * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(s->d_kphase, kphase.data(), 3 * n_k * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemsetAsync(s->vloc, 0, N * sizeof(double), s->stream) != cudaSuccess ||
       cudaMemsetAsync(s->aux, 0, N * sizeof(PointAux), s->stream) != cudaSuccess ||
       cudaMemsetAsync(s->psi, 0, s->state_bytes, s->stream) != cudaSuccess ||
@@ -615,11 +627,11 @@ int tdks_destroy(tdks_sys s) {
   cudaFree(s->d_err);
   for (int i = 0; i < 3; i++) cudaFree(s->term[i]);
   cudaFree(s->vloc); cudaFree(s->aux); cudaFree(s->dens_part); cudaFree(s->lda_part);
-  cudaFree(s->obs_part); cudaFree(s->ring); cudaFree(s->fin_part);
+  cudaFree(s->obs_part); cudaFree(s->ring);
   for (int j = 0; j < 4; j++) cudaFree(s->vx_hist[j]);
   cudaFree(s->etrs_save); cudaFree(s->etrs_save_lo);
   cudaFree(s->n_total); cudaFree(s->fin_sum);
-  cudaFree(s->obs_rec); cudaFree(s->d_kvec); cudaFree(s->d_wocc);
+  cudaFree(s->obs_rec); cudaFree(s->d_kvec); cudaFree(s->d_kphase); cudaFree(s->d_wocc);
   cudaFree(s->staging);
   tsurff_free(s);
   hartree_free(s);
@@ -1065,7 +1077,7 @@ int tdks_apply_H(tdks_sys s, double t, const void *dev_in, void *dev_out) {
   else if (s->xc == TDKS_XC_LDA_X) return fail(TDKS_ESTATE, "LDA exchange needs the density of set orbitals");
   else CU(cudaMemsetAsync(s->dens_part, 0, (size_t)s->n_kb * s->N * sizeof(double), s->stream));
   if (rc) return rc;
-  if ((rc = run_lda(s, E, A))) return rc;
+  if ((rc = run_lda(s, E, A, false))) return rc;
   if ((rc = run_gather(s, dev_in, A))) return rc;
   SweepParams p{};
   sweep_common(s, p, A, 1);
@@ -1342,7 +1354,7 @@ static int apply_scaled(tdks_system *s, const void *in, void *out, double cr, do
   double E[3], A[3];
   field_at(s, t, E, A);
   int rc;
-  if ((rc = run_lda(s, E, A))) return rc;
+  if ((rc = run_lda(s, E, A, false))) return rc;
   if ((rc = run_gather(s, in, A))) return rc;
   SweepParams p{};
   sweep_common(s, p, A, 1);

@@ -145,7 +145,7 @@ struct GatherParams {
   const int *rowent;          // entry indices, point-major
   int n_ent;
   void *nl;                   // [kb][n_ent + 1][OVC] vectors, row r0 of each sphere point
-  const float2 *phase;        // complex64: [k][n_ent] (cos, sin) of k.T + A.d, or null
+  const void *phase;          // [k][n_ent] (cos, sin) of k.T + A.d as float2 or double2; null: no phases
 };
 
 // The projectors' share of a periodic cell's current (record time): partial records
@@ -157,9 +157,11 @@ struct NlCurrentParams {
   const int *atom_begin;      // [n_atoms + 1] entry ranges
   const ProjEntry *ent;
   const double *D;            // [n_atoms][4]
-  const double *kvec;         // [n_k][3]
+  const void *phase;          // [k][n_ent] entry phases (GatherParams)
+  int n_ent;
   const double *wocc;         // [n_k] k-weight times occupation
-  double A[3], h3;
+  double h3;
+  int n_chunks;               // CTAs per (atom, kb), set by the launcher
   double *out;
 };
 cudaError_t launch_nl_current(const NlCurrentParams &p, cudaStream_t s);
@@ -224,10 +226,9 @@ size_t sweep_smem(int M, int tx, int ty);
 // and 2) and the non-local term at every sphere point (skipped when no point is in a sphere).
 constexpr int NL_THREADS = 256;
 cudaError_t launch_gather(int prec, int bloch, const GatherParams &p, cudaStream_t s);
-// out[k * n_ent + e] = (cos, sin) of A.d_e (+ k.T_e in a periodic cell), as the complex64
-// projector kernels would form it per entry
-cudaError_t launch_phase_table(const ProjEntry *ent, int n_ent, int n_k, const double *kvec, const double A[3],
-                               int bloch, float2 *out, cudaStream_t s);
+// out[k * n_ent + e] = (cos, sin) of A.d_e (+ k.T_e in a periodic cell): float2 (complex64) or double2
+cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_k, const double *kvec,
+                               const double A[3], int bloch, void *out, cudaStream_t s);
 // chunks per (atom, k-batch) that fill the GPU for n_atoms * n_kb units
 int gather_chunks(long units);
 cudaError_t launch_density(int prec, long N, int n_kb, int n_batches, const void *psi, const void *psi_lo,
@@ -247,8 +248,6 @@ cudaError_t launch_rk4_finish(long n, void *psi, const void *acc, const void *k,
 // n_out[r] = sum over this system's states of w_k f |psi_ik(r)|^2 (FP64), from dens_part
 cudaError_t launch_density_sum(int prec, long N, int n_kb, int n_batches, const double *wocc,
                                const double *dens_part, double *n_out, cudaStream_t s);
-// fin_part: device scratch of FIN_BLOCKS * 10 doubles for the first of the two stages
-constexpr int FIN_BLOCKS = 64;
 // CFM4 exchange history: v[j] is v_x at the start of the j-th latest sub-step (v[0] the
 // newest), w[j] its weight in an exponential's effective potential, nh the points in use.
 struct CfmHist {
@@ -263,12 +262,12 @@ cudaError_t launch_cfm_veff(int prec, int bloch, long N, int nx, int ny, int nz,
 cudaError_t launch_finalize(const double *obs_part, long n_items, const double *lda_part,
                             int n_lda_blocks, double *record, double t_state, double h3,
                             double occ, int bloch, double omega_cell, const double A[3],
-                            double field_val, double *fin_part, cudaStream_t s);
+                            double field_val, cudaStream_t s);
 // The same record in two parts, for state-parallel runs: the 10 sums into sums[0..9]
 // (sums[0..3]: this rank's band energy and current; sums[4..9]: from the summed density),
 // then, once the caller has summed sums[0..3] over the ranks, the record from sums.
 cudaError_t launch_finalize_sums(const double *obs_part, long n_items, const double *lda_part, int n_lda_blocks,
-                                 double *fin_part, double *sums, cudaStream_t s);
+                                 double *sums, cudaStream_t s);
 cudaError_t launch_record_from_sums(const double *sums, double *record, double t_state, double h3, double occ,
                                     int bloch, double omega_cell, const double A[3], double field_val,
                                     cudaStream_t s);

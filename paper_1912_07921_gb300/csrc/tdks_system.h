@@ -56,6 +56,7 @@ struct tdks_system {
   double *ring = nullptr;
   double *obs_rec = nullptr;    // single record for tdks_observe
   double *d_kvec = nullptr, *d_wocc = nullptr, *d_D = nullptr;
+  double2 *d_kphase = nullptr;  // [n_k][3] e^{i k_a L_a}
   int *d_rowent = nullptr, *d_atom_begin = nullptr;
   int2 *d_sp = nullptr;       // entry ranges of the points inside a sphere
   void *d_nl = nullptr;       // non-local term per sphere point, [n_kb][n_ent + 1][OVC]
@@ -63,12 +64,11 @@ struct tdks_system {
   tdks::ProjEntry *d_ent = nullptr;
   float4 *d_ent_beta = nullptr;  // compact copies of the entries' FP32 beta and (cell, atom)
   int2 *d_ent_ca = nullptr;
-  // complex64 projector phases e^{i (k.T + A.d)} of every entry and k-point, built once per
-  // vector potential (a sub-step's Taylor terms share one)
-  float2 *d_phase = nullptr;
+  // projector phases e^{i (k.T + A.d)} of every entry and k-point (float2 or double2 by precision),
+  // built once per vector potential (a sub-step's Taylor terms share one)
+  void *d_phase = nullptr;
   double phase_A[3] = {0.0, 0.0, 0.0};
   bool phase_ok = false;
-  double *fin_part = nullptr;    // first-stage partials of the observable record
   void *d_q = nullptr;
   double2 *d_qpart = nullptr;   // gather partial sums, gchunks per (atom, k-batch)
   int gchunks = 1;

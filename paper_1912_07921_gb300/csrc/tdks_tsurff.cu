@@ -131,9 +131,11 @@ __global__ void __launch_bounds__(TS_THREADS) tsurff_flux_kernel(const TsFlux f)
         const double2 x = g0[(long)j * f.n_orb], y = g1[(long)j * f.n_orb], w = sW[j * np + pl];
         const int ax = sAx[j];
         const double k = ax == 0 ? k0 : (ax == 1 ? k1 : k2);
-        const double tr = k * x.x + y.x, ti = k * x.y + y.y;
-        ar += w.x * tr - w.y * ti;
-        ai += w.x * ti + w.y * tr;
+        const double tr = fma(k, x.x, y.x), ti = fma(k, x.y, y.y);
+        ar = fma(w.x, tr, ar);  // (as written with + and -, a product and a sum more)
+        ai = fma(w.x, ti, ai);
+        ar = fma(-w.y, ti, ar);
+        ai = fma(w.y, tr, ai);
       }
     }
   }
