@@ -978,23 +978,26 @@ __device__ __forceinline__ void write_record(const double O[4], const double Lq[
   rec[7] = field_val;
 }
 
-// Sum of the 10 per-thread values v over the CTA: a fixed xor tree
-// within each warp, then the warps in order; thread c < 10 returns component c.
-constexpr int FIN_THREADS = 128;       // batches: one CTA per system
+// Sum of the 10 per-thread values v over the CTA in a fixed order: 16 threads per component, each
+// adding every 16th thread's value, then a tree of four; thread c < 10 returns component c.  (A
+// shuffle tree in every warp is 50 FP64 sums a warp, most of whose lanes are not needed.)
+constexpr int FIN_THREADS = 160;       // batches: one CTA per system
 constexpr int FIN_MAX_THREADS = 256;   // one system: a cluster of CTAs
 __device__ __forceinline__ double block_sum10(double v[10], int t) {
-  __shared__ double red[FIN_MAX_THREADS / 32][10];
+  __shared__ double all[10][FIN_MAX_THREADS + 1];
+  __shared__ double red[10];
 #pragma unroll
-  for (int c = 0; c < 10; c++) {
-    double x = v[c];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if ((t & 31) == 0) red[t >> 5][c] = x;
+  for (int c = 0; c < 10; c++) all[c][t] = v[c];
+  __syncthreads();
+  if (t < 160) {
+    const int c = t / 16, l = t % 16;
+    double x = 0.0;
+    for (int i = l; i < (int)blockDim.x; i += 16) x += all[c][i];
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (l == 0) red[c] = x;
   }
   __syncthreads();
-  double x = 0.0;
-  if (t < 10)
-    for (int w = 0; w < (int)blockDim.x / 32; w++) x += red[w][t];
-  return x;
+  return t < 10 ? red[t] : 0.0;
 }
 
 // Partials of records [i0, i1) and LDA blocks [l0, l1), summed by one CTA.

@@ -164,7 +164,7 @@ void sweep_geometry(const tdks_system *s, SweepParams &p, int sweep) {
     // arithmetic of a complex128 plane they are small.
     const long per_plane = (long)p.n_tx * p.n_ty * p.n_kb;
     const bool c64 = s->prec == TDKS_C64;
-    const int step = sweep >= 0 ? ws_shape_planes(kernel_shape(s, s->wshape[sweep], sweep)) : 1;
+    const int step = sweep >= 0 ? ws_shape_planes(kernel_shape(s, s->wshape[sweep], sweep), s->M, s->bc == TDKS_BC_BLOCH) : 1;
     const double extra = c64 ? 0.5 * s->M : 0.3, spread = c64 ? 1.0 : 0.1;
     double best = -1.0;
     for (int n = 1; n <= s->nz; n++) {
@@ -560,6 +560,7 @@ int tdks_create_grid(int nx, int ny, int nz, double h, int fd_order, int bc, int
   if (kweights) for (int i = 0; i < n_k; i++) s->kw[i] = kweights[i];
   cudaGetDevice(&s->dev);
   const size_t pts = (size_t)s->n_kb * N;
+  for (int i = 0; i < 4; i++) s->wshape[i] = ws_default_shape(prec, bc == TDKS_BC_BLOCH, (long)pts, i == 3);
   s->term_bytes = pts * OVC * 16;
   s->state_bytes = s->term_bytes;
   const int nlda = lda_blocks(N);

@@ -28,6 +28,7 @@
 #include <atomic>
 #include <cmath>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "tdks_system.h"
@@ -147,7 +148,8 @@ __device__ __forceinline__ void fft_pass(const double2 *a, double2 *b, const Fft
 }
 
 // Transform of the LB lines in a (b: as much scratch); the result is in a again on return.
-template <int SIGN, int LB>
+// BIG: lengths with prime factors above 5 (periodic cells); the others' kernels keep half the registers.
+template <int SIGN, int LB, bool BIG>
 __device__ __forceinline__ void fft_lines(double2 *&a, double2 *&b, const FftPlan &p) {
   int Ns = 1;
   for (int i = 0; i < p.nrad; i++) {
@@ -157,10 +159,13 @@ __device__ __forceinline__ void fft_lines(double2 *&a, double2 *&b, const FftPla
       case 3: fft_pass<3, SIGN, LB>(a, b, p, Ns); break;
       case 4: fft_pass<4, SIGN, LB>(a, b, p, Ns); break;
       case 5: fft_pass<5, SIGN, LB>(a, b, p, Ns); break;
-      case 7: fft_pass<7, SIGN, LB>(a, b, p, Ns); break;
       case 8: fft_pass<8, SIGN, LB>(a, b, p, Ns); break;
-      case 11: fft_pass<11, SIGN, LB>(a, b, p, Ns); break;
-      default: fft_pass<13, SIGN, LB>(a, b, p, Ns); break;
+      default:
+        if constexpr (BIG) {
+          if (p.rad[i] == 7) fft_pass<7, SIGN, LB>(a, b, p, Ns);
+          else if (p.rad[i] == 11) fft_pass<11, SIGN, LB>(a, b, p, Ns);
+          else fft_pass<13, SIGN, LB>(a, b, p, Ns);
+        }
     }
     Ns *= p.rad[i];
     double2 *t = a;
@@ -172,8 +177,8 @@ __device__ __forceinline__ void fft_lines(double2 *&a, double2 *&b, const FftPla
 
 // Real x lines -> half spectrum.  Line l = z ny + y of src (nx values, zeros beyond) goes to row
 // z py + y of buf (hx values); lines 2q and 2q + 1 are one complex line.
-template <int LB>
-__global__ void __launch_bounds__(FFT_THREADS)
+template <int LB, bool BIG>
+__global__ void __launch_bounds__(FFT_THREADS, BIG ? 1 : 6)
 fft_x_forward(const double *src, double2 *buf, const FftPlan p, int nx, int ny, int py, long lines) {
   extern __shared__ double2 sm[];
   double2 *a = sm, *b = sm + p.n * LB;
@@ -189,7 +194,7 @@ fft_x_forward(const double *src, double2 *buf, const FftPlan p, int nx, int ny, 
     }
     a[t] = v;
   }
-  fft_lines<-1, LB>(a, b, p);
+  fft_lines<-1, LB, BIG>(a, b, p);
   for (int t = threadIdx.x; t < hx * LB; t += FFT_THREADS) {
     const int l = t % LB, k = t / LB;
     const long la = l0 + 2 * l, lb = la + 1;
@@ -201,8 +206,8 @@ fft_x_forward(const double *src, double2 *buf, const FftPlan p, int nx, int ny, 
 }
 
 // The inverse of fft_x_forward: half spectra -> real lines, times scale.
-template <int LB>
-__global__ void __launch_bounds__(FFT_THREADS)
+template <int LB, bool BIG>
+__global__ void __launch_bounds__(FFT_THREADS, BIG ? 1 : 6)
 fft_x_inverse(const double2 *buf, double *dst, const FftPlan p, int nx, int ny, int py, long lines, double scale) {
   extern __shared__ double2 sm[];
   double2 *a = sm, *b = sm + p.n * LB;
@@ -219,7 +224,7 @@ fft_x_inverse(const double2 *buf, double *dst, const FftPlan p, int nx, int ny, 
     a[k * LB + l] = make_double2(A.x - B.y, A.y + B.x);
     if (k > 0 && 2 * k < n) a[(n - k) * LB + l] = make_double2(A.x + B.y, B.x - A.y);
   }
-  fft_lines<1, LB>(a, b, p);
+  fft_lines<1, LB, BIG>(a, b, p);
   for (int t = threadIdx.x; t < nx * LB; t += FFT_THREADS) {
     const int l = t % LB, i = t / LB;
     const long la = l0 + 2 * l, lb = la + 1;
@@ -230,8 +235,8 @@ fft_x_inverse(const double2 *buf, double *dst, const FftPlan p, int nx, int ny, 
 }
 
 // Lines along y (SIGN -1: n_in = ny values in, py out; +1: py in, ny out) of LB adjacent columns.
-template <int SIGN, int LB>
-__global__ void __launch_bounds__(FFT_THREADS) fft_y(double2 *buf, const FftPlan p, int hx, int n_in, int n_out) {
+template <int SIGN, int LB, bool BIG>
+__global__ void __launch_bounds__(FFT_THREADS, BIG ? 1 : 6) fft_y(double2 *buf, const FftPlan p, int hx, int n_in, int n_out) {
   extern __shared__ double2 sm[];
   double2 *a = sm, *b = sm + p.n * LB;
   const int n = p.n, x0 = blockIdx.x * LB;
@@ -240,7 +245,7 @@ __global__ void __launch_bounds__(FFT_THREADS) fft_y(double2 *buf, const FftPlan
     const int l = t % LB, i = t / LB;
     a[t] = i < n_in && x0 + l < hx ? base[(long)i * hx + l] : make_double2(0.0, 0.0);
   }
-  fft_lines<SIGN, LB>(a, b, p);
+  fft_lines<SIGN, LB, BIG>(a, b, p);
   for (int t = threadIdx.x; t < n_out * LB; t += FFT_THREADS) {
     const int l = t % LB, i = t / LB;
     if (x0 + l < hx) base[(long)i * hx + l] = a[t];
@@ -249,8 +254,8 @@ __global__ void __launch_bounds__(FFT_THREADS) fft_y(double2 *buf, const FftPlan
 
 // Lines along z: forward, times the kernel's transform, inverse (nz values in and out).
 // kout: forward only, the real part of the transform of a kernel's lines (pz values in) to kout.
-template <int LB>
-__global__ void __launch_bounds__(FFT_THREADS)
+template <int LB, bool BIG>
+__global__ void __launch_bounds__(FFT_THREADS, BIG ? 1 : 6)
 fft_z(double2 *buf, const FftPlan p, int hx, int nz, const double *kern, double *kout) {
   extern __shared__ double2 sm[];
   double2 *a = sm, *b = sm + p.n * LB;
@@ -260,7 +265,7 @@ fft_z(double2 *buf, const FftPlan p, int hx, int nz, const double *kern, double 
     const int l = t % LB, i = t / LB;
     a[t] = i < nz && x0 + l < hx ? buf[at + i * stride + l] : make_double2(0.0, 0.0);
   }
-  fft_lines<-1, LB>(a, b, p);
+  fft_lines<-1, LB, BIG>(a, b, p);
   for (int t = threadIdx.x; t < n * LB; t += FFT_THREADS) {
     const int l = t % LB, i = t / LB;
     if (x0 + l >= hx) continue;
@@ -272,7 +277,7 @@ fft_z(double2 *buf, const FftPlan p, int hx, int nz, const double *kern, double 
     }
   }
   if (kout) return;
-  fft_lines<1, LB>(a, b, p);
+  fft_lines<1, LB, BIG>(a, b, p);
   for (int t = threadIdx.x; t < nz * LB; t += FFT_THREADS) {
     const int l = t % LB, i = t / LB;
     if (x0 + l < hx) buf[at + i * stride + l] = a[t];
@@ -364,45 +369,59 @@ cudaError_t big_smem() {
   return ensure_smem_attr(K, 2ul * 8 * 512 * sizeof(double2), done);
 }
 
+// f(LB, BIG) as compile-time constants for a line length
+template <class F>
+cudaError_t by_length(const FftPlan &p, F f) {
+  const bool big = p.n > 1 && p.rad[p.nrad - 1] > 5 && p.rad[p.nrad - 1] != 8;
+  if (lines_of(p.n) == 8)
+    return big ? f(std::integral_constant<int, 8>{}, std::true_type{}) : f(std::integral_constant<int, 8>{}, std::false_type{});
+  return big ? f(std::integral_constant<int, 4>{}, std::true_type{}) : f(std::integral_constant<int, 4>{}, std::false_type{});
+}
+
 cudaError_t x_forward(const double *src, double2 *buf, const FftPlan &p, int nx, int ny, int nz, int py, cudaStream_t s) {
-  const long lines = (long)ny * nz;
-  const int LB = lines_of(p.n);
-  const unsigned grid = (unsigned)((lines + 2 * LB - 1) / (2 * LB));
-  auto k = LB == 8 ? fft_x_forward<8> : fft_x_forward<4>;
-  if (cudaError_t e = LB == 8 ? big_smem<fft_x_forward<8>>() : big_smem<fft_x_forward<4>>()) return e;
-  k<<<grid, FFT_THREADS, smem_of(p.n), s>>>(src, buf, p, nx, ny, py, lines);
-  return cudaGetLastError();
+  return by_length(p, [&](auto lb, auto big) {
+    constexpr int LB = decltype(lb)::value;
+    constexpr auto k = fft_x_forward<LB, decltype(big)::value>;
+    const long lines = (long)ny * nz;
+    if (cudaError_t e = big_smem<k>()) return e;
+    k<<<(unsigned)((lines + 2 * LB - 1) / (2 * LB)), FFT_THREADS, smem_of(p.n), s>>>(src, buf, p, nx, ny, py, lines);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t x_inverse(const double2 *buf, double *dst, const FftPlan &p, int nx, int ny, int nz, int py, double scale,
                       cudaStream_t s) {
-  const long lines = (long)ny * nz;
-  const int LB = lines_of(p.n);
-  const unsigned grid = (unsigned)((lines + 2 * LB - 1) / (2 * LB));
-  auto k = LB == 8 ? fft_x_inverse<8> : fft_x_inverse<4>;
-  if (cudaError_t e = LB == 8 ? big_smem<fft_x_inverse<8>>() : big_smem<fft_x_inverse<4>>()) return e;
-  k<<<grid, FFT_THREADS, smem_of(p.n), s>>>(buf, dst, p, nx, ny, py, lines, scale);
-  return cudaGetLastError();
+  return by_length(p, [&](auto lb, auto big) {
+    constexpr int LB = decltype(lb)::value;
+    constexpr auto k = fft_x_inverse<LB, decltype(big)::value>;
+    const long lines = (long)ny * nz;
+    if (cudaError_t e = big_smem<k>()) return e;
+    k<<<(unsigned)((lines + 2 * LB - 1) / (2 * LB)), FFT_THREADS, smem_of(p.n), s>>>(buf, dst, p, nx, ny, py, lines,
+                                                                                 scale);
+    return cudaGetLastError();
+  });
 }
 
 template <int SIGN>
 cudaError_t y_lines(double2 *buf, const FftPlan &p, int hx, int nz, int n_in, int n_out, cudaStream_t s) {
-  const int LB = lines_of(p.n);
-  const dim3 grid((hx + LB - 1) / LB, nz);
-  auto k = LB == 8 ? fft_y<SIGN, 8> : fft_y<SIGN, 4>;
-  if (cudaError_t e = LB == 8 ? big_smem<fft_y<SIGN, 8>>() : big_smem<fft_y<SIGN, 4>>()) return e;
-  k<<<grid, FFT_THREADS, smem_of(p.n), s>>>(buf, p, hx, n_in, n_out);
-  return cudaGetLastError();
+  return by_length(p, [&](auto lb, auto big) {
+    constexpr int LB = decltype(lb)::value;
+    constexpr auto k = fft_y<SIGN, LB, decltype(big)::value>;
+    if (cudaError_t e = big_smem<k>()) return e;
+    k<<<dim3((hx + LB - 1) / LB, nz), FFT_THREADS, smem_of(p.n), s>>>(buf, p, hx, n_in, n_out);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t z_lines(double2 *buf, const FftPlan &p, int hx, int py, int nz, const double *kern, double *kout,
                     cudaStream_t s) {
-  const int LB = lines_of(p.n);
-  const dim3 grid((hx + LB - 1) / LB, py);
-  auto k = LB == 8 ? fft_z<8> : fft_z<4>;
-  if (cudaError_t e = LB == 8 ? big_smem<fft_z<8>>() : big_smem<fft_z<4>>()) return e;
-  k<<<grid, FFT_THREADS, smem_of(p.n), s>>>(buf, p, hx, nz, kern, kout);
-  return cudaGetLastError();
+  return by_length(p, [&](auto lb, auto big) {
+    constexpr int LB = decltype(lb)::value;
+    constexpr auto k = fft_z<LB, decltype(big)::value>;
+    if (cudaError_t e = big_smem<k>()) return e;
+    k<<<dim3((hx + LB - 1) / LB, py), FFT_THREADS, smem_of(p.n), s>>>(buf, p, hx, nz, kern, kout);
+    return cudaGetLastError();
+  });
 }
 
 }  // namespace

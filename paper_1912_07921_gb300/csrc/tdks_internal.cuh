@@ -297,8 +297,18 @@ bool ws_shape_info(int shape, int *tx, int *ty, int *rows, int *warps);
 // run one that does.  Tiles, tensor maps and record counts follow the result.
 // last: the sweep of the last Taylor term.
 int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last);
+// The shape a sweep takes until one is set or tuned.  complex64, terms 1 to 3: shape 6 once the grid has
+// work for its larger tile (medium molecule 0.316 -> 0.250 ms, 48^3 with 16 orbitals 18.4 -> 17.2 us; at
+// 24^3 shape 0 is still ahead, 9.6 against 10.4 us, and in cells up to 32^3); last term: shape 3 while the
+// sweep is short (64^3, 24 orbitals 96 -> 82 us), shape 2 for long ones (medium molecule 0.54 -> 0.48 ms).
+// complex128 is bound by the FP64 pipe in every shape and stays with shape 0's smaller tile.
+inline int ws_default_shape(int prec, int bloch, long points, bool last) {
+  if (prec != P_C64) return 0;
+  if (last) return points < 1500000 ? 3 : 2;
+  return points >= (bloch ? 60000 : 30000) ? 6 : 0;
+}
 // planes a shape's kernel takes per iteration
-int ws_shape_planes(int shape);
+int ws_shape_planes(int shape, int M, int bloch);
 bool tma_supported(int M, int tx, int ty);
 int tma_planes(int prec, int mode, bool lockstep = false);
 int lda_blocks(long N);

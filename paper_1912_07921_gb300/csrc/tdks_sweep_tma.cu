@@ -333,7 +333,10 @@ bool ws_shape_info(int shape, int *tx, int *ty, int *rows, int *warps) {
   return false;
 }
 
-int ws_shape_planes(int shape) { return shape == 6 || shape == 8 ? 2 : 1; }
+int ws_shape_planes(int shape, int M, int bloch) {
+  if (shape == 7) return M == 4 || bloch ? 1 : 2;
+  return shape == 6 || shape == 8 ? 2 : 1;
+}
 
 int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last) {
   if (shape < 5) return shape;
@@ -341,7 +344,6 @@ int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool 
   if (shape == 5) return bloch ? 2 : 5;
   if (bloch && (M != 2 || nx % 2 != 0 || ny % 2 != 0)) return 2;     // blocks must not straddle a face
   if (last) return 2;                                                // their operands would not fit
-  if (shape == 7 && M != 2) return 6;                                // its z queues would not fit
   return shape;
 }
 

@@ -101,6 +101,10 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *tmap, 
       : "memory");
 }
 
+__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap *tmap) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
+}
+
 }  // namespace
 
 // Compile-time loop: f(integral_constant<int, 0>) ... f(integral_constant<int, N-1>).
@@ -377,17 +381,22 @@ template <> struct WsShape<3> { static constexpr int U = 1, TX = 16, TY = 8, R =
 template <> struct WsShape<4> { static constexpr int U = 1, TX = 14, TY = 8, R = 2, RX = 1; };   //  7
 template <> struct WsShape<5> { static constexpr int U = 1, TX = 16, TY = 12, R = 4, RX = 1; };  // 12 (complex64, 8-byte vectors)
 template <> struct WsShape<6> { static constexpr int U = 2, TX = 16, TY = 12, R = 2, RX = 1; };  // 12 (complex64, terms 1-3)
-template <> struct WsShape<7> { static constexpr int U = 1, TX = 16, TY = 24, R = 2, RX = 2; };  // 12 (complex64, order 4, terms 1-3)
+template <> struct WsShape<7> { static constexpr int U = 2, TX = 16, TY = 16, R = 2, RX = 2; };  //  8 (complex64, terms 1-3)
 template <> struct WsShape<8> { static constexpr int U = 2, TX = 16, TY = 12, R = 2, RX = 2; };  // 12 (complex64, 8-byte vectors, terms 1-3)
+// planes per iteration of a shape's kernels
+template <int SHAPE, int M, int BLOCH> struct WsPlanes {
+  static constexpr int U = SHAPE == 7 && (M == 4 || BLOCH) ? 1 : WsShape<SHAPE>::U;
+};
 template <int TX, int TY, int R, int OV = OVC, int RX = 1, bool SPL = false> struct WsWarps {
   static constexpr int CW = OV * TX * TY / (32 * R * RX);  // consumer warps
-  // Blocks of 2 x 2 points want more registers than 65536 / threads: their twelve consumer warps and the
-  // four service warps start with 128 per thread each, all there are, and the service warpgroup
-  // gives most of its share to the consumers, whose z queues would spill at 128 (M = 4: 72 of them):
-  // 384 * 152 + 128 * 56 = 512 * 128.
+  // Blocks of 2 x 2 points, and two planes at a time, want more registers than 65536 / threads: the
+  // consumer warps and the four service warps start with equal shares, all there are, and the service
+  // warpgroup gives most of its share to the consumers, whose z queues would spill:
+  // 384 * 152 + 128 * 56 = 512 * 128 (M = 4: queues of 72 registers), 256 * 232 + 128 * 40 = 384 * 168
+  // (queues of 144).
   static constexpr bool SPLIT = RX == 2 || SPL;
-  static_assert(!SPLIT || CW == 12, "the register split is for twelve consumer warps");
-  static constexpr int CONSUMER_REGS = 152, PRODUCER_REGS = 56;
+  static_assert(!SPLIT || CW == 12 || CW == 8, "the register splits are for twelve or eight consumer warps");
+  static constexpr int CONSUMER_REGS = CW == 12 ? 152 : 232, PRODUCER_REGS = CW == 12 ? 56 : 40;
   static constexpr int THREADS = 32 * CW + 128;            // + three producer warps and the patcher
   // consumer thread t owns vector t % OV of block (t / OV) % (TX / RX) of row group t / (OV TX / RX),
   // whose R rows are y-adjacent: the row groups must fill the tile and the warps exactly
@@ -545,11 +554,21 @@ __device__ __forceinline__ void stencil_block(const SweepParams &p, const typena
   }
 #pragma unroll
   for (int m = 1; m <= M; m++) {
-    V xln[2], xhn[2], yln[2], yhn[2];
+    // (x arms first, then y arms: half of the neighbours live at a time)
+    V xln[2], xhn[2], yln[2], yhn[2], szx[4];
 #pragma unroll
     for (int i = 0; i < 2; i++) {
       xln[i] = (S0 - m * sx)[i * SXO];
       xhn[i] = (S0 + (m + 1) * sx)[i * SXO];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const int r = q >> 1, c = q & 1;
+      const V xm = c == 0 ? xln[r] : xl[r], xp = c == 0 ? xh[r] : xhn[r];
+      szx[q] = T::add(T::add(Q[q][(QB + M - m) % QN], Q[q][(QB + M + m) % QN]), T::add(xm, xp));
+    }
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
       yln[i] = (S0 + i * sx)[-m * SXO];
       yhn[i] = (S0 + i * sx)[(m + 1) * SXO];
     }
@@ -559,7 +578,7 @@ __device__ __forceinline__ void stencil_block(const SweepParams &p, const typena
       const V xm = c == 0 ? xln[r] : xl[r], xp = c == 0 ? xh[r] : xhn[r];
       const V ym = r == 0 ? yln[c] : yl[c], yp = r == 0 ? yh[c] : yhn[c];
       const V zm = Q[q][(QB + M - m) % QN], zp = Q[q][(QB + M + m) % QN];
-      const V s6 = T::add(T::add(T::add(zm, zp), T::add(xm, xp)), T::add(ym, yp));
+      const V s6 = T::add(szx[q], T::add(ym, yp));
       acc[q] = T::fma(W[m], s6, acc[q]);
       if (BLOCH && need_grad) {
         const V dx = T::sub(xp, xm), dy = T::sub(yp, ym), dz = T::sub(zp, zm);
@@ -605,6 +624,8 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
   constexpr int SO = G::SO > 0 ? G::SO : 1;
   constexpr int QN = 2 * M + U;   // z-queue entries
   constexpr int LP = 2 * M / U;   // priming centre loads per item
+  // order-8 blocks of 16-byte vectors: their queues leave no registers for projector terms in flight
+  constexpr bool LATE_NL = RX == 2 && M == 4 && T::OV == 4;
   constexpr int IR = 16;          // claimed-item ring (the producer runs at most a few items ahead)
   extern __shared__ unsigned char smem_raw[];
   unsigned char *cbase = smem_raw + ((0u - smem_u32(smem_raw)) & 127u);
@@ -656,11 +677,16 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
     bool gave_up = false;
     for (unsigned seq = 0; !gave_up; seq++) {
       if constexpr (KIND == 0) {
-        const unsigned int t = atomicAdd(work, 1u);
-        // every CTA ends with one claim past the last item: the launch's last claim returns the
-        // counter to zero for the next launch
-        if ((long)t == n_items_all + (long)gridDim.x - 1) atomicExch(work, 0u);
-        s_item[seq % IR] = (long)t < n_items_all ? (long)t : -1;
+        // (a CTA's first item is its own number, without a round trip to the counter; then every CTA
+        // claims until one claim is past the last item: n_items claims in all, the last of which
+        // returns the counter to zero for the next launch)
+        long t = blockIdx.x;
+        if (seq > 0) {
+          const unsigned int r = atomicAdd(work, 1u);
+          if ((long)r == n_items_all - 1) atomicExch(work, 0u);
+          t = (long)gridDim.x + (long)r;
+        }
+        s_item[seq % IR] = t < n_items_all ? t : -1;
         mbar_arrive(&ibar[seq % IR]);
       } else if (!mbar_wait_or_abort(&ibar[seq % IR], (seq / IR) & 1u, abort_flag)) {
         gave_up = true;
@@ -681,6 +707,8 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
       cu.nz = qp->nz;
       cu.wrap = qp->bloch;
       const int n = loads_of<M, U>(KIND, cu.z0, z1);
+      // (sending the last term's operand tiles to L2 four or eight planes ahead of their loads made it
+      // 18% and 36% slower on the medium molecule: eight streams per CTA are enough for the DRAM)
       for (cu.l = 0; cu.l < n;) {
         // the slot is free once the consumers have released its previous use (at once the first time)
         if (!mbar_wait_or_abort(&empty[rp.slot], rp.phase ^ 1u, abort_flag)) {
@@ -701,6 +729,16 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
   };
   if (warp >= CW && warp < CW + 3) {
     if (lane == 0 && !src.withhold()) {
+      if constexpr (!BATCH) {
+        const SweepMaps *mp = src.maps_of(0);
+        if (warp == CW) tma_prefetch_map(&mp->ctr);
+        if (warp == CW + 1) {
+          tma_prefetch_map(&mp->in);
+          tma_prefetch_map(&mp->aux);
+        }
+        if (OPS && warp == CW + 2)
+          for (int j = 0; j < 4; j++) tma_prefetch_map(&mp->op[j]);
+      }
       if (warp == CW) serve(std::integral_constant<int, 0>{});
       if (warp == CW + 1) serve(std::integral_constant<int, 1>{});
       if (OPS && warp == CW + 2) serve(std::integral_constant<int, 2>{});
@@ -944,11 +982,15 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
           constexpr int QB = (RQ + U + u) % QN;  // queue position of plane (zf + u) - M
           Rv ve[NP];
           V nlv[NP], acc[NP];
+          [[maybe_unused]] bool in_sphere = false;
 #pragma unroll
           for (int q = 0; q < NP; q++) {
             const PointAux a = (ax + (q % RX) * dx1)[u * TX * TY + tsl0 + (q / RX) * TX];
             ve[q] = *reinterpret_cast<const Rv *>(&a.veff);
-            if constexpr (G::NLS) {
+            if constexpr (P == P_C128) in_sphere = in_sphere || a.r1 > a.r0;
+            if constexpr (LATE_NL) {
+              // (loaded after the stencil, below)
+            } else if constexpr (G::NLS) {
               // (gathered into the slot by the patcher warp)
               const V *nla = reinterpret_cast<const V *>(hslot + G::IN_BYTES + G::AUX_BYTES + G::STRIP_BYTES);
               nlv[q] = has_proj && a.r1 > a.r0 ? (nla + (q % RX) * sx)[(u * TX * TY + tsl0 + (q / RX) * TX) * OV + v] : T::zero();
@@ -965,11 +1007,20 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
           } else {
             stencil_rows<M, P, QB, QN, R>(W, w0, Q, xs + u * G::SX * G::SY * OV, hs0, SXO, ve, acc);
           }
+          if constexpr (LATE_NL) {
+#pragma unroll
+            for (int q = 0; q < NP; q++) {
+              const PointAux a = (ax + (q % RX) * dx1)[u * TX * TY + tsl0 + (q / RX) * TX];
+              nlv[q] = has_proj ? nl_term<P>(nlk, a.r0, a.r1) : T::zero();
+            }
+          }
           const long iu = idx + (long)u * plane_pts * OV;
+          // (complex128: two FP64 sums per value are worth a vote; most warps meet no sphere)
+          const bool add_nl = has_proj && (P != P_C128 || __any_sync(0xffffffffu, in_sphere));
 #pragma unroll
           for (int q = 0; q < NP; q++) {
             const bool live = own[q] && (zf + u < z1);
-            if (has_proj) acc[q] = T::add(acc[q], nlv[q]);
+            if (add_nl) acc[q] = T::add(acc[q], nlv[q]);
             const V c0 = Q[q][(QB + M) % QN];
             if (MODE == MODE_FIRST && do_obs && live) {
               oa.add_e(c0, acc[q]);
@@ -1039,7 +1090,7 @@ ws_sweep_batch_kernel(const __grid_constant__ BatchSweepArgs a) {
 template <int SHAPE, int M, int P, int MODE, int BLOCH>
 static cudaError_t launch_ws_t(const SweepMaps &maps, const SweepParams &p, int grid, cudaStream_t s) {
   constexpr int TX = WsShape<SHAPE>::TX, TY = WsShape<SHAPE>::TY, R = WsShape<SHAPE>::R, RX = WsShape<SHAPE>::RX;
-  constexpr int U = WsShape<SHAPE>::U;
+  constexpr int U = WsPlanes<SHAPE, M, BLOCH>::U;
   typedef TmaGeom<M, TX, TY, U, MODE == MODE_LAST, BLOCH != 0, MODE == MODE_FIRST> G;
   auto k = ws_sweep_kernel<M, P, MODE, TX, TY, R, RX, U, BLOCH>;
   static std::atomic<unsigned> attr_done{0};
@@ -1059,7 +1110,7 @@ static cudaError_t launch_ws_t(const SweepMaps &maps, const SweepParams &p, int 
 template <int SHAPE, int M, int P, int MODE>
 static cudaError_t launch_ws_batch_t(const BatchSweepArgs &a, cudaStream_t s) {
   constexpr int TX = WsShape<SHAPE>::TX, TY = WsShape<SHAPE>::TY, R = WsShape<SHAPE>::R, RX = WsShape<SHAPE>::RX;
-  constexpr int U = WsShape<SHAPE>::U;
+  constexpr int U = WsPlanes<SHAPE, M, 0>::U;
   typedef TmaGeom<M, TX, TY, U, MODE == MODE_LAST, false, MODE == MODE_FIRST> G;
   auto k = ws_sweep_batch_kernel<M, P, MODE, TX, TY, R, RX, U>;
   static std::atomic<unsigned> attr_done{0};
@@ -1079,7 +1130,7 @@ static cudaError_t launch_ws_batch_t(const BatchSweepArgs &a, cudaStream_t s) {
 template <int SHAPE> struct C64Shape {
   static constexpr bool ONLY = SHAPE >= 5;
   static constexpr int P = SHAPE == 7 || SHAPE == 6 ? P_C64 : P_C64S;
-  static constexpr bool M4 = SHAPE != 7;       // has order-8 kernels
+  static constexpr bool M4 = true;             // has order-8 kernels
   static constexpr bool CELL = SHAPE >= 6;     // has periodic-cell kernels (order 4)
   static constexpr bool LAST = SHAPE == 5;     // has last-term kernels
 };
