@@ -599,7 +599,7 @@ template <typename R>
 __device__ __forceinline__ void lda_body(long N, int nx, int ny, int nz, double h, int bloch, int n_kb,
                                          int n_batches, const double *wocc, const double *dens_part,
                                          const double *vloc, int xc, double Ex, double Ey, double Ez,
-                                         double half_A2, PointAux *aux, double *lda_part, int blk, int nblk,
+                                         double half_A2, double w0, PointAux *aux, double *lda_part, int blk, int nblk,
                                          const double *n_in = nullptr, const double *vh = nullptr,
                                          bool sums = true) {
   constexpr bool F32 = sizeof(R) == 4;
@@ -660,7 +660,7 @@ __device__ __forceinline__ void lda_body(long N, int nx, int ny, int nz, double 
       const float vhf = vh ? (float)vh[p] : 0.0f;
       float v = (float)vloc[p] + vx + vhf + hA2f;
       if (!bloch) v += Exf * x + Eyf * y + Ezf * z;
-      *reinterpret_cast<float *>(&aux[p].veff) = v;
+      *reinterpret_cast<float *>(&aux[p].veff) = v + (float)w0;
       if (sums) {
         // (with the Hartree potential the record subtracts int n (v_x + v_H) and adds E_H =
         // 1/2 int n v_H: the third sum is int n (v_x + v_H / 2))
@@ -676,7 +676,7 @@ __device__ __forceinline__ void lda_body(long N, int nx, int ny, int nz, double 
       const double vhd = vh ? vh[p] : 0.0;
       double v = vloc[p] + vx + vhd + half_A2;
       if (!bloch) v += Ex * x + Ey * y + Ez * z;
-      *reinterpret_cast<double *>(&aux[p].veff) = v;
+      *reinterpret_cast<double *>(&aux[p].veff) = v + w0;
       if (sums) {
         acc[0] += n;
         acc[1] += n * 0.75 * vx;
@@ -718,8 +718,8 @@ template <typename R>
 __global__ void __launch_bounds__(LDA_THREADS)
 lda_kernel(long N, int nx, int ny, int nz, double h, int bloch, int n_kb, int n_batches, const double *wocc,
            const double *dens_part, const double *vloc, int xc, double Ex, double Ey, double Ez, double half_A2,
-           PointAux *aux, double *lda_part, const double *n_in, const double *vh, int sums) {
-  lda_body<R>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part, vloc, xc, Ex, Ey, Ez, half_A2, aux,
+           double w0, PointAux *aux, double *lda_part, const double *n_in, const double *vh, int sums) {
+  lda_body<R>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part, vloc, xc, Ex, Ey, Ez, half_A2, w0, aux,
               lda_part, blockIdx.x, gridDim.x, n_in, vh, sums != 0);
 }
 
@@ -814,7 +814,7 @@ template <typename R>
 __global__ void __launch_bounds__(LDA_THREADS)
 cfm_veff_kernel(long N, int nx, int ny, int nz, double h, int bloch, int n_kb, int n_batches, const double *wocc,
                 const double *dens_part, const double *vloc, int xc, int push, CfmHist hist, double Ex, double Ey,
-                double Ez, PointAux *aux, const double *vh, const double *n_in) {
+                double Ez, double w0, PointAux *aux, const double *vh, const double *n_in) {
   constexpr bool F32 = sizeof(R) == 4;
   const int n_k = n_kb / n_batches;
   __shared__ float2 s_w[LDA_MAXK];
@@ -872,21 +872,21 @@ cfm_veff_kernel(long N, int nx, int ny, int nz, double h, int bloch, int n_kb, i
     double v = vloc[p];
     for (int j = 0; j < hist.nh; j++) v += hist.w[j] * hist.v[j][p];
     v += Ex * ((ix - cx) * h) + Ey * ((iy - cy) * h) + Ez * ((iz - cz) * h);
-    *reinterpret_cast<R *>(&aux[p].veff) = (R)v;
+    *reinterpret_cast<R *>(&aux[p].veff) = (R)v + (R)w0;
   }
 }
 
 cudaError_t launch_cfm_veff(int prec, int bloch, long N, int nx, int ny, int nz, double h, int n_kb, int n_batches,
                             const double *wocc, const double *dens_part, const double *vloc, int xc, int push,
-                            const CfmHist &hist, const double E[3], PointAux *aux, cudaStream_t s,
+                            const CfmHist &hist, const double E[3], double w0, PointAux *aux, cudaStream_t s,
                             const double *vh, const double *n_in) {
   const int blocks = lda_blocks(N);
   if (prec == P_C64)
     cfm_veff_kernel<float><<<blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
-                                                          vloc, xc, push, hist, E[0], E[1], E[2], aux, vh, n_in);
+                                                          vloc, xc, push, hist, E[0], E[1], E[2], w0, aux, vh, n_in);
   else
     cfm_veff_kernel<double><<<blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
-                                                           vloc, xc, push, hist, E[0], E[1], E[2], aux, vh, n_in);
+                                                           vloc, xc, push, hist, E[0], E[1], E[2], w0, aux, vh, n_in);
   return cudaGetLastError();
 }
 
@@ -924,7 +924,7 @@ lda_batch_kernel(const BatchAux *aux, const BatchClock *clk, const long *begin, 
   __syncthreads();
   const double E = f;
   lda_body<R>(a.N, a.nx, a.ny, a.nz, a.h, 0, a.n_kb, a.n_batches, a.wocc, a.dens_part, a.vloc, a.xc,
-              E * a.pol[0], E * a.pol[1], E * a.pol[2], 0.0, a.aux, a.lda_part, (int)(blockIdx.x - begin[s]),
+              E * a.pol[0], E * a.pol[1], E * a.pol[2], 0.0, a.w0, a.aux, a.lda_part, (int)(blockIdx.x - begin[s]),
               a.n_lda);
 }
 
@@ -937,15 +937,15 @@ cudaError_t launch_lda_batch(int prec, const BatchAux *aux, const BatchClock *cl
 
 cudaError_t launch_lda(int prec, int bloch, long N, int nx, int ny, int nz, double h, int n_kb, int n_batches,
                        const double *wocc, const double *dens_part, const double *vloc, int xc, const double E[3],
-                       double half_A2, PointAux *aux, double *lda_part, int n_blocks, cudaStream_t s,
+                       double half_A2, double w0, PointAux *aux, double *lda_part, int n_blocks, cudaStream_t s,
                        const double *n_in, const double *vh, int sums) {
   if (prec == P_C64)
     lda_kernel<float><<<n_blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
-                                                       vloc, xc, E[0], E[1], E[2], half_A2, aux, lda_part, n_in, vh,
+                                                       vloc, xc, E[0], E[1], E[2], half_A2, w0, aux, lda_part, n_in, vh,
                                                        sums);
   else
     lda_kernel<double><<<n_blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
-                                                        vloc, xc, E[0], E[1], E[2], half_A2, aux, lda_part, n_in, vh,
+                                                        vloc, xc, E[0], E[1], E[2], half_A2, w0, aux, lda_part, n_in, vh,
                                                         sums);
   return cudaGetLastError();
 }

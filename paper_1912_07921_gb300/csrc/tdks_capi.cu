@@ -193,6 +193,12 @@ void sweep_geometry(const tdks_system *s, SweepParams &p, int sweep) {
   p.n_items = (long)p.n_tx * p.n_ty * p.n_kb * p.n_zc;
 }
 
+double centre_weight(const tdks_system *s) {
+  double c[MAXM + 1], d[MAXM + 1];
+  fd_weights(s->M, c, d);
+  return -1.5 * c[0] / (s->h * s->h);
+}
+
 long n_items_of(const tdks_system *s) {
   SweepParams p{};
   sweep_geometry(s, p);
@@ -217,6 +223,7 @@ void sweep_common(const tdks_system *s, SweepParams &p, const double A[3], int s
   p.nl = s->d_nl;
   p.n_ent = s->n_ent;
   p.kvec = s->d_kvec;
+  p.kphase = s->d_kphase;
   p.bloch = s->bc == TDKS_BC_BLOCH;
   p.L[0] = s->nx * s->h; p.L[1] = s->ny * s->h; p.L[2] = s->nz * s->h;
   for (int a = 0; a < 3; a++) p.A[a] = A[a];
@@ -396,7 +403,7 @@ int run_lda(tdks_system *s, const double E[3], const double A[3], bool sums = tr
   Timed tm(s, 2);
   cudaError_t e = launch_lda(s->prec, s->bc == TDKS_BC_BLOCH, s->N, s->nx, s->ny, s->nz, s->h, s->n_kb,
                              s->n_batches, s->d_wocc, s->dens_part, s->vloc, s->xc != TDKS_XC_NONE, El, half_A2,
-                             s->aux, s->lda_part, lda_blocks(s->N), s->stream,
+                             centre_weight(s), s->aux, s->lda_part, lda_blocks(s->N), s->stream,
                              (s->xfn || hartree) ? s->n_total : nullptr, hartree ? s->d_vh : nullptr, sums ? 1 : 0);
   s->launches++;
   if (e != cudaSuccess) return fail(TDKS_EDEVICE, std::string("lda: ") + cudaGetErrorString(e));
@@ -1218,7 +1225,7 @@ static int run_cfm_veff(tdks_system *s, bool push, int nh, const double w[4], co
   Timed tm(s, 2);
   cudaError_t e = launch_cfm_veff(s->prec, s->bc == TDKS_BC_BLOCH, s->N, s->nx, s->ny, s->nz, s->h, s->n_kb,
                                   s->n_batches, s->d_wocc, s->dens_part, s->vloc, s->xc != TDKS_XC_NONE,
-                                  push ? 1 : 0, h, El, s->aux, s->stream, total && hartree ? s->d_vh : nullptr,
+                                  push ? 1 : 0, h, El, centre_weight(s), s->aux, s->stream, total && hartree ? s->d_vh : nullptr,
                                   total ? s->n_total : nullptr);
   s->launches++;
   if (e != cudaSuccess) return fail(TDKS_EDEVICE, std::string("cfm4 potential: ") + cudaGetErrorString(e));

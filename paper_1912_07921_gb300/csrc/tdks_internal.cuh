@@ -65,8 +65,9 @@ struct TsEntry {
   double ws;
 };
 
-// Per-point record read by the sweeps (16 bytes): the diagonal potential V_eff (double
-// for complex128 systems; float in the first 4 bytes for complex64 systems) and the point's
+// Per-point record read by the sweeps (16 bytes): the diagonal of H, V_eff + w0 with w0 the stencil's
+// centre weight, summed in the compute precision (double for complex128 systems; float in the first 4
+// bytes for complex64 systems; formed once per point here, not once per value in the sweeps), and the point's
 // range [r0, r1) in the point-major projector entry list.
 struct __align__(16) PointAux {
   double veff;
@@ -100,6 +101,7 @@ struct SweepParams {
   // Bloch boundary
   int bloch;                  // periodic cell: values across a face carry exp(i k.L) per wrap
   const double *kvec;         // [n_k][3]
+  const double2 *kphase;      // [n_k][3] e^{i k_a L_a}
   double L[3];
   double A[3];                // vector potential (velocity gauge)
   int grad_mask;              // bit a: add -i A_a grad_a; bit 3: observables need all grads
@@ -170,7 +172,7 @@ cudaError_t launch_nl_current(const NlCurrentParams &p, cudaStream_t s);
 struct BatchAux {
   long N;
   int nx, ny, nz, n_kb, n_batches, xc;
-  double h, occ;
+  double h, occ, w0;
   const double *wocc;       // [n_k] k-weight times occupation
   int gauge, envelope;
   double pol[3], amp, omega, t_total;
@@ -236,7 +238,7 @@ cudaError_t launch_density(int prec, long N, int n_kb, int n_batches, const void
 cudaError_t launch_lda(int prec, int bloch, long N, int nx, int ny, int nz, double h,
                        int n_kb, int n_batches, const double *wocc, const double *dens_part,
                        const double *vloc, int xc,
-                       const double E[3], double half_A2, PointAux *aux, double *lda_part,
+                       const double E[3], double half_A2, double w0, PointAux *aux, double *lda_part,
                        int n_blocks, cudaStream_t s, const double *n_in = nullptr, const double *vh = nullptr,
                        int sums = 1);
 // Classical Runge-Kutta stage update over n complex128 values (complex128 systems):
@@ -257,7 +259,7 @@ struct CfmHist {
 };
 cudaError_t launch_cfm_veff(int prec, int bloch, long N, int nx, int ny, int nz, double h, int n_kb, int n_batches,
                             const double *wocc, const double *dens_part, const double *vloc, int xc, int push,
-                            const CfmHist &hist, const double E[3], PointAux *aux, cudaStream_t s,
+                            const CfmHist &hist, const double E[3], double w0, PointAux *aux, cudaStream_t s,
                             const double *vh = nullptr, const double *n_in = nullptr);
 cudaError_t launch_finalize(const double *obs_part, long n_items, const double *lda_part,
                             int n_lda_blocks, double *record, double t_state, double h3,

@@ -54,7 +54,7 @@ int scratch_address(void **out) {
 }
 
 template <typename R>
-__global__ void noalloc_prepare(long N, const double *vloc, PointAux *aux, int *err) {
+__global__ void noalloc_prepare(long N, const double *vloc, double w0, PointAux *aux, int *err) {
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i == 0) {  // the error word and the sweep's work counter must start at zero on every call
     err[0] = 0;
@@ -62,7 +62,7 @@ __global__ void noalloc_prepare(long N, const double *vloc, PointAux *aux, int *
   }
   if (i < N) {
     PointAux a{0.0, 0, 0};
-    *reinterpret_cast<R *>(&a.veff) = (R)vloc[i];
+    *reinterpret_cast<R *>(&a.veff) = (R)vloc[i] + (R)w0;
     aux[i] = a;
   }
 }
@@ -99,8 +99,8 @@ extern "C" int tdks_apply_H_noalloc(int nx, int ny, int nz, double h, int fd_ord
   s.stream = st;
 
   const int blocks = (int)((N + 255) / 256);
-  if (prec == TDKS_C64) noalloc_prepare<float><<<blocks, 256, 0, st>>>(N, dev_vloc, aux, err);
-  else noalloc_prepare<double><<<blocks, 256, 0, st>>>(N, dev_vloc, aux, err);
+  if (prec == TDKS_C64) noalloc_prepare<float><<<blocks, 256, 0, st>>>(N, dev_vloc, centre_weight(&s), aux, err);
+  else noalloc_prepare<double><<<blocks, 256, 0, st>>>(N, dev_vloc, centre_weight(&s), aux, err);
   CU(cudaGetLastError());
 
   const double A0[3] = {0.0, 0.0, 0.0};

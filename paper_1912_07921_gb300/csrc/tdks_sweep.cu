@@ -61,7 +61,6 @@ sweep_kernel(const SweepParams p) {
   S W[M + 1];
 #pragma unroll
   for (int m = 0; m <= M; m++) W[m] = T::coef(p.w[m], p.wf[m]);
-  const typename W0T<P>::type w0 = P == P_C64 ? (typename W0T<P>::type)p.wf[0] : (typename W0T<P>::type)p.w[0];
   const bool kim = p.coef_im != 0;
   const typename T::K KC = T::kcoef(p.coef, p.coeff, kim);
   const bool need_grad = BLOCH && (p.grad_mask != 0);
@@ -168,7 +167,7 @@ sweep_kernel(const SweepParams p) {
       }
       __syncthreads();
       V gax[3] = {T::zero(), T::zero(), T::zero()};
-      V acc = stencil_point<M, P, BLOCH>(p, W, w0, Q, sm + buf * PLANE, csl, SX * OVC, ve, need_grad, grads, gax);
+      V acc = stencil_point<M, P, BLOCH>(p, W, Q, sm + buf * PLANE, csl, SX * OVC, ve, need_grad, grads, gax);
       if (own && r1 > r0) acc = T::add(acc, T::ld(nlk + (long)r0 * OVC));
       if (MODE == MODE_FIRST && p.do_obs && own) {
         oa.add_e(Q[M], acc);

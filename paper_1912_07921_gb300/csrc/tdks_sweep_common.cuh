@@ -52,10 +52,6 @@ template <> struct ObsAcc<P_C64S> {
   __device__ __forceinline__ double get_j(int a) const { return (double)jh[a] + (double)jl[a]; }
 };
 
-// Diagonal weight w0 in the compute precision.
-template <int P> struct W0T { typedef float type; };
-template <> struct W0T<P_C128> { typedef double type; };
-
 // H applied at one point.  The z-column queue is the circular register array Q of QN
 // (>= 2M+1) entries; plane z+j (j = -M..M) sits in Q[(QB + M + j) % QN] (QB: compile-time
 // rotation, so no register moves per plane).  Sp = shared plane z (vectors, row stride SXO
@@ -63,13 +59,13 @@ template <> struct W0T<P_C128> { typedef double type; };
 // is set (observables of periodic cells).
 template <int M, int P, int BLOCH, int QB = 0, int QN = 2 * M + 1>
 __device__ __forceinline__ typename VT<P>::V
-stencil_point(const SweepParams &p, const typename VT<P>::S *W, typename W0T<P>::type w0,
+stencil_point(const SweepParams &p, const typename VT<P>::S *W,
               const typename VT<P>::V *Q, const typename VT<P>::V *Sp, int csl, int SXO,
               typename VT<P>::R ve, bool need_grad, bool grads, typename VT<P>::V *gax) {
   typedef VT<P> T;
   typedef typename T::V V;
   const V c0 = Q[(QB + M) % QN];
-  V acc = T::mul(T::diag(ve, w0), c0);
+  V acc = T::mul(T::diag(ve), c0);
   V gsum = T::zero();
 #pragma unroll
   for (int m = 1; m <= M; m++) {

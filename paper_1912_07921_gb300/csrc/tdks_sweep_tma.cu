@@ -98,7 +98,6 @@ __device__ __forceinline__ void tma_sweep_body(const Src &src) {
     S_ W[M + 1];
 #pragma unroll
     for (int m = 0; m <= M; m++) W[m] = T::coef(p.w[m], p.wf[m]);
-    const typename W0T<P>::type w0 = P == P_C64 ? (typename W0T<P>::type)p.wf[0] : (typename W0T<P>::type)p.w[0];
     const bool kim = p.coef_im != 0;
     const typename T::K KC = T::kcoef(p.coef, p.coeff, kim);
     int tx, ty, kb, z0, z1;
@@ -154,7 +153,7 @@ __device__ __forceinline__ void tma_sweep_body(const Src &src) {
           const R ve = *reinterpret_cast<const R *>(&a.veff);
           const V nlv = has_proj ? nl_term<P>(nlk, a.r0, a.r1) : T::zero();
           V gax[3];
-          V acc = stencil_point<M, P, 0, QB, QN>(p, W, w0, Q, xs + u * G::PLANE, hsl, G::SX * OVC, ve, false,
+          V acc = stencil_point<M, P, 0, QB, QN>(p, W, Q, xs + u * G::PLANE, hsl, G::SX * OVC, ve, false,
                                                  false, gax);
           const bool live = own && (zf + u < z1);
           if (has_proj) acc = T::add(acc, nlv);
@@ -340,9 +339,9 @@ int ws_shape_planes(int shape, int M, int bloch) {
 
 int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last) {
   if (shape < 5) return shape;
-  if (prec != P_C64) return 2;                                       // the FP64 pipe bounds every shape alike
+  if (prec != P_C64) return shape == 6 && !last && !(bloch && M != 2) ? 6 : 2;
   if (shape == 5) return bloch ? 2 : 5;
-  if (bloch && (M != 2 || nx % 2 != 0 || ny % 2 != 0)) return 2;     // blocks must not straddle a face
+  if (bloch && (M != 2 || (shape != 6 && (nx % 2 != 0 || ny % 2 != 0)))) return 2;  // blocks must not straddle a face
   if (last) return 2;                                                // their operands would not fit
   return shape;
 }

@@ -152,6 +152,8 @@ bool ws_path(const tdks_system *s);
 int kernel_shape(const tdks_system *s, int shape, int sweep);
 void sweep_geometry(const tdks_system *s, tdks::SweepParams &p, int sweep = -1);
 void sweep_common(const tdks_system *s, tdks::SweepParams &p, const double A[3], int sweep = -1);
+// centre weight -3 c_0 / (2 h^2) of the kinetic stencil
+double centre_weight(const tdks_system *s);
 long n_items_of(const tdks_system *s);
 bool encode_map(const tdks_system *s, const void *ptr, int mode, CUtensorMap *out, bool lockstep, int tx, int ty);
 // tile box (no halo) of z depth `depth` over a packed array

@@ -409,8 +409,8 @@ template <int TX, int TY, int R, int OV = OVC, int RX = 1, bool SPL = false> str
 // the halo plane Sp (row 0's own vector at hs0, row stride SXO vectors).  Same terms and
 // summation order as stencil_point.
 template <int M, int P, int QB, int QN, int R>
-__device__ __forceinline__ void stencil_rows(const typename VT<P>::S *W, typename W0T<P>::type w0,
-                                             const typename VT<P>::V (*Q)[QN], const typename VT<P>::V *Sp, int hs0,
+__device__ __forceinline__ void stencil_rows(const typename VT<P>::S *W,
+                                                   const typename VT<P>::V (*Q)[QN], const typename VT<P>::V *Sp, int hs0,
                                              int SXO, const typename VT<P>::R *ve, typename VT<P>::V *acc) {
   typedef VT<P> T;
   typedef typename T::V V;
@@ -418,7 +418,7 @@ __device__ __forceinline__ void stencil_rows(const typename VT<P>::S *W, typenam
 #pragma unroll
   for (int k = 0; k < 2 * M + R; k++) col[k] = Sp[hs0 + (k - M) * SXO];
 #pragma unroll
-  for (int r = 0; r < R; r++) acc[r] = T::mul(T::diag(ve[r], w0), Q[r][(QB + M) % QN]);
+  for (int r = 0; r < R; r++) acc[r] = T::mul(T::diag(ve[r]), Q[r][(QB + M) % QN]);
 #pragma unroll
   for (int m = 1; m <= M; m++) {
 #pragma unroll
@@ -432,20 +432,12 @@ __device__ __forceinline__ void stencil_rows(const typename VT<P>::S *W, typenam
   }
 }
 
-// Bloch phase of one wrap, e^{i ang} = c + i s, in the compute precision.
+// Bloch phase of one wrap, e^{i k_a L_a} = c + i s, in the compute precision (from the table: a sine and
+// cosine in here cost registers, and the FP64 pair is a function call).
 template <int P>
-__device__ __forceinline__ void bloch_phase(double ang, typename VT<P>::S &c, typename VT<P>::S &s) {
-  if constexpr (P != P_C128) {
-    float sn, cs;
-    sincosf((float)ang, &sn, &cs);
-    c = pk2(cs, cs);
-    s = pk2(sn, sn);
-  } else {
-    double sn, cs;
-    sincos(ang, &sn, &cs);
-    c = cs;
-    s = sn;
-  }
+__device__ __forceinline__ void bloch_phase(double2 ph, typename VT<P>::S &c, typename VT<P>::S &s) {
+  c = VT<P>::bc(ph.x);
+  s = VT<P>::bc(ph.y);
 }
 // a times the phase of w wraps, (c + i s)^w (w = +-1 except in grids smaller than the stencil)
 template <int P>
@@ -465,7 +457,7 @@ __device__ __forceinline__ typename VT<P>::V apply_phase(typename VT<P>::S c, ty
 // them), so the neighbours are read as in a finite box.
 template <int M, int P, int QB, int QN, int R>
 __device__ __forceinline__ void stencil_rows_bloch(const SweepParams &p, const typename VT<P>::S *W,
-                                                   typename W0T<P>::type w0, const typename VT<P>::V (*Q)[QN],
+                                              const typename VT<P>::V (*Q)[QN],
                                                    const typename VT<P>::V *S, int hs0, int SXO,
                                                    const typename VT<P>::R *ve, typename VT<P>::V *acc,
                                                    typename VT<P>::V (*gax)[3], bool need_grad, bool grads) {
@@ -483,7 +475,7 @@ __device__ __forceinline__ void stencil_rows_bloch(const SweepParams &p, const t
   V gsum[R];
 #pragma unroll
   for (int r = 0; r < R; r++) {
-    acc[r] = T::mul(T::diag(ve[r], w0), Q[r][(QB + M) % QN]);
+    acc[r] = T::mul(T::diag(ve[r]), Q[r][(QB + M) % QN]);
     gsum[r] = T::zero();
     gax[r][0] = gax[r][1] = gax[r][2] = T::zero();
   }
@@ -523,7 +515,7 @@ __device__ __forceinline__ void stencil_rows_bloch(const SweepParams &p, const t
 // block lies inside the cell or outside it as a whole.
 template <int M, int P, int BLOCH, int QB, int QN>
 __device__ __forceinline__ void stencil_block(const SweepParams &p, const typename VT<P>::S *W,
-                                              typename W0T<P>::type w0, const typename VT<P>::V (*Q)[QN],
+                                              const typename VT<P>::V (*Q)[QN],
                                               const typename VT<P>::V *S0, int SXO, int sx,
                                               const typename VT<P>::R *ve, typename VT<P>::V *acc,
                                               typename VT<P>::V (*gax)[3], bool need_grad, bool grads) {
@@ -537,7 +529,7 @@ __device__ __forceinline__ void stencil_block(const SweepParams &p, const typena
   V gsum[4];
 #pragma unroll
   for (int q = 0; q < 4; q++) {
-    acc[q] = T::mul(T::diag(ve[q], w0), Q[q][(QB + M) % QN]);
+    acc[q] = T::mul(T::diag(ve[q]), Q[q][(QB + M) % QN]);
     if (BLOCH) {
       gsum[q] = T::zero();
       gax[q][0] = gax[q][1] = gax[q][2] = T::zero();
@@ -770,8 +762,8 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
       const bool sl = x0 - M < 0, sr = x0 + TX + M > nx, st = y0 - M < 0, sb = y0 + TY + M > ny;
       const int kidx = kb / p.n_batches;
       S_ cx, sx, cy, sy;
-      bloch_phase<P>(p.kvec[3 * kidx] * p.L[0], cx, sx);
-      bloch_phase<P>(p.kvec[3 * kidx + 1] * p.L[1], cy, sy);
+      bloch_phase<P>(p.kphase[3 * kidx], cx, sx);
+      bloch_phase<P>(p.kphase[3 * kidx + 1], cy, sy);
       constexpr int VB = (int)sizeof(V);  // bytes per thread vector
       constexpr int SRB = (int)(G::STRIPX_BYTES / VB);
       constexpr int STB = SRB + (int)(G::STRIPX_BYTES / VB);
@@ -879,7 +871,6 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
     S_ W[M + 1];
 #pragma unroll
     for (int m = 0; m <= M; m++) W[m] = T::coef(p.w[m], p.wf[m]);
-    const typename W0T<P>::type w0 = P != P_C128 ? (typename W0T<P>::type)p.wf[0] : (typename W0T<P>::type)p.w[0];
     const bool kim = p.coef_im != 0;
     const typename T::K KC = T::kcoef(p.coef, p.coeff, kim);
     int tx, ty, kb, z0, z1;
@@ -892,7 +883,7 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
     // periodic cell: the Bloch phase of one wrap along z, e^{i k_z L_z} = cz + i sz, applied to
     // the queue planes loaded from beyond a z face (the patcher warp handles x and y)
     S_ cz{}, sz{};
-    if constexpr (BLOCH) bloch_phase<P>(p.kvec[3 * kidx + 2] * p.L[2], cz, sz);
+    if constexpr (BLOCH) bloch_phase<P>(p.kphase[3 * kidx + 2], cz, sz);
     S_ szm = sz;  // -sz: one wrap the other way
     if constexpr (P != P_C128) szm ^= SIGN2; else szm = -szm;
     const bool need_grad = BLOCH && p.grad_mask != 0;
@@ -1000,12 +991,12 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
           }
           [[maybe_unused]] V gax[BLOCH ? NP : 1][3];
           if constexpr (RX == 2) {
-            stencil_block<M, P, BLOCH, QB, QN>(p, W, w0, Q, xs + u * G::SX * G::SY * OV + hs0, SXO, sx, ve, acc, gax,
+            stencil_block<M, P, BLOCH, QB, QN>(p, W, Q, xs + u * G::SX * G::SY * OV + hs0, SXO, sx, ve, acc, gax,
                                                need_grad, grads);
           } else if constexpr (BLOCH) {
-            stencil_rows_bloch<M, P, QB, QN, R>(p, W, w0, Q, xs + u * G::SX * G::SY * OV, hs0, SXO, ve, acc, gax, need_grad, grads);
+            stencil_rows_bloch<M, P, QB, QN, R>(p, W, Q, xs + u * G::SX * G::SY * OV, hs0, SXO, ve, acc, gax, need_grad, grads);
           } else {
-            stencil_rows<M, P, QB, QN, R>(W, w0, Q, xs + u * G::SX * G::SY * OV, hs0, SXO, ve, acc);
+            stencil_rows<M, P, QB, QN, R>(W, Q, xs + u * G::SX * G::SY * OV, hs0, SXO, ve, acc);
           }
           if constexpr (LATE_NL) {
 #pragma unroll
@@ -1020,7 +1011,10 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
 #pragma unroll
           for (int q = 0; q < NP; q++) {
             const bool live = own[q] && (zf + u < z1);
-            if (add_nl) acc[q] = T::add(acc[q], nlv[q]);
+            if (add_nl) {
+              if constexpr (P == P_C128) asm volatile("");  // (a branch: speculated, the sums are not saved)
+              acc[q] = T::add(acc[q], nlv[q]);
+            }
             const V c0 = Q[q][(QB + M) % QN];
             if (MODE == MODE_FIRST && do_obs && live) {
               oa.add_e(c0, acc[q]);
@@ -1145,8 +1139,14 @@ cudaError_t launch_ws_batch_shape(int M, int prec, int mode, const BatchSweepArg
   }                                                                               \
   return cudaErrorInvalidValue;
   if constexpr (C64Shape<SHAPE>::ONLY) {
-    if (prec != P_C64) return cudaErrorInvalidValue;
     constexpr int P = C64Shape<SHAPE>::P;
+    if constexpr (SHAPE == 6) {
+      if (prec == P_C128 && M == 2 && mode == MODE_FIRST) return launch_ws_batch_t<SHAPE, 2, P_C128, MODE_FIRST>(a, s);
+      if (prec == P_C128 && M == 2 && mode == MODE_MID) return launch_ws_batch_t<SHAPE, 2, P_C128, MODE_MID>(a, s);
+      if (prec == P_C128 && M == 4 && mode == MODE_FIRST) return launch_ws_batch_t<SHAPE, 4, P_C128, MODE_FIRST>(a, s);
+      if (prec == P_C128 && M == 4 && mode == MODE_MID) return launch_ws_batch_t<SHAPE, 4, P_C128, MODE_MID>(a, s);
+    }
+    if (prec != P_C64) return cudaErrorInvalidValue;
     if constexpr (C64Shape<SHAPE>::LAST) {
       if (M == 2 && mode == MODE_LAST) return launch_ws_batch_t<SHAPE, 2, P, MODE_LAST>(a, s);
       if constexpr (C64Shape<SHAPE>::M4)
@@ -1197,6 +1197,21 @@ template <int SHAPE>
 cudaError_t launch_ws_shape(int M, int prec, int mode, int bloch, const SweepMaps &maps, const SweepParams &p,
                             int grid, cudaStream_t s) {
   if constexpr (C64Shape<SHAPE>::ONLY) {
+    if constexpr (SHAPE == 6) {
+      if (prec == P_C128) {
+        if (mode == MODE_LAST) return cudaErrorInvalidValue;
+        const bool first = mode == MODE_FIRST;
+        if (bloch && M == 2)
+          return first ? launch_ws_t<SHAPE, 2, P_C128, MODE_FIRST, 1>(maps, p, grid, s)
+                       : launch_ws_t<SHAPE, 2, P_C128, MODE_MID, 1>(maps, p, grid, s);
+        if (bloch) return cudaErrorInvalidValue;
+        if (M == 2)
+          return first ? launch_ws_t<SHAPE, 2, P_C128, MODE_FIRST, 0>(maps, p, grid, s)
+                       : launch_ws_t<SHAPE, 2, P_C128, MODE_MID, 0>(maps, p, grid, s);
+        return first ? launch_ws_t<SHAPE, 4, P_C128, MODE_FIRST, 0>(maps, p, grid, s)
+                     : launch_ws_t<SHAPE, 4, P_C128, MODE_MID, 0>(maps, p, grid, s);
+      }
+    }
     constexpr int P = C64Shape<SHAPE>::P;
     if (prec != P_C64) return cudaErrorInvalidValue;
 #define TDKS_WS5_MODES(MM, BL)                                                                   \

@@ -96,8 +96,8 @@ template <> struct VT<P_C128> {
   static __device__ __forceinline__ S bc(double s) { return s; }
   // a coefficient from its FP64 value (the FP32 copy is for complex64)
   static __device__ __forceinline__ S coef(double d, float) { return d; }
-  // diagonal (V_eff(r) + w0) broadcast, in the compute precision
-  static __device__ __forceinline__ S diag(R ve, double w0) { return ve + w0; }
+  // the point record's diagonal, broadcast
+  static __device__ __forceinline__ S diag(R ve) { return ve; }
   static __device__ __forceinline__ V add(V a, V b) { return make_double2(a.x + b.x, a.y + b.y); }
   static __device__ __forceinline__ V sub(V a, V b) { return make_double2(a.x - b.x, a.y - b.y); }
   static __device__ __forceinline__ V mul(S s, V a) { return make_double2(s * a.x, s * a.y); }
@@ -137,7 +137,7 @@ template <> struct VT<P_C64> {
   static __device__ __forceinline__ S bc(double s) { float f = (float)s; return pk2(f, f); }
   // a coefficient from its FP32 copy (no FP64 conversion in the kernel)
   static __device__ __forceinline__ S coef(double, float f) { return pk2(f, f); }
-  static __device__ __forceinline__ S diag(R ve, float w0) { const float d = ve + w0; return pk2(d, d); }
+  static __device__ __forceinline__ S diag(R ve) { return pk2(ve, ve); }
   static __device__ __forceinline__ V add(V a, V b) { return make_ulonglong2(add2(a.x, b.x), add2(a.y, b.y)); }
   static __device__ __forceinline__ V sub(V a, V b) { return make_ulonglong2(sub2(a.x, b.x), sub2(a.y, b.y)); }
   static __device__ __forceinline__ V mul(S s, V a) { return make_ulonglong2(mul2(s, a.x), mul2(s, a.y)); }
@@ -183,7 +183,7 @@ template <> struct VT<P_C64S> {
   static __device__ __forceinline__ V zero() { return 0ull; }
   static __device__ __forceinline__ S bc(double s) { float f = (float)s; return pk2(f, f); }
   static __device__ __forceinline__ S coef(double, float f) { return pk2(f, f); }
-  static __device__ __forceinline__ S diag(R ve, float w0) { const float d = ve + w0; return pk2(d, d); }
+  static __device__ __forceinline__ S diag(R ve) { return pk2(ve, ve); }
   static __device__ __forceinline__ V add(V a, V b) { return add2(a, b); }
   static __device__ __forceinline__ V sub(V a, V b) { return sub2(a, b); }
   static __device__ __forceinline__ V mul(S s, V a) { return mul2(s, a); }
