@@ -24,9 +24,15 @@ namespace tdks {
 // ---------------------------------------------------------------------------------
 constexpr int GATHER_THREADS = 256;
 
-int gather_chunks(long units) {
+// CTAs of a unit.  Of a batch: as many as fill the GPU.  Of a system alone (a cluster): 8 while all units
+// are resident at once that way, else 4, also where the units alone would fill the GPU, as a CTA's loop is
+// a chain of dependent loads.  Gather and non-local kernel of 8 atoms x 16 k-batches in a 64^3 cell: 115 us
+// with 1 CTA a unit, 78, 68, 62 with 2, 3, 4, then 77, 74, 70 with 5, 6, 8 (clusters of 5 to 7 leave SMs of a
+// GPC over); 16 atoms x 8: 42, 33, 31, 30, 38, 38, 39.
+int gather_chunks(long units, bool cluster) {
+  if (cluster) return units * 16 <= 152L * 4 ? 8 : 4;  // (8 CTAs: the portable cluster size)
   const long want = (152L * 4 + units - 1) / units;
-  return (int)(want < 1 ? 1 : (want > 8 ? 8 : want));  // (8 CTAs: the portable cluster size)
+  return (int)(want < 1 ? 1 : (want > 8 ? 8 : want));
 }
 
 // (out: this CTA's 4 x OVC x 2 sums, index (j OVC + v) 2 + c)
@@ -45,6 +51,7 @@ __device__ __forceinline__ void gather_body(const GatherParams &p, int a, int kb
   const int len = (a1 - a0 + p.n_chunks - 1) / p.n_chunks;
   const int e0 = a0 + chunk * len, e1 = min(a1, e0 + len);
   const bool phase = BLOCH || (p.A[0] != 0.0 || p.A[1] != 0.0 || p.A[2] != 0.0);
+#pragma unroll 4
   for (int e = e0 + lane; e < e1; e += LANES) {
     if constexpr (P == P_C64) {
       // compact entry arrays: 8 + 16 bytes per entry instead of the full record
@@ -220,21 +227,70 @@ __device__ __forceinline__ void nl_body(const GatherParams &p, long t, int kb) {
   reinterpret_cast<V *>(p.nl)[((long)kb * (p.n_ent + 1) + r.x) * OVC + v] = acc;
 }
 
-// (with many k-batches each thread takes its (sphere point, vector) through a run of them: the
-// point's entry data stays in L1 across the run, and a periodic cell's 64 k-batches need 8x
-// fewer CTAs; a molecule's few k-batches keep one per CTA row, for parallelism)
-constexpr int NL_KB_RUN = 8;
-inline unsigned nl_kb_rows(int n_kb) { return n_kb >= 4 * NL_KB_RUN ? (n_kb + NL_KB_RUN - 1) / NL_KB_RUN : n_kb; }
-template <int P, int BLOCH>
-__global__ void __launch_bounds__(NL_THREADS) nl_kernel(const GatherParams p) {
-  const long t = (long)blockIdx.x * NL_THREADS + threadIdx.x;
-  if ((int)gridDim.y == p.n_kb) {
-    nl_body<P, BLOCH>(p, t, blockIdx.y);
-    return;
+// The same at RUN k-batches kb0 .. at once (a single system's kernel): the point's entries, their
+// strengths and phases are read once for all of them, and the loads of RUN k-batches are in flight together.
+template <int P, int BLOCH, int RUN>
+__device__ __forceinline__ void nl_run(const GatherParams &p, long t, int kb0) {
+  typedef VT<P> T;
+  typedef typename T::V V;
+  const long sidx = t / OVC;
+  const int v = (int)(t % OVC);
+  if (sidx >= p.n_sp) return;
+  const int2 r = p.sp[sidx];
+  const bool phase = BLOCH || (p.A[0] != 0.0 || p.A[1] != 0.0 || p.A[2] != 0.0);
+  V acc[RUN];
+#pragma unroll
+  for (int i = 0; i < RUN; i++) acc[i] = T::zero();
+  for (int e = r.x; e < r.y; e++) {
+    const int ei = p.rowent[e];
+    typename T::S b[4];
+    int atom;
+    if constexpr (P == P_C64) {
+      atom = p.ent_ca[ei].y;
+      const float4 b4 = p.ent_beta[ei];
+      b[0] = T::coef(0.0, b4.x); b[1] = T::coef(0.0, b4.y); b[2] = T::coef(0.0, b4.z); b[3] = T::coef(0.0, b4.w);
+    } else {
+      const ProjEntry &E = p.ent[ei];
+      atom = E.atom;
+#pragma unroll
+      for (int j = 0; j < 4; j++) b[j] = E.betad[j];
+    }
+#pragma unroll
+    for (int i = 0; i < RUN; i++) {
+      const int kb = kb0 + i;
+      if (RUN > 1 && kb >= p.n_kb) break;
+      const V *qa = reinterpret_cast<const V *>(p.q) + ((long)(kb * p.n_atoms + atom) * 4) * OVC + v;
+      V x = T::mul(b[0], T::ld(qa));
+#pragma unroll
+      for (int j = 1; j < 4; j++) x = T::fma(b[j], T::ld(qa + j * OVC), x);
+      if (phase) {
+        const long pi = (long)(kb / p.n_batches) * p.n_ent + ei;
+        if constexpr (P == P_C64) {
+          const float2 ph = reinterpret_cast<const float2 *>(p.phase)[pi];
+          x = T::cmul(pk2(ph.x, ph.x), pk2(-ph.y, -ph.y), x);
+        } else {
+          const double2 ph = reinterpret_cast<const double2 *>(p.phase)[pi];
+          x = T::cmul(ph.x, -ph.y, x);
+        }
+      }
+      acc[i] = T::add(acc[i], x);
+    }
   }
-  const int run = (p.n_kb + gridDim.y - 1) / gridDim.y;
-  const int kb0 = blockIdx.y * run, kb1 = min(p.n_kb, kb0 + run);
-  for (int kb = kb0; kb < kb1; kb++) nl_body<P, BLOCH>(p, t, kb);
+#pragma unroll
+  for (int i = 0; i < RUN; i++)
+    if (RUN == 1 || kb0 + i < p.n_kb)
+      reinterpret_cast<V *>(p.nl)[((long)(kb0 + i) * (p.n_ent + 1) + r.x) * OVC + v] = acc[i];
+}
+
+// k-batches a thread takes: up to 4 as long as ~6 CTAs per SM are left (8 is slower: registers).
+inline int nl_run_of(int n_sp, int n_kb) {
+  int run = 4;
+  while (run > 1 && ((long)n_sp * OVC + NL_THREADS - 1) / NL_THREADS * ((n_kb + run - 1) / run) < 152 * 6) run /= 2;
+  return run;
+}
+template <int P, int BLOCH, int RUN>
+__global__ void __launch_bounds__(NL_THREADS) nl_kernel(const GatherParams p) {
+  nl_run<P, BLOCH, RUN>(p, (long)blockIdx.x * NL_THREADS + threadIdx.x, blockIdx.y * RUN);
 }
 
 // Batched gather: stage 1 over every system's (atom, kb, chunk) CTAs, stage 2 over every
@@ -422,18 +478,8 @@ __global__ void __launch_bounds__(NLC_THREADS) nl_current_kernel(const NlCurrent
 
 cudaError_t launch_nl_current(const NlCurrentParams &q, cudaStream_t s) {
   NlCurrentParams p = q;
-  p.n_chunks = gather_chunks((long)p.n_atoms * p.n_kb);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(p.n_atoms * p.n_chunks, p.n_kb);
-  cfg.blockDim = dim3(NLC_THREADS);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = p.n_chunks;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, nl_current_kernel, p);
+  p.n_chunks = gather_chunks((long)p.n_atoms * p.n_kb, true);
+  return launch_cluster(nl_current_kernel, dim3(p.n_atoms * p.n_chunks, p.n_kb), NLC_THREADS, s, p.n_chunks, p);
 }
 
 // Entry phases (cos, sin) of k.T + A.d, as the projector kernels read them: for complex64 systems the
@@ -465,29 +511,23 @@ cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_
   const long n = (long)n_ent * n_k;
   if (n <= 0) return cudaSuccess;
   const unsigned grid = (unsigned)((n + 127) / 128);
-  if (prec == P_C64)
-    phase_table_kernel<P_C64><<<grid, 128, 0, s>>>(ent, n_ent, n_k, kvec, A[0], A[1], A[2], bloch, out);
-  else
-    phase_table_kernel<P_C128><<<grid, 128, 0, s>>>(ent, n_ent, n_k, kvec, A[0], A[1], A[2], bloch, out);
+  const auto kern = prec == P_C64 ? phase_table_kernel<P_C64> : phase_table_kernel<P_C128>;
+  kern<<<grid, 128, 0, s>>>(ent, n_ent, n_k, kvec, A[0], A[1], A[2], bloch, out);
   return cudaGetLastError();
 }
 
 template <int P, int BLOCH>
 static cudaError_t launch_gather_t(const GatherParams &p, cudaStream_t s) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(p.n_atoms * p.n_chunks, p.n_kb);
-  cfg.blockDim = dim3(GATHER_THREADS);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = p.n_chunks;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cudaError_t e = cudaLaunchKernelEx(&cfg, gather_kernel<P, BLOCH>, p)) return e;
-  if (p.n_sp > 0) {
-    const dim3 grid((unsigned)(((long)p.n_sp * OVC + NL_THREADS - 1) / NL_THREADS), nl_kb_rows(p.n_kb));
-    nl_kernel<P, BLOCH><<<grid, NL_THREADS, 0, s>>>(p);
+  if (cudaError_t e = launch_cluster(gather_kernel<P, BLOCH>, dim3(p.n_atoms * p.n_chunks, p.n_kb), GATHER_THREADS, s,
+                                     p.n_chunks, p))
+    return e;
+  if (p.n_sp <= 0) return cudaSuccess;
+  const int run = nl_run_of(p.n_sp, p.n_kb);
+  const dim3 grid((unsigned)(((long)p.n_sp * OVC + NL_THREADS - 1) / NL_THREADS), (p.n_kb + run - 1) / run);
+  switch (run) {
+    case 1: nl_kernel<P, BLOCH, 1><<<grid, NL_THREADS, 0, s>>>(p); break;
+    case 2: nl_kernel<P, BLOCH, 2><<<grid, NL_THREADS, 0, s>>>(p); break;
+    default: nl_kernel<P, BLOCH, 4><<<grid, NL_THREADS, 0, s>>>(p);
   }
   return cudaGetLastError();
 }
@@ -794,10 +834,8 @@ cudaError_t launch_rk4_finish(long n, void *psi, const void *acc, const void *k,
 
 cudaError_t launch_density_sum(int prec, long N, int n_kb, int n_batches, const double *wocc,
                                const double *dens_part, double *n_out, cudaStream_t s) {
-  if (prec == P_C64)
-    density_sum_kernel<float><<<lda_blocks(N), lda_threads(N), 0, s>>>(N, n_kb, n_batches, wocc, dens_part, n_out);
-  else
-    density_sum_kernel<double><<<lda_blocks(N), lda_threads(N), 0, s>>>(N, n_kb, n_batches, wocc, dens_part, n_out);
+  const auto kern = prec == P_C64 ? density_sum_kernel<float> : density_sum_kernel<double>;
+  kern<<<lda_blocks(N), lda_threads(N), 0, s>>>(N, n_kb, n_batches, wocc, dens_part, n_out);
   return cudaGetLastError();
 }
 
@@ -881,12 +919,8 @@ cudaError_t launch_cfm_veff(int prec, int bloch, long N, int nx, int ny, int nz,
                             const CfmHist &hist, const double E[3], double w0, PointAux *aux, cudaStream_t s,
                             const double *vh, const double *n_in) {
   const int blocks = lda_blocks(N);
-  if (prec == P_C64)
-    cfm_veff_kernel<float><<<blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
-                                                          vloc, xc, push, hist, E[0], E[1], E[2], w0, aux, vh, n_in);
-  else
-    cfm_veff_kernel<double><<<blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
-                                                           vloc, xc, push, hist, E[0], E[1], E[2], w0, aux, vh, n_in);
+  const auto kern = prec == P_C64 ? cfm_veff_kernel<float> : cfm_veff_kernel<double>;
+  kern<<<blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part, vloc, xc, push, hist, E[0], E[1], E[2], w0, aux, vh, n_in);
   return cudaGetLastError();
 }
 
@@ -939,14 +973,8 @@ cudaError_t launch_lda(int prec, int bloch, long N, int nx, int ny, int nz, doub
                        const double *wocc, const double *dens_part, const double *vloc, int xc, const double E[3],
                        double half_A2, double w0, PointAux *aux, double *lda_part, int n_blocks, cudaStream_t s,
                        const double *n_in, const double *vh, int sums) {
-  if (prec == P_C64)
-    lda_kernel<float><<<n_blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
-                                                       vloc, xc, E[0], E[1], E[2], half_A2, w0, aux, lda_part, n_in, vh,
-                                                       sums);
-  else
-    lda_kernel<double><<<n_blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part,
-                                                        vloc, xc, E[0], E[1], E[2], half_A2, w0, aux, lda_part, n_in, vh,
-                                                        sums);
+  const auto kern = prec == P_C64 ? lda_kernel<float> : lda_kernel<double>;
+  kern<<<n_blocks, lda_threads(N), 0, s>>>(N, nx, ny, nz, h, bloch, n_kb, n_batches, wocc, dens_part, vloc, xc, E[0], E[1], E[2], half_A2, w0, aux, lda_part, n_in, vh, sums);
   return cudaGetLastError();
 }
 
@@ -1098,18 +1126,8 @@ static cudaError_t launch_finalize_cluster(const double *obs_part, long n_items,
                                            double field_val, cudaStream_t s) {
   const long want = (n_items + n_lda + 4L * FIN_MAX_THREADS - 1) / (4L * FIN_MAX_THREADS);
   const unsigned nb = (unsigned)(want < 1 ? 1 : (want > 8 ? 8 : want));
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(nb);
-  cfg.blockDim = dim3(FIN_MAX_THREADS);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = nb;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, finalize_kernel, obs_part, n_items, lda_part, n_lda, sums, rec, t_state, h3, occ,
-                            bloch, omega_cell, Ax, Ay, Az, field_val);
+  return launch_cluster(finalize_kernel, nb, FIN_MAX_THREADS, s, (int)nb, obs_part, n_items, lda_part, n_lda, sums, rec,
+                        t_state, h3, occ, bloch, omega_cell, Ax, Ay, Az, field_val);
 }
 
 cudaError_t launch_finalize_sums(const double *obs_part, long n_items, const double *lda_part, int n_lda,
@@ -1139,36 +1157,25 @@ cudaError_t launch_finalize(const double *obs_part, long n_items, const double *
 // into hi = fl32(x) and lo = fl32(x - hi) (the double-float state); unpacking returns
 // hi + lo in FP64.
 // ---------------------------------------------------------------------------------
-__global__ void pack_kernel(int to_internal, int c64, long N, int n_k, int n_orb, int n_batches, int BS,
-                            void *internal, void *internal_lo, double2 *plain) {
-  const long total = (long)n_k * n_batches * N * BS;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const int j = (int)(i % BS);
-    long r = i / BS;
-    const long pt = r % N;
-    r /= N;
-    const int b = (int)(r % n_batches);
-    const int k = (int)(r / n_batches);
-    const int o = b * BS + j;
-    const long pidx = ((long)k * N + pt) * n_orb + o;
-    if (to_internal) {
-      const double2 x = o < n_orb ? plain[pidx] : make_double2(0.0, 0.0);
-      if (c64) {
-        const float hx = (float)x.x, hy = (float)x.y;
-        reinterpret_cast<float2 *>(internal)[i] = make_float2(hx, hy);
-        reinterpret_cast<float2 *>(internal_lo)[i] = make_float2((float)(x.x - (double)hx), (float)(x.y - (double)hy));
-      } else {
-        reinterpret_cast<double2 *>(internal)[i] = x;
-      }
-    } else if (o < n_orb) {
-      if (c64) {
-        const float2 h = reinterpret_cast<const float2 *>(internal)[i];
-        const float2 l = reinterpret_cast<const float2 *>(internal_lo)[i];
-        plain[pidx] = make_double2((double)h.x + (double)l.x, (double)h.y + (double)l.y);
-      } else {
-        plain[pidx] = reinterpret_cast<const double2 *>(internal)[i];
-      }
+// Internal layout -> host layout for the points [g0, g0 + npts) of all k-points' points one after another
+// (chunks, so that the copy to the host of one overlaps the unpacking of the next).  Thread = one value
+// of the host layout.
+__global__ void unpack_kernel(int c64, long N, long g0, long npts, int n_orb, int n_batches, int BS,
+                              const void *internal, const void *internal_lo, double2 *plain) {
+  const unsigned stride = gridDim.x * blockDim.x;
+  const unsigned long long total = (unsigned long long)npts * n_orb;
+  for (unsigned long long i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+    const long pt = (long)(i / (unsigned)n_orb), g = g0 + pt, k = g / N;
+    const unsigned o = (unsigned)(i - (unsigned long long)pt * n_orb), b = o / BS, j = o - b * BS;
+    const long src = ((k * n_batches + b) * N + (g - k * N)) * BS + j;
+    double2 x;
+    if (c64) {
+      const float2 h = reinterpret_cast<const float2 *>(internal)[src], l = reinterpret_cast<const float2 *>(internal_lo)[src];
+      x = make_double2((double)h.x + (double)l.x, (double)h.y + (double)l.y);
+    } else {
+      x = reinterpret_cast<const double2 *>(internal)[src];
     }
+    plain[g0 * n_orb + i] = x;
   }
 }
 
@@ -1229,14 +1236,14 @@ cudaError_t launch_pack_in(int prec, long N, int k, long pt0, long npts, int n_o
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack(int prec, int to_internal, long N, int n_k, int n_orb, int n_batches, void *internal,
-                        void *internal_lo, double *plain, cudaStream_t s) {
+cudaError_t launch_unpack(int prec, long N, long g0, long npts, int n_orb, int n_batches, const void *internal,
+                          const void *internal_lo, double *plain, cudaStream_t s) {
   const int BS = prec == P_C64 ? 2 * OVC : OVC;
-  const long total = (long)n_k * n_batches * N * BS;
-  long g = (total + 255) / 256;
+  long g = (npts * n_orb + 255) / 256;
   if (g > 152 * 32) g = 152 * 32;
-  pack_kernel<<<(int)g, 256, 0, s>>>(to_internal, prec == P_C64, N, n_k, n_orb, n_batches, BS, internal,
-                                     internal_lo, (double2 *)plain);
+  if (g <= 0) return cudaSuccess;
+  unpack_kernel<<<(int)g, 256, 0, s>>>(prec == P_C64, N, g0, npts, n_orb, n_batches, BS, internal, internal_lo,
+                                       (double2 *)plain);
   return cudaGetLastError();
 }
 

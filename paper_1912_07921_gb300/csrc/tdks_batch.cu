@@ -242,7 +242,7 @@ int tdks_batch_create(const tdks_sys *systems, int n, void *stream, tdks_batch_t
   // partial-sum buffer holds
   long batch_units = 0;
   for (tdks_system *s : b->sys) batch_units += (long)s->n_atoms * s->n_kb;
-  const int bchunks = gather_chunks(std::max(batch_units, 1L));
+  const int bchunks = gather_chunks(std::max(batch_units, 1L), false);
   for (int i = 0; i < n; i++) {
     tdks_system *s = b->sys[i];
     const void *ins[4] = {s->psi, s->term[0], s->term[1], s->term[2]};
@@ -392,7 +392,8 @@ int tdks_batch_autotune(tdks_batch_t b, int reps, double *ms) {
   const int n = (int)b->sys.size();
   const int saved[4] = {b->shape[0], b->shape[1], b->shape[2], b->shape[3]};
   int pick[4] = {saved[0], saved[1], saved[2], saved[3]};
-  double best[4] = {-1.0, -1.0, -1.0, -1.0};
+  double best[4] = {-1.0, -1.0, -1.0, -1.0}, took[WS_SHAPES][4];
+  for (int i = 0; i < WS_SHAPES * 4; i++) took[i / 4][i % 4] = -1.0;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   CU(cudaEventCreate(&e0));
   if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -405,12 +406,18 @@ int tdks_batch_autotune(tdks_batch_t b, int reps, double *ms) {
     for (int k = 0; k < 4; k++) b->shape[k] = sh;
     if ((rc = build_sweep_tables(b, true))) break;
     for (int k = 0; k < 4 && !rc; k++) {
+      const int ks = kernel_shape(b->sys[0], sh, k);
+      double &per = took[ks][k];  // shapes that run one kernel are timed once
+      if (per >= 0.0) {
+        if (ms) ms[sh * 4 + k] = per;
+        continue;
+      }
       BatchSweepArgs a{b->d_sweep[k], b->d_maps, k, b->d_item_begin[k],
                       n, b->total_items[k], b->d_work, b->d_item_sys[k]};
-      cudaError_t e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, kernel_shape(b->sys[0], sh, k));  // warm-up
+      cudaError_t e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, ks);  // warm-up
       cudaEventRecord(e0, b->work);
       for (int r = 0; r < reps && e == cudaSuccess; r++)
-        e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, kernel_shape(b->sys[0], sh, k));
+        e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, ks);
       cudaEventRecord(e1, b->work);
       if (e != cudaSuccess) { rc = fail(TDKS_EDEVICE, std::string("batched sweep: ") + cudaGetErrorString(e)); break; }
       if (cudaEventSynchronize(e1) != cudaSuccess) { rc = fail(TDKS_EDEVICE, "batch autotune timing"); break; }
@@ -419,7 +426,7 @@ int tdks_batch_autotune(tdks_batch_t b, int reps, double *ms) {
       if (rc) break;
       float t = 0.f;
       cudaEventElapsedTime(&t, e0, e1);
-      const double per = (double)t / reps;
+      per = (double)t / reps;
       if (ms) ms[sh * 4 + k] = per;
       if (best[k] < 0.0 || per < best[k]) { best[k] = per; pick[k] = sh; }
     }

@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <utility>
 
 namespace tdks {
 
@@ -35,6 +36,22 @@ inline cudaError_t ensure_smem_attr(K k, size_t smem, std::atomic<unsigned> &don
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_acq_rel);
   return e;
+}
+
+// Launch with thread-block clusters of `cluster` CTAs along x.
+template <typename... Par, typename... Arg>
+inline cudaError_t launch_cluster(void (*k)(Par...), dim3 grid, dim3 block, cudaStream_t s, int cluster, Arg &&...arg) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, std::forward<Arg>(arg)...);
 }
 
 constexpr int OVC = 4;        // 16-byte vectors per (point, batch)
@@ -232,7 +249,7 @@ cudaError_t launch_gather(int prec, int bloch, const GatherParams &p, cudaStream
 cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_k, const double *kvec,
                                const double A[3], int bloch, void *out, cudaStream_t s);
 // chunks per (atom, k-batch) that fill the GPU for n_atoms * n_kb units
-int gather_chunks(long units);
+int gather_chunks(long units, bool cluster);
 cudaError_t launch_density(int prec, long N, int n_kb, int n_batches, const void *psi, const void *psi_lo,
                            const double *wocc, double *dens_part, cudaStream_t s);
 cudaError_t launch_lda(int prec, int bloch, long N, int nx, int ny, int nz, double h,
@@ -277,8 +294,8 @@ cudaError_t launch_record_from_sums(const double *sums, double *record, double t
 cudaError_t launch_pack_in(int prec, long N, int k, long pt0, long npts, int n_orb, int n_batches,
                            const double *plain, void *internal, void *internal_lo, const double *wocc,
                            double *dens_part, cudaStream_t s);
-cudaError_t launch_pack(int prec, int to_internal, long N, int n_k, int n_orb, int n_batches,
-                        void *internal, void *internal_lo, double *plain, cudaStream_t s);
+cudaError_t launch_unpack(int prec, long N, long g0, long npts, int n_orb, int n_batches, const void *internal,
+                          const void *internal_lo, double *plain, cudaStream_t s);
 
 // TMA sweep for finite boxes (tdks_sweep_tma.cu).  maps.in: dims {16 floats, nx, ny, nz,
 // n_kb}, box {16, TX+2M, TY+2M, tma_planes(prec, mode), 1} (TY: the shape's tile height); maps.aux: dims {4, nx, ny, nz}

@@ -338,6 +338,11 @@ int ws_shape_planes(int shape, int M, int bloch) {
 }
 
 int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last) {
+  // The tile of 16 x 12 points: with four service warps the complex64 kernels of shape 1 have 168
+  // registers and spill (order 8: 0.56 ms where shape 2 takes 0.27), as do shape 2's records in periodic
+  // cells (0.55 ms against 0.22 with shape 6).
+  if (prec == P_C64 && (shape == 1 || (bloch && (shape == 2 || shape == 5))))
+    return last || (bloch && M != 2) ? 2 : 6;
   if (shape < 5) return shape;
   if (prec != P_C64) return shape == 6 && !last && !(bloch && M != 2) ? 6 : 2;
   if (shape == 5) return bloch ? 2 : 5;

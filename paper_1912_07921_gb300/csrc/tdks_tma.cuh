@@ -1159,11 +1159,17 @@ cudaError_t launch_ws_batch_shape(int M, int prec, int mode, const BatchSweepArg
       if (M == 4 && mode == MODE_MID) return launch_ws_batch_t<SHAPE, 4, P, MODE_MID>(a, s);
     }
   } else {
+    if constexpr (SHAPE == 1)
+      if (prec == P_C64) return cudaErrorInvalidValue;  // (complex128 only)
     if (M == 2) {
-      if (prec == P_C64) { TDKS_WSB_MODES(2, P_C64) } else { TDKS_WSB_MODES(2, P_C128) }
+      if constexpr (SHAPE != 1)
+        if (prec == P_C64) { TDKS_WSB_MODES(2, P_C64) }
+      TDKS_WSB_MODES(2, P_C128)
     }
     if (M == 4) {
-      if (prec == P_C64) { TDKS_WSB_MODES(4, P_C64) } else { TDKS_WSB_MODES(4, P_C128) }
+      if constexpr (SHAPE != 1)
+        if (prec == P_C64) { TDKS_WSB_MODES(4, P_C64) }
+      TDKS_WSB_MODES(4, P_C128)
     }
   }
 #undef TDKS_WSB_MODES
@@ -1181,11 +1187,17 @@ static cudaError_t launch_ws_bc(int M, int prec, int mode, const SweepMaps &maps
     case MODE_LAST: return launch_ws_t<SHAPE, MM, PP, MODE_LAST, BLOCH>(maps, p, grid, s);   \
   }                                                                                          \
   return cudaErrorInvalidValue;
+  if constexpr (SHAPE == 1)
+    if (prec == P_C64) return cudaErrorInvalidValue;  // (complex128 only)
   if (M == 2) {
-    if (prec == P_C64) { TDKS_WS_MODES(2, P_C64) } else { TDKS_WS_MODES(2, P_C128) }
+    if constexpr (SHAPE != 1)
+      if (prec == P_C64) { TDKS_WS_MODES(2, P_C64) }
+    TDKS_WS_MODES(2, P_C128)
   }
   if (M == 4) {
-    if (prec == P_C64) { TDKS_WS_MODES(4, P_C64) } else { TDKS_WS_MODES(4, P_C128) }
+    if constexpr (SHAPE != 1)
+      if (prec == P_C64) { TDKS_WS_MODES(4, P_C64) }
+    TDKS_WS_MODES(4, P_C128)
   }
 #undef TDKS_WS_MODES
   return cudaErrorInvalidValue;
