@@ -338,17 +338,19 @@ int ws_shape_planes(int shape, int M, int bloch) {
 }
 
 int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last) {
-  // The tile of 16 x 12 points: with four service warps the complex64 kernels of shape 1 have 168
-  // registers and spill (order 8: 0.56 ms where shape 2 takes 0.27), as do shape 2's records in periodic
-  // cells (0.55 ms against 0.22 with shape 6).
-  if (prec == P_C64 && (shape == 1 || (bloch && (shape == 2 || shape == 5))))
-    return last || (bloch && M != 2) ? 2 : 6;
-  if (shape < 5) return shape;
-  if (prec != P_C64) return shape == 6 && !last && !(bloch && M != 2) ? 6 : 2;
-  if (shape == 5) return bloch ? 2 : 5;
-  if (bloch && (M != 2 || (shape != 6 && (nx % 2 != 0 || ny % 2 != 0)))) return 2;  // blocks must not straddle a face
-  if (last) return 2;                                                // their operands would not fit
-  return shape;
+  if (prec != P_C64) {
+    if (shape < 5) return shape;
+    return shape == 6 && !last && !(bloch && M != 2) ? 6 : 2;
+  }
+  // In cells of order 8 the tile of 16 x 12 points spills beside four service warps (64^3, 8 k-points: 0.92,
+  // 0.57, 0.95 ms in the first, middle and last term; shape 0 0.69, 0.36, 0.74, shape 3 0.69 in the last).
+  if (bloch && M != 2) return shape == 0 || shape == 3 || shape == 4 ? shape : (last ? 3 : 0);
+  // So does shape 1 (168 registers; order 8 in a box 0.56 ms where shape 2 takes 0.27), and shape 2's records
+  // in cells (0.55 ms, shape 6 0.22).
+  if (shape == 1 || (bloch && (shape == 2 || shape == 5))) return last ? 2 : 6;
+  if (shape <= 5) return shape;
+  if (last) return 2;                                                        // their operands would not fit
+  return bloch && shape != 6 && (nx % 2 != 0 || ny % 2 != 0) ? 6 : shape;  // blocks must not straddle a face
 }
 
 cudaError_t launch_sweep_tma(int M, int prec, int mode, int tx, int ty, const SweepMaps &maps, const SweepParams &p,

@@ -648,7 +648,10 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
   }
   __syncthreads();  // the only CTA-wide barrier: from here on the warps run decoupled
 
-  typedef WsWarps<TX, TY, R, OV, RX, U == 2> WW;
+  // (Records, and the last term's operands, beside the queues and face phases of order 8 in a cell spill at
+  // eight warps' 168 registers: 64^3, 8 k-points, 16 orbitals 0.80 -> 0.69 and 0.81 -> 0.74 ms.  The middle
+  // terms lose by the split, 0.364 -> 0.373.)
+  typedef WsWarps<TX, TY, R, OV, RX, U == 2 || (BLOCH && M == 4 && CW == 8 && MODE != MODE_MID)> WW;
   if (warp >= CW) {
   if constexpr (WW::SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(WW::PRODUCER_REGS));
   // ---- producers: one warp per ring (warp CW the centre planes, CW + 1 the halo planes, CW + 2 the
@@ -1118,13 +1121,12 @@ static cudaError_t launch_ws_batch_t(const BatchSweepArgs &a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Shapes 5 to 7 are complex64 kernels; what runs where is decided by ws_kernel_shape, which the
-// launchers below rely on: shape 5 finite boxes, 6 (order 4 or 8) and 7 (order 4) also periodic
-// cells of order 4.  Shapes 5 and 6 compute one complex value per thread vector, shape 7 two.
+// Shapes 5 to 8 exist for some systems; what runs where is decided by ws_kernel_shape, which the
+// launchers below rely on: shape 5 complex64 boxes, 6 to 8 terms 1 to 3 of complex64 boxes and order-4
+// cells, 6 also of complex128.  Shapes 5 and 8 compute one complex64 value per thread vector, 6 and 7 two.
 template <int SHAPE> struct C64Shape {
   static constexpr bool ONLY = SHAPE >= 5;
   static constexpr int P = SHAPE == 7 || SHAPE == 6 ? P_C64 : P_C64S;
-  static constexpr bool M4 = true;             // has order-8 kernels
   static constexpr bool CELL = SHAPE >= 6;     // has periodic-cell kernels (order 4)
   static constexpr bool LAST = SHAPE == 5;     // has last-term kernels
 };
@@ -1149,28 +1151,22 @@ cudaError_t launch_ws_batch_shape(int M, int prec, int mode, const BatchSweepArg
     if (prec != P_C64) return cudaErrorInvalidValue;
     if constexpr (C64Shape<SHAPE>::LAST) {
       if (M == 2 && mode == MODE_LAST) return launch_ws_batch_t<SHAPE, 2, P, MODE_LAST>(a, s);
-      if constexpr (C64Shape<SHAPE>::M4)
-        if (M == 4 && mode == MODE_LAST) return launch_ws_batch_t<SHAPE, 4, P, MODE_LAST>(a, s);
+      if (M == 4 && mode == MODE_LAST) return launch_ws_batch_t<SHAPE, 4, P, MODE_LAST>(a, s);
     }
     if (M == 2 && mode == MODE_FIRST) return launch_ws_batch_t<SHAPE, 2, P, MODE_FIRST>(a, s);
     if (M == 2 && mode == MODE_MID) return launch_ws_batch_t<SHAPE, 2, P, MODE_MID>(a, s);
-    if constexpr (C64Shape<SHAPE>::M4) {
-      if (M == 4 && mode == MODE_FIRST) return launch_ws_batch_t<SHAPE, 4, P, MODE_FIRST>(a, s);
-      if (M == 4 && mode == MODE_MID) return launch_ws_batch_t<SHAPE, 4, P, MODE_MID>(a, s);
-    }
+    if (M == 4 && mode == MODE_FIRST) return launch_ws_batch_t<SHAPE, 4, P, MODE_FIRST>(a, s);
+    if (M == 4 && mode == MODE_MID) return launch_ws_batch_t<SHAPE, 4, P, MODE_MID>(a, s);
   } else {
-    if constexpr (SHAPE == 1)
-      if (prec == P_C64) return cudaErrorInvalidValue;  // (complex128 only)
-    if (M == 2) {
-      if constexpr (SHAPE != 1)
-        if (prec == P_C64) { TDKS_WSB_MODES(2, P_C64) }
-      TDKS_WSB_MODES(2, P_C128)
+    if (prec == P_C64) {
+      if constexpr (SHAPE != 1) {
+        if (M == 2) { TDKS_WSB_MODES(2, P_C64) }
+        if (M == 4) { TDKS_WSB_MODES(4, P_C64) }
+      }
+      return cudaErrorInvalidValue;
     }
-    if (M == 4) {
-      if constexpr (SHAPE != 1)
-        if (prec == P_C64) { TDKS_WSB_MODES(4, P_C64) }
-      TDKS_WSB_MODES(4, P_C128)
-    }
+    if (M == 2) { TDKS_WSB_MODES(2, P_C128) }
+    if (M == 4) { TDKS_WSB_MODES(4, P_C128) }
   }
 #undef TDKS_WSB_MODES
   return cudaErrorInvalidValue;
@@ -1187,18 +1183,18 @@ static cudaError_t launch_ws_bc(int M, int prec, int mode, const SweepMaps &maps
     case MODE_LAST: return launch_ws_t<SHAPE, MM, PP, MODE_LAST, BLOCH>(maps, p, grid, s);   \
   }                                                                                          \
   return cudaErrorInvalidValue;
-  if constexpr (SHAPE == 1)
-    if (prec == P_C64) return cudaErrorInvalidValue;  // (complex128 only)
-  if (M == 2) {
-    if constexpr (SHAPE != 1)
-      if (prec == P_C64) { TDKS_WS_MODES(2, P_C64) }
-    TDKS_WS_MODES(2, P_C128)
+  // (complex64: shape 1 not at all, shape 2 in cells the last term of order 4 only)
+  if (prec == P_C64) {
+    if constexpr (SHAPE == 2 && BLOCH) {
+      if (M == 2 && mode == MODE_LAST) return launch_ws_t<SHAPE, 2, P_C64, MODE_LAST, BLOCH>(maps, p, grid, s);
+    } else if constexpr (SHAPE != 1) {
+      if (M == 2) { TDKS_WS_MODES(2, P_C64) }
+      if (M == 4) { TDKS_WS_MODES(4, P_C64) }
+    }
+    return cudaErrorInvalidValue;
   }
-  if (M == 4) {
-    if constexpr (SHAPE != 1)
-      if (prec == P_C64) { TDKS_WS_MODES(4, P_C64) }
-    TDKS_WS_MODES(4, P_C128)
-  }
+  if (M == 2) { TDKS_WS_MODES(2, P_C128) }
+  if (M == 4) { TDKS_WS_MODES(4, P_C128) }
 #undef TDKS_WS_MODES
   return cudaErrorInvalidValue;
 }
@@ -1239,9 +1235,7 @@ cudaError_t launch_ws_shape(int M, int prec, int mode, int bloch, const SweepMap
     }
     if (bloch) return cudaErrorInvalidValue;
     if (M == 2) { TDKS_WS5_MODES(2, 0) }
-    if constexpr (C64Shape<SHAPE>::M4) {
-      if (M == 4) { TDKS_WS5_MODES(4, 0) }
-    }
+    if (M == 4) { TDKS_WS5_MODES(4, 0) }
 #undef TDKS_WS5_MODES
     return cudaErrorInvalidValue;
   } else {

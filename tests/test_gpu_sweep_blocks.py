@@ -1,5 +1,5 @@
-"""Sweep shapes whose threads own 2 x 2 blocks of points (6: one complex64 value per thread
-vector; 7: two, order 4), against the FP64 oracle where blocks, tiles and periodic images can
+"""Sweep shapes that take two planes at a time or blocks of 2 x 2 points, and every shape in cells of order
+8 (where some run another's kernel), against the FP64 oracle where blocks, tiles and periodic images can
 go wrong: odd edges (blocks half outside a box), edges below and just past a tile, cells smaller
 than the tile, odd cells (which run another shape), spheres across the faces, the velocity gauge
 with all three components and the current's gradients.
@@ -57,4 +57,12 @@ def test_blocks_in_a_box(shape, order, grid):
 def test_blocks_in_a_cell(shape, grid):
     nx, ny, nz = grid
     spec = bloch_cell(I.PREC_C64, n_orb=2 if nx == 2 else 5, n_k=2, nx=nx, ny=ny, nz=nz)
+    _check(spec, bloch_inputs(spec), shape)
+
+
+@pytest.mark.parametrize("shape", range(9))
+@pytest.mark.parametrize("order,grid", [(4, (18, 14, 9)), (8, (18, 14, 9)), (8, (17, 25, 10))])
+def test_every_shape_in_a_cell(shape, order, grid):
+    nx, ny, nz = grid
+    spec = bloch_cell(I.PREC_C64, n_orb=5, n_k=2, nx=nx, ny=ny, nz=nz, fd_order=order)
     _check(spec, bloch_inputs(spec), shape)
