@@ -184,51 +184,9 @@ __device__ __forceinline__ void gather_finish(const GatherParams &p, int a, int 
 //   nl(r) = sum over the point's entries (a, j) of beta_aj(r) e^{-i phi} q_aj,
 //   phi = k . T + A . d (Bloch cells / velocity gauge), q_aj = D_aj h^3 <beta_aj|in>,
 // summed in entry order from zero and stored at row r0 (the point's first entry) of
-// nl[kb]; the sweeps add it to H in at the point.  Thread = (sphere point, v).
-template <int P, int BLOCH>
-__device__ __forceinline__ void nl_body(const GatherParams &p, long t, int kb) {
-  typedef VT<P> T;
-  typedef typename T::V V;
-  const long sidx = t / OVC;
-  const int v = (int)(t % OVC);
-  if (sidx >= p.n_sp) return;
-  const int2 r = p.sp[sidx];
-  const int kidx = kb / p.n_batches;
-  const bool phase = BLOCH || (p.A[0] != 0.0 || p.A[1] != 0.0 || p.A[2] != 0.0);
-  V acc = T::zero();
-  for (int e = r.x; e < r.y; e++) {
-    const int ei = p.rowent[e];
-    V x;
-    if constexpr (P == P_C64) {
-      const int2 ca = p.ent_ca[ei];
-      const float4 b4 = p.ent_beta[ei];
-      const V *qa = reinterpret_cast<const V *>(p.q) + ((long)(kb * p.n_atoms + ca.y) * 4) * OVC + v;
-      x = T::mul(T::coef(0.0, b4.x), T::ld(qa));
-      x = T::fma(T::coef(0.0, b4.y), T::ld(qa + OVC), x);
-      x = T::fma(T::coef(0.0, b4.z), T::ld(qa + 2 * OVC), x);
-      x = T::fma(T::coef(0.0, b4.w), T::ld(qa + 3 * OVC), x);
-      if (phase) {
-        const float2 ph = reinterpret_cast<const float2 *>(p.phase)[(long)kidx * p.n_ent + ei];
-        x = T::cmul(pk2(ph.x, ph.x), pk2(-ph.y, -ph.y), x);
-      }
-    } else {
-      const ProjEntry &E = p.ent[ei];
-      const V *qa = reinterpret_cast<const V *>(p.q) + ((long)(kb * p.n_atoms + E.atom) * 4) * OVC + v;
-      x = T::mul(E.betad[0], T::ld(qa));
-#pragma unroll
-      for (int j = 1; j < 4; j++) x = T::fma(E.betad[j], T::ld(qa + j * OVC), x);
-      if (phase) {
-        const double2 ph = reinterpret_cast<const double2 *>(p.phase)[(long)kidx * p.n_ent + ei];
-        x = T::cmul(ph.x, -ph.y, x);
-      }
-    }
-    acc = T::add(acc, x);
-  }
-  reinterpret_cast<V *>(p.nl)[((long)kb * (p.n_ent + 1) + r.x) * OVC + v] = acc;
-}
-
-// The same at RUN k-batches kb0 .. at once (a single system's kernel): the point's entries, their
-// strengths and phases are read once for all of them, and the loads of RUN k-batches are in flight together.
+// nl[kb]; the sweeps add it to H in at the point.  Thread = (sphere point, v) at RUN k-batches kb0 .. at
+// once: the point's entries, their strengths and phases are read once for all of them, and the loads of RUN
+// k-batches are in flight together.
 template <int P, int BLOCH, int RUN>
 __device__ __forceinline__ void nl_run(const GatherParams &p, long t, int kb0) {
   typedef VT<P> T;
@@ -318,20 +276,17 @@ gather_finish_batch_kernel(const GatherParams *gp, const long *ubegin, const int
   gather_finish<P>(p, (int)(local % p.n_atoms), (int)(local / p.n_atoms), threadIdx.x % 16);
 }
 
-// CTA c of the batched non-local kernel: system s with nbegin[s] <= c < nbegin[s+1]; within
-// it, kb = local / chunks, chunk = local % chunks.
+// CTA c of the batched non-local kernel: system s with nbegin[s] <= c < nbegin[s+1], sphere points from
+// (c - nbegin[s]) NL_BATCH_RUNS NL_THREADS / OVC on, all k-batches.  (A copy of the parameters: read through
+// the pointer they are loaded again after every store.)
 template <int P>
 __global__ void __launch_bounds__(NL_THREADS)
 nl_batch_kernel(const GatherParams *gp, const long *nbegin, const int *sys_of) {
   const int s = sys_of[blockIdx.x];
-  const GatherParams &p = gp[s];
-  const long local = blockIdx.x - nbegin[s];
-  constexpr long RUN = (long)NL_THREADS * NL_BATCH_RUNS;
-  const long chunks = ((long)p.n_sp * OVC + RUN - 1) / RUN;
-  const int kb = (int)(local / chunks);
-  const long t0 = (local % chunks) * RUN + threadIdx.x;
-#pragma unroll 2
-  for (int i = 0; i < NL_BATCH_RUNS; i++) nl_body<P, 0>(p, t0 + (long)i * NL_THREADS, kb);
+  const GatherParams p = gp[s];
+  const long t0 = (blockIdx.x - nbegin[s]) * NL_THREADS * NL_BATCH_RUNS + threadIdx.x;
+  for (int kb = 0; kb < p.n_kb; kb += 4)
+    for (int i = 0; i < NL_BATCH_RUNS; i++) nl_run<P, 0, 4>(p, t0 + (long)i * NL_THREADS, kb);
 }
 
 cudaError_t launch_gather_batch(int prec, const GatherParams *gp, const long *begin, const long *ubegin,
@@ -658,21 +613,44 @@ __device__ __forceinline__ void lda_body(long N, int nx, int ny, int nz, double 
                cz = bloch ? 0.0 : 0.5 * (nz - 1);
   const float hf = (float)h, cxf = (float)cx, cyf = (float)cy, czf = (float)cz;
   const float Exf = (float)Ex, Eyf = (float)Ey, Ezf = (float)Ez, hA2f = (float)half_A2;
-  for (long p = blk * (long)blockDim.x + threadIdx.x; p < N; p += (long)nblk * blockDim.x) {
-    double n = 0.0;
-    float nh = 0.f, nl = 0.f;  // complex64: n = nh + nl
+  // (32-bit index arithmetic, as the grids here have far fewer than 2^32 points, and the coordinates step
+  // with the index: the divisions of a point cost more than its potential)
+  const long stride = (long)nblk * blockDim.x;
+  long p = blk * (long)blockDim.x + threadIdx.x;
+  const unsigned up = (unsigned)p, us = (unsigned)stride, unx = (unsigned)nx, uny = (unsigned)ny;
+  int ix = (int)(up % unx), iy = (int)((up / unx) % uny), iz = (int)(up / (unx * uny));
+  const int sx = (int)(us % unx), sy = (int)((us / unx) % uny), sz = (int)(us / (unx * uny));
+  // Two points at a time, a stride apart, their loads together: a point is a chain of dependent loads and
+  // of sums.  (The second one of the last pair reads the first again.)
+  for (; p < N; p += 2 * stride) {
+    const long pp[2] = {p, p + stride < N ? p + stride : p};
+    double n[2] = {0.0, 0.0}, vl[2], vhd[2];
+    float nh[2] = {0.f, 0.f}, nl[2] = {0.f, 0.f};  // complex64: n = nh + nl
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      vl[u] = vloc[pp[u]];
+      vhd[u] = vh ? vh[pp[u]] : 0.0;
+    }
     if (n_in) {
       // the density summed over every rank's states (state-parallel propagation)
-      n = n_in[p];
-      nh = (float)n;
-      nl = (float)(n - (double)nh);
+#pragma unroll
+      for (int u = 0; u < 2; u++) {
+        n[u] = n_in[pp[u]];
+        nh[u] = (float)n[u];
+        nl[u] = (float)(n[u] - (double)nh[u]);
+      }
     } else if constexpr (F32) {
       const float2 *d2 = reinterpret_cast<const float2 *>(dens_part);
       for (int k = 0; k < n_k; k++) {
-        float sh = 0.f, sl = 0.f;  // sum over the k-point's batches of sum |psi|^2
+        float sh[2] = {0.f, 0.f}, sl[2] = {0.f, 0.f};  // sum over the k-point's batches of sum |psi|^2
+#pragma unroll 4
         for (int b = 0; b < n_batches; b++) {
-          const float2 d = d2[(long)(k * n_batches + b) * N + p];
-          df_add_df(sh, sl, d.x, d.y);
+          const float2 *db = d2 + (long)(k * n_batches + b) * N;
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            const float2 d = db[pp[u]];
+            df_add_df(sh[u], sl[u], d.x, d.y);
+          }
         }
         float2 w;
         if (k < LDA_MAXK) {
@@ -681,50 +659,60 @@ __device__ __forceinline__ void lda_body(long N, int nx, int ny, int nz, double 
           const float hi = (float)wocc[k];
           w = make_float2(hi, (float)(wocc[k] - (double)hi));
         }
-        // (sh + sl)(w.x + w.y): the leading product exactly (FMA residual), the cross terms rounded
-        const float ph = sh * w.x;
-        const float pl = fmaf(sh, w.x, -ph) + (sh * w.y + sl * w.x);
-        df_add_df(nh, nl, ph, pl);
-      }
-    } else {
-      for (int kb = 0; kb < n_kb; kb++) n += dens_part[(long)kb * N + p];
-    }
-    // (32-bit index arithmetic: a 64-bit division per coordinate cost more than the point's
-    // arithmetic; the grids here have far fewer than 2^32 points)
-    const unsigned up = (unsigned)p, unx = (unsigned)nx, uny = (unsigned)ny;
-    const int ix = (int)(up % unx), iy = (int)((up / unx) % uny), iz = (int)(up / (unx * uny));
-    if constexpr (F32) {
-      const float nf = nh;
-      const float x = (ix - cxf) * hf, y = (iy - cyf) * hf, z = (iz - czf) * hf;
-      const float vx = xc ? -cbrtf(3.0f * nf * 0.318309886f) : 0.0f;
-      const float vhf = vh ? (float)vh[p] : 0.0f;
-      float v = (float)vloc[p] + vx + vhf + hA2f;
-      if (!bloch) v += Exf * x + Eyf * y + Ezf * z;
-      *reinterpret_cast<float *>(&aux[p].veff) = v + (float)w0;
-      if (sums) {
-        // (with the Hartree potential the record subtracts int n (v_x + v_H) and adds E_H =
-        // 1/2 int n v_H: the third sum is int n (v_x + v_H / 2))
-        const float t[6] = {nf, nf * 0.75f * vx, nf * (vx + 0.5f * vhf), x * nf, y * nf, z * nf};
 #pragma unroll
-        for (int c = 0; c < 6; c++) df_acc(fh[c], fl[c], t[c]);
-        fl[0] += nl;  // the electron count keeps the double-float density in full
+        for (int u = 0; u < 2; u++) {
+          // (sh + sl)(w.x + w.y): the leading product exactly (FMA residual), the cross terms rounded
+          const float ph = sh[u] * w.x;
+          const float pl = fmaf(sh[u], w.x, -ph) + (sh[u] * w.y + sl[u] * w.x);
+          df_add_df(nh[u], nl[u], ph, pl);
+        }
       }
     } else {
-      const double x = (ix - cx) * h, y = (iy - cy) * h, z = (iz - cz) * h;
-      double vx = 0.0;
-      if (xc) vx = -cbrt(3.0 * n * 0.31830988618379067154);  // 1/pi
-      const double vhd = vh ? vh[p] : 0.0;
-      double v = vloc[p] + vx + vhd + half_A2;
-      if (!bloch) v += Ex * x + Ey * y + Ez * z;
-      *reinterpret_cast<double *>(&aux[p].veff) = v + w0;
-      if (sums) {
-        acc[0] += n;
-        acc[1] += n * 0.75 * vx;
-        acc[2] += n * (vx + 0.5 * vhd);
-        acc[3] += x * n;
-        acc[4] += y * n;
-        acc[5] += z * n;
+#pragma unroll 4
+      for (int kb = 0; kb < n_kb; kb++)
+#pragma unroll
+        for (int u = 0; u < 2; u++) n[u] += dens_part[(long)kb * N + pp[u]];
+    }
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const bool live = u == 0 || p + stride < N;
+      if constexpr (F32) {
+        const float nf = nh[u];
+        const float x = (ix - cxf) * hf, y = (iy - cyf) * hf, z = (iz - czf) * hf;
+        const float vx = xc ? -cbrtf(3.0f * nf * 0.318309886f) : 0.0f;
+        const float vhf = (float)vhd[u];
+        float v = (float)vl[u] + vx + vhf + hA2f;
+        if (!bloch) v += Exf * x + Eyf * y + Ezf * z;
+        if (live) *reinterpret_cast<float *>(&aux[pp[u]].veff) = v + (float)w0;
+        if (sums && live) {
+          // (with the Hartree potential the record subtracts int n (v_x + v_H) and adds E_H =
+          // 1/2 int n v_H: the third sum is int n (v_x + v_H / 2))
+          const float t[6] = {nf, nf * 0.75f * vx, nf * (vx + 0.5f * vhf), x * nf, y * nf, z * nf};
+#pragma unroll
+          for (int c = 0; c < 6; c++) df_acc(fh[c], fl[c], t[c]);
+          fl[0] += nl[u];  // the electron count keeps the double-float density in full
+        }
+      } else if (live) {
+        const double x = (ix - cx) * h, y = (iy - cy) * h, z = (iz - cz) * h;
+        double vx = 0.0;
+        if (xc) vx = -cbrt(3.0 * n[u] * 0.31830988618379067154);  // 1/pi
+        double v = vl[u] + vx + vhd[u] + half_A2;
+        if (!bloch) v += Ex * x + Ey * y + Ez * z;
+        *reinterpret_cast<double *>(&aux[pp[u]].veff) = v + w0;
+        if (sums) {
+          acc[0] += n[u];
+          acc[1] += n[u] * 0.75 * vx;
+          acc[2] += n[u] * (vx + 0.5 * vhd[u]);
+          acc[3] += x * n[u];
+          acc[4] += y * n[u];
+          acc[5] += z * n[u];
+        }
       }
+      ix += sx;
+      iy += sy;
+      iz += sz;
+      if (ix >= nx) { ix -= nx; iy++; }
+      if (iy >= ny) { iy -= ny; iz++; }
     }
   }
   if (!sums) return;  // (uniform over the grid: V_eff only, no record follows)
@@ -755,7 +743,7 @@ __device__ __forceinline__ void lda_body(long N, int nx, int ny, int nz, double 
 }
 
 template <typename R>
-__global__ void __launch_bounds__(LDA_THREADS)
+__global__ void __launch_bounds__(LDA_THREADS, 4)
 lda_kernel(long N, int nx, int ny, int nz, double h, int bloch, int n_kb, int n_batches, const double *wocc,
            const double *dens_part, const double *vloc, int xc, double Ex, double Ey, double Ez, double half_A2,
            double w0, PointAux *aux, double *lda_part, const double *n_in, const double *vh, int sums) {
@@ -939,7 +927,7 @@ __device__ __forceinline__ double batch_field(const BatchAux &a, double t) {
 // Batched LDA: the systems' CTA ranges are concatenated; the field is evaluated at each
 // system's current sub-step midpoint from its device clock.
 template <typename R>
-__global__ void __launch_bounds__(LDA_THREADS)
+__global__ void __launch_bounds__(LDA_THREADS, 4)
 lda_batch_kernel(const BatchAux *aux, const BatchClock *clk, const long *begin, int n_sys) {
   __shared__ double f;
   // the CTA's system: a binary search over the systems' CTA ranges (a table lookup, as the

@@ -60,11 +60,13 @@ void batch_free(tdks_batch *b) {
   if (b->work) cudaStreamDestroy(b->work);
 }
 
-// CTAs of one system in the batched LDA launch: a sixteenth of the single-system count (whose
-// partial buffer it fills), i.e. ~16 points per thread, so that the launch over all systems pays
-// each CTA's setup (system lookup, field, weight staging) a few times per SM rather than once per
-// CTA-sized run of points.
-static int lda_batch_blocks(long N) { return (int)std::max(1L, (std::min((N + 255) / 256, 608L) + 15) / 16); }
+// CTAs of one system in the batched LDA launch: its share of the 4 per SM that are resident at once, at
+// most the single-system count (whose partial buffer it fills).  A CTA's setup (system lookup, field, weight
+// staging) is paid once, and no second round of CTAs runs on a part of the SMs.
+static long lda_work(const tdks_system *s) { return s->N * (4 + s->n_kb); }
+static int lda_batch_blocks(const tdks_system *s, long total) {
+  return (int)std::max(1L, std::min((long)lda_blocks(s->N), 152L * 4 * lda_work(s) / total));
+}
 
 // Kernels one sub-step launches: the LDA/V_eff kernel, per Taylor term the projector step
 // (gather stages 1 and 2 and the non-local term, where any system has atoms) and the sweep,
@@ -242,6 +244,8 @@ int tdks_batch_create(const tdks_sys *systems, int n, void *stream, tdks_batch_t
   // partial-sum buffer holds
   long batch_units = 0;
   for (tdks_system *s : b->sys) batch_units += (long)s->n_atoms * s->n_kb;
+  long all_lda = 0;
+  for (tdks_system *s : b->sys) all_lda += lda_work(s);
   const int bchunks = gather_chunks(std::max(batch_units, 1L), false);
   for (int i = 0; i < n; i++) {
     tdks_system *s = b->sys[i];
@@ -259,8 +263,8 @@ int tdks_batch_create(const tdks_sys *systems, int n, void *stream, tdks_batch_t
     }
     gather_begin[i + 1] = gather_begin[i] + (long)s->n_atoms * s->n_kb * (s->n_atoms > 0 ? nch : 0);
     unit_begin[i + 1] = unit_begin[i] + (long)s->n_atoms * s->n_kb;
-    nl_begin[i + 1] = nl_begin[i] + (s->n_atoms > 0 ? nl_batch_blocks(s->n_sp, s->n_kb) : 0);
-    const int nl = lda_batch_blocks(s->N);
+    nl_begin[i + 1] = nl_begin[i] + (s->n_atoms > 0 ? nl_batch_blocks(s->n_sp) : 0);
+    const int nl = lda_batch_blocks(s, all_lda);
     lda_begin[i + 1] = lda_begin[i] + nl;
     BatchAux &a = aux[i];
     a.N = s->N; a.nx = s->nx; a.ny = s->ny; a.nz = s->nz; a.n_kb = s->n_kb; a.xc = s->xc;

@@ -334,18 +334,17 @@ int lda_blocks(long N);
 cudaError_t launch_sweep_tma_batch(int M, int prec, int mode, const BatchSweepArgs &a, cudaStream_t s,
                                    int shape = 0);
 // begin: prefix sums of n_atoms * n_kb * n_chunks (stage 1 CTAs); ubegin: of n_atoms * n_kb;
-// nbegin: of the non-local kernel's CTAs, n_kb * ceil(n_sp * OVC / NL_THREADS).  gsys, usys,
+// nbegin: of the non-local kernel's CTAs (nl_batch_blocks).  gsys, usys,
 // nsys: the system of each stage-1 CTA, unit and non-local CTA (one table load instead of a
 // binary search over the prefix sums in every CTA).
 cudaError_t launch_gather_batch(int prec, const GatherParams *gp, const long *begin, const long *ubegin,
                                 const long *nbegin, const int *gsys, const int *usys, const int *nsys,
                                 long total, long total_units, long total_nl, cudaStream_t s);
-// CTAs of the non-local kernel of one system; in a batch each CTA covers NL_BATCH_RUNS runs of
-// NL_THREADS (sphere point, vector) pairs, so that its setup is paid once per several runs
-inline long nl_blocks(int n_sp, int n_kb) { return (long)n_kb * (((long)n_sp * OVC + NL_THREADS - 1) / NL_THREADS); }
-constexpr int NL_BATCH_RUNS = 8;
-inline long nl_batch_blocks(int n_sp, int n_kb) {
-  return (long)n_kb * (((long)n_sp * OVC + NL_THREADS * NL_BATCH_RUNS - 1) / (NL_THREADS * NL_BATCH_RUNS));
+// CTAs of one system in a batch's non-local kernel: each covers NL_BATCH_RUNS runs of NL_THREADS (sphere
+// point, vector) pairs, so that its setup is paid once per several runs
+constexpr int NL_BATCH_RUNS = 2;
+inline long nl_batch_blocks(int n_sp) {
+  return ((long)n_sp * OVC + NL_THREADS * NL_BATCH_RUNS - 1) / (NL_THREADS * NL_BATCH_RUNS);
 }
 cudaError_t launch_lda_batch(int prec, const BatchAux *aux, const BatchClock *clk, const long *begin, int n_sys,
                              long total, cudaStream_t s);
