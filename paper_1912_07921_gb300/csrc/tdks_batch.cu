@@ -217,7 +217,8 @@ int tdks_batch_create(const tdks_sys *systems, int n, void *stream, tdks_batch_t
   b->substeps = s0->clock_substeps;
   long points = 0;  // (every system's points and orbital batches share a launch)
   for (tdks_system *s : b->sys) points += s ? (long)s->n_kb * s->N : 0;
-  for (int k = 0; k < 4; k++) b->shape[k] = ws_default_shape(b->prec, 0, points, k == 3);
+  // (48 x 48: the systems differ in size, so no tile fits better)
+  for (int k = 0; k < 4; k++) b->shape[k] = ws_default_shape(b->prec, 0, 48, 48, points, k == 3);
   auto bad = [&](const char *m) { delete b; return fail(TDKS_EINVAL, m); };
   for (tdks_system *s : b->sys) {
     if (!s) return bad("NULL system in batch");

@@ -567,7 +567,7 @@ int tdks_create_grid(int nx, int ny, int nz, double h, int fd_order, int bc, int
   if (kweights) for (int i = 0; i < n_k; i++) s->kw[i] = kweights[i];
   cudaGetDevice(&s->dev);
   const size_t pts = (size_t)s->n_kb * N;
-  for (int i = 0; i < 4; i++) s->wshape[i] = ws_default_shape(prec, bc == TDKS_BC_BLOCH, (long)pts, i == 3);
+  for (int i = 0; i < 4; i++) s->wshape[i] = ws_default_shape(prec, bc == TDKS_BC_BLOCH, nx, ny, (long)pts, i == 3);
   s->term_bytes = pts * OVC * 16;
   s->state_bytes = s->term_bytes;
   const int nlda = lda_blocks(N);

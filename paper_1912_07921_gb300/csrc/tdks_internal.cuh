@@ -320,9 +320,14 @@ int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool 
 // work for its larger tile (medium molecule 0.316 -> 0.250 ms, 48^3 with 16 orbitals 18.4 -> 17.2 us; at
 // 24^3 shape 0 is still ahead, 9.6 against 10.4 us, and in cells up to 32^3); last term: shape 3 while the
 // sweep is short (64^3, 24 orbitals 96 -> 82 us), shape 2 for long ones (medium molecule 0.54 -> 0.48 ms).
-// complex128 is bound by the FP64 pipe in every shape and stays with shape 0's smaller tile.
-inline int ws_default_shape(int prec, int bloch, long points, bool last) {
-  if (prec != P_C64) return 0;
+// complex128 is bound by the FP64 pipe in every shape (96^3, 16 orbitals 1.513 ms with shape 0, 1.531 with 2) and
+// takes the tile that leaves fewer of its points outside the grid (cell of 30 x 36 x 32, 3 k-points, 10 orbitals:
+// 16 x 12 has 6% and 16 x 8 18% outside, 0.175 against 0.193 ms); short sweeps keep the smaller one.
+inline int ws_default_shape(int prec, int bloch, int nx, int ny, long points, bool last) {
+  if (prec != P_C64) {
+    const long wx = (nx + 15) / 16 * 16L, a0 = wx * ((ny + 7) / 8 * 8), a2 = wx * ((ny + 11) / 12 * 12);
+    return points >= 60000 && 51 * a2 < 50 * a0 ? 2 : 0;
+  }
   if (last) return points < 1500000 ? 3 : 2;
   return points >= (bloch ? 60000 : 30000) ? 6 : 0;
 }
