@@ -40,8 +40,8 @@ METRIC = "H.psi orbital-gridpoint updates/s (medium molecule, Taylor-4 step)"
 UNIT = "updates/s"
 
 
-SWEEP_SOURCES = ["tdks_sweep_tma.cu", "tdks_tma.cuh", "tdks_sweep_ws1.cu", "tdks_sweep_ws2.cu", "tdks_sweep_ws3.cu", "tdks_sweep_ws5.cu",
-                 "tdks_sweep_ws4.cu", "tdks_sweep_common.cuh", "tdks_vec.cuh", "tdks_internal.cuh"]
+SWEEP_SOURCES = ["tdks_sweep_tma.cu", "tdks_tma.cuh", "tdks_sweep_ws1.cu", "tdks_sweep_ws2.cu", "tdks_sweep_ws3.cu", "tdks_sweep_ws4.cu",
+                 "tdks_sweep_ws5.cu", "tdks_sweep_ws6.cu", "tdks_sweep_ws7.cu", "tdks_sweep_ws8.cu", "tdks_sweep_common.cuh", "tdks_vec.cuh", "tdks_internal.cuh"]
 WORKLOAD = ("medium molecule 96^3 h=0.25 order-8 FD, 64 orbitals, 16 atoms x 4 KB projectors, sin^2 pulse, "
             "LDA exchange, dt=0.05 as 4 Taylor-4 sub-steps")
 NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e data-sheet bandwidth, for context beside the measured peak

@@ -334,15 +334,15 @@ int tdks_set_tile(tdks_sys sys, int tx, int ty, int zc);
 int tdks_set_failure_injection(tdks_sys sys, int withhold);
 
 /* Stencil sweep implementation: 0 (default) streams the input planes with TMA bulk
- * tensor copies where that applies (finite boxes, 16x8 tiles) into a warp-specialised
- * kernel (one producer warp, eight consumer warps); 1 always uses the general sweep (loads
- * through L1/L2; the only one for periodic cells); 2 is the TMA sweep in which all warps of
+ * tensor copies where that applies (16x8 system tiles) into a warp-specialised
+ * kernel (four service warps, 6 to 16 consumer warps); 1 always uses the general sweep (loads
+ * through L1/L2); 2 is the TMA sweep (finite boxes) in which all warps of
  * a CTA advance plane by plane together.  All compute the same values (to the last bits of
  * FP64 rounding in the energy and current sums). */
 int tdks_set_sweep_path(tdks_sys sys, int path);
 
 /*
- * Tile shapes of the warp-specialised TMA sweep (path 0, finite boxes, 16x8 system tile)
+ * Tile shapes of the warp-specialised TMA sweep (path 0, 16x8 system tile)
  * and the autotuner that picks one per Taylor-term sweep.  No passage of the paper
  * defines these: they choose how the stencil (Sec. "Maxwell ... coupling", finite
  * differences on a uniform grid) is tiled on the GPU and do not change its values (each
@@ -350,14 +350,18 @@ int tdks_set_sweep_path(tdks_sys sys, int path);
  * partial sums are grouped per consumer warp, so those change in the last bits).
  *
  * tdks_sweep_shape_info: shape s (0 .. count-1) covers tx x ty points of one orbital batch
- * per work item with `warps` consumer warps, each thread computing `rows` y-adjacent
- * points of one 16-byte vector (two complex64 or one complex128 values; 4 vectors per point,
- * so warps x 32 = 4 tx ty / rows).  Shape 5 computes complex64 finite boxes with one
- * complex64 value (8 bytes) per thread vector, 8 vectors per point (warps x 32 = 8 tx ty /
- * rows): fewer shared-memory bytes per value at the same register budget; complex128
- * systems and periodic cells run it as shape 2 (the same tile and warp count).  *count (if
- * not NULL) receives the number of shapes; tx/ty/rows/warps may be NULL.  TDKS_EINVAL for a
- * shape out of range.
+ * per work item with `warps` consumer warps, each thread computing `rows` points of one
+ * 16-byte vector (two complex64 or one complex128 values; 4 vectors per point, so
+ * warps x 32 = 4 tx ty / rows): y-adjacent ones in shapes 0 to 4 and 6, a block of 2 x 2 in
+ * shape 7.  Shapes 5 (columns) and 8 (blocks) take 8-byte vectors of one complex64 value, 8 per
+ * point (shape 5: warps x 32 = 8 tx ty / rows).  Shapes 6 to 8 take two planes at a time where
+ * the registers allow.  Every shape can be chosen for every system; one without a kernel for
+ * a system's precision, order, boundary or term runs the kernel of another (complex128: 5, 7, 8
+ * and 6 in the last term as 2; complex64: 1 as 6 or 2, 6 to 8 in the last term as 2, all but 0,
+ * 3 and 4 in cells of order 8 as 0 or 3).  Until one is set or tuned, complex64 takes 6 (0 on
+ * small grids) and 2 (3 on smaller grids) for the last term, complex128 0 or 2, whichever tile leaves
+ * fewer points outside the grid.  *count (if not NULL) receives the number of shapes;
+ * tx/ty/rows/warps may be NULL.  TDKS_EINVAL for a shape out of range.
  */
 int tdks_sweep_shape_info(int shape, int *count, int *tx, int *ty, int *rows, int *warps);
 /* Shape of Taylor-term sweep `sweep` (0 = t1 from psi, 1 = t2, 2 = t3, 3 = t4 and the
@@ -367,7 +371,8 @@ int tdks_get_sweep_shape(tdks_sys sys, int sweep, int *shape);
 /* Autotuner: times every shape on each of the four Taylor-term sweeps of this system, on
  * its own grid, orbitals and projectors (in the velocity gauge with a vector potential
  * amp * pol, so that the gauge term is timed too; reps launches each after one warm-up
- * launch, CUDA events on the system's stream), and keeps the fastest shape per sweep.  The state psi is
+ * launch, CUDA events on the system's stream; shapes that run one kernel are timed once), and
+ * keeps the fastest shape per sweep.  The state psi is
  * not changed; the Taylor-term buffers and the density partials are overwritten (the next
  * propagation or H application rebuilds them).  ms (if not NULL) receives the mean
  * milliseconds per launch as ms[shape * 4 + sweep] (count * 4 values).  Systems that do not

@@ -19,7 +19,7 @@ namespace tdks {
 // memory in a fixed order); their sums are added in chunk order and take D_aj h^3.  For one system
 // the chunks of a unit are a thread-block cluster whose first CTA reads the others' sums from their
 // shared memory; a second launch for that sum, a chain of 16 dependent loads, took longer than the
-// gather itself (64^3, 4 atoms, 2 k-batches: 8.2 + 10 us against 9.5).  Batches keep two launches (their
+// gather itself (64^3, 4 atoms, 2 k-batches: 8.2 + 10 us against 11.2).  Batches keep two launches (their
 // units differ in size).  No atomics: the result does not depend on timing.
 // ---------------------------------------------------------------------------------
 constexpr int GATHER_THREADS = 256;
@@ -574,7 +574,7 @@ constexpr int LDA_THREADS = 256;  // most threads of a CTA (and those of a batch
 
 // Threads per CTA of one system's launch: a small grid's points are spread over all SMs (a complex128
 // point's cube root is ~150 FP64 instructions at 2 per clock and SM: 24^3 points in 54 CTAs of 256
-// threads took 10.4 us, in 432 of 32 4.3 us).
+// threads took 10.4 us, in 432 of 32 7.5 us).
 static int lda_threads(long N) { return N <= 608 * 32 ? 32 : (N <= 608 * 64 ? 64 : (N <= 608 * 256 ? 128 : LDA_THREADS)); }
 int lda_blocks(long N) {
   const int t = lda_threads(N);
@@ -1043,7 +1043,7 @@ __device__ __forceinline__ void finalize_body(const double *obs_part, long n_ite
 // One system: a cluster of CTAs, CTA b of which sums the b-th contiguous share of the partials; the
 // first adds the CTAs' sums in order and writes the record (rec), or the 10 sums (sums).  The shares
 // depend only on the counts, so the record is the same on every run.  (Two launches with the sums
-// in between, 64 CTAs and one, took 7.4 + 4.0 us on the tiny molecule.)
+// in between, 64 CTAs and one, took 7.4 + 4.0 us on the tiny molecule, this one 8.7.)
 __global__ void __launch_bounds__(FIN_MAX_THREADS)
 finalize_kernel(const double *obs_part, long n_items, const double *lda_part, int n_lda, double *sums, double *rec,
                 double t_state, double h3, double occ, int bloch, double omega_cell, double Ax, double Ay, double Az,

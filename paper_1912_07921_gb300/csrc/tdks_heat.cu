@@ -50,7 +50,7 @@ __device__ __forceinline__ double2 value(const HeatParams &p, int kb, int j, lon
 
 // phi at grid offset s along axis a from (x, y, z): the periodic image with its Bloch phase
 // (the phase of one wrap comes from a table: a sine and cosine per wrapped neighbour cost more than
-// the rest of the point, 1.01 -> 0.35 ms for 30x36x32 points and 36 complex128 values each)
+// the rest of the point, 1.01 -> 0.41 ms for 30x36x32 points and 36 complex128 values each)
 __device__ __forceinline__ double2 neighbour(const HeatParams &p, int kb, int j, int x, int y, int z, int a, int s,
                                             const double2 *kph) {
   int c[3] = {x, y, z};

@@ -297,23 +297,22 @@ cudaError_t launch_pack_in(int prec, long N, int k, long pt0, long npts, int n_o
 cudaError_t launch_unpack(int prec, long N, long g0, long npts, int n_orb, int n_batches, const void *internal,
                           const void *internal_lo, double *plain, cudaStream_t s);
 
-// TMA sweep for finite boxes (tdks_sweep_tma.cu).  maps.in: dims {16 floats, nx, ny, nz,
-// n_kb}, box {16, TX+2M, TY+2M, tma_planes(prec, mode), 1} (TY: the shape's tile height); maps.aux: dims {4, nx, ny, nz}
-// (4-byte words), box {4, TX, TY, tma_planes}; maps.op[i]: dims as maps.in, box
-// {16, TX, TY, 1, 1}; maps.ctr: as maps.op with tma_planes planes.  Default: the
-// warp-specialised kernel (a producer warp and eight consumer warps); lockstep: the variant
-// in which all warps of a CTA advance plane by plane together.
+// TMA sweep (tdks_sweep_tma.cu).  maps.in: 8-byte words, dims {8 nx, ny, nz, n_kb}, box {8 (TX + 2M), TY + 2M,
+// tma_planes(prec, mode), 1} (TX, TY: the shape's tile); maps.aux: dims {2 nx, ny, nz}, box {2 TX, TY,
+// tma_planes}; maps.op[i]: dims as maps.in, box {8 TX, TY, 1, 1}; maps.ctr: as maps.op with tma_planes planes.
+// (A tile row is one run of the innermost dimension: with a dimension of its own per point the copies moved 64
+// bytes at a time, last term of the medium molecule 653 -> 620 us.)  Default: the warp-specialised kernel;
+// lockstep: the variant in which all warps of a CTA advance plane by plane together.
 cudaError_t launch_sweep_tma(int M, int prec, int mode, int tx, int ty, const SweepMaps &maps,
                              const SweepParams &p, int grid, cudaStream_t s, bool lockstep = false,
                              int shape = 0);
 // Tile shapes of the warp-specialised sweep: shape s covers tx x ty points of one orbital
-// block with `warps` consumer warps, each thread computing `rows` y-adjacent points.
-// Shape 0 (16 x 8, two points per thread, eight consumer warps) is the default and the one
-// the batched sweep uses.  Null outputs are skipped; false for a shape out of range.
+// block with `warps` consumer warps, each thread computing `rows` points of a 16-byte vector.
+// Null outputs are skipped; false for a shape out of range.
 constexpr int WS_SHAPES = 9;
 bool ws_shape_info(int shape, int *tx, int *ty, int *rows, int *warps);
-// The shape whose kernel a sweep of `shape` runs: shapes 5 to 8 exist for some systems only, the others
-// run one that does.  Tiles, tensor maps and record counts follow the result.
+// The shape whose kernel a sweep of `shape` runs: some shapes exist for some systems only, the others run one
+// that does.  Tiles, tensor maps and record counts follow the result.
 // last: the sweep of the last Taylor term.
 int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool last);
 // The shape a sweep takes until one is set or tuned.  complex64, terms 1 to 3: shape 6 once the grid has

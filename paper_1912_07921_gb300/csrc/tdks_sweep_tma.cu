@@ -1,8 +1,9 @@
-// TMA-fed Taylor-term sweep for finite boxes (zero boundary).
+// TMA-fed Taylor-term sweeps: the rules for the warp-specialised kernels (tdks_tma.cuh), and the variant for
+// finite boxes (zero boundary) in which a CTA's warps advance together.
 //
 // Same arithmetic as the general sweep (tdks_sweep.cu; see tdks_sweep_common.cuh), with
 // the stencil input streamed by the Tensor Memory Accelerator:
-//   * a 5D tensor map views the input as {16 floats, nx, ny, nz, k*batch}; one
+//   * a 4D tensor map views the input as {8-byte words of a row of points, ny, nz, k*batch}; one
 //     cp.async.bulk.tensor copy brings a whole (TX+2M) x (TY+2M) plane tile with its halo
 //     into shared memory, and out-of-box coordinates arrive as zeros, which is exactly
 //     the zero boundary condition of a finite box;

@@ -342,37 +342,33 @@ struct Loader {
 };
 
 // ---------------------------------------------------------------------------------------
-// Warp-specialised variant: one producer warp keeps the three rings full, CW consumer
-// warps compute.  A ring slot is handed back by an "empty" mbarrier that each consumer
-// warp arrives on once it has read the slot, so the consumer warps never wait for one
-// another inside a work item: while some warps read their shared-memory neighbours,
-// others do arithmetic or store.  Each consumer thread computes one 16-byte vector of R
-// y-adjacent points, which share the y-column values they read (R points need 2M+R column
-// loads instead of 2M R).
+// Warp-specialised variant: service warps keep the rings full, CW consumer warps compute.  Four of them, a
+// warpgroup: the centre ring (and the claims of work items), the halo ring, the last term's operand ring,
+// and in periodic cells the patcher of the images (a single producer for all rings was late: a wait on one
+// ring held the others up; middle term of the medium molecule 0.287 -> 0.275 ms, 24 boxes of order 4 0.424
+// -> 0.374).  A ring slot is handed back by an "empty" mbarrier that each consumer warp arrives on once it
+// has read the slot, so the consumer warps never wait for one another inside a work item: while some warps
+// read their shared-memory neighbours, others do arithmetic or store.
 //
-// Shapes (tile TX x TY points of one orbital block; R y-adjacent points per consumer
-// thread; CW = 4 TX TY / (32 R) consumer warps, plus the producer warp).  More points per
-// thread share more y-column loads and give each warp more independent arithmetic; more
-// warps hide more latency.  The register budget of a thread is set by the warps that share
-// one of the SM's four scheduler partitions (16K registers each): 7 or 8 warps in all leave
-// 255 registers per thread, 9 leave 168, 13 leave 128, 17 leave 96.  tdks_autotune times
-// the shapes on the system's own data.
-//
-// Shape 5 computes complex64 systems with one complex value per thread vector (8 bytes, 8
-// vectors per point, P_C64S): at the same register budget a thread then holds the z queues
-// of 4 y-adjacent points, which share their y-column loads, while a warp still spans 4
-// consecutive points in x (conflict-free 256-byte shared loads).  Per output value that is
-// 2M x-arm loads, 2M/4 y-arm loads and one queue load of 8 bytes, against 2M, (2M+2)/2 and
-// one of 16 bytes for two values in the two-complex shapes: about a third fewer shared-memory
-// bytes per value.  Complex128 systems and periodic cells run shape 5 as shape 2.
-//
-// Shapes 6 and 7 give a thread a block of 2 x 2 points (RX = 2 x-adjacent, R = 2 y-adjacent): the
-// block shares its x-arm loads too, 2M per row and 2M per column for four points, so a value costs
-// 2M + 1 shared loads where two y-adjacent points cost 3M + 2 and one point 4M + 1.  The block's
-// inner neighbours come from the z queues.  To keep the loads free of bank conflicts (a point is 64
-// bytes, half of the banks) the odd blocks of a row are mirrored: their first point is the right
-// one and their x offsets count downwards, so that two blocks side by side always read different
-// halves of the banks.  The x arm is symmetric, so mirrored values are the same bit for bit.
+// Shapes: a tile of TX x TY points of one orbital block; a thread owns a column of R y-adjacent points, or
+// (RX = 2) a block of 2 x 2, of one vector of 16 bytes (8 in shapes 5 and 8), at U planes an iteration.  The
+// points of a thread share the arm values they read.  Shared-memory reads, not HBM, bound the complex64
+// middle terms of order 8: a value costs 4M + 1 loads alone, (3M + 2) with two y-adjacent points, 2M + 1 in
+// a block, whose inner neighbours come from the z queues.  Threads have 65536 / (32 (CW + 4)) registers:
+// 168 with 6 to 8 consumer warps, 128 with 12, 96 with 16; the kernels whose queues need more split them
+// (WsWarps).  tdks_autotune times the shapes on the system's own data.
+//   5: 8-byte vectors (one complex64 value), four y-adjacent points in the registers of two.
+//   6: shape 2 at two planes an iteration: one wait and one release per ring and two planes, and two planes'
+//      loads to overlap.  Medium molecule, middle term: 0.275 -> 0.255 ms.
+//   7: blocks of 2 x 2 of 16-byte vectors on 232 registers.  The fastest in cells and boxes of order 4 (64^3
+//      cell, 8 k-points, 16 orbitals: 0.184 ms, shape 6 0.206, shape 3 0.230); at order 8 its 144 queue
+//      registers leave one plane an iteration and 8 warps to hide the loads' latency: 0.272 against 0.255.
+//   8: blocks of 2 x 2 of 8-byte vectors, two planes: 0.254 to 0.257 at order 8, 0.342 for 24 boxes of order 4
+//      where shape 6 takes 0.347.
+// To keep a block's loads free of bank conflicts (a point is 64 bytes, half of the banks) the odd blocks of
+// a row are mirrored: their first point is the right one and their x offsets count downwards, so that two
+// blocks side by side always read different halves of the banks.  The x arm is symmetric, so mirrored values
+// are the same bit for bit.
 template <int SHAPE> struct WsShape;
 template <> struct WsShape<0> { static constexpr int U = 1, TX = 16, TY = 8, R = 2, RX = 1; };   //  8 consumer warps
 template <> struct WsShape<1> { static constexpr int U = 1, TX = 16, TY = 12, R = 4, RX = 1; };  //  6
@@ -397,7 +393,7 @@ template <int TX, int TY, int R, int OV = OVC, int RX = 1, bool SPL = false> str
   static constexpr bool SPLIT = RX == 2 || SPL;
   static_assert(!SPLIT || CW == 12 || CW == 8, "the register splits are for twelve or eight consumer warps");
   static constexpr int CONSUMER_REGS = CW == 12 ? 152 : 232, PRODUCER_REGS = CW == 12 ? 56 : 40;
-  static constexpr int THREADS = 32 * CW + 128;            // + three producer warps and the patcher
+  static constexpr int THREADS = 32 * CW + 128;            // + the four service warps
   // consumer thread t owns vector t % OV of block (t / OV) % (TX / RX) of row group t / (OV TX / RX),
   // whose R rows are y-adjacent: the row groups must fill the tile and the warps exactly
   static_assert(TY % R == 0 && TX % RX == 0 && CW * 32 == OV * (TX / RX) * (TY / R),
