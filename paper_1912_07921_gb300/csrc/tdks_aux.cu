@@ -14,35 +14,34 @@ namespace tdks {
 //                                         exp(+i (k.T_u + A.d_u)) in(cell(u))[v]
 // (the <beta_aj|psi> of V_NL = sum |beta> D <beta|; the paper's norm-conserving
 // pseudopotentials, Sec. "Magneto-optics" and Sec. "Periodic systems", with synthetic
-// Gaussian-times-polynomial projectors).  n_chunks CTAs per (atom, kb), each summing a contiguous
-// share of the sphere with 64 point lanes x OVC vectors (warp shuffles, then warps through shared
-// memory in a fixed order); their sums are added in chunk order and take D_aj h^3.  For one system
-// the chunks of a unit are a thread-block cluster whose first CTA reads the others' sums from their
-// shared memory; a second launch for that sum, a chain of 16 dependent loads, took longer than the
-// gather itself (64^3, 4 atoms, 2 k-batches: 8.2 + 10 us against 11.2).  Batches keep two launches (their
-// units differ in size).  No atomics: the result does not depend on timing.
+// Gaussian-times-polynomial projectors).  An atom's entries are split into n_chunks contiguous shares, a
+// share over 8 warps of 8 point lanes x OVC vectors.  A warp sums its entries (complex64: in FP32, so this
+// grouping is part of the result), its lanes meet by shuffles, then the warps of a share and the shares are
+// added in order in FP64, times D_aj h^3.  For one system a thread-block cluster takes the 8 n_chunks warps of a
+// unit, and its first CTA reads the others' sums from their shared memory; a second launch for that sum, a
+// chain of 16 dependent loads, took longer than the gather itself (64^3, 4 atoms, 2 k-batches: 8.2 + 10 us
+// against 11.2).  Batches keep two launches (their units differ in size).  No atomics: the result does not
+// depend on timing.
 // ---------------------------------------------------------------------------------
-constexpr int GATHER_THREADS = 256;
+constexpr int GATHER_THREADS = 256;   // of a share
+constexpr int GATHER_CHUNKS = 16;     // most shares
 
-// CTAs of a unit.  Of a batch: as many as fill the GPU.  Of a system alone (a cluster): 8 while all units
-// are resident at once that way, else 4, also where the units alone would fill the GPU, as a CTA's loop is
-// a chain of dependent loads.  Gather and non-local kernel of 8 atoms x 16 k-batches in a 64^3 cell: 115 us
-// with 1 CTA a unit, 78, 68, 62 with 2, 3, 4, then 77, 74, 70 with 5, 6, 8 (clusters of 5 to 7 leave SMs of a
-// GPC over); 16 atoms x 8: 42, 33, 31, 30, 38, 38, 39.
-int gather_chunks(long units, bool cluster) {
-  if (cluster) return units * 16 <= 152L * 4 ? 8 : 4;  // (8 CTAs: the portable cluster size)
+int gather_chunks(long units) {
   const long want = (152L * 4 + units - 1) / units;
-  return (int)(want < 1 ? 1 : (want > 8 ? 8 : want));
+  return (int)(want < 1 ? 1 : (want > GATHER_CHUNKS ? GATHER_CHUNKS : want));
 }
+// CTAs of a unit's cluster (the portable sizes; clusters of 3 or 5 to 7 leave SMs of a GPC over: 8 atoms x 16
+// k-batches in a 64^3 cell, gather and non-local kernel, 78 us with 2, 62 with 4, 77 with 5, 74 with 6)
+static int gather_cluster(int n_chunks) { return n_chunks < 2 ? 1 : (n_chunks < 4 ? 2 : (n_chunks <= 8 ? 4 : 8)); }
 
-// (out: this CTA's 4 x OVC x 2 sums, index (j OVC + v) 2 + c)
+// One warp's share: warp w (0 .. 8 n_chunks - 1) of unit (a, kb).  (out: 4 x OVC x 2 sums, index (j OVC + v) 2 + c)
 template <int P, int BLOCH>
-__device__ __forceinline__ void gather_body(const GatherParams &p, int a, int kb, int chunk, double2 *out) {
+__device__ __forceinline__ void gather_warp(const GatherParams &p, int a, int kb, int w, double2 *out) {
   typedef VT<P> T;
   typedef typename T::V V;
   const int kidx = kb / p.n_batches;
-  const int tid = threadIdx.x, v = tid % OVC, lane = tid / OVC;
-  constexpr int LANES = GATHER_THREADS / OVC;
+  constexpr int LANES = GATHER_THREADS / OVC, WARPS = GATHER_THREADS / 32;
+  const int tid = threadIdx.x, v = tid % OVC, chunk = w / WARPS, lane = w % WARPS * (32 / OVC) + tid % 32 / OVC;
   // per-lane sums: FP64 for complex128 systems, FP32 for complex64 systems; the cross-lane
   // sums below are FP64 for both.
   double2 accd[4] = {};
@@ -92,10 +91,9 @@ __device__ __forceinline__ void gather_body(const GatherParams &p, int a, int kb
       }
     }
   }
-  // reduce over lanes with equal v (they differ in bits 2..4 of the lane id), then over the
-  // warps in a fixed order.  complex64: the lane sums are FP32 (as the per-lane sums), so
-  // the shuffles stay off GB300's slow FP64 pipe; the warp partials are FP64.
-  __shared__ double2 red[GATHER_THREADS / 32][4][OVC][2];
+  // reduce over lanes with equal v (they differ in bits 2..4 of the lane id).  complex64: the
+  // lane sums are FP32 (as the per-lane sums), so the shuffles stay off GB300's slow FP64 pipe;
+  // the warp partials are FP64.
 #pragma unroll
   for (int j = 0; j < 4; j++)
 #pragma unroll
@@ -106,30 +104,19 @@ __device__ __forceinline__ void gather_body(const GatherParams &p, int a, int kb
           x.x += __shfl_xor_sync(0xffffffffu, x.x, o);
           x.y += __shfl_xor_sync(0xffffffffu, x.y, o);
         }
-        if ((tid & 31) < OVC) red[tid >> 5][j][v][cc] = make_double2(x.x, x.y);
+        if (tid % 32 < OVC) out[(j * OVC + v) * 2 + cc] = make_double2(x.x, x.y);
       } else if (cc == 0) {
         double2 x = accd[j];
         for (int o = 4; o < 32; o <<= 1) {
           x.x += __shfl_xor_sync(0xffffffffu, x.x, o);
           x.y += __shfl_xor_sync(0xffffffffu, x.y, o);
         }
-        if ((tid & 31) < OVC) {
-          red[tid >> 5][j][v][0] = x;
-          red[tid >> 5][j][v][1] = make_double2(0.0, 0.0);
+        if (tid % 32 < OVC) {
+          out[(j * OVC + v) * 2] = x;
+          out[(j * OVC + v) * 2 + 1] = make_double2(0.0, 0.0);
         }
       }
     }
-  __syncthreads();
-  if (tid < 4 * OVC) {
-    const int j = tid / OVC, vv = tid % OVC;
-    double2 s0 = make_double2(0.0, 0.0), s1 = make_double2(0.0, 0.0);
-    for (int w = 0; w < GATHER_THREADS / 32; w++) {
-      s0.x += red[w][j][vv][0].x; s0.y += red[w][j][vv][0].y;
-      s1.x += red[w][j][vv][1].x; s1.y += red[w][j][vv][1].y;
-    }
-    out[2 * tid] = s0;
-    out[2 * tid + 1] = s1;
-  }
 }
 
 // q of one (atom, kb, j, v) from its sums, times D h^3.
@@ -146,23 +133,37 @@ __device__ __forceinline__ void store_q(const GatherParams &p, int a, int kb, in
   }
 }
 
-// One system: a cluster of n_chunks CTAs per (atom, kb).
+// One system: a cluster of `ctas` CTAs per (atom, kb).
+constexpr int GATHER_SUMS = 8 * OVC;  // of a warp
 template <int P, int BLOCH>
-__global__ void __launch_bounds__(GATHER_THREADS) gather_kernel(const GatherParams p) {
-  __shared__ double2 part[4 * OVC * 2];
-  const int a = blockIdx.x / p.n_chunks, kb = blockIdx.y, chunk = blockIdx.x % p.n_chunks, t = threadIdx.x;
-  gather_body<P, BLOCH>(p, a, kb, chunk, part);
+__global__ void __launch_bounds__(2 * GATHER_THREADS, 2) gather_kernel(const GatherParams p, int ctas) {
+  constexpr int WARPS = GATHER_THREADS / 32;
+  __shared__ double2 red[2 * WARPS][GATHER_SUMS], part[GATHER_CHUNKS][GATHER_SUMS];
+  const int a = blockIdx.x / ctas, rank = blockIdx.x % ctas, kb = blockIdx.y, t = threadIdx.x;
+  const int warps = blockDim.x / 32, warp = t / 32;
+  gather_warp<P, BLOCH>(p, a, kb, rank * warps + warp, red[warp]);
   cg::cluster_group cl = cg::this_cluster();
   cl.sync();
-  if (chunk == 0 && t < 4 * OVC) {
-    double2 s0 = part[2 * t], s1 = part[2 * t + 1];
-    for (int c = 1; c < p.n_chunks; c++) {
-      const double2 *r = cl.map_shared_rank(part, c);
-      const double2 x = r[2 * t], y = r[2 * t + 1];
-      s0.x += x.x; s0.y += x.y;
-      s1.x += y.x; s1.y += y.y;
+  if (rank == 0) {
+    for (int i = t; i < p.n_chunks * GATHER_SUMS; i += blockDim.x) {
+      const int c = i / GATHER_SUMS, k = i % GATHER_SUMS;
+      double2 x[WARPS], s = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int w = 0; w < WARPS; w++)
+        x[w] = cl.map_shared_rank(&red[0][0], (c * WARPS + w) / warps)[(c * WARPS + w) % warps * GATHER_SUMS + k];
+#pragma unroll
+      for (int w = 0; w < WARPS; w++) { s.x += x[w].x; s.y += x[w].y; }
+      part[c][k] = s;
     }
-    store_q<P>(p, a, kb, t, s0, s1);
+    __syncthreads();
+    if (t < 4 * OVC) {
+      double2 s0 = make_double2(0.0, 0.0), s1 = make_double2(0.0, 0.0);
+      for (int c = 0; c < p.n_chunks; c++) {
+        s0.x += part[c][2 * t].x; s0.y += part[c][2 * t].y;
+        s1.x += part[c][2 * t + 1].x; s1.y += part[c][2 * t + 1].y;
+      }
+      store_q<P>(p, a, kb, t, s0, s1);
+    }
   }
   cl.sync();  // the others' shared memory stays until it has been read
 }
@@ -261,8 +262,16 @@ gather_batch_kernel(const GatherParams *gp, const long *begin, const int *sys_of
   const long u = blockIdx.x - begin[s];
   const long unit = u / p.n_chunks;
   const int chunk = (int)(u % p.n_chunks);
-  gather_body<P, 0>(p, (int)(unit % p.n_atoms), (int)(unit / p.n_atoms), chunk,
-                    p.qpart + ((long)(unit / p.n_atoms * p.n_atoms + unit % p.n_atoms) * p.n_chunks + chunk) * 8 * OVC);
+  __shared__ double2 red[GATHER_THREADS / 32][GATHER_SUMS];
+  const int t = threadIdx.x;
+  gather_warp<P, 0>(p, (int)(unit % p.n_atoms), (int)(unit / p.n_atoms), chunk * (GATHER_THREADS / 32) + t / 32,
+                    red[t / 32]);
+  __syncthreads();
+  if (t < GATHER_SUMS) {
+    double2 x = make_double2(0.0, 0.0);
+    for (int w = 0; w < GATHER_THREADS / 32; w++) { x.x += red[w][t].x; x.y += red[w][t].y; }
+    p.qpart[((unit / p.n_atoms * p.n_atoms + unit % p.n_atoms) * p.n_chunks + chunk) * GATHER_SUMS + t] = x;
+  }
 }
 
 template <int P>
@@ -433,7 +442,8 @@ __global__ void __launch_bounds__(NLC_THREADS) nl_current_kernel(const NlCurrent
 
 cudaError_t launch_nl_current(const NlCurrentParams &q, cudaStream_t s) {
   NlCurrentParams p = q;
-  p.n_chunks = gather_chunks((long)p.n_atoms * p.n_kb, true);
+  // (complex64: the lanes' FP32 sums run over all of an atom's entries)
+  p.n_chunks = p.prec != P_C128 ? 1 : ((long)p.n_atoms * p.n_kb * 16 <= 152L * 4 ? 8 : 4);
   return launch_cluster(nl_current_kernel, dim3(p.n_atoms * p.n_chunks, p.n_kb), NLC_THREADS, s, p.n_chunks, p);
 }
 
@@ -461,6 +471,19 @@ __global__ void phase_table_kernel(const ProjEntry *ent, int n_ent, int n_k, con
   }
 }
 
+// e^{i k_a L_a} of the complex64 sweeps, [n_k][3] in FP64 from the FP32 sine and cosine.
+__global__ void face_phase_kernel(int n, const double *kvec, double Lx, double Ly, double Lz, double2 *out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  float sn, cs;
+  sincosf((float)(kvec[i] * (i % 3 == 0 ? Lx : (i % 3 == 1 ? Ly : Lz))), &sn, &cs);
+  out[i] = make_double2(cs, sn);
+}
+cudaError_t launch_face_phase(int n_k, const double *kvec, const double L[3], double2 *out, cudaStream_t s) {
+  face_phase_kernel<<<(3 * n_k + 127) / 128, 128, 0, s>>>(3 * n_k, kvec, L[0], L[1], L[2], out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_k, const double *kvec,
                                const double A[3], int bloch, void *out, cudaStream_t s) {
   const long n = (long)n_ent * n_k;
@@ -473,8 +496,8 @@ cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_
 
 template <int P, int BLOCH>
 static cudaError_t launch_gather_t(const GatherParams &p, cudaStream_t s) {
-  if (cudaError_t e = launch_cluster(gather_kernel<P, BLOCH>, dim3(p.n_atoms * p.n_chunks, p.n_kb), GATHER_THREADS, s,
-                                     p.n_chunks, p))
+  const int ctas = gather_cluster(p.n_chunks), threads = GATHER_THREADS * p.n_chunks / ctas;
+  if (cudaError_t e = launch_cluster(gather_kernel<P, BLOCH>, dim3(p.n_atoms * ctas, p.n_kb), threads, s, ctas, p, ctas))
     return e;
   if (p.n_sp <= 0) return cudaSuccess;
   const int run = nl_run_of(p.n_sp, p.n_kb);

@@ -247,7 +247,7 @@ int tdks_batch_create(const tdks_sys *systems, int n, void *stream, tdks_batch_t
   for (tdks_system *s : b->sys) batch_units += (long)s->n_atoms * s->n_kb;
   long all_lda = 0;
   for (tdks_system *s : b->sys) all_lda += lda_work(s);
-  const int bchunks = gather_chunks(std::max(batch_units, 1L), false);
+  const int bchunks = gather_chunks(std::max(batch_units, 1L));
   for (int i = 0; i < n; i++) {
     tdks_system *s = b->sys[i];
     const void *ins[4] = {s->psi, s->term[0], s->term[1], s->term[2]};

@@ -223,7 +223,7 @@ void sweep_common(const tdks_system *s, SweepParams &p, const double A[3], int s
   p.nl = s->d_nl;
   p.n_ent = s->n_ent;
   p.kvec = s->d_kvec;
-  p.kphase = s->d_kphase;
+  p.kphase = s->d_kphase + (s->prec == TDKS_C64 ? 3 * s->n_k : 0);
   p.bloch = s->bc == TDKS_BC_BLOCH;
   p.L[0] = s->nx * s->h; p.L[1] = s->ny * s->h; p.L[2] = s->nz * s->h;
   for (int a = 0; a < 3; a++) p.A[a] = A[a];
@@ -602,7 +602,7 @@ int tdks_create_grid(int nx, int ny, int nz, double h, int fd_order, int bc, int
   ALLOC(s->ring, (size_t)tdks_system::RING * TDKS_RECORD * sizeof(double));
   ALLOC(s->obs_rec, TDKS_RECORD * sizeof(double));
   ALLOC(s->d_kvec, 3 * n_k * sizeof(double));
-  ALLOC(s->d_kphase, 3 * n_k * sizeof(double2));
+  ALLOC(s->d_kphase, (prec == TDKS_C64 ? 6 : 3) * n_k * sizeof(double2));
   ALLOC(s->d_wocc, n_k * sizeof(double));
 #undef ALLOC
   std::vector<double2> kphase(3 * n_k);
@@ -611,6 +611,7 @@ int tdks_create_grid(int nx, int ny, int nz, double h, int fd_order, int bc, int
     kphase[i] = make_double2(std::cos(s->kpts[i] * L[i % 3]), std::sin(s->kpts[i] * L[i % 3]));
   if (cudaMemcpy(s->d_kvec, s->kpts.data(), 3 * n_k * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(s->d_kphase, kphase.data(), 3 * n_k * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
+      (prec == TDKS_C64 && launch_face_phase(n_k, s->d_kvec, L, s->d_kphase + 3 * n_k, s->stream) != cudaSuccess) ||
       cudaMemsetAsync(s->vloc, 0, N * sizeof(double), s->stream) != cudaSuccess ||
       cudaMemsetAsync(s->aux, 0, N * sizeof(PointAux), s->stream) != cudaSuccess ||
       cudaMemsetAsync(s->psi, 0, s->state_bytes, s->stream) != cudaSuccess ||
@@ -872,7 +873,7 @@ int tdks_set_atoms_projectors(tdks_sys s, int n_atoms, const double *pos, const 
   CU(cudaMalloc((void **)&s->d_atom_begin, (n_atoms + 1) * sizeof(int)));
   CU(cudaMalloc((void **)&s->d_ent, ent.size() * sizeof(ProjEntry)));
   CU(cudaMalloc((void **)&s->d_q, (size_t)s->n_kb * n_atoms * 4 * OVC * 16));
-  s->gchunks = gather_chunks((long)n_atoms * s->n_kb, true);
+  s->gchunks = gather_chunks((long)n_atoms * s->n_kb);
   CU(cudaMalloc((void **)&s->d_qpart, (size_t)s->n_kb * n_atoms * s->gchunks * 4 * OVC * 2 * sizeof(double2)));
   CU(cudaMalloc((void **)&s->d_D, (size_t)n_atoms * 4 * sizeof(double)));
   {

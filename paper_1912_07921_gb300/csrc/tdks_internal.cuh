@@ -118,7 +118,7 @@ struct SweepParams {
   // Bloch boundary
   int bloch;                  // periodic cell: values across a face carry exp(i k.L) per wrap
   const double *kvec;         // [n_k][3]
-  const double2 *kphase;      // [n_k][3] e^{i k_a L_a}
+  const double2 *kphase;      // [n_k][3] e^{i k_a L_a} in the compute precision
   double L[3];
   double A[3];                // vector potential (velocity gauge)
   int grad_mask;              // bit a: add -i A_a grad_a; bit 3: observables need all grads
@@ -246,10 +246,11 @@ size_t sweep_smem(int M, int tx, int ty);
 constexpr int NL_THREADS = 256;
 cudaError_t launch_gather(int prec, int bloch, const GatherParams &p, cudaStream_t s);
 // out[k * n_ent + e] = (cos, sin) of A.d_e (+ k.T_e in a periodic cell): float2 (complex64) or double2
+cudaError_t launch_face_phase(int n_k, const double *kvec, const double L[3], double2 *out, cudaStream_t s);
 cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_k, const double *kvec,
                                const double A[3], int bloch, void *out, cudaStream_t s);
 // chunks per (atom, k-batch) that fill the GPU for n_atoms * n_kb units
-int gather_chunks(long units, bool cluster);
+int gather_chunks(long units);
 cudaError_t launch_density(int prec, long N, int n_kb, int n_batches, const void *psi, const void *psi_lo,
                            const double *wocc, double *dens_part, cudaStream_t s);
 cudaError_t launch_lda(int prec, int bloch, long N, int nx, int ny, int nz, double h,

@@ -56,7 +56,7 @@ struct tdks_system {
   double *ring = nullptr;
   double *obs_rec = nullptr;    // single record for tdks_observe
   double *d_kvec = nullptr, *d_wocc = nullptr, *d_D = nullptr;
-  double2 *d_kphase = nullptr;  // [n_k][3] e^{i k_a L_a}
+  double2 *d_kphase = nullptr;  // [n_k][3] e^{i k_a L_a}; complex64 systems: then the same from FP32 functions
   int *d_rowent = nullptr, *d_atom_begin = nullptr;
   int2 *d_sp = nullptr;       // entry ranges of the points inside a sphere
   void *d_nl = nullptr;       // non-local term per sphere point, [n_kb][n_ent + 1][OVC]

@@ -148,8 +148,9 @@ template <> struct VT<P_C64> {
   typedef u64 K;
   static __device__ __forceinline__ K kcoef(double, float f, bool im) { return pk2(im ? -f : f, f); }
   static __device__ __forceinline__ u64 kmul1(K k, bool im, u64 a) {
+    // (plus zero: the assembler joins a bare product with the sum that takes it, which then rounds once)
     const float2 f = up2(a);
-    return mul2(k, im ? pk2(f.y, f.x) : a);
+    return fma2(k, im ? pk2(f.y, f.x) : a, 0ull);
   }
   static __device__ __forceinline__ V kmul(K k, bool im, V a) {
     return make_ulonglong2(kmul1(k, im, a.x), kmul1(k, im, a.y));
@@ -193,7 +194,7 @@ template <> struct VT<P_C64S> {
   static __device__ __forceinline__ K kcoef(double, float f, bool im) { return pk2(im ? -f : f, f); }
   static __device__ __forceinline__ V kmul(K k, bool im, V a) {
     const float2 f = up2(a);
-    return mul2(k, im ? pk2(f.y, f.x) : a);
+    return fma2(k, im ? pk2(f.y, f.x) : a, 0ull);  // (plus zero: as VT<P_C64>::kmul1)
   }
   static __device__ __forceinline__ V negi(V a) {
     const float2 p = up2(a);
