@@ -30,12 +30,21 @@ int gather_chunks(long units) {
   const long want = (152L * 4 + units - 1) / units;
   return (int)(want < 1 ? 1 : (want > GATHER_CHUNKS ? GATHER_CHUNKS : want));
 }
+// Shares for a system alone: complex128, whose sums do not depend on the grouping in any digit that counts, in
+// as many as its cluster has CTAs, 8 while all units are resident at once that way, else 4 (96^3, 16 atoms, 4
+// k-batches: gather and non-local kernel 50 us, with the 10 shares of the rule above 63).
+int gather_chunks_alone(int prec, long units) {
+  return prec == P_C64 ? gather_chunks(units) : (units * 16 <= 152L * 4 ? 8 : 4);
+}
 // CTAs of a unit's cluster (the portable sizes; clusters of 3 or 5 to 7 leave SMs of a GPC over: 8 atoms x 16
-// k-batches in a 64^3 cell, gather and non-local kernel, 78 us with 2, 62 with 4, 77 with 5, 74 with 6)
-static int gather_cluster(int n_chunks) { return n_chunks < 2 ? 1 : (n_chunks < 4 ? 2 : (n_chunks <= 8 ? 4 : 8)); }
+// k-batches in a 64^3 cell, both kernels, 115 us with 1, 78 with 2, 62 with 4, 77 with 5, 74 with 6)
+static int gather_cluster(int prec, int n_chunks) {
+  if (prec != P_C64) return n_chunks;
+  return n_chunks < 2 ? 1 : (n_chunks < 4 ? 2 : (n_chunks <= 8 ? 4 : 8));
+}
 
 // One warp's share: warp w (0 .. 8 n_chunks - 1) of unit (a, kb).  (out: 4 x OVC x 2 sums, index (j OVC + v) 2 + c)
-template <int P, int BLOCH>
+template <int P, int BLOCH, int UN>
 __device__ __forceinline__ void gather_warp(const GatherParams &p, int a, int kb, int w, double2 *out) {
   typedef VT<P> T;
   typedef typename T::V V;
@@ -50,7 +59,7 @@ __device__ __forceinline__ void gather_warp(const GatherParams &p, int a, int kb
   const int len = (a1 - a0 + p.n_chunks - 1) / p.n_chunks;
   const int e0 = a0 + chunk * len, e1 = min(a1, e0 + len);
   const bool phase = BLOCH || (p.A[0] != 0.0 || p.A[1] != 0.0 || p.A[2] != 0.0);
-#pragma unroll 4
+#pragma unroll UN
   for (int e = e0 + lane; e < e1; e += LANES) {
     if constexpr (P == P_C64) {
       // compact entry arrays: 8 + 16 bytes per entry instead of the full record
@@ -133,36 +142,55 @@ __device__ __forceinline__ void store_q(const GatherParams &p, int a, int kb, in
   }
 }
 
-// One system: a cluster of `ctas` CTAs per (atom, kb).
+// One system: a cluster of `ctas` CTAs per (atom, kb).  complex64: 48 registers, so that the 5 shares of 128 units (16 atoms
+// and 8 k-batches) are resident at once.
 constexpr int GATHER_SUMS = 8 * OVC;  // of a warp
 template <int P, int BLOCH>
-__global__ void __launch_bounds__(2 * GATHER_THREADS, 2) gather_kernel(const GatherParams p, int ctas) {
+__global__ void __maxnreg__(P == P_C64 ? 48 : 64) gather_kernel(const GatherParams p, int ctas) {
   constexpr int WARPS = GATHER_THREADS / 32;
-  __shared__ double2 red[2 * WARPS][GATHER_SUMS], part[GATHER_CHUNKS][GATHER_SUMS];
+  __shared__ double2 red[2 * WARPS][GATHER_SUMS], part[GATHER_CHUNKS][GATHER_SUMS], tot[GATHER_SUMS];
   const int a = blockIdx.x / ctas, rank = blockIdx.x % ctas, kb = blockIdx.y, t = threadIdx.x;
   const int warps = blockDim.x / 32, warp = t / 32;
-  gather_warp<P, BLOCH>(p, a, kb, rank * warps + warp, red[warp]);
+  gather_warp<P, BLOCH, P == P_C64 ? 2 : 4>(p, a, kb, rank * warps + warp, red[warp]);
   cg::cluster_group cl = cg::this_cluster();
-  cl.sync();
-  if (rank == 0) {
-    for (int i = t; i < p.n_chunks * GATHER_SUMS; i += blockDim.x) {
+  const bool whole = warps % WARPS == 0;  // a share's warps are one CTA's
+  const int own = warps / WARPS;
+  if (whole) {
+    __syncthreads();
+    for (int i = t; i < own * GATHER_SUMS; i += blockDim.x) {
       const int c = i / GATHER_SUMS, k = i % GATHER_SUMS;
-      double2 x[WARPS], s = make_double2(0.0, 0.0);
+      double2 s = make_double2(0.0, 0.0);
 #pragma unroll
-      for (int w = 0; w < WARPS; w++)
-        x[w] = cl.map_shared_rank(&red[0][0], (c * WARPS + w) / warps)[(c * WARPS + w) % warps * GATHER_SUMS + k];
-#pragma unroll
-      for (int w = 0; w < WARPS; w++) { s.x += x[w].x; s.y += x[w].y; }
+      for (int w = 0; w < WARPS; w++) { s.x += red[c * WARPS + w][k].x; s.y += red[c * WARPS + w][k].y; }
       part[c][k] = s;
     }
-    __syncthreads();
-    if (t < 4 * OVC) {
-      double2 s0 = make_double2(0.0, 0.0), s1 = make_double2(0.0, 0.0);
-      for (int c = 0; c < p.n_chunks; c++) {
-        s0.x += part[c][2 * t].x; s0.y += part[c][2 * t].y;
-        s1.x += part[c][2 * t + 1].x; s1.y += part[c][2 * t + 1].y;
+  }
+  cl.sync();
+  if (rank == 0) {
+    if (!whole) {
+      for (int i = t; i < p.n_chunks * GATHER_SUMS; i += blockDim.x) {
+        const int c = i / GATHER_SUMS, k = i % GATHER_SUMS;
+        double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int w = 0; w < WARPS; w++) {
+          const int q = c * WARPS + w;
+          const double2 x = cl.map_shared_rank(&red[0][0], q / warps)[q % warps * GATHER_SUMS + k];
+          s.x += x.x; s.y += x.y;
+        }
+        part[c][k] = s;
       }
-      store_q<P>(p, a, kb, t, s0, s1);
+      __syncthreads();
+    }
+    if (t < GATHER_SUMS) {
+      double2 s = make_double2(0.0, 0.0);
+#pragma unroll 4
+      for (int c = 0; c < p.n_chunks; c++) {
+        const double2 x = whole ? cl.map_shared_rank(&part[0][0], c / own)[c % own * GATHER_SUMS + t] : part[c][t];
+        s.x += x.x; s.y += x.y;
+      }
+      tot[t] = s;
+      __syncwarp();
+      if (t < 4 * OVC) store_q<P>(p, a, kb, t, tot[2 * t], tot[2 * t + 1]);
     }
   }
   cl.sync();  // the others' shared memory stays until it has been read
@@ -264,7 +292,7 @@ gather_batch_kernel(const GatherParams *gp, const long *begin, const int *sys_of
   const int chunk = (int)(u % p.n_chunks);
   __shared__ double2 red[GATHER_THREADS / 32][GATHER_SUMS];
   const int t = threadIdx.x;
-  gather_warp<P, 0>(p, (int)(unit % p.n_atoms), (int)(unit / p.n_atoms), chunk * (GATHER_THREADS / 32) + t / 32,
+  gather_warp<P, 0, 4>(p, (int)(unit % p.n_atoms), (int)(unit / p.n_atoms), chunk * (GATHER_THREADS / 32) + t / 32,
                     red[t / 32]);
   __syncthreads();
   if (t < GATHER_SUMS) {
@@ -443,7 +471,7 @@ __global__ void __launch_bounds__(NLC_THREADS) nl_current_kernel(const NlCurrent
 cudaError_t launch_nl_current(const NlCurrentParams &q, cudaStream_t s) {
   NlCurrentParams p = q;
   // (complex64: the lanes' FP32 sums run over all of an atom's entries)
-  p.n_chunks = p.prec != P_C128 ? 1 : ((long)p.n_atoms * p.n_kb * 16 <= 152L * 4 ? 8 : 4);
+  p.n_chunks = p.prec != P_C128 ? 1 : gather_chunks_alone(P_C128, (long)p.n_atoms * p.n_kb);
   return launch_cluster(nl_current_kernel, dim3(p.n_atoms * p.n_chunks, p.n_kb), NLC_THREADS, s, p.n_chunks, p);
 }
 
@@ -496,7 +524,7 @@ cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_
 
 template <int P, int BLOCH>
 static cudaError_t launch_gather_t(const GatherParams &p, cudaStream_t s) {
-  const int ctas = gather_cluster(p.n_chunks), threads = GATHER_THREADS * p.n_chunks / ctas;
+  const int ctas = gather_cluster(P, p.n_chunks), threads = GATHER_THREADS * p.n_chunks / ctas;
   if (cudaError_t e = launch_cluster(gather_kernel<P, BLOCH>, dim3(p.n_atoms * ctas, p.n_kb), threads, s, ctas, p, ctas))
     return e;
   if (p.n_sp <= 0) return cudaSuccess;

@@ -873,7 +873,7 @@ int tdks_set_atoms_projectors(tdks_sys s, int n_atoms, const double *pos, const 
   CU(cudaMalloc((void **)&s->d_atom_begin, (n_atoms + 1) * sizeof(int)));
   CU(cudaMalloc((void **)&s->d_ent, ent.size() * sizeof(ProjEntry)));
   CU(cudaMalloc((void **)&s->d_q, (size_t)s->n_kb * n_atoms * 4 * OVC * 16));
-  s->gchunks = gather_chunks((long)n_atoms * s->n_kb);
+  s->gchunks = gather_chunks_alone(s->prec, (long)n_atoms * s->n_kb);
   CU(cudaMalloc((void **)&s->d_qpart, (size_t)s->n_kb * n_atoms * s->gchunks * 4 * OVC * 2 * sizeof(double2)));
   CU(cudaMalloc((void **)&s->d_D, (size_t)n_atoms * 4 * sizeof(double)));
   {
@@ -1080,15 +1080,21 @@ int tdks_autotune(tdks_sys s, int reps, double *ms) {
         continue;
       }
       if ((rc = tune_launch(s, sw))) break;  // warm-up (and fills this sweep's output)
-      cudaEventRecord(e0, s->stream);
-      for (int r = 0; r < reps && rc == TDKS_OK; r++) rc = tune_launch(s, sw);
-      cudaEventRecord(e1, s->stream);
+      // one launch first: a shape that it shows to be well behind the best is timed no further
+      for (int part = 0; part < 2 && rc == TDKS_OK; part++) {
+        const int n = part == 0 ? 1 : reps;
+        if (part == 1 && (reps == 1 || (best[sw] >= 0.0 && per > 1.15 * best[sw]))) break;
+        cudaEventRecord(e0, s->stream);
+        for (int r = 0; r < n && rc == TDKS_OK; r++) rc = tune_launch(s, sw);
+        cudaEventRecord(e1, s->stream);
+        if (rc) break;
+        if (cudaEventSynchronize(e1) != cudaSuccess) { rc = fail(TDKS_EDEVICE, "autotune timing"); break; }
+        if ((rc = check_err(s))) break;
+        float t = 0.f;
+        cudaEventElapsedTime(&t, e0, e1);
+        per = (double)t / n;
+      }
       if (rc) break;
-      if (cudaEventSynchronize(e1) != cudaSuccess) { rc = fail(TDKS_EDEVICE, "autotune timing"); break; }
-      if ((rc = check_err(s))) break;
-      float t = 0.f;
-      cudaEventElapsedTime(&t, e0, e1);
-      per = (double)t / reps;
       if (ms) ms[sh * 4 + sw] = per;
       if (best[sw] < 0.0 || per < best[sw]) { best[sw] = per; pick[sw] = sh; }
     }

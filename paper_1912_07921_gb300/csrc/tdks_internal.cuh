@@ -251,6 +251,7 @@ cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_
                                const double A[3], int bloch, void *out, cudaStream_t s);
 // chunks per (atom, k-batch) that fill the GPU for n_atoms * n_kb units
 int gather_chunks(long units);
+int gather_chunks_alone(int prec, long units);
 cudaError_t launch_density(int prec, long N, int n_kb, int n_batches, const void *psi, const void *psi_lo,
                            const double *wocc, double *dens_part, cudaStream_t s);
 cudaError_t launch_lda(int prec, int bloch, long N, int nx, int ny, int nz, double h,
