@@ -365,10 +365,10 @@ def run_ours(args, rank, world, local_rank):
 
 # FP64 instructions (thread level: DADD, DMUL, DFMA) per orbital value of one complex128
 # Taylor sub-step in the stencil sweeps, counted from the sweep source: per sweep the diagonal
-# term (1 add, 2 mul), M = 4 stencil distances of 5 complex adds and 1 complex FMA (12 each),
-# the Taylor coefficient (4); the last sweep adds the series combine (8 adds) and the density
-# (|psi|^2: 2, the lane sum and weight: ~2).  3 x 55 + 67 = 232.
-C128_FP64_INSTR_PER_VALUE_SUBSTEP = 232.0
+# term (2 mul), M = 4 stencil distances of 5 complex adds and 1 complex FMA (12 each),
+# the real or imaginary Taylor coefficient (2); the last sweep adds the series combine (8 adds) and the
+# density (|psi|^2: 2, the lane sum and weight: ~2).  3 x 52 + 64 = 220.
+C128_FP64_INSTR_PER_VALUE_SUBSTEP = 220.0
 
 
 def fp64_peak():
