@@ -324,12 +324,14 @@ int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool 
 // complex128 is bound by the FP64 pipe in every shape (96^3, 16 orbitals 1.513 ms with shape 0, 1.531 with 2) and
 // takes the tile that leaves fewer of its points outside the grid (cell of 30 x 36 x 32, 3 k-points, 10 orbitals:
 // 16 x 12 has 6% and 16 x 8 18% outside, 0.175 against 0.193 ms); short sweeps keep the smaller one.
+// A small complex64 cell also goes by the fit (first and middle term, 40^3 with 2 k-batches, 20% more of 16 x 12
+// tiles outside: 20.8 and 18.4 us with shape 0, 23.0 and 19.2 with 6; 48^3 with 1: 16.6 and 14.5, 15.6 and 14.6;
+// 36 x 30 x 32 with 2, 12.5% more outside: 18.7 and 16.3, 15.5 and 14.4).
 inline int ws_default_shape(int prec, int bloch, int nx, int ny, long points, bool last) {
-  if (prec != P_C64) {
-    const long wx = (nx + 15) / 16 * 16L, a0 = wx * ((ny + 7) / 8 * 8), a2 = wx * ((ny + 11) / 12 * 12);
-    return points >= 60000 && 51 * a2 < 50 * a0 ? 2 : 0;
-  }
+  const long wx = (nx + 15) / 16 * 16L, a0 = wx * ((ny + 7) / 8 * 8), a2 = wx * ((ny + 11) / 12 * 12);
+  if (prec != P_C64) return points >= 60000 && 51 * a2 < 50 * a0 ? 2 : 0;
   if (last) return points < 1500000 ? 3 : 2;
+  if (bloch && points < 150000 && 20 * a2 > 23 * a0) return 0;
   return points >= (bloch ? 60000 : 30000) ? 6 : 0;
 }
 // planes a shape's kernel takes per iteration
