@@ -435,10 +435,8 @@ void hartree_free(tdks_system *s) {
   s->d_vh = nullptr;
 }
 
-// Workspace, twiddle tables and the transformed kernel of the system's grid (once, when the Hartree
-// term is turned on).
-int hartree_setup(tdks_system *s) {
-  if (s->d_vh) return TDKS_OK;
+// Workspace, twiddle tables and the transformed kernel of the system's grid.
+static int hartree_build(tdks_system *s) {
   int hp[3];
   const int n[3] = {s->nx, s->ny, s->nz};
   const bool box = s->bc == TDKS_BC_ZERO;
@@ -456,14 +454,13 @@ int hartree_setup(tdks_system *s) {
       const double ang = 2.0 * M_PI * (double)(2 * j <= hp[a] ? j : j - hp[a]) / (double)hp[a];
       tw.push_back(make_double2(std::cos(ang), std::sin(ang)));
     }
-  // (the larger of the density's spectrum and, while the box's kernel is transformed, the kernel's)
   CU(cudaMalloc((void **)&s->d_htw, tw.size() * sizeof(double2)));
   CU(cudaMemcpy(s->d_htw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice));
   CU(cudaMalloc((void **)&s->d_hbuf, row * s->nz * sizeof(double2)));
   CU(cudaMalloc((void **)&s->d_hkern, row * hp[2] * sizeof(double)));
   CU(cudaMalloc((void **)&s->d_vh, s->N * sizeof(double)));
-  if (!s->n_total) CU(cudaMalloc((void **)&s->n_total, (size_t)s->N * sizeof(double)));
   if (box) {
+    // the sampled kernel and its half spectrum: the largest allocations here, for the length of this call
     const double self = 3.0 * std::log(2.0 + std::sqrt(3.0)) - 0.5 * M_PI;
     plans(hp, s->d_htw, p);
     double *k = nullptr;
@@ -479,14 +476,29 @@ int hartree_setup(tdks_system *s) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     cudaFree(k);
     cudaFree(kb);
-    CU(e);
+    if (e != cudaSuccess)
+      return fail(e == cudaErrorMemoryAllocation ? TDKS_ENOMEM : TDKS_EDEVICE,
+                  std::string("Hartree kernel transform: ") + cudaGetErrorString(e));
   } else {
     hartree_kernel_cell<<<grid_blocks(P), 256, 0, s->stream>>>(s->nx, s->ny, s->nz, s->nx * s->h, s->ny * s->h,
                                                                s->nz * s->h, s->d_hkern);
     CU(cudaGetLastError());
     CU(cudaStreamSynchronize(s->stream));
   }
+  if (!s->n_total) CU(cudaMalloc((void **)&s->n_total, (size_t)s->N * sizeof(double)));
   return TDKS_OK;
+}
+
+// Once, when the Hartree term is turned on: d_vh says that all of it is there, so a set-up that fails
+// leaves nothing behind and is done from the beginning the next time.
+int hartree_setup(tdks_system *s) {
+  if (s->d_vh) return TDKS_OK;
+  const int rc = hartree_build(s);
+  if (rc) {
+    hartree_free(s);
+    cudaGetLastError();  // (reported by rc)
+  }
+  return rc;
 }
 
 // v_H of the density in n_total (FP64, N points) into d_vh.
