@@ -19,8 +19,8 @@
 //   * Line transforms are mixed-radix Stockham passes in shared memory (Govindaraju et al., SC 2008:
 //     each pass takes R values N/R apart, twiddles them, does an R-point DFT and stores them in
 //     autosorted order), radices 8, 4, 2, 3, 5, 7, 11, 13, twiddles from a table.  A CTA takes LB
-//     adjacent lines, value-major ([i][line]), so that strided axes are read in runs of LB values and
-//     no pass has a bank conflict.
+//     adjacent lines, value-major ([i][line]), so that strided axes are read in runs of LB values and,
+//     with LB = 8 (lengths up to 512), no pass has a bank conflict.
 // Bound by the FP64 pipe (2 instructions per clock per SM) and, at small grids, by five launches: a
 // 128^3 padded transform pair is ~8e7 FP64 instructions, 0.13 ms.
 #include <cuda_runtime.h>
@@ -318,10 +318,12 @@ __global__ void hartree_kernel_cell(int nx, int ny, int nz, double Lx, double Ly
   }
 }
 
-// radices of a line length: 8, 4 and 2 for its powers of two, then its odd primes (<= 13)
+// radices of a line length: 8, 4 and 2 for its powers of two, then its odd primes (<= 13).  (At most six
+// for lengths up to FFT_MAXN; longer ones, which have no room for theirs, are refused first.)
 bool factor(int n, FftPlan &p) {
   p.n = n;
   p.nrad = 0;
+  if (n > FFT_MAXN) return false;
   int m = n;
   const int rad[] = {8, 4, 2, 3, 5, 7, 11, 13};
   for (int r : rad)
@@ -331,7 +333,7 @@ bool factor(int n, FftPlan &p) {
       p.rad[p.nrad++] = r;
       m /= r;
     }
-  return m == 1 && n <= FFT_MAXN;
+  return m == 1;
 }
 
 // smallest length >= m whose prime factors are 2 and 3
