@@ -38,7 +38,8 @@ inline cudaError_t ensure_smem_attr(K k, size_t smem, std::atomic<unsigned> &don
   return e;
 }
 
-// Launch with thread-block clusters of `cluster` CTAs along x.
+// Launch with thread-block clusters of `cluster` CTAs along x.  (An error is returned and, as by a
+// cudaGetLastError() after a launch, no longer pending.)
 template <typename... Par, typename... Arg>
 inline cudaError_t launch_cluster(void (*k)(Par...), dim3 grid, dim3 block, cudaStream_t s, int cluster, Arg &&...arg) {
   cudaLaunchConfig_t cfg{};
@@ -51,7 +52,9 @@ inline cudaError_t launch_cluster(void (*k)(Par...), dim3 grid, dim3 block, cuda
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, std::forward<Arg>(arg)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k, std::forward<Arg>(arg)...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 constexpr int OVC = 4;        // 16-byte vectors per (point, batch)

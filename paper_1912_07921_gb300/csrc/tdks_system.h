@@ -18,9 +18,11 @@ int fail(int code, const std::string &msg);
 #define CU(call)                                                                             \
   do {                                                                                       \
     cudaError_t e_ = (call);                                                                 \
-    if (e_ != cudaSuccess)                                                                   \
+    if (e_ != cudaSuccess) {                                                                 \
+      cudaGetLastError(); /* reported here, not by the next launch's check as well */        \
       return tdks_host::fail(e_ == cudaErrorMemoryAllocation ? TDKS_ENOMEM : TDKS_EDEVICE,   \
                              std::string(#call) + ": " + cudaGetErrorString(e_));            \
+    }                                                                                        \
   } while (0)
 
 }  // namespace tdks_host

@@ -26,6 +26,7 @@ def load(tmp_path):
     for name, (args, res) in _lib.SIGNATURES.items():
         getattr(lib, name).argtypes, getattr(lib, name).restype = args, res
     lib.fake_fail_malloc.argtypes = [ctypes.c_long]
+    lib.fake_fail_launch.argtypes = [ctypes.c_long]
     lib.fake_live_blocks.restype = ctypes.c_long
     lib.fake_set_hook.argtypes = [HOOK]
     lib.fake_host_us.argtypes = [ctypes.c_double]

@@ -2,6 +2,7 @@
 // files in place of the real runtime.  Device memory is host memory (copies above 16 MB are skipped), kernels
 // do not run.  What a test needs to see or to cause:
 //   * fake_fail_malloc(n): the n-th cudaMalloc from now returns cudaErrorMemoryAllocation (0: none does);
+//   * fake_fail_launch(n): the n-th kernel launch from now is refused;
 //   * fake_set_hook(f): every launch calls f(kernel's mangled name, grid, block, arguments), whose result is
 //     the kernel's time in microseconds on a modelled device.  fake_host_us(x): host time per launch.  Events
 //     read the modelled device's clock: work starts when the host has enqueued it and the device is free.
@@ -19,7 +20,7 @@ std::map<void *, size_t> blocks;  // every live allocation
 std::map<const void *, std::string> names;
 std::mutex names_lock;
 cudaError_t last = cudaSuccess;
-long fail_at = 0;
+long fail_at = 0, fail_launch = 0;
 double host_now = 0.0, busy_until = 0.0, host_us = 0.0;
 double (*hook)(const char *, const unsigned *, const unsigned *, void **) = nullptr;
 struct { dim3 grid, block; size_t smem; cudaStream_t s; } conf;
@@ -29,6 +30,7 @@ cudaError_t report(cudaError_t e) {
 }
 cudaError_t launch(const void *f, dim3 g, dim3 b, void **args) {
   const unsigned gg[3] = {g.x, g.y, g.z}, bb[3] = {b.x, b.y, b.z};
+  if (fail_launch > 0 && --fail_launch == 0) return report(cudaErrorInvalidConfiguration);
   host_now += host_us;
   const double t = hook ? hook(names[f].c_str(), gg, bb, args) : 0.0;
   busy_until = std::max(busy_until, host_now) + t;
@@ -44,6 +46,7 @@ int encode_tiled(...) { return 0; }
 extern "C" {
 
 void fake_fail_malloc(long n) { fail_at = n; }
+void fake_fail_launch(long n) { fail_launch = n; }
 long fake_live_blocks() { return (long)blocks.size(); }
 void fake_set_hook(double (*f)(const char *, const unsigned *, const unsigned *, void **)) { hook = f; }
 void fake_host_us(double us) { host_us = us; }
