@@ -1480,10 +1480,9 @@ int tdks_set_propagator(tdks_sys s, int propagator) {
 
 int tdks_set_exchange(tdks_sys s, tdks_exchange_fn fn, void *ctx) {
   if (!s) return fail(TDKS_EINVAL, "NULL system");
-  if (fn && !s->n_total) {
-    CU(cudaMalloc((void **)&s->n_total, (size_t)s->N * sizeof(double)));
-    CU(cudaMalloc((void **)&s->fin_sum, 10 * sizeof(double)));
-  }
+  // (each by itself: the Hartree term too allocates n_total)
+  if (fn && !s->n_total) CU(cudaMalloc((void **)&s->n_total, (size_t)s->N * sizeof(double)));
+  if (fn && !s->fin_sum) CU(cudaMalloc((void **)&s->fin_sum, 10 * sizeof(double)));
   s->xfn = fn;
   s->xctx = fn ? ctx : nullptr;
   return TDKS_OK;
