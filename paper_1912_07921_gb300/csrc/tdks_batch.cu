@@ -102,6 +102,13 @@ int enqueue_substep(tdks_batch *b) {
   return TDKS_OK;
 }
 
+// The sweeps' claim counter back to zero, where the last claim of every sweep leaves it, unless one of its CTAs
+// gave up a bounded wait (they claim nothing more): the next sweep would skip the items already counted.
+int reset_claims(tdks_batch *b) {
+  CU(cudaMemsetAsync(b->d_work, 0, sizeof(unsigned int), b->work));
+  return TDKS_OK;
+}
+
 template <class T>
 int upload(T **dst, const std::vector<T> &v) {
   CU(cudaMalloc((void **)dst, std::max<size_t>(1, v.size()) * sizeof(T)));
@@ -338,6 +345,7 @@ int tdks_batch_propagate(tdks_batch_t b, int n_steps, int use_graph) {
   CU(cudaEventRecord(b->ev_in, b->stream));
   CU(cudaStreamWaitEvent(b->work, b->ev_in, 0));
   CU(cudaMemcpyAsync(b->d_clock, clk.data(), n * sizeof(BatchClock), cudaMemcpyHostToDevice, b->work));
+  if (int rc = reset_claims(b)) return rc;
   if (use_graph && !b->exec) {
     CU(cudaStreamBeginCapture(b->work, cudaStreamCaptureModeThreadLocal));
     const int rc = enqueue_substep(b);
@@ -394,6 +402,7 @@ int tdks_batch_autotune(tdks_batch_t b, int reps, double *ms) {
     for (int i = 0; i < WS_SHAPES * 4; i++) ms[i] = -1.0;
   CU(cudaStreamSynchronize(b->stream));
   CU(cudaStreamSynchronize(b->work));
+  if (int rc = reset_claims(b)) return rc;
   const int n = (int)b->sys.size();
   const int saved[4] = {b->shape[0], b->shape[1], b->shape[2], b->shape[3]};
   int pick[4] = {saved[0], saved[1], saved[2], saved[3]};
