@@ -767,29 +767,37 @@ __device__ __forceinline__ void lda_body(long N, int nx, int ny, int nz, double 
     }
   }
   if (!sums) return;  // (uniform over the grid: V_eff only, no record follows)
-  __shared__ double red[LDA_THREADS / 32][6];
+  if constexpr (F32) {
+    // The threads' sums meet in FP64 in a fixed order: G = blockDim / 8 threads a component, each adding
+    // every G-th thread's value, then a tree: 8 sums a component and 8 threads on the FP64 pipe, where a shuffle
+    // tree in every warp has 40.  Medium molecule, a record's launch: 41.3 us (44.5 with shuffle trees in FP64
+    // and the kernel as it was then; 35.9 with sums that carry 48 bits only); 48^3, 16 orbitals: 11.4 (17.6; 10.4).
+    __shared__ double all[6][LDA_THREADS];
+    const int t = threadIdx.x, G = blockDim.x / 8, c = t / G, l = t % G;
 #pragma unroll
-  for (int i = 0; i < 6; i++) {
-    double x;
-    if constexpr (F32) {
-      // (lanes meet as double-float: five FP64 sums per value and warp cost more than the points)
-      float h = fh[i], l = fl[i];
-      for (int o = 16; o > 0; o >>= 1) {
-        const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
-        df_add_df(h, l, oh, ol);
-      }
-      x = (double)h + (double)l;
-    } else {
-      x = acc[i];
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    }
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][i] = x;
-  }
-  __syncthreads();
-  if (threadIdx.x < 6) {
+    for (int i = 0; i < 6; i++) all[i][t] = (double)fh[i] + (double)fl[i];
+    __syncthreads();
     double x = 0.0;
-    for (int w = 0; w < (int)blockDim.x / 32; w++) x += red[w][threadIdx.x];
-    lda_part[blk * 6 + threadIdx.x] = x;
+    if (c < 6) {
+#pragma unroll
+      for (int i = 0; i < 8; i++) x += all[c][l + i * G];
+    }
+    for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (c < 6 && l == 0) lda_part[blk * 6 + c] = x;
+  } else {
+    __shared__ double red[LDA_THREADS / 32][6];
+#pragma unroll
+    for (int i = 0; i < 6; i++) {
+      double x = acc[i];
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][i] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+      double x = 0.0;
+      for (int w = 0; w < (int)blockDim.x / 32; w++) x += red[w][threadIdx.x];
+      lda_part[blk * 6 + threadIdx.x] = x;
+    }
   }
 }
 
