@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <utility>
 #include <vector>
 
 #include "tdks_system.h"
@@ -60,12 +61,34 @@ void batch_free(tdks_batch *b) {
   if (b->work) cudaStreamDestroy(b->work);
 }
 
-// CTAs of one system in the batched LDA launch: its share of the 4 per SM that are resident at once, at
-// most the single-system count (whose partial buffer it fills).  A CTA's setup (system lookup, field, weight
-// staging) is paid once, and no second round of CTAs runs on a part of the SMs.
-static long lda_work(const tdks_system *s) { return s->N * (4 + s->n_kb); }
-static int lda_batch_blocks(const tdks_system *s, long total) {
-  return (int)std::max(1L, std::min((long)lda_blocks(s->N), 152L * 4 * lda_work(s) / total));
+// CTAs of each system in the batched LDA launch: whole rounds of the 4 per SM that are resident at once, as
+// many as leave a system 8 CTAs on average, handed out one by one where a CTA has most to do (no more than the
+// single-system count, whose partial buffer they fill).  A CTA's setup (system lookup, field, weight staging) is
+// paid once a round, no CTA has more than 6% above the even share, and no round runs on a part of the SMs.  (A
+// point of a complex64 system is bound by its loads, of a complex128 system by the cube root's FP64 instructions.)
+// complex64, 24 / 64 / 128 / 256 systems: 87 / 214 / 390 / 735 us, where one round with every system's share
+// rounded down took 87 / 222 / 519 / 1086 (1.1 to 2 times the even share on the slowest CTA) and CTAs of ~16
+// points a thread, without rounds, 124 / 266 / 496 / 952; a floor of 16 CTAs a system in place of 8 gives 212 at 64.
+// complex128, 8 / 24 / 64 systems: 153 / 404 / 1050, before 158 / 444 / 1389.
+std::vector<int> lda_batch_blocks(const std::vector<tdks_system *> &sys) {
+  const long n = (long)sys.size(), slots = 152L * 4, ctas = slots * std::max(1L, (8 * n + slots - 1) / slots);
+  std::vector<int> k(n, 1);
+  std::vector<std::pair<double, long>> heap;  // (work of a CTA, system), the largest on top
+  auto put = [&](long i) {
+    const tdks_system *s = sys[i];
+    if (k[i] >= lda_blocks(s->N)) return;
+    heap.push_back({(double)s->N * (s->prec == TDKS_C64 ? 4 + s->n_kb : 1) / k[i], i});
+    std::push_heap(heap.begin(), heap.end());
+  };
+  for (long i = 0; i < n; i++) put(i);
+  for (long c = n; c < ctas && !heap.empty(); c++) {
+    std::pop_heap(heap.begin(), heap.end());
+    const long i = heap.back().second;
+    heap.pop_back();
+    k[i]++;
+    put(i);
+  }
+  return k;
 }
 
 // Kernels one sub-step launches: the LDA/V_eff kernel, per Taylor term the projector step
@@ -252,8 +275,7 @@ int tdks_batch_create(const tdks_sys *systems, int n, void *stream, tdks_batch_t
   // partial-sum buffer holds
   long batch_units = 0;
   for (tdks_system *s : b->sys) batch_units += (long)s->n_atoms * s->n_kb;
-  long all_lda = 0;
-  for (tdks_system *s : b->sys) all_lda += lda_work(s);
+  const std::vector<int> lda_ctas = lda_batch_blocks(b->sys);
   const int bchunks = gather_chunks(std::max(batch_units, 1L));
   for (int i = 0; i < n; i++) {
     tdks_system *s = b->sys[i];
@@ -272,7 +294,7 @@ int tdks_batch_create(const tdks_sys *systems, int n, void *stream, tdks_batch_t
     gather_begin[i + 1] = gather_begin[i] + (long)s->n_atoms * s->n_kb * (s->n_atoms > 0 ? nch : 0);
     unit_begin[i + 1] = unit_begin[i] + (long)s->n_atoms * s->n_kb;
     nl_begin[i + 1] = nl_begin[i] + (s->n_atoms > 0 ? nl_batch_blocks(s->n_sp) : 0);
-    const int nl = lda_batch_blocks(s, all_lda);
+    const int nl = lda_ctas[i];
     lda_begin[i + 1] = lda_begin[i] + nl;
     BatchAux &a = aux[i];
     a.N = s->N; a.nx = s->nx; a.ny = s->ny; a.nz = s->nz; a.n_kb = s->n_kb; a.xc = s->xc;
