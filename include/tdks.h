@@ -371,7 +371,7 @@ int tdks_get_sweep_shape(tdks_sys sys, int sweep, int *shape);
 /* Autotuner: times every shape on each of the four Taylor-term sweeps of this system, on
  * its own grid, orbitals and projectors (in the velocity gauge with a vector potential
  * amp * pol, so that the gauge term is timed too; after one warm-up launch one launch, and
- * reps more unless that one is 15% behind the best; CUDA events on the system's stream; shapes
+ * reps more unless that one is 15% and 0.03 ms behind the shortest such launch; CUDA events on the system's stream; shapes
  * that run one kernel are timed once), and keeps the fastest shape per sweep.  The state psi is
  * not changed; the Taylor-term buffers and the density partials are overwritten (the next
  * propagation or H application rebuilds them).  ms (if not NULL) receives the mean

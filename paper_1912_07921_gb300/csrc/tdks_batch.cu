@@ -428,7 +428,7 @@ int tdks_batch_autotune(tdks_batch_t b, int reps, double *ms) {
   const int n = (int)b->sys.size();
   const int saved[4] = {b->shape[0], b->shape[1], b->shape[2], b->shape[3]};
   int pick[4] = {saved[0], saved[1], saved[2], saved[3]};
-  double best[4] = {-1.0, -1.0, -1.0, -1.0}, took[WS_SHAPES][4];
+  double best[4] = {-1.0, -1.0, -1.0, -1.0}, best_one[4] = {-1.0, -1.0, -1.0, -1.0}, took[WS_SHAPES][4];
   for (int i = 0; i < WS_SHAPES * 4; i++) took[i / 4][i % 4] = -1.0;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   CU(cudaEventCreate(&e0));
@@ -452,9 +452,11 @@ int tdks_batch_autotune(tdks_batch_t b, int reps, double *ms) {
                       n, b->total_items[k], b->d_work, b->d_item_sys[k]};
       cudaError_t e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, ks);  // warm-up
       // (one launch first, as for a system alone)
+      bool in_full = reps == 1;
       for (int part = 0; part < 2 && !rc; part++) {
         const int m = part == 0 ? 1 : reps;
-        if (part == 1 && (reps == 1 || (best[k] >= 0.0 && per > 1.15 * best[k]))) break;
+        if (part == 1 && (reps == 1 || !(in_full = tune_further(per, best_one[k])))) break;
+        if (part == 1 && (best_one[k] < 0.0 || per < best_one[k])) best_one[k] = per;
         cudaEventRecord(e0, b->work);
         for (int r = 0; r < m && e == cudaSuccess; r++)
           e = launch_sweep_tma_batch(b->M, b->prec, modes[k], a, b->work, ks);
@@ -470,7 +472,7 @@ int tdks_batch_autotune(tdks_batch_t b, int reps, double *ms) {
       }
       if (rc) break;
       if (ms) ms[sh * 4 + k] = per;
-      if (best[k] < 0.0 || per < best[k]) { best[k] = per; pick[k] = sh; }
+      if (in_full && (best[k] < 0.0 || per < best[k])) { best[k] = per; pick[k] = sh; }
     }
   }
   cudaEventDestroy(e0);

@@ -1020,24 +1020,30 @@ int tdks_get_sweep_shape(tdks_sys s, int sweep, int *shape) {
   return TDKS_OK;
 }
 
-// One timed Taylor-term sweep of the autotuner: sweep 0 reads the state and writes t1,
-// sweeps 1 and 2 read t(k-1) and write t(k); sweep 3 reads t3 and combines into t1/t2 in
-// place of the state (state hi <- t1, state lo <- t2), so the state itself is untouched.
-static int tune_launch(tdks_system *s, int sweep) {
+// A Taylor-term sweep of the autotuner: sweep 0 reads the state and writes t1, sweeps 1 and 2
+// read t(k-1) and write t(k); sweep 3 reads t3 and combines into t1/t2 in place of the state
+// (state hi <- t1, state lo <- t2), so the state itself is untouched.  Its parameters and maps
+// are made once per shape, as a propagation's are, so that the timed launches follow one another.
+struct TuneSweep {
+  SweepParams p{};
+  SweepMaps tm;
+  int mode;
+};
+static int tune_prepare(tdks_system *s, int sweep, TuneSweep &t) {
   // in the velocity gauge, a vector potential along the field's polarisation, so that the
   // timed sweeps carry the gauge term the propagation's sweeps carry
   double At[3] = {0.0, 0.0, 0.0};
   if (s->gauge == TDKS_GAUGE_VELOCITY)
     for (int a = 0; a < 3; a++) At[a] = s->amp * s->pol[a];
   const int modes[4] = {MODE_FIRST, MODE_MID, MODE_MID, MODE_LAST};
-  const int mode = modes[sweep];
-  SweepParams p{};
+  t.mode = modes[sweep];
+  SweepParams &p = t.p;
   sweep_common(s, p, At, sweep);
   set_coef(p, 0.0, -0.01 / (sweep + 1));
   p.in = sweep == 0 ? s->psi : s->term[sweep - 1];
-  SweepMaps tm;
-  if (!encode_sweep_maps(s, p.in, mode, &tm, false, sweep)) return fail(TDKS_EDEVICE, "tensor map encoding failed");
-  if (mode == MODE_LAST) {
+  SweepMaps &tm = t.tm;
+  if (!encode_sweep_maps(s, p.in, t.mode, &tm, false, sweep)) return fail(TDKS_EDEVICE, "tensor map encoding failed");
+  if (t.mode == MODE_LAST) {
     int tx = 16, ty = 8;
     ws_shape_info(kernel_shape(s, s->wshape[sweep], sweep), &tx, &ty, nullptr, nullptr);
     const void *ops[4] = {s->term[0], s->term[1], s->term[0], s->term[1]};
@@ -1050,7 +1056,7 @@ static int tune_launch(tdks_system *s, int sweep) {
   } else {
     p.out = s->term[sweep];
   }
-  return run_sweep(s, mode, p, &tm, sweep);
+  return TDKS_OK;
 }
 
 int tdks_autotune(tdks_sys s, int reps, double *ms) {
@@ -1067,7 +1073,7 @@ int tdks_autotune(tdks_sys s, int reps, double *ms) {
     cudaEventDestroy(e0);
     return fail(TDKS_EDEVICE, "cudaEventCreate");
   }
-  double best[4] = {-1.0, -1.0, -1.0, -1.0}, took[WS_SHAPES][4];
+  double best[4] = {-1.0, -1.0, -1.0, -1.0}, best_one[4] = {-1.0, -1.0, -1.0, -1.0}, took[WS_SHAPES][4];
   int pick[4] = {saved[0], saved[1], saved[2], saved[3]};
   int rc = TDKS_OK;
   for (int i = 0; i < WS_SHAPES * 4; i++) took[i / 4][i % 4] = -1.0;
@@ -1079,24 +1085,29 @@ int tdks_autotune(tdks_sys s, int reps, double *ms) {
         if (ms) ms[sh * 4 + sw] = per;
         continue;
       }
-      if ((rc = tune_launch(s, sw))) break;  // warm-up (and fills this sweep's output)
-      // one launch first: a shape that it shows to be well behind the best is timed no further
+      TuneSweep t;
+      if ((rc = tune_prepare(s, sw, t))) break;
+      auto launch = [&]() { return run_sweep(s, t.mode, t.p, &t.tm, sw); };
+      if ((rc = launch())) break;  // warm-up (and fills this sweep's output)
+      // one launch first: a shape that it shows to be well behind is timed no further
+      bool in_full = reps == 1;
       for (int part = 0; part < 2 && rc == TDKS_OK; part++) {
         const int n = part == 0 ? 1 : reps;
-        if (part == 1 && (reps == 1 || (best[sw] >= 0.0 && per > 1.15 * best[sw]))) break;
+        if (part == 1 && (reps == 1 || !(in_full = tune_further(per, best_one[sw])))) break;
+        if (part == 1 && (best_one[sw] < 0.0 || per < best_one[sw])) best_one[sw] = per;
         cudaEventRecord(e0, s->stream);
-        for (int r = 0; r < n && rc == TDKS_OK; r++) rc = tune_launch(s, sw);
+        for (int r = 0; r < n && rc == TDKS_OK; r++) rc = launch();
         cudaEventRecord(e1, s->stream);
         if (rc) break;
         if (cudaEventSynchronize(e1) != cudaSuccess) { rc = fail(TDKS_EDEVICE, "autotune timing"); break; }
         if ((rc = check_err(s))) break;
-        float t = 0.f;
-        cudaEventElapsedTime(&t, e0, e1);
-        per = (double)t / n;
+        float ms_n = 0.f;
+        cudaEventElapsedTime(&ms_n, e0, e1);
+        per = (double)ms_n / n;
       }
       if (rc) break;
       if (ms) ms[sh * 4 + sw] = per;
-      if (best[sw] < 0.0 || per < best[sw]) { best[sw] = per; pick[sw] = sh; }
+      if (in_full && (best[sw] < 0.0 || per < best[sw])) { best[sw] = per; pick[sw] = sh; }
     }
   }
   cudaEventDestroy(e0);

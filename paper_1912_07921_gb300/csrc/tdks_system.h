@@ -176,6 +176,12 @@ int hartree_setup(tdks_system *s);
 int hartree_solve(tdks_system *s);
 void hartree_free(tdks_system *s);
 int check_err(tdks_system *s);
+// The autotuners' rule: whether a shape whose first timed launch took `one` ms gets the repeats, best_one being
+// the shortest first launch of a shape so far (< 0: none).  First launches are compared with one another: alone
+// between two events a launch takes 2 to 3 us longer than among others, and events count in steps of ~2 us, so a
+// comparison with the best mean dropped every shape after the first of a sweep below ~20 us (24^3, 8 orbitals: 8.9
+// us alone, 6.3 among others).  Short sweeps are always timed in full: it costs next to nothing.
+inline bool tune_further(double one, double best_one) { return best_one < 0.0 || one < 1.15 * best_one + 0.03; }
 double kinetic_max(const tdks_system *s);
 
 }  // namespace tdks_host

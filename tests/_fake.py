@@ -29,7 +29,7 @@ def load(tmp_path):
     lib.fake_fail_launch.argtypes = [ctypes.c_long]
     lib.fake_live_blocks.restype = ctypes.c_long
     lib.fake_set_hook.argtypes = [HOOK]
-    lib.fake_host_us.argtypes = [ctypes.c_double]
+    lib.fake_times.argtypes = [ctypes.c_double, ctypes.c_double]
     return lib
 
 

@@ -4,8 +4,9 @@
 //   * fake_fail_malloc(n): the n-th cudaMalloc from now returns cudaErrorMemoryAllocation (0: none does);
 //   * fake_fail_launch(n): the n-th kernel launch from now is refused;
 //   * fake_set_hook(f): every launch calls f(kernel's mangled name, grid, block, arguments), whose result is
-//     the kernel's time in microseconds on a modelled device.  fake_host_us(x): host time per launch.  Events
-//     read the modelled device's clock: work starts when the host has enqueued it and the device is free.
+//     the kernel's time in microseconds on a modelled device.  Work starts when the host has enqueued it and
+//     the device is free; fake_times(h, e): host time per launch, and the device's time between an event and
+//     the kernel after it.  Events read the modelled device's clock.
 #include <cuda_runtime_api.h>
 #include <sys/mman.h>
 
@@ -21,7 +22,7 @@ std::map<const void *, std::string> names;
 std::mutex names_lock;
 cudaError_t last = cudaSuccess;
 long fail_at = 0, fail_launch = 0;
-double host_now = 0.0, busy_until = 0.0, host_us = 0.0;
+double host_now = 0.0, busy_until = 0.0, host_us = 0.0, event_us = 0.0;
 double (*hook)(const char *, const unsigned *, const unsigned *, void **) = nullptr;
 struct { dim3 grid, block; size_t smem; cudaStream_t s; } conf;
 cudaError_t report(cudaError_t e) {
@@ -49,7 +50,7 @@ void fake_fail_malloc(long n) { fail_at = n; }
 void fake_fail_launch(long n) { fail_launch = n; }
 long fake_live_blocks() { return (long)blocks.size(); }
 void fake_set_hook(double (*f)(const char *, const unsigned *, const unsigned *, void **)) { hook = f; }
-void fake_host_us(double us) { host_us = us; }
+void fake_times(double host, double event) { host_us = host, event_us = event; }
 
 cudaError_t cudaMalloc(void **p, size_t n) {
   *p = nullptr;
@@ -131,6 +132,7 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) {
 }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) {
   *reinterpret_cast<double *>(e) = std::max(host_now, busy_until);
+  busy_until = *reinterpret_cast<double *>(e) + event_us;
   return cudaSuccess;
 }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaStreamSynchronize(nullptr); }
