@@ -330,16 +330,24 @@ int run_sweep(tdks_system *s, int mode, SweepParams &p, const SweepMaps *tm, int
   return TDKS_OK;
 }
 
-// The entries' phases for vector potential A, built where they are not the ones at hand.
+// The entries' phases for vector potential A, built where they are not the ones at hand.  What is at hand is
+// known while the table is written by calls only: a captured call takes a table built in its own capture (a
+// replay does not know what other calls left), and once there is a graph, which may be replayed at any time,
+// every call outside builds its own.
 int entry_phases(tdks_system *s, const double A[3], const void **out) {
-  const size_t bytes = (size_t)s->n_ent * s->n_k * (s->prec == TDKS_C64 ? sizeof(float2) : sizeof(double2));
-  if (!s->d_phase) CU(cudaMalloc(&s->d_phase, bytes));
-  if (!s->phase_ok || A[0] != s->phase_A[0] || A[1] != s->phase_A[1] || A[2] != s->phase_A[2]) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  unsigned long long capture = 0;
+  if (cudaStreamGetCaptureInfo(s->stream, &st, &capture) != cudaSuccess) cudaGetLastError();
+  if (st == cudaStreamCaptureStatusNone) capture = 0;
+  else s->phase_graphs = true;
+  const bool known = s->phase_ok && s->phase_capture == capture && (capture != 0 || !s->phase_graphs);
+  if (!known || A[0] != s->phase_A[0] || A[1] != s->phase_A[1] || A[2] != s->phase_A[2]) {
     CU(launch_phase_table(s->prec, s->d_ent, s->n_ent, s->n_k, s->d_kvec, A, s->bc == TDKS_BC_BLOCH, s->d_phase,
                           s->stream));
     s->launches++;
     for (int a = 0; a < 3; a++) s->phase_A[a] = A[a];
     s->phase_ok = true;
+    s->phase_capture = capture;
   }
   *out = s->d_phase;
   return TDKS_OK;
@@ -911,6 +919,8 @@ int tdks_set_atoms_projectors(tdks_sys s, int n_atoms, const double *pos, const 
   }
   CU(cudaMemcpy(s->d_D, D, (size_t)n_atoms * 4 * sizeof(double), cudaMemcpyHostToDevice));
   if (s->bc == TDKS_BC_BLOCH) {
+    // (here, so that a first propagation can be captured; boxes have no vector potential, and no phases)
+    CU(cudaMalloc(&s->d_phase, ent.size() * s->n_k * (s->prec == TDKS_C64 ? sizeof(float2) : sizeof(double2))));
     // room for the projectors' current records after the sweep partials
     const long need = s->obs_base + (long)n_atoms * s->n_kb * s->BS;
     double *grown = nullptr;

@@ -67,10 +67,12 @@ struct tdks_system {
   float4 *d_ent_beta = nullptr;  // compact copies of the entries' FP32 beta and (cell, atom)
   int2 *d_ent_ca = nullptr;
   // projector phases e^{i (k.T + A.d)} of every entry and k-point (float2 or double2 by precision),
-  // built once per vector potential (a sub-step's Taylor terms share one)
+  // built once per vector potential (a sub-step's Taylor terms share one); the capture that built
+  // the table (0: none), and whether any capture has (entry_phases)
   void *d_phase = nullptr;
   double phase_A[3] = {0.0, 0.0, 0.0};
-  bool phase_ok = false;
+  bool phase_ok = false, phase_graphs = false;
+  unsigned long long phase_capture = 0;
   void *d_q = nullptr;
   double2 *d_qpart = nullptr;   // gather partial sums, gchunks per (atom, k-batch)
   int gchunks = 1;
