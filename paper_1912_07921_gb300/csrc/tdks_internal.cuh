@@ -326,7 +326,10 @@ int ws_kernel_shape(int shape, int M, int prec, int bloch, int nx, int ny, bool 
 // sweep is short (64^3, 24 orbitals 96 -> 82 us), shape 2 for long ones (medium molecule 0.54 -> 0.48 ms).
 // complex128 is bound by the FP64 pipe in every shape (96^3, 16 orbitals 1.513 ms with shape 0, 1.531 with 2) and
 // takes the tile that leaves fewer of its points outside the grid (cell of 30 x 36 x 32, 3 k-points, 10 orbitals:
-// 16 x 12 has 6% and 16 x 8 18% outside, 0.175 against 0.193 ms); short sweeps keep the smaller one.
+// 16 x 12 has 6% and 16 x 8 18% outside, 0.175 against 0.193 ms); short sweeps keep the smaller one.  Of both
+// orders: in cells of order 8 shape 2's kernels spill beside four service warps and shape 0's do not, and it is
+// still the faster one wherever this rule takes it (middle term, 8 orbitals, 2 k-points: 30 x 36 x 32 168 against
+// 173 us, 64 x 36 x 40 376 against 430, 60^3 854 against 927; where both fit as well, 48^3, 430 against 437).
 // A small complex64 cell also goes by the fit (first and middle term, 40^3 with 2 k-batches, 20% more of 16 x 12
 // tiles outside: 20.8 and 18.4 us with shape 0, 23.0 and 19.2 with 6; 48^3 with 1: 16.6 and 14.5, 15.6 and 14.6;
 // 36 x 30 x 32 with 2, 12.5% more outside: 18.7 and 16.3, 15.5 and 14.4).
