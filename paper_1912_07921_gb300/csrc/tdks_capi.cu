@@ -682,6 +682,13 @@ static int ensure_staging(tdks_system *s) {
   return TDKS_OK;
 }
 
+// Waits for a stream at the end of a scope: a call that fails between its copies from or to the caller's buffer
+// returns with none of them in flight.
+struct Drain {
+  cudaStream_t s;
+  ~Drain() { cudaStreamSynchronize(s); }
+};
+
 // The upload runs in chunks (point ranges of each k-point) on a copy stream; each chunk is
 // packed into the internal layout, with its density partials, on the system stream as soon
 // as it has landed, so packing overlaps the remaining copies.
@@ -702,6 +709,7 @@ int tdks_set_orbitals(tdks_sys s, const double *psi) {
     CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     s->ev_chunk.push_back(e);
   }
+  const Drain drain{s->copy_stream};
   // With two upload buffers the upload packs into the spares on their own stream, so that the
   // packing too overlaps the work enqueued before this call; the system then switches to them
   // for the work enqueued after it.  With one, it packs in place on the system's stream.
@@ -792,6 +800,7 @@ int tdks_get_orbitals(tdks_sys s, double *psi_out) {
     CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     s->ev_chunk.push_back(e);
   }
+  const Drain drain{s->copy_stream};
   int c = 0;
   for (long g0 = 0; g0 < points; g0 += len, c++) {
     const long npts = std::min(len, points - g0);

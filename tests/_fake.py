@@ -28,6 +28,7 @@ def load(tmp_path):
     lib.fake_fail_malloc.argtypes = [ctypes.c_long]
     lib.fake_fail_launch.argtypes = [ctypes.c_long]
     lib.fake_live_blocks.restype = ctypes.c_long
+    lib.fake_copies_in_flight.restype = ctypes.c_long
     lib.fake_set_hook.argtypes = [HOOK]
     lib.fake_times.argtypes = [ctypes.c_double, ctypes.c_double]
     return lib

@@ -3,6 +3,7 @@
 // do not run.  What a test needs to see or to cause:
 //   * fake_fail_malloc(n): the n-th cudaMalloc from now returns cudaErrorMemoryAllocation (0: none does);
 //   * fake_fail_launch(n): the n-th kernel launch from now is refused;
+//   * fake_copies_in_flight(): asynchronous copies on streams that have not been waited for since;
 //   * fake_set_hook(f): every launch calls f(kernel's mangled name, grid, block, arguments), whose result is
 //     the kernel's time in microseconds on a modelled device.  Work starts when the host has enqueued it and
 //     the device is free; fake_times(h, e): host time per launch, and the device's time between an event and
@@ -20,6 +21,7 @@ namespace {
 std::map<void *, size_t> blocks;  // every live allocation
 std::map<const void *, std::string> names;
 std::mutex names_lock;
+std::map<cudaStream_t, long> copies;  // enqueued since the stream was last waited for
 cudaError_t last = cudaSuccess;
 long fail_at = 0, fail_launch = 0;
 double host_now = 0.0, busy_until = 0.0, host_us = 0.0, event_us = 0.0;
@@ -49,6 +51,11 @@ extern "C" {
 void fake_fail_malloc(long n) { fail_at = n; }
 void fake_fail_launch(long n) { fail_launch = n; }
 long fake_live_blocks() { return (long)blocks.size(); }
+long fake_copies_in_flight() {
+  long n = 0;
+  for (auto &c : copies) n += c.second;
+  return n;
+}
 void fake_set_hook(double (*f)(const char *, const unsigned *, const unsigned *, void **)) { hook = f; }
 void fake_times(double host, double event) { host_us = host, event_us = event; }
 
@@ -71,7 +78,10 @@ cudaError_t cudaFree(void *p) {
   return cudaSuccess;
 }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { return copy(d, s, n); }
-cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) { return copy(d, s, n); }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t st) {
+  copies[st]++;
+  return copy(d, s, n);
+}
 cudaError_t cudaMemset(void *p, int v, size_t n) {
   if (n <= (16u << 20)) memset(p, v, n);
   return cudaSuccess;
@@ -116,7 +126,8 @@ cudaError_t cudaStreamDestroy(cudaStream_t s) {
   delete reinterpret_cast<char *>(s);
   return cudaSuccess;
 }
-cudaError_t cudaStreamSynchronize(cudaStream_t) {
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+  copies.erase(s);
   host_now = std::max(host_now, busy_until);
   return cudaSuccess;
 }
@@ -135,7 +146,10 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) {
   busy_until = *reinterpret_cast<double *>(e) + event_us;
   return cudaSuccess;
 }
-cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaStreamSynchronize(nullptr); }
+cudaError_t cudaEventSynchronize(cudaEvent_t) {
+  host_now = std::max(host_now, busy_until);
+  return cudaSuccess;
+}
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t a, cudaEvent_t b) {
   *ms = (float)((*reinterpret_cast<double *>(b) - *reinterpret_cast<double *>(a)) * 1e-3);
   return cudaSuccess;
