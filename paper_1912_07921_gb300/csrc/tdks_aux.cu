@@ -282,8 +282,8 @@ __global__ void __launch_bounds__(NL_THREADS) nl_kernel(const GatherParams p) {
 
 // Batched gather: stage 1 over every system's (atom, kb, chunk) CTAs, stage 2 over every
 // system's (atom, kb) units.  The system of a CTA (or unit) comes from a table.
-// (Bound by the latency of entry and state loads: five CTAs on an SM, at 48 registers with 60 bytes spilled outside
-// the loop, hide more of it than three at the 70 the kernel takes by itself.  complex64, 24 / 64 / 128 / 256 systems:
+// (Bound by the latency of entry and state loads: five CTAs on an SM, at 48 registers with 60 bytes of them spilled,
+// hide more of it than three at the 70 the kernel takes by itself.  complex64, 24 / 64 / 128 / 256 systems:
 // 22.8 / 59.4 / 91 / 151 us against 40 / 72 / 149 / 250; six CTAs 27 / 49 / 112 / 169.  complex128 (64 registers by
 // itself): 8 / 24 / 64 systems 73 / 146 / 316 either way.)
 template <int P>

@@ -361,7 +361,6 @@ int run_gather(tdks_system *s, const void *in, const double A[3]) {
   g.atom_begin = s->d_atom_begin; g.ent = s->d_ent; g.D = s->d_D;
   g.ent_beta = s->d_ent_beta; g.ent_ca = s->d_ent_ca;
   g.h3 = s->h * s->h * s->h;
-  g.kvec = s->d_kvec;
   for (int a = 0; a < 3; a++) g.A[a] = s->gauge == TDKS_GAUGE_VELOCITY ? A[a] : 0.0;
   g.q = s->d_q;
   g.n_chunks = s->gchunks;

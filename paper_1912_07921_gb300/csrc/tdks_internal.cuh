@@ -156,7 +156,6 @@ struct GatherParams {
   const int2 *ent_ca;         // [n_ent] (cell, atom) of each entry
   const double *D;            // [n_atoms][4]
   double h3;
-  const double *kvec;
   double A[3];
   void *q;                    // [kb][atom][4][OVC] vectors
   int n_chunks;               // CTAs per (atom, kb): each sums a contiguous share of the sphere
@@ -244,15 +243,17 @@ cudaError_t launch_sweep(int M, int prec, int mode, int bloch, int tx, int ty,
 int sweep_threads(int tx, int ty);
 size_t sweep_smem(int M, int tx, int ty);
 
-// Launchers (tdks_aux.cu).  The projector step is three kernels: the gather-dot (stages 1
-// and 2) and the non-local term at every sphere point (skipped when no point is in a sphere).
+// Launchers (tdks_aux.cu).  The projector step of a system alone is two kernels: the gather-dot (a cluster per
+// unit) and the non-local term at every sphere point (skipped when no point is in a sphere); a batch's gather
+// has a second stage as a launch of its own.
 constexpr int NL_THREADS = 256;
 cudaError_t launch_gather(int prec, int bloch, const GatherParams &p, cudaStream_t s);
-// out[k * n_ent + e] = (cos, sin) of A.d_e (+ k.T_e in a periodic cell): float2 (complex64) or double2
+// out[3 k + a] = e^{i k_a L_a} from FP32 functions (complex64 sweeps)
 cudaError_t launch_face_phase(int n_k, const double *kvec, const double L[3], double2 *out, cudaStream_t s);
+// out[k * n_ent + e] = (cos, sin) of A.d_e (+ k.T_e in a periodic cell): float2 (complex64) or double2
 cudaError_t launch_phase_table(int prec, const ProjEntry *ent, int n_ent, int n_k, const double *kvec,
                                const double A[3], int bloch, void *out, cudaStream_t s);
-// chunks per (atom, k-batch) that fill the GPU for n_atoms * n_kb units
+// chunks per (atom, k-batch) that fill the GPU for n_atoms * n_kb units; those of a system alone
 int gather_chunks(long units);
 int gather_chunks_alone(int prec, long units);
 cudaError_t launch_density(int prec, long N, int n_kb, int n_batches, const void *psi, const void *psi_lo,

@@ -288,7 +288,7 @@ static cudaError_t lockstep_by_mode(int mode, const SweepMaps &maps, const Sweep
   return cudaErrorInvalidValue;
 }
 
-// Shapes 1..4 are compiled in translation units of their own (tdks_sweep_ws*.cu).
+// Shapes 1 to 8 are compiled in translation units of their own (tdks_sweep_ws*.cu).
 extern template cudaError_t launch_ws_shape<1>(int, int, int, int, const SweepMaps &, const SweepParams &, int,
                                                  cudaStream_t);
 extern template cudaError_t launch_ws_shape<2>(int, int, int, int, const SweepMaps &, const SweepParams &, int,

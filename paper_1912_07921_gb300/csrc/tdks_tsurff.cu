@@ -99,7 +99,7 @@ constexpr int TS_WMAX = 1024;  // Volkov factors of one shared-memory tile (mome
 // bounds it, so every lane holds a pair (pairs are numbered through, orbital fastest) and the entries
 // are split over enough CTAs to fill the GPU.  The tile's factors are formed once per CTA; G is read
 // through L1 in runs of orbitals.  One CTA per momentum with a thread per orbital, as before, left
-// 112 of 128 threads idle with 16 orbitals: 48^3 box, 400 momenta, 6.3 ms per flux
+// 112 of 128 threads idle with 16 orbitals: 64^3 grid, 400 momenta, 6.3 ms per flux
 // against 1.05; the multiply-adds alone take 0.85.
 __global__ void __launch_bounds__(TS_THREADS) tsurff_flux_kernel(const TsFlux f) {
   __shared__ double2 sW[TS_WMAX];
