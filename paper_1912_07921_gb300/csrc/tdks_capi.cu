@@ -765,9 +765,9 @@ int tdks_set_upload_buffers(tdks_sys s, int n) {
   CU(cudaStreamSynchronize(s->stream));
   if (s->pack_stream) CU(cudaStreamSynchronize(s->pack_stream));
   if (n == 2) {
-    CU(cudaMalloc(&s->psi_b, s->state_bytes));
-    if (s->psi_lo) CU(cudaMalloc(&s->psi_lo_b, s->state_bytes));
-    CU(cudaMalloc((void **)&s->dens_b, (size_t)s->n_kb * s->N * sizeof(double)));
+    if (!s->psi_b) CU(cudaMalloc(&s->psi_b, s->state_bytes));
+    if (s->psi_lo && !s->psi_lo_b) CU(cudaMalloc(&s->psi_lo_b, s->state_bytes));
+    if (!s->dens_b) CU(cudaMalloc((void **)&s->dens_b, (size_t)s->n_kb * s->N * sizeof(double)));
     if (!s->pack_stream) {
       CU(cudaStreamCreateWithFlags(&s->pack_stream, cudaStreamNonBlocking));
       CU(cudaEventCreateWithFlags(&s->ev_spare_free, cudaEventDisableTiming));
@@ -1496,11 +1496,13 @@ int tdks_set_propagator(tdks_sys s, int propagator) {
   if (propagator == TDKS_PROP_RK4 && s->prec != TDKS_C128)
     return fail(TDKS_EINVAL, "RK4 runs on complex128 systems");
   CU(cudaStreamSynchronize(s->stream));
-  if (propagator != TDKS_PROP_TAYLOR4 && propagator != TDKS_PROP_RK4 && !s->vx_hist[0])
-    for (int j = 0; j < 4; j++) CU(cudaMalloc((void **)&s->vx_hist[j], (size_t)s->N * sizeof(double)));
-  if (propagator == TDKS_PROP_ETRS && !s->etrs_save) {
-    CU(cudaMalloc(&s->etrs_save, s->state_bytes));
-    if (s->psi_lo) CU(cudaMalloc(&s->etrs_save_lo, s->state_bytes));
+  // (each buffer by itself: an earlier call may have run out of memory between two of them)
+  if (propagator != TDKS_PROP_TAYLOR4 && propagator != TDKS_PROP_RK4)
+    for (int j = 0; j < 4; j++)
+      if (!s->vx_hist[j]) CU(cudaMalloc((void **)&s->vx_hist[j], (size_t)s->N * sizeof(double)));
+  if (propagator == TDKS_PROP_ETRS) {
+    if (!s->etrs_save) CU(cudaMalloc(&s->etrs_save, s->state_bytes));
+    if (s->psi_lo && !s->etrs_save_lo) CU(cudaMalloc(&s->etrs_save_lo, s->state_bytes));
   }
   s->prop = propagator;
   s->n_hist = 0;
