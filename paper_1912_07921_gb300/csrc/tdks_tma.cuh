@@ -706,8 +706,10 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
           gave_up = true;
           break;
         }
-        // (the patcher warp writes halo slots: its writes come before the copy that follows them)
-        if (BLOCH && KIND == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        // The copy writes the slot through the asynchronous proxy, the consumers read it (and the patcher warp
+        // writes it) through the generic one: across the two, only this fence orders what came before the
+        // release with the copy that follows it.
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         ld.emit_at(cu, KIND, rp.slot);
         rp.next<S>();
         issued++;
