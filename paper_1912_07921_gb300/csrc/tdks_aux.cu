@@ -772,22 +772,28 @@ __device__ __forceinline__ void lda_body(long N, int nx, int ny, int nz, double 
   }
   if (!sums) return;  // (uniform over the grid: V_eff only, no record follows)
   if constexpr (F32) {
-    // The threads' sums meet in FP64 in a fixed order: G = blockDim / 8 threads a component, each adding
-    // every G-th thread's value, then a tree: 8 sums a component and 8 threads on the FP64 pipe, where a shuffle
-    // tree in every warp has 40.  Medium molecule, a record's launch: 41.3 us (44.5 with shuffle trees in FP64
-    // and the kernel as it was then; 35.9 with sums that carry 48 bits only); 48^3, 16 orbitals: 11.4 (17.6; 10.4).
-    __shared__ double all[6][LDA_THREADS];
+    // The threads' sums meet in FP64 in a fixed order, two components at a time: G = blockDim / 8 threads a
+    // component, each adding every G-th thread's value, then a tree: 8 sums a component and 8 threads on the FP64
+    // pipe, where a shuffle tree in every warp has 40.  Medium molecule, a record's launch: 41.0 us (44.5 with
+    // shuffle trees in FP64 and the kernel as it was then; 35.9 with sums that carry 48 bits only); 48^3, 16
+    // orbitals: 11.0 (17.6; 10.4).  Launches without a record: 30.0 and 5.5; with all six components at once the
+    // compiler's point loop was slower there, 35.6 and 8.5.
+    __shared__ double all[2][LDA_THREADS];
     const int t = threadIdx.x, G = blockDim.x / 8, c = t / G, l = t % G;
 #pragma unroll
-    for (int i = 0; i < 6; i++) all[i][t] = (double)fh[i] + (double)fl[i];
-    __syncthreads();
-    double x = 0.0;
-    if (c < 6) {
+    for (int r = 0; r < 6; r += 2) {
+      if (r) __syncthreads();
+      all[0][t] = (double)fh[r] + (double)fl[r];
+      all[1][t] = (double)fh[r + 1] + (double)fl[r + 1];
+      __syncthreads();
+      double x = 0.0;
+      if (c < 2) {
 #pragma unroll
-      for (int i = 0; i < 8; i++) x += all[c][l + i * G];
+        for (int i = 0; i < 8; i++) x += all[c][l + i * G];
+      }
+      for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if (c < 2 && l == 0) lda_part[blk * 6 + r + c] = x;
     }
-    for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (c < 6 && l == 0) lda_part[blk * 6 + c] = x;
   } else {
     __shared__ double red[LDA_THREADS / 32][6];
 #pragma unroll
