@@ -105,6 +105,13 @@ __device__ __forceinline__ void tma_prefetch_map(const CUtensorMap *tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
 }
 
+// Before a thread's first use of a tensor map in global memory (not needed for maps in kernel parameters): maps
+// are read through a proxy of their own, which may still hold what an earlier table had at the address.
+__device__ __forceinline__ void tma_acquire_map(const CUtensorMap *tmap) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(tmap))
+               : "memory");
+}
+
 }  // namespace
 
 // Compile-time loop: f(integral_constant<int, 0>) ... f(integral_constant<int, N-1>).
@@ -666,6 +673,7 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
     RingPos rp;
     unsigned issued = 0;
     bool gave_up = false;
+    [[maybe_unused]] int mapped = -1;  // batch: the system whose maps this thread has acquired last
     for (unsigned seq = 0; !gave_up; seq++) {
       if constexpr (KIND == 0) {
         // (a CTA's first item is its own number, without a round trip to the counter; then every CTA
@@ -697,6 +705,17 @@ __device__ __forceinline__ void ws_sweep_body(const Src &src, unsigned int *work
       cu.ny = qp->ny;
       cu.nz = qp->nz;
       cu.wrap = qp->bloch;
+      if (BATCH && cu.sys != mapped) {
+        mapped = cu.sys;
+        const SweepMaps *mp = src.maps_of(mapped);
+        if constexpr (KIND == 0) tma_acquire_map(&mp->ctr);
+        if constexpr (KIND == 1) {
+          tma_acquire_map(&mp->in);
+          tma_acquire_map(&mp->aux);
+        }
+        if constexpr (KIND == 2)
+          for (int j = 0; j < 4; j++) tma_acquire_map(&mp->op[j]);
+      }
       const int n = loads_of<M, U>(KIND, cu.z0, z1);
       // (sending the last term's operand tiles to L2 four or eight planes ahead of their loads made it
       // 18% and 36% slower on the medium molecule: eight streams per CTA are enough for the DRAM)
