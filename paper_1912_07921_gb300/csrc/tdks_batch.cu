@@ -133,9 +133,9 @@ int reset_claims(tdks_batch *b) {
 }
 
 template <class T>
-int upload(T **dst, const std::vector<T> &v) {
+int upload(const tdks_batch *b, T **dst, const std::vector<T> &v) {
   CU(cudaMalloc((void **)dst, std::max<size_t>(1, v.size()) * sizeof(T)));
-  if (!v.empty()) CU(cudaMemcpy(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
+  if (!v.empty()) CU(to_device(*dst, v.data(), v.size() * sizeof(T), b->work));
   return TDKS_OK;
 }
 
@@ -197,16 +197,16 @@ int build_sweep_tables(tdks_batch *b, bool tune) {
   cudaFree(b->d_maps); b->d_maps = nullptr;
   int rc = TDKS_OK;
   for (int k = 0; k < 4 && !rc; k++) {
-    rc = upload(&b->d_sweep[k], sp[k]);
-    if (!rc) rc = upload(&b->d_item_begin[k], ib[k]);
+    rc = upload(b, &b->d_sweep[k], sp[k]);
+    if (!rc) rc = upload(b, &b->d_item_begin[k], ib[k]);
     b->total_items[k] = ib[k][n];
     std::vector<int> owner((size_t)ib[k][n]);
     for (int i = 0; i < n; i++)
       for (long it = ib[k][i]; it < ib[k][i + 1]; it++) owner[(size_t)it] = i;
-    if (!rc) rc = upload(&b->d_item_sys[k], owner);
+    if (!rc) rc = upload(b, &b->d_item_sys[k], owner);
   }
-  if (!rc) rc = upload(&b->d_maps, maps);
-  if (!rc && b->d_aux) CU(cudaMemcpy(b->d_aux, b->aux_h.data(), n * sizeof(BatchAux), cudaMemcpyHostToDevice));
+  if (!rc) rc = upload(b, &b->d_maps, maps);
+  if (!rc && b->d_aux) CU(to_device(b->d_aux, b->aux_h.data(), n * sizeof(BatchAux), b->work));
   if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
   if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
   return rc;
@@ -306,16 +306,22 @@ int tdks_batch_create(const tdks_sys *systems, int n, void *stream, tdks_batch_t
     a.obs_part = s->obs_part; a.ring = s->ring;  // a.n_items: set with the sweep tables
     a.ring_len = tdks_system::RING;
   }
-  int rc = build_sweep_tables(b, false);
+  // (the stream first: the tables are copied on it)
+  int rc = TDKS_OK;
+  if (cudaStreamCreateWithFlags(&b->work, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming) != cudaSuccess)
+    rc = fail(TDKS_EDEVICE, "batch stream/event creation");
+  if (!rc) rc = build_sweep_tables(b, false);
   b->total_gather = gather_begin[n];
   b->total_units = unit_begin[n];
   b->total_lda = lda_begin[n];
   b->total_nl = nl_begin[n];
-  for (int k = 0; k < 4 && !rc; k++) rc = upload(&b->d_gather[k], gp[k]);
-  if (!rc) rc = upload(&b->d_gather_begin, gather_begin);
-  if (!rc) rc = upload(&b->d_unit_begin, unit_begin);
-  if (!rc) rc = upload(&b->d_lda_begin, lda_begin);
-  if (!rc) rc = upload(&b->d_nl_begin, nl_begin);
+  for (int k = 0; k < 4 && !rc; k++) rc = upload(b, &b->d_gather[k], gp[k]);
+  if (!rc) rc = upload(b, &b->d_gather_begin, gather_begin);
+  if (!rc) rc = upload(b, &b->d_unit_begin, unit_begin);
+  if (!rc) rc = upload(b, &b->d_lda_begin, lda_begin);
+  if (!rc) rc = upload(b, &b->d_nl_begin, nl_begin);
   // the system of every CTA (or unit) of the batched projector launches
   auto owners = [&](const std::vector<long> &beg) {
     std::vector<int> o((size_t)beg[n]);
@@ -323,16 +329,12 @@ int tdks_batch_create(const tdks_sys *systems, int n, void *stream, tdks_batch_t
       for (long c = beg[i]; c < beg[i + 1]; c++) o[(size_t)c] = i;
     return o;
   };
-  if (!rc) rc = upload(&b->d_gather_sys, owners(gather_begin));
-  if (!rc) rc = upload(&b->d_unit_sys, owners(unit_begin));
-  if (!rc) rc = upload(&b->d_nl_sys, owners(nl_begin));
-  if (!rc) rc = upload(&b->d_work, std::vector<unsigned int>(1, 0u));
-  if (!rc) rc = upload(&b->d_aux, aux);
-  if (!rc) rc = upload(&b->d_clock, clk);
-  if (!rc && (cudaStreamCreateWithFlags(&b->work, cudaStreamNonBlocking) != cudaSuccess ||
-              cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming) != cudaSuccess ||
-              cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming) != cudaSuccess))
-    rc = fail(TDKS_EDEVICE, "batch stream/event creation");
+  if (!rc) rc = upload(b, &b->d_gather_sys, owners(gather_begin));
+  if (!rc) rc = upload(b, &b->d_unit_sys, owners(unit_begin));
+  if (!rc) rc = upload(b, &b->d_nl_sys, owners(nl_begin));
+  if (!rc) rc = upload(b, &b->d_work, std::vector<unsigned int>(1, 0u));
+  if (!rc) rc = upload(b, &b->d_aux, aux);
+  if (!rc) rc = upload(b, &b->d_clock, clk);
   if (rc) {
     batch_free(b);
     delete b;

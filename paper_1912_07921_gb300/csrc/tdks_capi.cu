@@ -527,7 +527,7 @@ int check_err(tdks_system *s) {
   int h = 0;
   CU(cudaMemcpy(&h, s->d_err, sizeof(int), cudaMemcpyDeviceToHost));
   if (h) {
-    CU(cudaMemset(s->d_err, 0, 2 * sizeof(int)));  // and the work counter an aborted sweep left
+    CU(cudaMemsetAsync(s->d_err, 0, 2 * sizeof(int), s->stream));  // and the work counter an aborted sweep left
     return fail(TDKS_ETIMEOUT, "a sweep kernel gave up waiting for its TMA copies");
   }
   return TDKS_OK;
@@ -616,8 +616,8 @@ int tdks_create_grid(int nx, int ny, int nz, double h, int fd_order, int bc, int
   const double L[3] = {nx * h, ny * h, nz * h};
   for (int i = 0; i < 3 * n_k; i++)
     kphase[i] = make_double2(std::cos(s->kpts[i] * L[i % 3]), std::sin(s->kpts[i] * L[i % 3]));
-  if (cudaMemcpy(s->d_kvec, s->kpts.data(), 3 * n_k * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(s->d_kphase, kphase.data(), 3 * n_k * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
+  if (to_device(s->d_kvec, s->kpts.data(), 3 * n_k * sizeof(double), s->stream) != cudaSuccess ||
+      to_device(s->d_kphase, kphase.data(), 3 * n_k * sizeof(double2), s->stream) != cudaSuccess ||
       (prec == TDKS_C64 && launch_face_phase(n_k, s->d_kvec, L, s->d_kphase + 3 * n_k, s->stream) != cudaSuccess) ||
       cudaMemsetAsync(s->vloc, 0, N * sizeof(double), s->stream) != cudaSuccess ||
       cudaMemsetAsync(s->aux, 0, N * sizeof(PointAux), s->stream) != cudaSuccess ||
@@ -628,7 +628,7 @@ int tdks_create_grid(int nx, int ny, int nz, double h, int fd_order, int bc, int
   build_tmaps(s);
   std::vector<double> wocc(n_k);
   for (int i = 0; i < n_k; i++) wocc[i] = s->kw[i] * s->occ;
-  if (cudaMemcpy(s->d_wocc, wocc.data(), n_k * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (to_device(s->d_wocc, wocc.data(), n_k * sizeof(double), s->stream) != cudaSuccess)
     return cleanup(TDKS_EDEVICE, "initial copies");
   *out = s;
   return TDKS_OK;
@@ -900,19 +900,19 @@ int tdks_set_atoms_projectors(tdks_sys s, int n_atoms, const double *pos, const 
       aux[i] = PointAux{0.0, rowptr[i], rowptr[i + 1]};
       if (rowptr[i + 1] > rowptr[i]) sp.push_back(make_int2(rowptr[i], rowptr[i + 1]));
     }
-    CU(cudaMemcpy(s->aux, aux.data(), s->N * sizeof(PointAux), cudaMemcpyHostToDevice));
+    CU(to_device(s->aux, aux.data(), s->N * sizeof(PointAux), s->stream));
     s->n_sp = (int)sp.size();
     s->n_ent = (int)ent.size();
     CU(cudaMalloc((void **)&s->d_sp, sp.size() * sizeof(int2)));
-    CU(cudaMemcpy(s->d_sp, sp.data(), sp.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    CU(to_device(s->d_sp, sp.data(), sp.size() * sizeof(int2), s->stream));
     // one 16-byte vector per (kb, entry row, v) plus a zero row per kb
     const size_t nl_bytes = (size_t)s->n_kb * (s->n_ent + 1) * OVC * 16;
     CU(cudaMalloc(&s->d_nl, nl_bytes));
-    CU(cudaMemset(s->d_nl, 0, nl_bytes));
+    CU(cudaMemsetAsync(s->d_nl, 0, nl_bytes, s->stream));
   }
-  CU(cudaMemcpy(s->d_rowent, rowent.data(), ent.size() * sizeof(int), cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(s->d_atom_begin, atom_begin.data(), (n_atoms + 1) * sizeof(int), cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(s->d_ent, ent.data(), ent.size() * sizeof(ProjEntry), cudaMemcpyHostToDevice));
+  CU(to_device(s->d_rowent, rowent.data(), ent.size() * sizeof(int), s->stream));
+  CU(to_device(s->d_atom_begin, atom_begin.data(), (n_atoms + 1) * sizeof(int), s->stream));
+  CU(to_device(s->d_ent, ent.data(), ent.size() * sizeof(ProjEntry), s->stream));
   {
     std::vector<float4> eb(ent.size());
     std::vector<int2> eca(ent.size());
@@ -922,10 +922,10 @@ int tdks_set_atoms_projectors(tdks_sys s, int n_atoms, const double *pos, const 
     }
     CU(cudaMalloc((void **)&s->d_ent_beta, ent.size() * sizeof(float4)));
     CU(cudaMalloc((void **)&s->d_ent_ca, ent.size() * sizeof(int2)));
-    CU(cudaMemcpy(s->d_ent_beta, eb.data(), ent.size() * sizeof(float4), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(s->d_ent_ca, eca.data(), ent.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    CU(to_device(s->d_ent_beta, eb.data(), ent.size() * sizeof(float4), s->stream));
+    CU(to_device(s->d_ent_ca, eca.data(), ent.size() * sizeof(int2), s->stream));
   }
-  CU(cudaMemcpy(s->d_D, D, (size_t)n_atoms * 4 * sizeof(double), cudaMemcpyHostToDevice));
+  CU(to_device(s->d_D, D, (size_t)n_atoms * 4 * sizeof(double), s->stream));
   if (s->bc == TDKS_BC_BLOCH) {
     // (here, so that a first propagation can be captured; boxes have no vector potential, and no phases)
     CU(cudaMalloc(&s->d_phase, ent.size() * s->n_k * (s->prec == TDKS_C64 ? sizeof(float2) : sizeof(double2))));

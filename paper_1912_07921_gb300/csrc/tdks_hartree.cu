@@ -457,7 +457,7 @@ static int hartree_build(tdks_system *s) {
       tw.push_back(make_double2(std::cos(ang), std::sin(ang)));
     }
   CU(cudaMalloc((void **)&s->d_htw, tw.size() * sizeof(double2)));
-  CU(cudaMemcpy(s->d_htw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice));
+  CU(to_device(s->d_htw, tw.data(), tw.size() * sizeof(double2), s->stream));
   CU(cudaMalloc((void **)&s->d_hbuf, row * s->nz * sizeof(double2)));
   CU(cudaMalloc((void **)&s->d_hkern, row * hp[2] * sizeof(double)));
   CU(cudaMalloc((void **)&s->d_vh, s->N * sizeof(double)));

@@ -25,6 +25,14 @@ int fail(int code, const std::string &msg);
     }                                                                                        \
   } while (0)
 
+// A table onto the device, there on return for the kernels of `stream`.  (A cudaMemcpy from pageable memory may
+// return with its transfer still to come on the default stream, which nothing orders before the kernels of a
+// stream created without that; and fills on a stream would not be ordered with it.)
+inline cudaError_t to_device(void *dst, const void *src, size_t bytes, cudaStream_t stream) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, stream);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(stream);
+}
+
 }  // namespace tdks_host
 
 struct tdks_system {

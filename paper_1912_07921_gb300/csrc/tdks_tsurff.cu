@@ -288,12 +288,12 @@ extern "C" int tdks_set_tsurff(tdks_sys s, const int *box, int n_p, const double
   }
   s->ts_ne = (int)ent.size();
   CU(cudaMalloc((void **)&s->d_ts_ent, ent.size() * sizeof(TsEntry)));
-  CU(cudaMemcpy(s->d_ts_ent, ent.data(), ent.size() * sizeof(TsEntry), cudaMemcpyHostToDevice));
+  CU(to_device(s->d_ts_ent, ent.data(), ent.size() * sizeof(TsEntry), s->stream));
   CU(cudaMalloc((void **)&s->d_ts_p, (size_t)n_p * 3 * sizeof(double)));
-  CU(cudaMemcpy(s->d_ts_p, p, (size_t)n_p * 3 * sizeof(double), cudaMemcpyHostToDevice));
+  CU(to_device(s->d_ts_p, p, (size_t)n_p * 3 * sizeof(double), s->stream));
   CU(cudaMalloc((void **)&s->d_ts_G, 2 * ent.size() * (size_t)s->n_orb * sizeof(double2)));
   CU(cudaMalloc((void **)&s->d_ts_b, (size_t)s->n_orb * n_p * sizeof(double2)));
-  CU(cudaMemset(s->d_ts_b, 0, (size_t)s->n_orb * n_p * sizeof(double2)));
+  CU(cudaMemsetAsync(s->d_ts_b, 0, (size_t)s->n_orb * n_p * sizeof(double2), s->stream));
   const long pairs = (long)s->n_orb * n_p;
   CU(cudaMalloc((void **)&s->d_ts_E, (size_t)n_p * (s->nx + s->ny + s->nz) * sizeof(double2)));
   CU(cudaMalloc((void **)&s->d_ts_part, (size_t)flux_splits(pairs, s->ts_ne) * pairs * sizeof(double2)));

@@ -29,13 +29,14 @@ def load(tmp_path):
     lib.fake_fail_launch.argtypes = [ctypes.c_long]
     lib.fake_live_blocks.restype = ctypes.c_long
     lib.fake_copies_in_flight.restype = ctypes.c_long
+    lib.fake_unordered_launches.restype = ctypes.c_long
     lib.fake_set_hook.argtypes = [HOOK]
     lib.fake_times.argtypes = [ctypes.c_double, ctypes.c_double]
     return lib
 
 
-def create(lib, nx, ny, nz, h=0.3, order=4, bc=0, prec=0, n_orb=1, n_k=1):
+def create(lib, nx, ny, nz, h=0.3, order=4, bc=0, prec=0, n_orb=1, n_k=1, stream=None):
     out = ctypes.c_void_p()
-    rc = lib.tdks_create_grid(nx, ny, nz, h, order, bc, prec, n_orb, n_k, None, None, None, ctypes.byref(out))
+    rc = lib.tdks_create_grid(nx, ny, nz, h, order, bc, prec, n_orb, n_k, None, None, stream, ctypes.byref(out))
     assert rc == 0, lib.tdks_last_error()
     return out

@@ -4,6 +4,8 @@
 //   * fake_fail_malloc(n): the n-th cudaMalloc from now returns cudaErrorMemoryAllocation (0: none does);
 //   * fake_fail_launch(n): the n-th kernel launch from now is refused;
 //   * fake_copies_in_flight(): asynchronous copies on streams that have not been waited for since;
+//   * fake_unordered_launches(): launches on another stream than the default one that nothing orders after the
+//     copies and fills enqueued on the default stream before (cudaMemcpy to the device, cudaMemset);
 //   * fake_set_hook(f): every launch calls f(kernel's mangled name, grid, block, arguments), whose result is
 //     the kernel's time in microseconds on a modelled device.  Work starts when the host has enqueued it and
 //     the device is free; fake_times(h, e): host time per launch, and the device's time between an event and
@@ -23,7 +25,8 @@ std::map<const void *, std::string> names;
 std::mutex names_lock;
 std::map<cudaStream_t, long> copies;  // enqueued since the stream was last waited for
 cudaError_t last = cudaSuccess;
-long fail_at = 0, fail_launch = 0;
+long fail_at = 0, fail_launch = 0, unordered = 0;
+bool default_pending = false;
 double host_now = 0.0, busy_until = 0.0, host_us = 0.0, event_us = 0.0;
 double (*hook)(const char *, const unsigned *, const unsigned *, void **) = nullptr;
 struct { dim3 grid, block; size_t smem; cudaStream_t s; } conf;
@@ -31,7 +34,8 @@ cudaError_t report(cudaError_t e) {
   if (e != cudaSuccess) last = e;
   return e;
 }
-cudaError_t launch(const void *f, dim3 g, dim3 b, void **args) {
+cudaError_t launch(const void *f, dim3 g, dim3 b, void **args, cudaStream_t s) {
+  if (s && default_pending) unordered++;
   const unsigned gg[3] = {g.x, g.y, g.z}, bb[3] = {b.x, b.y, b.z};
   if (fail_launch > 0 && --fail_launch == 0) return report(cudaErrorInvalidConfiguration);
   host_now += host_us;
@@ -56,6 +60,7 @@ long fake_copies_in_flight() {
   for (auto &c : copies) n += c.second;
   return n;
 }
+long fake_unordered_launches() { return unordered; }
 void fake_set_hook(double (*f)(const char *, const unsigned *, const unsigned *, void **)) { hook = f; }
 void fake_times(double host, double event) { host_us = host, event_us = event; }
 
@@ -77,16 +82,22 @@ cudaError_t cudaFree(void *p) {
   blocks.erase(it);
   return cudaSuccess;
 }
-cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { return copy(d, s, n); }
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind k) {
+  if (k == cudaMemcpyHostToDevice) default_pending = true;
+  return copy(d, s, n);
+}
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t st) {
   copies[st]++;
   return copy(d, s, n);
 }
-cudaError_t cudaMemset(void *p, int v, size_t n) {
+cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t) {
   if (n <= (16u << 20)) memset(p, v, n);
   return cudaSuccess;
 }
-cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t) { return cudaMemset(p, v, n); }
+cudaError_t cudaMemset(void *p, int v, size_t n) {
+  default_pending = true;
+  return cudaMemsetAsync(p, v, n, nullptr);
+}
 
 cudaError_t cudaGetLastError() {
   const cudaError_t e = last;
@@ -128,6 +139,7 @@ cudaError_t cudaStreamDestroy(cudaStream_t s) {
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
   copies.erase(s);
+  if (!s) default_pending = false;
   host_now = std::max(host_now, busy_until);
   return cudaSuccess;
 }
@@ -170,7 +182,7 @@ cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
 
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args) {
-  return launch(f, c->gridDim, c->blockDim, args);
+  return launch(f, c->gridDim, c->blockDim, args, c->stream);
 }
 unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, cudaStream_t s) {
   conf = {g, b, smem, s};
@@ -187,8 +199,8 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) {
   *k = reinterpret_cast<cudaKernel_t>(const_cast<void *>(f));
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **args, size_t, cudaStream_t) {
-  return launch(reinterpret_cast<const void *>(k), g, b, args);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **args, size_t, cudaStream_t s) {
+  return launch(reinterpret_cast<const void *>(k), g, b, args, s);
 }
 void **__cudaRegisterFatBinary(void *) {
   static void *handle;
