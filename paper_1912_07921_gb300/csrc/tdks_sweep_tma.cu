@@ -20,7 +20,7 @@
 
 namespace tdks {
 
-template <int M, int P, int MODE, int TX, int TY, int U, bool BATCH, class Src>
+template <int M, int P, int MODE, int TX, int TY, int U, class Src>
 __device__ __forceinline__ void tma_sweep_body(const Src &src) {
   typedef VT<P> T;
   typedef typename T::V V;
@@ -44,7 +44,6 @@ __device__ __forceinline__ void tma_sweep_body(const Src &src) {
   __shared__ __align__(8) uint64_t ofull[SO];
   __shared__ double red[NT / 32][4];
   __shared__ int s_abort;
-  __shared__ SweepParams s_params;  // batch: parameters of the current item's system
 
   const int tid = threadIdx.x;
   const int v = tid % OVC;
@@ -86,12 +85,6 @@ __device__ __forceinline__ void tma_sweep_body(const Src &src) {
     const SweepMaps *mp_unused;
     long local;
     src.item(item, pp, mp_unused, local);
-    if constexpr (BATCH) {
-      __syncthreads();  // everyone is done with the previous item's parameters
-      if (tid == 0) s_params = *pp;
-      __syncthreads();
-      pp = &s_params;
-    }
     const SweepParams &p = *pp;
     const int nx = p.nx, ny = p.ny;
     const long N = (long)nx * ny * p.nz;
@@ -219,14 +212,7 @@ template <int M, int P, int MODE, int TX, int TY, int U>
 __global__ void __launch_bounds__(OVC * TX * TY, 1)
 tma_sweep_kernel(const __grid_constant__ SweepMaps maps, const __grid_constant__ SweepParams p) {
   const SingleSrc src{&p, &maps};
-  tma_sweep_body<M, P, MODE, TX, TY, U, false>(src);
-}
-
-template <int M, int P, int MODE, int TX, int TY, int U>
-__global__ void __launch_bounds__(OVC * TX * TY, 1)
-tma_sweep_batch_kernel(const __grid_constant__ BatchSweepArgs a) {
-  const BatchSrc src{&a};
-  tma_sweep_body<M, P, MODE, TX, TY, U, true>(src);
+  tma_sweep_body<M, P, MODE, TX, TY, U>(src);
 }
 
 // Planes per TMA copy of a sweep mode (the z depth of its tensor-map boxes): the lockstep
