@@ -1,5 +1,5 @@
-// Warp-specialised TMA sweep, tile shape 6 (2 x 2 points per thread, complex64; see WsShape in
-// tdks_tma.cuh), compiled on its own so that the shapes build in parallel.
+// Warp-specialised TMA sweep, tile shape 6 (two y-adjacent points per thread, two planes at a time; see WsShape
+// in tdks_tma.cuh), compiled on its own so that the shapes build in parallel.
 #include "tdks_tma.cuh"
 
 namespace tdks {

@@ -366,7 +366,8 @@ struct Loader {
 // (WsWarps).  tdks_autotune times the shapes on the system's own data.
 //   5: 8-byte vectors (one complex64 value), four y-adjacent points in the registers of two.
 //   6: shape 2 at two planes an iteration: one wait and one release per ring and two planes, and two planes'
-//      loads to overlap.  Medium molecule, middle term: 0.275 -> 0.255 ms.
+//      loads to overlap.  Medium molecule, middle term: 0.275 -> 0.255 ms.  complex128, bound by the FP64 pipe,
+//      gains in the first term of order-4 cells only (60^3, 8 orbitals, 2 k-points: 446 against shape 2's 451 us).
 //   7: blocks of 2 x 2 of 16-byte vectors on 232 registers.  The fastest in cells and boxes of order 4 (64^3
 //      cell, 8 k-points, 16 orbitals: 0.184 ms, shape 6 0.206, shape 3 0.230); at order 8 its 144 queue
 //      registers leave one plane an iteration and 8 warps to hide the loads' latency: 0.272 against 0.255.
@@ -383,7 +384,7 @@ template <> struct WsShape<2> { static constexpr int U = 1, TX = 16, TY = 12, R 
 template <> struct WsShape<3> { static constexpr int U = 1, TX = 16, TY = 8, R = 1, RX = 1; };   // 16
 template <> struct WsShape<4> { static constexpr int U = 1, TX = 14, TY = 8, R = 2, RX = 1; };   //  7
 template <> struct WsShape<5> { static constexpr int U = 1, TX = 16, TY = 12, R = 4, RX = 1; };  // 12 (complex64, 8-byte vectors)
-template <> struct WsShape<6> { static constexpr int U = 2, TX = 16, TY = 12, R = 2, RX = 1; };  // 12 (complex64, terms 1-3)
+template <> struct WsShape<6> { static constexpr int U = 2, TX = 16, TY = 12, R = 2, RX = 1; };  // 12 (terms 1-3)
 template <> struct WsShape<7> { static constexpr int U = 2, TX = 16, TY = 16, R = 2, RX = 2; };  //  8 (complex64, terms 1-3)
 template <> struct WsShape<8> { static constexpr int U = 2, TX = 16, TY = 12, R = 2, RX = 2; };  // 12 (complex64, 8-byte vectors, terms 1-3)
 // planes per iteration of a shape's kernels
