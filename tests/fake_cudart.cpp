@@ -1,5 +1,5 @@
 // A CUDA runtime without a GPU, for tests of the library's host code: linked with the library's own object
-// files in place of the real runtime.  Device memory is host memory (copies above 16 MB are skipped), kernels
+// files in place of the real runtime.  Device memory is host memory (copies and fills above 1 MB are skipped), kernels
 // do not run.  What a test needs to see or to cause:
 //   * fake_fail_malloc(n): the n-th cudaMalloc from now returns cudaErrorMemoryAllocation (0: none does);
 //   * fake_fail_launch(n): the n-th kernel launch from now is refused;
@@ -44,7 +44,7 @@ cudaError_t launch(const void *f, dim3 g, dim3 b, void **args, cudaStream_t s) {
   return cudaSuccess;
 }
 cudaError_t copy(void *d, const void *s, size_t n) {
-  if (n <= (16u << 20)) memcpy(d, s, n);
+  if (n <= (1u << 20)) memcpy(d, s, n);
   return cudaSuccess;
 }
 int encode_tiled(...) { return 0; }
@@ -91,7 +91,7 @@ cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cu
   return copy(d, s, n);
 }
 cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t) {
-  if (n <= (16u << 20)) memset(p, v, n);
+  if (n <= (1u << 20)) memset(p, v, n);
   return cudaSuccess;
 }
 cudaError_t cudaMemset(void *p, int v, size_t n) {
