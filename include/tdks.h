@@ -357,8 +357,9 @@ int tdks_set_sweep_path(tdks_sys sys, int path);
  * point (shape 5: warps x 32 = 8 tx ty / rows).  Shapes 6 to 8 take two planes at a time where
  * the registers allow.  Every shape can be chosen for every system; one without a kernel for
  * a system's precision, order, boundary or term runs the kernel of another (complex128: 5, 7, 8
- * and 6 in the last term as 2; complex64: 1 as 6 or 2, 6 to 8 in the last term as 2, all but 0,
- * 3 and 4 in cells of order 8 as 0 or 3).  Until one is set or tuned, complex64 takes 6 (0 on
+ * and, in the last term and in cells of order 8, 6 as 2; complex64: 1, and in cells 2 and 5, as 6,
+ * or 2 in the last term; 6 to 8 in the last term as 2; 7 and 8 in cells of odd nx or ny as 6; all
+ * but 0, 3 and 4 in cells of order 8 as 0 or 3).  Until one is set or tuned, complex64 takes 6 (0 on
  * small grids) and 2 (3 on smaller grids) for the last term, complex128 0 or 2, whichever tile leaves
  * fewer points outside the grid.  *count (if not NULL) receives the number of shapes;
  * tx/ty/rows/warps may be NULL.  TDKS_EINVAL for a shape out of range.
@@ -371,9 +372,9 @@ int tdks_get_sweep_shape(tdks_sys sys, int sweep, int *shape);
 /* Autotuner: times every shape on each of the four Taylor-term sweeps of this system, on
  * its own grid, orbitals and projectors (in the velocity gauge with a vector potential
  * amp * pol, so that the gauge term is timed too; after one warm-up launch one launch, and
- * reps more unless that one is 15% and 0.03 ms behind the shortest such launch; CUDA events on the system's stream; shapes
- * that run one kernel are timed once), and keeps the fastest shape per sweep.  The state psi is
- * not changed; the Taylor-term buffers and the density partials are overwritten (the next
+ * reps more unless that one is 15% and 0.03 ms behind the shortest such launch; CUDA events on
+ * the system's stream; shapes that run one kernel are timed once), and keeps the fastest shape
+ * per sweep.  The state psi is not changed; the Taylor-term buffers and the density partials are overwritten (the next
  * propagation or H application rebuilds them).  ms (if not NULL) receives the mean
  * milliseconds per launch as ms[shape * 4 + sweep] (count * 4 values).  Systems that do not
  * take the warp-specialised sweep keep their settings and ms is filled with -1.
